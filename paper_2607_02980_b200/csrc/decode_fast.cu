@@ -1,5 +1,5 @@
-// Bandwidth-tuned decode kernels: bf16, d = 128, S = 64, G <= 8, one landmark per KV head, any local window of
-// up to 16 chunks (W <= 897).
+// Bandwidth-tuned decode kernels: bf16, d = 128, S = 64, G <= 8, one landmark per KV head or per query head, any local
+// window of up to 16 chunks (W <= 897).  One launch per step; the shapes decode_cluster.cu takes go there instead.
 //
 //   decode_score   streams the landmarks of every (sequence, KV head) once with 128-bit loads and
 //                  scores them against the G query heads with warp MMA (landmark rows are the A
@@ -1144,6 +1144,7 @@ size_t decode_fast_scratch_bytes(const Shape& s) {
 }
 
 int launch_decode_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
+    if (decode_cluster_supports(s)) return launch_decode_cluster(s, t, stream);
     const Plan p = make_plan(s, sm_count());
     if (t.scratch_bytes < p.total) return HILS_ERR_WORKSPACE;
     const int pairs = s.B * s.Hkv;

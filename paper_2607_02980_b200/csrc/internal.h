@@ -60,6 +60,10 @@ int launch_decode_fast(const Shape& s, const Tensors& t, cudaStream_t stream);
 bool decode_fast_supports(const Shape& s, int dtype);
 size_t decode_fast_scratch_bytes(const Shape& s);
 
+// Decode in one launch of thread-block clusters (one landmark row per KV head).
+bool decode_cluster_supports(const Shape& s);
+int launch_decode_cluster(const Shape& s, const Tensors& t, cudaStream_t stream);
+
 // Decode fast path run on the library's own static device scratch (see hils_decode_noalloc).
 int launch_decode_noalloc(const Shape& s, const Tensors& t, int32_t* device_status, cudaStream_t stream);
 size_t decode_noalloc_capacity();

@@ -1,0 +1,97 @@
+"""The one-launch decode kernel (clusters per (sequence, KV head)) against the CPU oracle at the sizes where
+it can go wrong: candidate lists around its tiles of 64, around the switch from ranking every candidate to the
+histogram, lists that agree in every score (the exact radix selection), ragged and invalid lengths, windows, every
+column packing, draft tokens apart and grouped, pages out of range."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2607_02980_b200 as hils
+from paper_2607_02980_b200 import workloads as wl
+from parity import TOL_LSE, TOL_OUT, check_decode
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.mark.parametrize("B,T,seq,K,W,G,marks", [
+    (3, 64 * 130, [64 * 17 + 1, 64 * 129, 64 * 130], 16, 1, 4, "random"),     # 17, 128 and 129 candidates
+    (2, 64 * 70, [64 * 70, 64 * 65 + 1], 64, 65, 8, "random"),                # lists a little longer than K
+    (2, 64 * 400, [64 * 400, 64 * 260 + 7], 128, 512, 2, "random"),
+    (2, 64 * 300, [64 * 300, 64 * 200], 16, 1, 4, "equal"),                   # every score ties: lowest ids
+    (2, 64 * 300, [64 * 300 - 1, 5], 20, 130, 3, "three values"),
+    (40, 64 * 150, None, 32, 1, 4, "three values"),                           # two CTAs per SM
+    (1, 64 * 150, [64 * 150], 16, 1, 1, "random"),
+    (2, 64 * 150, [64 * 150, 64 * 3], 1, 1, 5, "random"),
+])
+def test_against_the_oracle(B, T, seq, K, W, G, marks):
+    Hkv = 2 if B < 40 else 8
+    cfg = wl.HilsConfig("cluster", "decode", B, G * Hkv, Hkv, T, 128, 64, K, "bf16", 900 + K + B, n_needles=2, window=W)
+    seq = seq or [T - 211 * b for b in range(B)]
+    inp = wl.make_decode_inputs(cfg, "cpu", seq_lens=torch.tensor(seq, dtype=torch.int32))
+    if marks == "equal":
+        inp["landmarks"][:] = inp["landmarks"][:1, :1, :1].clone()
+    elif marks == "three values":
+        which = torch.randint(0, 3, (cfg.C,), generator=torch.Generator().manual_seed(3))
+        inp["landmarks"] = inp["landmarks"][:, :, which].contiguous()
+    bias = None if marks != "random" else wl.make_bias(cfg, "cpu")
+    g = {n: t.to(DEV) for n, t in inp.items()}
+    out, lse, sel = hils.hils_decode(g["q"], g["k"], g["v"], g["landmarks"], g["seq_lens"], 64, K, window=W,
+                                     bias=None if bias is None else bias.to(DEV))
+    torch.cuda.synchronize()
+    assert hils.last_launch_count() == 1
+    check_decode(cfg, inp, out, lse, sel, bias=bias, W=W)
+    if marks == "equal":
+        assert (sel.cpu() == torch.arange(K, dtype=torch.int32)).all()
+
+
+@pytest.mark.parametrize("B,M,W,Hkv", [(2, 3, 1, 4), (10, 4, 200, 8), (5, 7, 512, 8)])
+def test_draft_tokens_equal_single_calls_and_the_oracle(B, M, W, Hkv):
+    cfg = wl.HilsConfig("drafts", "decode", B, 4 * Hkv, Hkv, 64 * 80 + 3, 128, 64, 16, "bf16", 950 + M, window=W)
+    seq = [cfg.L - 331 * b for b in range(B)]
+    seq[1] = 64 * 40 + 1                                     # the tokens see different numbers of chunks
+    inp = wl.make_decode_inputs(cfg, "cpu", seq_lens=torch.tensor(seq, dtype=torch.int32))
+    q = inp["q"][:, None].float() + 0.3 * torch.randn((B, M, cfg.Hq, 128), generator=torch.Generator().manual_seed(M))
+    q = q.to(torch.bfloat16)
+    bias = wl.make_bias(cfg, "cpu")
+    g = {n: t.to(DEV) for n, t in inp.items()}
+    out, lse, sel = hils.hils_decode_multi(q.to(DEV), g["k"], g["v"], g["landmarks"], g["seq_lens"], 64, 16,
+                                           bias=bias.to(DEV), window=W)
+    torch.cuda.synchronize()
+    assert hils.last_launch_count() == 1
+    for m in range(M):
+        sl = torch.tensor([n - M + m + 1 for n in seq], dtype=torch.int32)
+        o1, l1, s1 = hils.hils_decode(q[:, m].contiguous().to(DEV), g["k"], g["v"], g["landmarks"], sl.to(DEV), 64, 16,
+                                      bias=bias.to(DEV), window=W)
+        torch.cuda.synchronize()
+        assert torch.equal(s1, sel[:, m])
+        assert (o1.float() - out[:, m].float()).abs().max() <= 1.6e-2 and (l1 - lse[:, m]).abs().max() <= 1e-4
+        ref = oracle.hils_decode(q[:, m], inp["k"], inp["v"], inp["landmarks"], bias, sl, S=64, K=16, W=W)
+        ok = np.repeat(ref["margin"] >= 1e-3, 4, axis=1)
+        assert np.abs(out[:, m].float().cpu().numpy() - ref["out"])[ok].max() <= TOL_OUT["bf16"]
+        assert np.abs(lse[:, m].cpu().numpy() - ref["lse"])[ok].max() <= TOL_LSE["bf16"]
+
+
+def test_invalid_lengths_and_pages_set_the_status_and_leave_the_rest_alone():
+    cfg = wl.HilsConfig("bad", "decode", 3, 8, 2, 64 * 40, 128, 64, 16, "bf16", 970)
+    inp = wl.make_decode_inputs(cfg, "cpu", seq_lens=torch.tensor([64 * 40, 64 * 20 + 9, 777], dtype=torch.int32))
+    g = {n: t.to(DEV) for n, t in inp.items()}
+    good = hils.hils_decode(g["q"], g["k"], g["v"], g["landmarks"], g["seq_lens"], 64, 16)
+    p = hils.make_params(B=3, Hq=8, Hkv=2, Hl=2, L=0, T_max=cfg.L, C=cfg.C, d=128, chunk_size=64, top_k=16, dtype=1)
+    ws = hils.alloc_workspace(p, True, DEV)
+    lens = g["seq_lens"].clone()
+    lens[1] = cfg.L + 1
+    out, lse, sel = hils.hils_decode(g["q"], g["k"], g["v"], g["landmarks"], lens, 64, 16, workspace=ws)
+    assert hils.poll_status(ws) == -7
+    assert (out[1] == 0).all() and (lse[1] == 0).all() and (sel[1] == -1).all()
+    for b in (0, 2):
+        assert torch.equal(out[b], good[0][b]) and torch.equal(sel[b], good[2][b])
+    from test_gpu_paged import paginate
+    kp, vp, table = paginate(inp, cfg, 3)
+    table[0, 39] = kp.shape[0]                                # the last token's own chunk of sequence 0
+    ws[:256].zero_()
+    out, lse, sel = hils.hils_decode_paged(g["q"], kp.to(DEV), vp.to(DEV), g["landmarks"], table.to(DEV), g["seq_lens"],
+                                           64, 16, workspace=ws)
+    assert hils.poll_status(ws) == -7
+    assert torch.equal(sel, good[2]) and torch.equal(out[1:], good[0][1:])
