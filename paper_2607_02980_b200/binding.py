@@ -8,6 +8,7 @@ There is no CPU or PyTorch fallback: if the shared library is missing, every cal
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 from typing import Dict, Optional, Tuple
 
@@ -132,10 +133,12 @@ def _dtype_code(t: torch.Tensor) -> int:
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()          # (the argument types make it a void pointer)
 
 
 def _check(t: torch.Tensor, name: str, shape: Tuple[int, ...], dtype, cuda: bool):
+    if t.is_cuda is cuda and t.dtype is dtype and t.shape == shape and t.is_contiguous():
+        return
     if tuple(t.shape) != tuple(shape):
         raise ValueError("%s has shape %s, expected %s" % (name, tuple(t.shape), tuple(shape)))
     if t.dtype != dtype:
@@ -148,6 +151,13 @@ def _check(t: torch.Tensor, name: str, shape: Tuple[int, ...], dtype, cuda: bool
 
 def make_params(*, B, Hq, Hkv, Hl, L, T_max, C, d, chunk_size, top_k, window=1, scale=0.0, dtype, impl="auto"):
     return HilsParams(B, Hq, Hkv, Hl, L, T_max, C, d, chunk_size, top_k, window, float(scale), dtype, _IMPL[impl])
+
+
+@functools.lru_cache(maxsize=256)
+def _params_ref(*fields):
+    """Reference to the parameter struct of one call shape (read only: the library takes it as const).  A decoding loop
+    makes the same call over and over, and filling the struct costs as much as the foreign call itself."""
+    return ctypes.byref(HilsParams(*fields))
 
 
 def workspace_bytes(params: HilsParams, is_decode: bool) -> int:
@@ -167,9 +177,18 @@ def alloc_workspace(params: HilsParams, is_decode: bool, device) -> torch.Tensor
     return ws
 
 
-def _stream_ptr(stream) -> ctypes.c_void_p:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+def _scratch(nbytes: int, where: str, device) -> torch.Tensor:
+    """Workspace of one call that did not bring its own.  Nobody can read its status word afterwards, so (unlike a
+    workspace that is kept, see alloc_workspace) it need not start at zero."""
+    if nbytes == 0:
+        raise HilsError(-2, where)
+    return torch.empty(nbytes, dtype=torch.uint8, device=device)
+
+
+def _stream_ptr(stream) -> int:
+    if stream is None:
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
 
 
 def hils_prefill(q, k, v, landmarks, chunk_size: int, top_k: int, out=None, lse=None, sel_idx=None, stream=None, *,
@@ -197,16 +216,16 @@ def hils_prefill(q, k, v, landmarks, chunk_size: int, top_k: int, out=None, lse=
     _check(out, "out", (B, Hq, L, d), dt, True)
     _check(lse, "lse", (B, Hq, L), torch.float32, True)
     _check(sel_idx, "sel_idx", (B, Hkv, L, top_k), torch.int32, True)
-    p = make_params(B=B, Hq=Hq, Hkv=Hkv, Hl=Hl, L=L, T_max=T, C=C, d=d, chunk_size=chunk_size, top_k=top_k,
-                    window=window, scale=scale, dtype=_dtype_code(q), impl=impl)
-    ws = alloc_workspace(p, False, q.device) if workspace is None else workspace
+    p = _params_ref(B, Hq, Hkv, Hl, L, T, C, d, chunk_size, top_k, window, float(scale), _dtype_code(q),
+                    _IMPL[impl])
+    ws = _scratch(lib.hils_workspace_bytes(p, 0), "hils_workspace_bytes", q.device) if workspace is None else workspace
     if q_route is not None:
         _check(q_route, "q_route", (B, Hq, L, d), dt, True)
-        rc = lib.hils_prefill_routed(ctypes.byref(p), _ptr(q), _ptr(q_route), _ptr(k), _ptr(v), _ptr(landmarks),
+        rc = lib.hils_prefill_routed(p, _ptr(q), _ptr(q_route), _ptr(k), _ptr(v), _ptr(landmarks),
                                      _ptr(bias), _ptr(out), _ptr(lse), _ptr(sel_idx), _ptr(ws), ws.numel(),
                                      _stream_ptr(stream))
     else:
-        rc = lib.hils_prefill(ctypes.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(landmarks), _ptr(bias), _ptr(out),
+        rc = lib.hils_prefill(p, _ptr(q), _ptr(k), _ptr(v), _ptr(landmarks), _ptr(bias), _ptr(out),
                               _ptr(lse), _ptr(sel_idx), _ptr(ws), ws.numel(), _stream_ptr(stream))
     if rc != 0:
         raise HilsError(rc, "hils_prefill")
@@ -237,16 +256,16 @@ def hils_decode(q, k_cache, v_cache, landmarks, seq_lens, chunk_size: int, top_k
     _check(out, "out", (B, Hq, d), dt, True)
     _check(lse, "lse", (B, Hq), torch.float32, True)
     _check(sel_idx, "sel_idx", (B, Hkv, top_k), torch.int32, True)
-    p = make_params(B=B, Hq=Hq, Hkv=Hkv, Hl=Hl, L=0, T_max=T, C=C, d=d, chunk_size=chunk_size, top_k=top_k,
-                    window=window, scale=scale, dtype=_dtype_code(q), impl=impl)
-    ws = alloc_workspace(p, True, q.device) if workspace is None else workspace
+    p = _params_ref(B, Hq, Hkv, Hl, 0, T, C, d, chunk_size, top_k, window, float(scale), _dtype_code(q),
+                    _IMPL[impl])
+    ws = _scratch(lib.hils_workspace_bytes(p, 1), "hils_workspace_bytes", q.device) if workspace is None else workspace
     if q_route is not None:
         _check(q_route, "q_route", tuple(q.shape), q.dtype, True)
-        rc = lib.hils_decode_routed(ctypes.byref(p), _ptr(q), _ptr(q_route), _ptr(k_cache), _ptr(v_cache), _ptr(landmarks),
+        rc = lib.hils_decode_routed(p, _ptr(q), _ptr(q_route), _ptr(k_cache), _ptr(v_cache), _ptr(landmarks),
                                     _ptr(bias), _ptr(seq_lens), _ptr(out), _ptr(lse), _ptr(sel_idx), _ptr(ws), ws.numel(),
                                     _stream_ptr(stream))
     else:
-        rc = lib.hils_decode(ctypes.byref(p), _ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(landmarks), _ptr(bias),
+        rc = lib.hils_decode(p, _ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(landmarks), _ptr(bias),
                              _ptr(seq_lens), _ptr(out), _ptr(lse), _ptr(sel_idx), _ptr(ws), ws.numel(),
                              _stream_ptr(stream))
     if rc != 0:
@@ -281,9 +300,9 @@ def hils_decode_noalloc(q, k_cache, v_cache, landmarks, seq_lens, chunk_size: in
     _check(sel_idx, "sel_idx", (B, Hkv, top_k), torch.int32, True)
     if device_status is not None:
         _check(device_status, "device_status", (1,), torch.int32, True)
-    p = make_params(B=B, Hq=Hq, Hkv=Hkv, Hl=Hl, L=0, T_max=T, C=C, d=d, chunk_size=chunk_size, top_k=top_k,
-                    window=1, scale=scale, dtype=_dtype_code(q), impl="auto")
-    rc = lib.hils_decode_noalloc(ctypes.byref(p), _ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(landmarks),
+    p = _params_ref(B, Hq, Hkv, Hl, 0, T, C, d, chunk_size, top_k, 1, float(scale), _dtype_code(q),
+                    _IMPL["auto"])
+    rc = lib.hils_decode_noalloc(p, _ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(landmarks),
                                  _ptr(bias), _ptr(seq_lens), _ptr(out), _ptr(lse), _ptr(sel_idx),
                                  _ptr(device_status), _stream_ptr(stream))
     if rc != 0:
@@ -307,19 +326,16 @@ def hils_prefill_at(q, k, v, landmarks, chunk_size: int, top_k: int, pos0: int, 
     _check(landmarks, "landmarks", (B, Hl, C, d), dt, True)
     if bias is not None:
         _check(bias, "bias", (B, Hl, C), torch.float32, True)
-    p = make_params(B=B, Hq=Hq, Hkv=Hkv, Hl=Hl, L=L, T_max=T, C=C, d=d, chunk_size=chunk_size, top_k=top_k,
-                    window=window, scale=scale, dtype=_dtype_code(q), impl=impl)
-    nbytes = int(lib.hils_prefill_at_workspace_bytes(ctypes.byref(p), int(pos0)))
+    p = _params_ref(B, Hq, Hkv, Hl, L, T, C, d, chunk_size, top_k, window, float(scale), _dtype_code(q),
+                    _IMPL[impl])
+    nbytes = int(lib.hils_prefill_at_workspace_bytes(p, int(pos0)))
     if nbytes == 0:
         raise HilsError(-2, "hils_prefill_at_workspace_bytes")
-    if workspace is None:
-        workspace = torch.empty(nbytes, dtype=torch.uint8, device=q.device)
-        workspace[:256].zero_()                   # only the status block has to start at zero
-    ws = workspace
+    ws = _scratch(nbytes, "hils_prefill_at_workspace_bytes", q.device) if workspace is None else workspace
     out = torch.empty((B, Hq, L, d), dtype=dt, device=q.device) if out is None else out
     lse = torch.empty((B, Hq, L), dtype=torch.float32, device=q.device) if lse is None else lse
     sel_idx = torch.empty((B, Hkv, L, top_k), dtype=torch.int32, device=q.device) if sel_idx is None else sel_idx
-    rc = lib.hils_prefill_at(ctypes.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(landmarks), _ptr(bias), int(pos0),
+    rc = lib.hils_prefill_at(p, _ptr(q), _ptr(k), _ptr(v), _ptr(landmarks), _ptr(bias), int(pos0),
                              _ptr(out), _ptr(lse), _ptr(sel_idx), _ptr(ws), nbytes, _stream_ptr(stream))
     if rc != 0:
         raise HilsError(rc, "hils_prefill_at")
@@ -343,13 +359,13 @@ def hils_decode_paged(q, k_pages, v_pages, landmarks, block_table, seq_lens, chu
     _check(seq_lens, "seq_lens", (B,), torch.int32, True)
     if bias is not None:
         _check(bias, "bias", (B, Hl, C), torch.float32, True)
-    p = make_params(B=B, Hq=Hq, Hkv=Hkv, Hl=Hl, L=0, T_max=C * chunk_size, C=C, d=d, chunk_size=chunk_size,
-                    top_k=top_k, window=window, scale=scale, dtype=_dtype_code(q), impl="auto")
-    ws = alloc_workspace(p, True, q.device) if workspace is None else workspace
+    p = _params_ref(B, Hq, Hkv, Hl, 0, C * chunk_size, C, d, chunk_size, top_k, window, float(scale),
+                    _dtype_code(q), _IMPL["auto"])
+    ws = _scratch(lib.hils_workspace_bytes(p, 1), "hils_workspace_bytes", q.device) if workspace is None else workspace
     out = torch.empty((B, Hq, d), dtype=dt, device=q.device) if out is None else out
     lse = torch.empty((B, Hq), dtype=torch.float32, device=q.device) if lse is None else lse
     sel_idx = torch.empty((B, Hkv, top_k), dtype=torch.int32, device=q.device) if sel_idx is None else sel_idx
-    rc = lib.hils_decode_paged(ctypes.byref(p), _ptr(q), _ptr(k_pages), _ptr(v_pages), _ptr(landmarks), _ptr(bias),
+    rc = lib.hils_decode_paged(p, _ptr(q), _ptr(k_pages), _ptr(v_pages), _ptr(landmarks), _ptr(bias),
                                _ptr(block_table), int(P), _ptr(seq_lens), _ptr(out), _ptr(lse), _ptr(sel_idx),
                                _ptr(ws), ws.numel() * ws.element_size(), _stream_ptr(stream))
     if rc != 0:
@@ -379,9 +395,8 @@ def hils_landmark_summary(landmark_queries, k, chunk_size: int, *, seq_lens=None
         bias = torch.zeros((B, Hl, C), dtype=torch.float32, device=k.device)
     _check(landmarks, "landmarks", (B, Hl, C, d), dt, True)
     _check(bias, "bias", (B, Hl, C), torch.float32, True)
-    p = make_params(B=B, Hq=Hl, Hkv=Hkv, Hl=Hl, L=0, T_max=T, C=C, d=d, chunk_size=chunk_size, top_k=1,
-                    window=1, scale=scale, dtype=_dtype_code(k), impl="auto")
-    rc = lib.hils_landmark_summary(ctypes.byref(p), _ptr(landmark_queries), _ptr(k), _ptr(seq_lens),
+    p = _params_ref(B, Hl, Hkv, Hl, 0, T, C, d, chunk_size, 1, 1, float(scale), _dtype_code(k), _IMPL["auto"])
+    rc = lib.hils_landmark_summary(p, _ptr(landmark_queries), _ptr(k), _ptr(seq_lens),
                                    int(chunk_begin), int(chunk_count), _ptr(landmarks), _ptr(bias), _stream_ptr(stream))
     if rc != 0:
         raise HilsError(rc, "hils_landmark_summary")
@@ -416,15 +431,11 @@ def hils_prefill_backward(q, k, v, landmarks, chunk_size: int, top_k: int, out, 
     dv = torch.empty((B, Hkv, T, d), **f32)
     dlm = torch.empty((B, Hl, C, d), **f32)
     dbias = torch.empty((B, Hl, C), **f32) if bias is not None else None
-    p = make_params(B=B, Hq=Hq, Hkv=Hkv, Hl=Hl, L=L, T_max=T, C=C, d=d, chunk_size=chunk_size, top_k=top_k,
-                    window=window, scale=scale, dtype=_dtype_code(q), impl=impl)
+    p = _params_ref(B, Hq, Hkv, Hl, L, T, C, d, chunk_size, top_k, window, float(scale), _dtype_code(q),
+                    _IMPL[impl])
     if workspace is None:
-        n = int(lib.hils_prefill_backward_workspace_bytes(ctypes.byref(p)))
-        if n == 0:
-            raise HilsError(-2, "hils_prefill_backward_workspace_bytes")
-        workspace = torch.empty(n, dtype=torch.uint8, device=q.device)
-        workspace[:256].zero_()
-    rc = lib.hils_prefill_backward(ctypes.byref(p), _ptr(q), _ptr(k), _ptr(v), _ptr(landmarks), _ptr(bias), _ptr(out),
+        workspace = _scratch(lib.hils_prefill_backward_workspace_bytes(p), "hils_prefill_backward_workspace_bytes", q.device)
+    rc = lib.hils_prefill_backward(p, _ptr(q), _ptr(k), _ptr(v), _ptr(landmarks), _ptr(bias), _ptr(out),
                                    _ptr(lse), _ptr(sel_idx), _ptr(dout), _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dlm),
                                    _ptr(dbias), _ptr(workspace), workspace.numel(), _stream_ptr(stream))
     if rc != 0:
@@ -480,9 +491,8 @@ def hils_chunk_overlap(sel_idx, block_queries: int, num_chunks: int, *, stats=No
         overlap = torch.empty((B, Hkv, nblk), dtype=torch.float32, device=sel_idx.device)
     _check(stats, "stats", (B, Hkv, nblk, 4), torch.int32, True)
     _check(overlap, "overlap", (B, Hkv, nblk), torch.float32, True)
-    p = make_params(B=B, Hq=Hkv, Hkv=Hkv, Hl=Hkv, L=L, T_max=0, C=int(num_chunks), d=1, chunk_size=1, top_k=K,
-                    window=1, scale=0.0, dtype=0, impl="auto")
-    rc = lib.hils_chunk_overlap(ctypes.byref(p), _ptr(sel_idx), int(block_queries), _ptr(stats), _ptr(overlap),
+    p = _params_ref(B, Hkv, Hkv, Hkv, L, 0, int(num_chunks), 1, 1, K, 1, 0.0, 0, _IMPL["auto"])
+    rc = lib.hils_chunk_overlap(p, _ptr(sel_idx), int(block_queries), _ptr(stats), _ptr(overlap),
                                 _stream_ptr(stream))
     if rc != 0:
         raise HilsError(rc, "hils_chunk_overlap")
@@ -522,15 +532,11 @@ def hils_decode_multi(q, k_cache, v_cache, landmarks, seq_lens, chunk_size: int,
     _check(out, "out", (B, M, Hq, d), dt, True)
     _check(lse, "lse", (B, M, Hq), torch.float32, True)
     _check(sel_idx, "sel_idx", (B, M, Hkv, top_k), torch.int32, True)
-    p = make_params(B=B, Hq=Hq, Hkv=Hkv, Hl=Hl, L=0, T_max=T, C=C, d=d, chunk_size=chunk_size, top_k=top_k,
-                    window=window, scale=scale, dtype=_dtype_code(q), impl="auto")
+    p = _params_ref(B, Hq, Hkv, Hl, 0, T, C, d, chunk_size, top_k, window, float(scale), _dtype_code(q),
+                    _IMPL["auto"])
     if workspace is None:
-        n = int(lib.hils_decode_multi_workspace_bytes(ctypes.byref(p), int(M)))
-        if n == 0:
-            raise HilsError(-2, "hils_decode_multi_workspace_bytes")
-        workspace = torch.empty(n, dtype=torch.uint8, device=q.device)
-        workspace[:256].zero_()
-    rc = lib.hils_decode_multi(ctypes.byref(p), int(M), _ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(landmarks),
+        workspace = _scratch(lib.hils_decode_multi_workspace_bytes(p, int(M)), "hils_decode_multi_workspace_bytes", q.device)
+    rc = lib.hils_decode_multi(p, int(M), _ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(landmarks),
                                _ptr(bias), _ptr(block_table), int(num_pages), _ptr(seq_lens), _ptr(out), _ptr(lse),
                                _ptr(sel_idx), _ptr(workspace), workspace.numel(), _stream_ptr(stream))
     if rc != 0:
