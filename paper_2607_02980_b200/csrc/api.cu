@@ -116,10 +116,11 @@ int pick_path(const Shape& s, const hils_params* p, Path* path) {
     return HILS_OK;
 }
 
-size_t scratch_bytes(const Shape& s, Path path) {
+size_t scratch_bytes(const Shape& s, Path path, int dtype) {
     switch (path) {
         case Path::DecodeFast: return decode_fast_scratch_bytes(s);
         case Path::PrefillFast: return prefill_fast_scratch_bytes(s);
+        case Path::Generic: return generic_scratch_bytes(s, dtype);
         default: return 0;
     }
 }
@@ -153,7 +154,7 @@ int run(const hils_params* p, int is_decode, const void* q, const void* k, const
         if (num_pages < 1 || static_cast<long long>(num_pages) * s.Hkv * s.S >= (1ll << 31)) return HILS_ERR_INVALID_ARG;
         if (reinterpret_cast<uintptr_t>(block_table) & 3u) return HILS_ERR_ALIGNMENT;
     }
-    const size_t need = kStatusBytes + scratch_bytes(s, path);
+    const size_t need = kStatusBytes + scratch_bytes(s, path, p->dtype);
     if (!ws || ws_bytes < need) return HILS_ERR_WORKSPACE;
     if (!aligned16(ws)) return HILS_ERR_ALIGNMENT;
     Tensors t{q, k, v, lm, bias, seq_lens, out, lse, sel, static_cast<int*>(ws),
@@ -396,7 +397,7 @@ size_t hils_workspace_bytes(const hils_params* params, int is_decode) {
     if (make_shape(params, is_decode, &s) != HILS_OK) return 0;
     Path path;
     if (pick_path(s, params, &path) != HILS_OK) return 0;
-    return kStatusBytes + align_up(scratch_bytes(s, path), 256);
+    return kStatusBytes + align_up(scratch_bytes(s, path, params->dtype), 256);
 }
 
 int hils_prefill(const hils_params* params, const void* q, const void* k, const void* v, const void* landmarks,
@@ -441,7 +442,7 @@ size_t hils_prefill_at_workspace_bytes(const hils_params* params, int64_t pos0) 
     if (make_shape(params, 0, &s, pos0) != HILS_OK) return 0;
     Path path;
     if (pick_path(s, params, &path) != HILS_OK) return 0;
-    return kStatusBytes + align_up(scratch_bytes(s, path), 256);
+    return kStatusBytes + align_up(scratch_bytes(s, path, params->dtype), 256);
 }
 
 int hils_decode_paged(const hils_params* params, const void* q, const void* k_pages, const void* v_pages,

@@ -1,9 +1,14 @@
-// Shape-agnostic HiLS kernels on CUDA cores: one warp per (sequence, KV group, query row) for
-// scoring + top-K selection, one warp per (sequence, query head, query row) for attention.
-// They cover fp32 and bf16, any head dim that is a multiple of 32 (<= 256), any chunk size and
-// any local window, prefill and decode.  They are the correctness anchor and the fall-back for
-// shapes the tensor-core / bandwidth-tuned kernels do not take.
+// Shape-agnostic HiLS kernels on CUDA cores: one warp per (sequence, KV group, query row) for scoring + top-K
+// selection, one CTA per (sequence, query head, query row) for attention, its warps sharing the row's chunks.
+// They cover fp32 and bf16, any head dim that is a multiple of 32 (<= 256), any chunk size and any local window,
+// prefill and decode.  They are the correctness anchor and the fall-back for shapes the tensor-core /
+// bandwidth-tuned kernels do not take.
+// Bound: the load path.  Every row reads its own K and V rows through L1, so a warp request has to cover whole
+// 64-byte runs: four lanes share a key (16-byte pieces, the quad's sum by two shuffles, the query in registers), where a
+// lane per key touched 32 lines per request; and a warp takes one chunk, where one warp walked all of a row's chunks.
+// fp32, 2048 tokens, d = 64, K = 4: 82 -> 38 us (attention by rows), 16 -> 10 us (selection).
 #include "internal.h"
+#include "tma.cuh"
 
 namespace hils {
 namespace {
@@ -33,6 +38,75 @@ __device__ inline int row_position(const GArgs& a, int b, int r) {
     return n - 1;
 }
 
+// One 16-byte piece of a row, widened.
+template <typename T> struct Piece;
+template <> struct Piece<float> {
+    static constexpr int kElems = 4;
+    __device__ static void load(const float* p, float (&x)[4]) {
+        const float4 a = *reinterpret_cast<const float4*>(p);
+        x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
+    }
+};
+template <> struct Piece<__nv_bfloat16> {
+    static constexpr int kElems = 8;
+    __device__ static void load(const __nv_bfloat16* p, float (&x)[8]) { load8(p, x); }
+};
+
+// A quad of lanes shares a row of D elements at most: lane j of the quad owns the 16-byte pieces j, j + 4, ..., npl of
+// them.  X: the head dimension is D itself (offsets inside a row are constants).
+template <typename T, int D, bool X>
+struct Quad {
+    static constexpr int kE = Piece<T>::kElems, kPl = D / kE / 4;
+    float x[kPl][kE];
+
+    __device__ __forceinline__ static int dim(int d) { return X ? D : d; }
+    // row: this lane's first piece
+    __device__ __forceinline__ void load(const T* row, int d) {
+#pragma unroll
+        for (int i = 0; i < kPl; ++i) {
+            if (X || i < d / (4 * kE)) {
+                Piece<T>::load(row + 4 * kE * i, x[i]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < kE; ++e) x[i][e] = 0.f;
+            }
+        }
+    }
+    __device__ __forceinline__ void fill(float v) {
+#pragma unroll
+        for (int i = 0; i < kPl; ++i)
+#pragma unroll
+            for (int e = 0; e < kE; ++e) x[i][e] = v;
+    }
+    // dot product over the quad (the sum in all four lanes)
+    __device__ __forceinline__ float dot(const Quad& o) const {
+        float a0 = 0.f, a1 = 0.f;
+#pragma unroll
+        for (int i = 0; i < kPl; ++i)
+#pragma unroll
+            for (int e = 0; e < kE; e += 2) {
+                a0 = fmaf(x[i][e], o.x[i][e], a0);
+                a1 = fmaf(x[i][e + 1], o.x[i][e + 1], a1);
+            }
+        a0 += a1;
+        a0 += __shfl_xor_sync(kFullMask, a0, 1);
+        a0 += __shfl_xor_sync(kFullMask, a0, 2);
+        return a0;
+    }
+    __device__ __forceinline__ void scale_by(float f) {
+#pragma unroll
+        for (int i = 0; i < kPl; ++i)
+#pragma unroll
+            for (int e = 0; e < kE; ++e) x[i][e] *= f;
+    }
+    __device__ __forceinline__ void add_scaled(float f, const Quad& o) {
+#pragma unroll
+        for (int i = 0; i < kPl; ++i)
+#pragma unroll
+            for (int e = 0; e < kE; ++e) x[i][e] = fmaf(f, o.x[i][e], x[i][e]);
+    }
+};
+
 // Insert key x into the descending list held as lst[j] of lane l <-> index j*32+l, keeping K entries.
 template <int NR>
 __device__ inline void list_insert(unsigned long long (&lst)[NR], unsigned long long x, int K, int lane) {
@@ -51,13 +125,47 @@ __device__ inline void list_insert(unsigned long long (&lst)[NR], unsigned long 
         lst[j] = nv;
     }
 }
+// Merges 32 keys (one per lane, any order) into the list: sorted across the warp, the larger of each list entry and
+// its mirror image taken, the bitonic result merged.
+template <int NR>
+__device__ inline void list_merge(unsigned long long (&lst)[NR], unsigned long long x, int K, int lane) {
+#pragma unroll
+    for (int k = 2; k <= 32; k <<= 1)
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            const unsigned long long o = __shfl_xor_sync(kFullMask, x, j);
+            const bool upper = (lane & j) != 0, desc = (lane & k) == 0;
+            x = (upper != desc) == (x > o) ? x : o;
+        }
+    const unsigned long long rev = __shfl_xor_sync(kFullMask, x, 31);
+    lst[NR - 1] = lst[NR - 1] > rev ? lst[NR - 1] : rev;
+#pragma unroll
+    for (int h = NR >> 1; h > 0; h >>= 1)
+#pragma unroll
+        for (int i = 0; i < NR; ++i)
+            if ((i & h) == 0) {
+                const unsigned long long a = lst[i], b = lst[i + h];
+                lst[i] = a > b ? a : b;
+                lst[i + h] = a > b ? b : a;
+            }
+#pragma unroll
+    for (int j = 16; j > 0; j >>= 1)
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            const unsigned long long o = __shfl_xor_sync(kFullMask, lst[i], j);
+            const bool upper = (lane & j) != 0;
+            lst[i] = upper == (lst[i] < o) ? lst[i] : o;
+        }
+#pragma unroll
+    for (int i = 0; i < NR; ++i)
+        if (i * 32 + lane >= K) lst[i] = 0ull;
+}
 
 // Scoring (Eq. surrogate top-k, per head), group max (App. C) and exact top-K with ties to the
-// lower chunk id.  One warp per (b, g, r); lane l scores chunk base+l.
-template <typename T, int NR>
+// lower chunk id.  One warp per (b, g, r), 32 chunks at a time.
+template <typename T, int D, bool X, int NR>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 generic_select_kernel(const GArgs a) {
-    extern __shared__ float smem[];
     const Shape& s = a.s;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const long long w = static_cast<long long>(blockIdx.x) * kWarpsPerBlock + wib;
@@ -74,44 +182,52 @@ generic_select_kernel(const GArgs a) {
         return;
     }
     const int ncand = local_lo(pos, s.W, s.S) / s.S;
-    const int d = s.d, G = s.G;
-    float* sq = smem + static_cast<size_t>(wib) * G * d;        // [G][d] queries of the group
-    const T* q = static_cast<const T*>(a.q_route);       // selection scores use the routing query
-    for (int x = lane; x < G * d; x += 32) {
-        const int rr = x / d, t = x % d;
-        sq[x] = to_f32(q[((static_cast<long long>(b) * s.Hq + g * G + rr) * s.R + r) * d + t]);
+    if (ncand <= s.K) {                       // nothing to choose
+        for (int t = lane; t < s.K; t += 32) sel[t] = t < ncand ? t : -1;
+        return;
     }
-    __syncwarp();
+    const int d = Quad<T, D, X>::dim(s.d), G = s.G, k8 = lane >> 2, at = (lane & 3) * Quad<T, D, X>::kE;
+    const T* q = static_cast<const T*>(a.q_route);       // selection scores use the routing query
+    const T* lm = static_cast<const T*>(a.lm);
 
     unsigned long long lst[NR];
 #pragma unroll
     for (int j = 0; j < NR; ++j) lst[j] = 0ull;
     unsigned long long thr = 0ull;
-    const T* lm = static_cast<const T*>(a.lm);
-
     for (int base = 0; base < ncand; base += 32) {
-        const int c = base + lane;
-        unsigned long long key = 0ull;
-        if (c < ncand) {
-            float u = -INFINITY;
-            for (int rr = 0; rr < G; ++rr) {
-                const int hl = (s.Hl == s.Hq) ? (g * G + rr) : g;
-                const T* row = lm + ((static_cast<long long>(b) * s.Hl + hl) * s.C + c) * d;
-                const float* qv = sq + rr * d;
-                float acc = 0.f;
-                for (int t = 0; t < d; t += 8) {
-                    float x[8];
-                    load8(row + t, x);
+        float u[4];                            // octet o: chunk base + 8 o + k8 (the same value in the quad's lanes)
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) acc = fmaf(x[e], qv[t + e], acc);
-                }
-                float sc = acc * s.scale;
-                if (a.bias) sc += a.bias[(static_cast<long long>(b) * s.Hl + hl) * s.C + c];
-                u = fmaxf(u, sc);
+        for (int o = 0; o < 4; ++o) u[o] = -INFINITY;
+        for (int rr = 0; rr < G; ++rr) {
+            Quad<T, D, X> qr;
+            qr.load(q + ((static_cast<long long>(b) * s.Hq + g * G + rr) * s.R + r) * d + at, d);
+            const int hl = (s.Hl == s.Hq) ? (g * G + rr) : g;
+            const long long lrow = (static_cast<long long>(b) * s.Hl + hl) * s.C;
+#pragma unroll
+            for (int o = 0; o < 4; ++o) {
+                if (base + o * 8 >= ncand) break;
+                const int c = min(base + o * 8 + k8, ncand - 1);
+                Quad<T, D, X> x;
+                x.load(lm + (lrow + c) * d + at, d);
+                float sc = x.dot(qr) * s.scale;
+                if (a.bias) sc += a.bias[lrow + c];
+                u[o] = fmaxf(u[o], sc);
             }
-            key = select_key(u, c);
         }
+        // lane l: chunk base + l
+        float mine = -INFINITY;
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+            const float v = __shfl_sync(kFullMask, u[o], (lane & 7) * 4);
+            if ((lane >> 3) == o) mine = v;
+        }
+        const unsigned long long key = base + lane < ncand ? select_key(mine, base + lane) : 0ull;
         unsigned pass = __ballot_sync(kFullMask, key > thr);
+        if (__popc(pass) > 4) {
+            list_merge<NR>(lst, key, s.K, lane);
+            thr = __shfl_sync(kFullMask, lst[(s.K - 1) >> 5], (s.K - 1) & 31);
+            pass = 0u;
+        }
         while (pass) {
             const int src = __ffs(pass) - 1;
             pass &= pass - 1;
@@ -123,165 +239,470 @@ generic_select_kernel(const GArgs a) {
         }
     }
 
-    // emit ascending chunk ids: rank of an id = number of selected ids below it
-    const int n = ncand < s.K ? ncand : s.K;
+    // emit ascending chunk ids: rank of an id = number of selected ids below it (all K places are taken)
 #pragma unroll
     for (int j = 0; j < NR; ++j) {
-        const int idx = j * 32 + lane;
-        const int mine = (idx < n) ? key_chunk(lst[j]) : 0x7fffffff;
+        const int mine = key_chunk(lst[j]);
         int rank = 0;
 #pragma unroll
         for (int j2 = 0; j2 < NR; ++j2) {
-            for (int l = 0; l < 32; ++l) {
-                const unsigned long long o = __shfl_sync(kFullMask, lst[j2], l);
-                const int oi = (j2 * 32 + l < n) ? key_chunk(o) : 0x7fffffff;
-                rank += (oi < mine) ? 1 : 0;
-            }
+            const int ids = key_chunk(lst[j2]);
+            for (int l = 0; l < min(32, s.K - j2 * 32); ++l) rank += __shfl_sync(kFullMask, ids, l) < mine ? 1 : 0;
         }
-        if (idx < n) sel[rank] = mine;
-    }
-    for (int t = n + lane; t < s.K; t += 32) sel[t] = -1;
-}
-
-// Softmax attention of the warp's query (in shared memory) over rows [lo, hi) of one KV head,
-// 32 keys at a time with a running max.  Returns m and Z; acc holds sum exp(s - m) * v.
-// Lane l owns output elements e*32 + l.
-template <typename T, int NE>
-__device__ inline void attend_span(const float* sq, const T* kbase, const T* vbase, int lo, int hi, int d,
-                                   float scale, int lane, float& m, float& Z, float (&acc)[NE]) {
-    m = -INFINITY;
-    Z = 0.f;
-#pragma unroll
-    for (int e = 0; e < NE; ++e) acc[e] = 0.f;
-    for (int base = lo; base < hi; base += 32) {
-        const int j = base + lane;
-        float sc = -INFINITY;
-        if (j < hi) {
-            const T* row = kbase + static_cast<long long>(j) * d;
-            float a0 = 0.f;
-            for (int t = 0; t < d; t += 8) {
-                float x[8];
-                load8(row + t, x);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) a0 = fmaf(x[e], sq[t + e], a0);
-            }
-            sc = a0 * scale;
-        }
-        const float mb = warp_max(sc);
-        const float mn = fmaxf(m, mb);
-        const float corr = __expf(m - mn);          // m = -inf on the first block -> 0
-        const float p = (j < hi) ? __expf(sc - mn) : 0.f;
-        Z = Z * corr + warp_sum(p);
-#pragma unroll
-        for (int e = 0; e < NE; ++e) acc[e] *= corr;
-        const int cnt = min(32, hi - base);
-        for (int jj = 0; jj < cnt; ++jj) {
-            const float pj = __shfl_sync(kFullMask, p, jj);
-            const T* vrow = vbase + static_cast<long long>(base + jj) * d;
-#pragma unroll
-            for (int e = 0; e < NE; ++e)
-                if (e * 32 < d) acc[e] = fmaf(pj, to_f32(vrow[e * 32 + lane]), acc[e]);
-        }
-        m = mn;
+        if (j * 32 + lane < s.K) sel[rank] = mine;
     }
 }
 
-// Per-chunk attention, local attention and fusion (Eq. HiLS weights; App. C per-head weights).
-// One warp per (b, h, r).
-template <typename T, int NE>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+// Scores of 64 keys from `base` on: octet o of the result holds key base + 8 o + lane / 4 (the same value in the quad's
+// lanes), -inf from `hi` on.  k: this lane's piece of row 0.
+template <typename T, int D, bool X>
+__device__ __forceinline__ void score_64(const Quad<T, D, X>& q, const T* k, int base, int hi, int d, float scale, int k8, float (&sc)[8]) {
+    if (base + 64 <= hi) {
+        const T* row = k + static_cast<long long>(base + k8) * d;
+#pragma unroll
+        for (int o = 0; o < 8; ++o) {
+            Quad<T, D, X> x;
+            x.load(row + static_cast<long long>(8 * o) * d, d);
+            sc[o] = x.dot(q) * scale;
+        }
+    } else {
+#pragma unroll
+        for (int o = 0; o < 8; ++o) {
+            const int j = base + o * 8 + k8;
+            sc[o] = -INFINITY;
+            if (base + o * 8 < hi) {
+                Quad<T, D, X> x;
+                x.load(k + static_cast<long long>(min(j, hi - 1)) * d, d);
+                const float v = x.dot(q) * scale;
+                if (j < hi) sc[o] = v;
+            }
+        }
+    }
+}
+__device__ __forceinline__ float octets_max(const float (&v)[8]) {
+    float m = v[0];
+#pragma unroll
+    for (int o = 1; o < 8; ++o) m = fmaxf(m, v[o]);
+#pragma unroll
+    for (int x = 4; x < 32; x <<= 1) m = fmaxf(m, __shfl_xor_sync(kFullMask, m, x));
+    return m;
+}
+__device__ __forceinline__ float octets_sum(const float (&v)[8]) {
+    float m = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+#pragma unroll
+    for (int x = 4; x < 32; x <<= 1) m += __shfl_xor_sync(kFullMask, m, x);
+    return m;
+}
+
+// Per-chunk attention, local attention and fusion (Eq. HiLS weights; App. C per-head weights).  One CTA per (b, h, r);
+// its warps take the row's items in turn: pieces of 64 tokens of the local window (their masses are exact, so mixing
+// by the masses reproduces the window's single softmax), then the selected chunks.  The sums over the keys stay spread
+// over the quads (a quad adds up its own keys) until the row is complete.
+constexpr int kAttWarps = 8;
+template <typename T, int D, bool X>
+__global__ void __launch_bounds__(kAttWarps * 32, D <= 64 ? 3 : 1)
 generic_attend_kernel(const GArgs a) {
-    extern __shared__ float smem[];
+    using Q = Quad<T, D, X>;
+    __shared__ float part[kAttWarps][D];
+    __shared__ float part_m[kAttWarps], part_d[kAttWarps];
+    pdl_wait();
     const Shape& s = a.s;
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const long long w = static_cast<long long>(blockIdx.x) * kWarpsPerBlock + wib;
-    const long long total = static_cast<long long>(s.B) * s.Hq * s.R;
-    if (w >= total) return;
-    const int r = static_cast<int>(w % s.R);
-    const int h = static_cast<int>((w / s.R) % s.Hq);
-    const int b = static_cast<int>(w / (static_cast<long long>(s.R) * s.Hq));
-    const int g = h / s.G, d = s.d;
-    const long long orow = (static_cast<long long>(b) * s.Hq + h) * s.R + r;
-    T* out = static_cast<T*>(a.out) + orow * d;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const unsigned orow = blockIdx.x;                           // (b Hq + h) R + r
+    const int r = static_cast<int>(orow % static_cast<unsigned>(s.R));
+    const int bh = static_cast<int>(orow / static_cast<unsigned>(s.R));
+    const int h = bh % s.Hq, b = bh / s.Hq;
+    const int g = h / s.G, d = Q::dim(s.d);
+    T* out = static_cast<T*>(a.out) + static_cast<long long>(orow) * d;
     const int pos = row_position(a, b, r);
     if (pos < 0) {
-        for (int t = lane; t < d; t += 32) out[t] = from_f32<T>(0.f);
-        if (lane == 0) a.lse[orow] = 0.f;
+        for (int t = threadIdx.x; t < d; t += blockDim.x) out[t] = from_f32<T>(0.f);
+        if (threadIdx.x == 0) a.lse[orow] = 0.f;
         return;
     }
     const int lo = local_lo(pos, s.W, s.S);
     const int ncand = lo / s.S;
-    float* sq = smem + static_cast<size_t>(wib) * 2 * d;        // attention query, then routing query
-    float* sr = sq + d;
-    const T* q = static_cast<const T*>(a.q) + orow * d;
-    const T* qr = static_cast<const T*>(a.q_route) + orow * d;
-    for (int t = lane; t < d; t += 32) { sq[t] = to_f32(q[t]); sr[t] = to_f32(qr[t]); }
-    __syncwarp();
+    const int k8 = lane >> 2, at = (lane & 3) * Q::kE;
+    Q q;
+    q.load(static_cast<const T*>(a.q) + static_cast<long long>(orow) * d + at, d);
 
-    const T* kg = static_cast<const T*>(a.k) + (static_cast<long long>(b) * s.Hkv + g) * s.T * d;
-    const T* vg = static_cast<const T*>(a.v) + (static_cast<long long>(b) * s.Hkv + g) * s.T * d;
+    const T* kg = static_cast<const T*>(a.k) + (static_cast<long long>(b) * s.Hkv + g) * s.T * d + at;
+    const T* vg = static_cast<const T*>(a.v) + (static_cast<long long>(b) * s.Hkv + g) * s.T * d + at;
     const int hl = (s.Hl == s.Hq) ? h : g;
-    const T* lm = static_cast<const T*>(a.lm) + (static_cast<long long>(b) * s.Hl + hl) * s.C * d;
-    const float* bias = a.bias ? a.bias + (static_cast<long long>(b) * s.Hl + hl) * s.C : nullptr;
+    const long long lrow = (static_cast<long long>(b) * s.Hl + hl) * s.C;
     const int32_t* sel = a.sel + ((static_cast<long long>(b) * s.Hkv + g) * s.R + r) * s.K;
 
-    // local branch first: lambda_loc = log Z_swa
-    float m, Z, acc[NE], part[NE];
-    attend_span<T, NE>(sq, kg, vg, lo, pos + 1, d, s.scale, lane, m, Z, part);
-    float Mx = m + __logf(Z);
-    float D = 1.f;
-#pragma unroll
-    for (int e = 0; e < NE; ++e) acc[e] = part[e] / Z;
-
-    for (int t = 0; t < s.K; ++t) {
-        const int c = sel[t];
-        if (c < 0) continue;
-        if (c >= ncand) {                       // never produced by the selection kernel
-            if (lane == 0) set_status(a.status, kDevBadIndex);
-            continue;
+    const int n_loc = (pos - lo) / 64 + 1, n_items = n_loc + min(s.K, ncand);
+    float Mx = -INFINITY, Dn = 0.f;
+    Q acc;
+    acc.fill(0.f);
+    for (int it = warp; it < n_items; it += nw) {
+        int k0, k1;
+        float lam = 0.f;
+        if (it < n_loc) {
+            k0 = lo + it * 64;
+            k1 = min(pos + 1, k0 + 64);
+        } else {
+            const int c = sel[it - n_loc];
+            if (c < 0 || c >= ncand) {              // never produced by the selection kernel
+                if (lane == 0) set_status(a.status, kDevBadIndex);
+                continue;
+            }
+            k0 = c * s.S;
+            k1 = k0 + s.S;
+            Q x, y;
+            x.load(static_cast<const T*>(a.q_route) + static_cast<long long>(orow) * d + at, d);
+            y.load(static_cast<const T*>(a.lm) + (lrow + c) * d + at, d);
+            lam = x.dot(y) * s.scale + (a.bias ? a.bias[lrow + c] : 0.f);
         }
-        float dotp = 0.f;
-        for (int x = lane; x < d; x += 32) dotp = fmaf(sr[x], to_f32(lm[static_cast<long long>(c) * d + x]), dotp);
-        float lam = warp_sum(dotp) * s.scale;
-        if (bias) lam += bias[c];
-        attend_span<T, NE>(sq, kg, vg, c * s.S, (c + 1) * s.S, d, s.scale, lane, m, Z, part);
+        float sc[8];
+        score_64<T, D, X>(q, kg, k0, k1, d, s.scale, k8, sc);
+        float m = octets_max(sc);
+        if (k1 - k0 > 64)                          // chunks of more than 64 tokens: the maximum over the whole chunk first
+            for (int base = k0 + 64; base < k1; base += 64) {
+                float sx[8];
+                score_64<T, D, X>(q, kg, base, k1, d, s.scale, k8, sx);
+                m = fmaxf(m, octets_max(sx));
+            }
+#pragma unroll
+        for (int o = 0; o < 8; ++o) sc[o] = __expf(sc[o] - m);
+        float Z = octets_sum(sc);
+        if (k1 - k0 > 64)
+            for (int base = k0 + 64; base < k1; base += 64) {
+                float sx[8];
+                score_64<T, D, X>(q, kg, base, k1, d, s.scale, k8, sx);
+#pragma unroll
+                for (int o = 0; o < 8; ++o) sx[o] = __expf(sx[o] - m);
+                Z += octets_sum(sx);
+            }
+        if (it < n_loc) lam = m + __logf(Z);
         const float Mn = fmaxf(Mx, lam);
-        const float c_old = __expf(Mx - Mn), c_new = __expf(lam - Mn);
-        D = D * c_old + c_new;
-        const float wnew = c_new / Z;
-#pragma unroll
-        for (int e = 0; e < NE; ++e) acc[e] = acc[e] * c_old + part[e] * wnew;
+        const float c_old = __expf(Mx - Mn), c_new = __expf(lam - Mn), w = c_new / Z;
+        Dn = Dn * c_old + c_new;
         Mx = Mn;
-    }
-    const float inv = 1.f / D;
+        acc.scale_by(c_old);
+        for (int base = k0;;) {
 #pragma unroll
-    for (int e = 0; e < NE; ++e)
-        if (e * 32 < d) out[e * 32 + lane] = from_f32<T>(acc[e] * inv);
-    if (lane == 0) a.lse[orow] = Mx + __logf(D);
+            for (int o = 0; o < 8; ++o) {
+                if (base + o * 8 >= k1) break;
+                Q x;
+                x.load(vg + static_cast<long long>(min(base + o * 8 + k8, k1 - 1)) * d, d);
+                acc.add_scaled(sc[o] * w, x);
+            }
+            base += 64;
+            if (base >= k1) break;
+            score_64<T, D, X>(q, kg, base, k1, d, s.scale, k8, sc);
+#pragma unroll
+            for (int o = 0; o < 8; ++o) sc[o] = __expf(sc[o] - m);
+        }
+    }
+    // the quads of the warp, then the warps (fixed order: deterministic)
+#pragma unroll
+    for (int i = 0; i < Q::kPl; ++i)
+#pragma unroll
+        for (int e = 0; e < Q::kE; ++e) {
+            float v = acc.x[i][e];
+#pragma unroll
+            for (int x = 4; x < 32; x <<= 1) v += __shfl_xor_sync(kFullMask, v, x);
+            acc.x[i][e] = v;
+        }
+    if (k8 == 0) {
+#pragma unroll
+        for (int i = 0; i < Q::kPl; ++i)
+#pragma unroll
+            for (int e = 0; e < Q::kE; ++e) part[warp][4 * Q::kE * i + at + e] = acc.x[i][e];
+    }
+    if (lane == 0) { part_m[warp] = Mx; part_d[warp] = Dn; }
+    __syncthreads();
+    float M = -INFINITY, den = 0.f;
+    for (int w = 0; w < nw; ++w) M = fmaxf(M, part_m[w]);
+    for (int w = 0; w < nw; ++w) den += part_d[w] * __expf(part_m[w] - M);
+    for (int t = threadIdx.x; t < d; t += blockDim.x) {
+        float v = 0.f;
+        for (int w = 0; w < nw; ++w) v = fmaf(part[w][t], __expf(part_m[w] - M), v);
+        out[t] = from_f32<T>(v / den);
+    }
+    if (threadIdx.x == 0) a.lse[orow] = M + __logf(den);
+}
+
+// ---- fp32 prefill on small shapes: chunk-major ------------------------------------------------------------------
+// The row kernel above reads (K + 1) chunks per row, mostly from L2 (61 % of its requests on 2048 tokens, d = 64, K = 4;
+// 38 us).  Here a CTA takes one chunk and the rows of a block that attend it: it looks its rows' selections through,
+// keeps K and V in shared memory and scores four rows at a time (lane = key, then lane = dimension), so that a K or V
+// value read from shared memory meets four rows.  Partial outputs and masses per (row, slot) go through global memory
+// to generic_fuse_kernel.  Same shape: 38 -> 26 us for the two kernels (bound by shared-memory reads while all CTAs
+// score, by latencies at both ends).
+constexpr int kRowBlock = 32;                // (early chunks are attended by every row of a block: two groups of four per warp)
+constexpr int kChunkWarps = 4;
+static_assert(kRowBlock <= kChunkWarps * 32, "one row per thread in the look-through");
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// Slots of a row: the selected chunks 0 .. K - 1, then the chunks of its local window.
+__host__ __device__ inline int chunk_slots(const Shape& s) { return s.K + (s.W + s.S - 2) / s.S + 1; }
+
+template <int D>
+struct ChunkSmem {
+    alignas(16) float k[64][D + 4];            // (padded: eight lanes reading the same piece of eight rows miss each other's banks)
+    alignas(16) float v[64][D];
+    alignas(16) float q[kChunkWarps][4][D];
+    alignas(16) float4 p[kChunkWarps][64][2];  // probabilities of four rows per key, each twice (pairs of a packed multiply)
+    int row[kRowBlock];                        // rows (of the block) that attend the chunk and the slot they hold it in
+    int slot[kRowBlock];
+    int cnt[kChunkWarps];
+};
+
+template <int D>
+__global__ void __launch_bounds__(kChunkWarps * 32)
+generic_chunk_kernel(const GArgs a, float* part, float* lam) {
+    extern __shared__ uint8_t chunk_raw[];
+    ChunkSmem<D>& sm = *reinterpret_cast<ChunkSmem<D>*>(chunk_raw);
+    constexpr int kV = D / 32;                 // dimensions per lane in the value pass
+    const Shape& s = a.s;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int c = blockIdx.y, r0 = blockIdx.x * kRowBlock, bh = blockIdx.z, h = bh % s.Hq, b = bh / s.Hq, g = h / s.G;
+    if (s.pos0 + min(s.R, r0 + kRowBlock) - 1 < c * s.S) return;            // the chunk lies after the block's last row
+    const float* kc = static_cast<const float*>(a.k) + ((static_cast<long long>(b) * s.Hkv + g) * s.T + static_cast<long long>(c) * s.S) * D;
+    const float* vc = static_cast<const float*>(a.v) + (kc - static_cast<const float*>(a.k));
+    const int rows_k = min(s.S, s.T - c * s.S);                             // rows of the chunk that exist
+    for (int x = tid; x < rows_k * (D / 4); x += blockDim.x)
+        cp_async16(smem_u32(&sm.k[x / (D / 4)][(x % (D / 4)) * 4]), kc + x * 4);
+    for (int x = tid; x < rows_k * (D / 4); x += blockDim.x)
+        cp_async16(smem_u32(&sm.v[x / (D / 4)][(x % (D / 4)) * 4]), vc + x * 4);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    for (int x = rows_k * D + tid; x < 64 * D; x += blockDim.x) { sm.k[x / D][x % D] = 0.f; sm.v[x / D][x % D] = 0.f; }
+    pdl_wait();                                 // the selection
+    int slot = -1;
+    {
+        const int r = r0 + tid, pos = s.pos0 + r;
+        if (tid < kRowBlock && r < s.R && c * s.S <= pos) {
+            const int lc = local_lo(pos, s.W, s.S) / s.S;
+            if (c >= lc) {
+                slot = s.K + c - lc;
+            } else {
+                const int32_t* sel = a.sel + ((static_cast<long long>(b) * s.Hkv + g) * s.R + r) * s.K;
+                for (int t = 0; t < s.K; ++t) if (sel[t] == c) slot = t;
+            }
+        }
+        const unsigned vote = __ballot_sync(kFullMask, slot >= 0);
+        if (lane == 0) sm.cnt[warp] = __popc(vote);
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        int at = __popc(vote & ((1u << lane) - 1u));
+        for (int w = 0; w < warp; ++w) at += sm.cnt[w];
+        if (slot >= 0) { sm.row[at] = r; sm.slot[at] = slot; }
+    }
+    int n = 0;
+    for (int w = 0; w < kChunkWarps; ++w) n += sm.cnt[w];
+    __syncthreads();
+    const int NS = chunk_slots(s), hl = (s.Hl == s.Hq) ? h : g;
+    const long long lrow = (static_cast<long long>(b) * s.Hl + hl) * s.C + c;
+    float lmv[kV];                              // the chunk's landmark
+#pragma unroll
+    for (int x = 0; x < kV; ++x) lmv[x] = c < s.C ? static_cast<const float*>(a.lm)[lrow * D + lane + 32 * x] : 0.f;
+    // query rows of a group of four, requested a group ahead
+    float qv[4][kV], rv[4][kV];
+    auto fetch = [&](int e0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const long long at = (static_cast<long long>(bh) * s.R + sm.row[min(e0 + i, n - 1)]) * D + lane;
+#pragma unroll
+            for (int x = 0; x < kV; ++x) {
+                qv[i][x] = static_cast<const float*>(a.q)[at + 32 * x];
+                rv[i][x] = static_cast<const float*>(a.q_route)[at + 32 * x];
+            }
+        }
+    };
+    if (warp * 4 < n) fetch(warp * 4);
+    for (int e0 = warp * 4; e0 < n; e0 += kChunkWarps * 4) {
+        int row[4], lim[4];
+        bool sel[4];
+        float lm[4];
+        float (*q)[D] = sm.q[warp];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int e = min(e0 + i, n - 1);
+            row[i] = sm.row[e];
+            sel[i] = sm.slot[e] < s.K;
+            lim[i] = sel[i] ? s.S - 1 : min(s.S - 1, s.pos0 + row[i] - c * s.S);
+            lm[i] = 0.f;
+#pragma unroll
+            for (int x = 0; x < kV; ++x) {
+                q[i][lane + 32 * x] = qv[i][x];
+                lm[i] = fmaf(rv[i][x], lmv[x], lm[i]);
+            }
+        }
+        if (e0 + kChunkWarps * 4 < n) fetch(e0 + kChunkWarps * 4);
+        __syncwarp();
+        // two dimensions per instruction: a pair's halves are added at the end
+        float2 a0[4], a1[4];                                                  // keys lane, lane + 32
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a0[i] = a1[i] = make_float2(0.f, 0.f);
+#pragma unroll 4
+        for (int x = 0; x < D; x += 4) {
+            const float4 k0 = *reinterpret_cast<const float4*>(&sm.k[lane][x]), k1 = *reinterpret_cast<const float4*>(&sm.k[lane + 32][x]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 qv = *reinterpret_cast<const float4*>(&q[i][x]);
+                const float2 ql = make_float2(qv.x, qv.y), qh = make_float2(qv.z, qv.w);
+                a0[i] = __ffma2_rn(ql, make_float2(k0.x, k0.y), a0[i]);
+                a1[i] = __ffma2_rn(ql, make_float2(k1.x, k1.y), a1[i]);
+                a0[i] = __ffma2_rn(qh, make_float2(k0.z, k0.w), a0[i]);
+                a1[i] = __ffma2_rn(qh, make_float2(k1.z, k1.w), a1[i]);
+            }
+        }
+        float s0[4], s1[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { s0[i] = a0[i].x + a0[i].y; s1[i] = a1[i].x + a1[i].y; }
+        float mx[4], z[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            s0[i] = lane <= lim[i] ? s0[i] * s.scale : -INFINITY;
+            s1[i] = lane + 32 <= lim[i] ? s1[i] * s.scale : -INFINITY;
+            mx[i] = warp_max(fmaxf(s0[i], s1[i]));
+            s0[i] = __expf(s0[i] - mx[i]);
+            s1[i] = __expf(s1[i] - mx[i]);
+            z[i] = warp_sum(s0[i] + s1[i]);
+            lm[i] = warp_sum(lm[i]);
+        }
+        sm.p[warp][lane][0] = make_float4(s0[0], s0[0], s0[1], s0[1]);
+        sm.p[warp][lane][1] = make_float4(s0[2], s0[2], s0[3], s0[3]);
+        sm.p[warp][lane + 32][0] = make_float4(s1[0], s1[0], s1[1], s1[1]);
+        sm.p[warp][lane + 32][1] = make_float4(s1[2], s1[2], s1[3], s1[3]);
+        __syncwarp();
+        float2 o[4][kV / 2];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int x = 0; x < kV / 2; ++x) o[i][x] = make_float2(0.f, 0.f);
+#pragma unroll 8
+        for (int j = 0; j < 64; ++j) {
+            const float4 p0 = sm.p[warp][j][0], p1 = sm.p[warp][j][1];
+#pragma unroll
+            for (int x = 0; x < kV / 2; ++x) {
+                const float2 v = *reinterpret_cast<const float2*>(&sm.v[j][2 * lane + 64 * x]);
+                o[0][x] = __ffma2_rn(make_float2(p0.x, p0.y), v, o[0][x]);
+                o[1][x] = __ffma2_rn(make_float2(p0.z, p0.w), v, o[1][x]);
+                o[2][x] = __ffma2_rn(make_float2(p1.x, p1.y), v, o[2][x]);
+                o[3][x] = __ffma2_rn(make_float2(p1.z, p1.w), v, o[3][x]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (e0 + i >= n) break;
+            const long long at = (static_cast<long long>(bh) * s.R + row[i]) * NS + sm.slot[e0 + i];
+            const float zi = 1.f / z[i];
+#pragma unroll
+            for (int x = 0; x < kV / 2; ++x)
+                *reinterpret_cast<float2*>(part + at * D + 2 * lane + 64 * x) = make_float2(o[i][x].x * zi, o[i][x].y * zi);
+            if (lane == 0) lam[at] = sel[i] ? lm[i] * s.scale + (a.bias ? a.bias[lrow] : 0.f) : mx[i] + __logf(z[i]);
+        }
+        __syncwarp();
+    }
+}
+
+// Mix of a row's slots (Eq. HiLS weights): one warp per (b, h, r).
+template <int D>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+generic_fuse_kernel(const GArgs a, const float* part, const float* lam) {
+    constexpr int kV = D / 32;
+    pdl_wait();
+    const Shape& s = a.s;
+    const int lane = threadIdx.x & 31;
+    const long long orow = static_cast<long long>(blockIdx.x) * kWarpsPerBlock + (threadIdx.x >> 5);
+    if (orow >= static_cast<long long>(s.B) * s.Hq * s.R) return;
+    const int pos = s.pos0 + static_cast<int>(orow % s.R), lc = local_lo(pos, s.W, s.S) / s.S;
+    const int NS = chunk_slots(s), nsel = min(s.K, lc), nl = pos / s.S - lc + 1;
+    const float* lr = lam + orow * NS;
+    auto slot_of = [&](int i) { return i < nsel ? i : s.K + (i - nsel); };
+    float M = -INFINITY;
+    for (int i = lane; i < nsel + nl; i += 32) M = fmaxf(M, lr[slot_of(i)]);
+    M = warp_max(M);
+    float den = 0.f, o[kV];
+#pragma unroll
+    for (int x = 0; x < kV; ++x) o[x] = 0.f;
+#pragma unroll 4
+    for (int i = 0; i < nsel + nl; ++i) {
+        const int t = slot_of(i);
+        const float w = __expf(lr[t] - M);
+        const float* src = part + (orow * NS + t) * D + lane;
+        den += w;
+#pragma unroll
+        for (int x = 0; x < kV; ++x) o[x] = fmaf(w, src[32 * x], o[x]);
+    }
+    float* out = static_cast<float*>(a.out) + orow * D + lane;
+#pragma unroll
+    for (int x = 0; x < kV; ++x) out[32 * x] = o[x] / den;
+    if (lane == 0) a.lse[orow] = M + __logf(den);
+}
+
+// The chunk-major kernels apply while the partial outputs stay small and looking every row's selection through once per
+// visible chunk stays cheap beside the attention itself (both hold up to about 4K tokens).
+bool chunk_major(const Shape& s, int dtype) {
+    if (dtype != HILS_F32 || s.is_decode || s.S > 64 || (s.d != 64 && s.d != 128)) return false;
+    const long long rows = static_cast<long long>(s.B) * s.Hq * s.R, chunks = (s.pos0 + s.R + s.S - 1) / s.S;
+    return chunks <= 65535 && static_cast<long long>(s.B) * s.Hq <= 65535 && rows * chunk_slots(s) * s.d * 4 <= (256ll << 20) &&
+           rows * chunks * s.K * 4 <= (256ll << 20);
+}
+size_t chunk_lam_offset(const Shape& s) {
+    return (static_cast<size_t>(s.B) * s.Hq * s.R * chunk_slots(s) * s.d * sizeof(float) + 255) / 256 * 256;
+}
+
+template <int D>
+int launch_chunk_major(const GArgs& a, void* scratch, cudaStream_t stream) {
+    const Shape& s = a.s;
+    static PerDeviceOnce once;
+    if (once.pending()) {
+        if (cudaFuncSetAttribute(generic_chunk_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(ChunkSmem<D>)) != cudaSuccess)
+            return HILS_ERR_CUDA;
+        once.done();
+    }
+    float* part = static_cast<float*>(scratch);
+    float* lam = reinterpret_cast<float*>(static_cast<char*>(scratch) + chunk_lam_offset(s));
+    const unsigned chunks = static_cast<unsigned>((s.pos0 + s.R + s.S - 1) / s.S), blocks = static_cast<unsigned>((s.R + kRowBlock - 1) / kRowBlock);
+    const long long rows = static_cast<long long>(s.B) * s.Hq * s.R;
+    if (launch_pdl(generic_chunk_kernel<D>, dim3(blocks, chunks, static_cast<unsigned>(s.B * s.Hq)), dim3(kChunkWarps * 32),
+                   sizeof(ChunkSmem<D>), stream, a, part, lam) != cudaSuccess)
+        return HILS_ERR_CUDA;
+    trace_mark("generic_attend", stream);
+    if (launch_pdl(generic_fuse_kernel<D>, dim3(static_cast<unsigned>((rows + kWarpsPerBlock - 1) / kWarpsPerBlock)),
+                   dim3(kWarpsPerBlock * 32), 0, stream, a, static_cast<const float*>(part), static_cast<const float*>(lam)) != cudaSuccess)
+        return HILS_ERR_CUDA;
+    trace_mark("generic_fuse", stream);
+    return 3;
+}
+
+template <typename T, int D, bool X>
+int launch_dim(const GArgs& a, int dtype, void* scratch, cudaStream_t stream) {
+    const Shape& s = a.s;
+    const long long sel_warps = static_cast<long long>(s.B) * s.Hkv * s.R;
+    const long long rows = static_cast<long long>(s.B) * s.Hq * s.R;
+    if (rows > 0x7fffffffll) return HILS_ERR_UNSUPPORTED;
+    const unsigned sel_blocks = static_cast<unsigned>((sel_warps + kWarpsPerBlock - 1) / kWarpsPerBlock);
+    const int nr = (s.K + 31) / 32;
+    if (nr <= 1) generic_select_kernel<T, D, X, 1><<<sel_blocks, kWarpsPerBlock * 32, 0, stream>>>(a);
+    else if (nr == 2) generic_select_kernel<T, D, X, 2><<<sel_blocks, kWarpsPerBlock * 32, 0, stream>>>(a);
+    else generic_select_kernel<T, D, X, 4><<<sel_blocks, kWarpsPerBlock * 32, 0, stream>>>(a);
+    if (cudaGetLastError() != cudaSuccess) return HILS_ERR_CUDA;
+    trace_mark("generic_select", stream);
+    if (chunk_major(s, dtype)) return s.d == 64 ? launch_chunk_major<64>(a, scratch, stream) : launch_chunk_major<128>(a, scratch, stream);
+    // a warp per item of the row, at most eight
+    const long long items = static_cast<long long>(s.K) + (s.W + s.S - 2) / 64 + 1;
+    const unsigned warps = static_cast<unsigned>(items < kAttWarps ? items : kAttWarps);
+    if (launch_pdl(generic_attend_kernel<T, D, X>, dim3(static_cast<unsigned>(rows)), dim3(warps * 32), 0, stream, a) != cudaSuccess)
+        return HILS_ERR_CUDA;
+    trace_mark("generic_attend", stream);
+    return 2;
 }
 
 template <typename T>
-int launch_typed(const GArgs& a, cudaStream_t stream) {
-    const Shape& s = a.s;
-    const long long sel_warps = static_cast<long long>(s.B) * s.Hkv * s.R;
-    const long long att_warps = static_cast<long long>(s.B) * s.Hq * s.R;
-    const unsigned sel_blocks = static_cast<unsigned>((sel_warps + kWarpsPerBlock - 1) / kWarpsPerBlock);
-    const unsigned att_blocks = static_cast<unsigned>((att_warps + kWarpsPerBlock - 1) / kWarpsPerBlock);
-    const size_t sel_smem = sizeof(float) * kWarpsPerBlock * s.G * s.d;
-    const size_t att_smem = sizeof(float) * kWarpsPerBlock * 2 * s.d;
-    const int nr = (s.K + 31) / 32;
-    if (nr <= 1) generic_select_kernel<T, 1><<<sel_blocks, kWarpsPerBlock * 32, sel_smem, stream>>>(a);
-    else if (nr == 2) generic_select_kernel<T, 2><<<sel_blocks, kWarpsPerBlock * 32, sel_smem, stream>>>(a);
-    else generic_select_kernel<T, 4><<<sel_blocks, kWarpsPerBlock * 32, sel_smem, stream>>>(a);
-    if (cudaGetLastError() != cudaSuccess) return HILS_ERR_CUDA;
-    trace_mark("generic_select", stream);
-    const int ne = s.d / 32;
-    if (ne <= 2) generic_attend_kernel<T, 2><<<att_blocks, kWarpsPerBlock * 32, att_smem, stream>>>(a);
-    else if (ne <= 4) generic_attend_kernel<T, 4><<<att_blocks, kWarpsPerBlock * 32, att_smem, stream>>>(a);
-    else generic_attend_kernel<T, 8><<<att_blocks, kWarpsPerBlock * 32, att_smem, stream>>>(a);
-    if (cudaGetLastError() != cudaSuccess) return HILS_ERR_CUDA;
-    trace_mark("generic_attend", stream);
-    return 2;
+int launch_typed(const GArgs& a, int dtype, void* scratch, cudaStream_t stream) {
+    if (a.s.d == 64) return launch_dim<T, 64, true>(a, dtype, scratch, stream);
+    if (a.s.d == 128) return launch_dim<T, 128, true>(a, dtype, scratch, stream);
+    if (a.s.d < 128) return launch_dim<T, 128, false>(a, dtype, scratch, stream);
+    return launch_dim<T, 256, false>(a, dtype, scratch, stream);
 }
 
 }  // namespace
@@ -291,11 +712,16 @@ bool generic_supports(const Shape& s) {
            s.S >= 1;
 }
 
+size_t generic_scratch_bytes(const Shape& s, int dtype) {
+    if (!chunk_major(s, dtype)) return 0;
+    return chunk_lam_offset(s) + sizeof(float) * static_cast<size_t>(s.B) * s.Hq * s.R * chunk_slots(s);
+}
+
 int launch_generic(const Shape& s, int dtype, const Tensors& t, cudaStream_t stream) {
     if (!generic_supports(s)) return HILS_ERR_UNSUPPORTED;
     GArgs a{s, t.q, t.q_route ? t.q_route : t.q, t.k, t.v, t.landmarks, t.bias, t.seq_lens, t.out, t.lse, t.sel_idx, t.status};
-    if (dtype == HILS_F32) return launch_typed<float>(a, stream);
-    return launch_typed<__nv_bfloat16>(a, stream);
+    if (dtype == HILS_F32) return launch_typed<float>(a, dtype, t.scratch, stream);
+    return launch_typed<__nv_bfloat16>(a, dtype, t.scratch, stream);
 }
 
 }  // namespace hils

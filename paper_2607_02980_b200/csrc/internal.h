@@ -55,6 +55,7 @@ bool trace_active();
 // Each launcher returns the number of kernels it enqueued, or a negative hils_status.
 int launch_generic(const Shape& s, int dtype, const Tensors& t, cudaStream_t stream);
 bool generic_supports(const Shape& s);
+size_t generic_scratch_bytes(const Shape& s, int dtype);
 
 int launch_decode_fast(const Shape& s, const Tensors& t, cudaStream_t stream);
 bool decode_fast_supports(const Shape& s, int dtype);
