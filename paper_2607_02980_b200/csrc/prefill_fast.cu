@@ -53,6 +53,7 @@ struct PArgs {
     int4* tiles;            // [max_tiles] {pair, chunk, first entry, rows}
     __nv_bfloat16* obuf;    // [entries of one block][G][128] normalised per-chunk outputs, in entry order
     float* lam;             // [entries of one block][G] per-head surrogate scores; local slot: log Z_swa
+    int t0;                 // first token of the chunk-major part (the ones before it go query-major)
     int i0, i1;             // token block [i0, i1) of the attend / fuse launch
     int blk;                // its index
     int n_blocks;           // query blocks of qb tokens
@@ -269,14 +270,14 @@ __device__ __forceinline__ int slot_chunk(const PArgs& a, int pair, int tok, int
 __global__ void invert_count_kernel(const PArgs a) {
     const Shape& s = a.s;
     const int K1 = s.K + max_local_slots(s.W), pairs = s.B * s.Hkv;
-    const long long total = static_cast<long long>(pairs) * s.R * K1;
+    const long long total = static_cast<long long>(pairs) * (s.R - a.t0) * K1;
     for (long long x = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; x < total;
          x += static_cast<long long>(gridDim.x) * blockDim.x) {
         const int slot = static_cast<int>(x % K1);
-        const int tok = static_cast<int>((x / K1) % s.R);
-        const int pair = static_cast<int>(x / (static_cast<long long>(K1) * s.R));
+        const int tok = a.t0 + static_cast<int>((x / K1) % (s.R - a.t0));
+        const int pair = static_cast<int>(x / (static_cast<long long>(K1) * (s.R - a.t0)));
         const int c = slot_chunk(a, pair, tok, slot);
-        if (c >= 0) atomicAdd(&a.cnt[(static_cast<long long>(tok / a.qb) * pairs + pair) * a.nc + c], 1);
+        if (c >= 0) atomicAdd(&a.cnt[(static_cast<long long>((tok - a.t0) / a.qb) * pairs + pair) * a.nc + c], 1);
     }
 }
 
@@ -349,16 +350,16 @@ __global__ void invert_fill_kernel(const PArgs a) {
     const Shape& s = a.s;
     const int K1 = s.K + max_local_slots(s.W), pairs = s.B * s.Hkv;
     const int lane = threadIdx.x & 31;
-    const int tblocks = (s.R + 31) / 32;
+    const int tblocks = (s.R - a.t0 + 31) / 32;                  // (t0 is a multiple of 32)
     const long long total = static_cast<long long>(pairs) * tblocks * K1;
     const long long nwarps = static_cast<long long>(gridDim.x) * (blockDim.x >> 5);
     for (long long w = static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); w < total; w += nwarps) {
         const int slot = static_cast<int>(w % K1);
         const int tb = static_cast<int>((w / K1) % tblocks);
         const int pair = static_cast<int>(w / (static_cast<long long>(K1) * tblocks));
-        const int tok = tb * 32 + lane;
+        const int tok = a.t0 + tb * 32 + lane;
         const int c = tok < s.R ? slot_chunk(a, pair, tok, slot) : -1;
-        const long long idx = c >= 0 ? (static_cast<long long>(tok / a.qb) * pairs + pair) * a.nc + c : -1 - lane;
+        const long long idx = c >= 0 ? (static_cast<long long>((tok - a.t0) / a.qb) * pairs + pair) * a.nc + c : -1 - lane;
         const unsigned same = __match_any_sync(kFullMask, idx);
         const int leader = __ffs(same) - 1;
         int base = 0;
@@ -368,7 +369,7 @@ __global__ void invert_fill_kernel(const PArgs a) {
             int pos = -1;
             if (c >= 0) {
                 pos = base + __popc(same & ((1u << lane) - 1u));
-                if (pos < a.max_tiles * a.tile_tok) a.entries[pos] = ((tok % a.qb) << 8) | slot;
+                if (pos < a.max_tiles * a.tile_tok) a.entries[pos] = (((tok - a.t0) % a.qb) << 8) | slot;
             }
             a.epos[(static_cast<long long>(pair) * s.R + tok) * K1 + slot] = pos;
         }
@@ -554,23 +555,24 @@ struct Plan {
         total, obuf_tiles;
 };
 
-Plan make_plan(const Shape& s, int qb_fixed = 0) {
+Plan make_plan(const Shape& s, int qb_fixed = 0, int t0 = 0) {
     Plan p;
+    const int R = s.R - t0;                      // tokens of the chunk-major part
     const size_t pairs = static_cast<size_t>(s.B) * s.Hkv;
     const int QB = qb_fixed > 0 ? qb_fixed : pick_query_block(s);
-    const size_t blk = static_cast<size_t>(s.R < QB ? (s.R + kS - 1) / kS * kS : QB);
+    const size_t blk = static_cast<size_t>(R < QB ? (R + 127) / 128 * 128 : QB);
     p.qb = static_cast<int>(blk);
     const size_t nchunks = (static_cast<size_t>(s.pos0) + s.R + kS - 1) / kS;     // chunks the queries can touch
     const size_t nc = static_cast<size_t>(s.C) > nchunks ? static_cast<size_t>(s.C) : nchunks;
     p.nc = static_cast<int>(nc);
-    const size_t nblocks = (static_cast<size_t>(s.R) + blk - 1) / blk;
+    const size_t nblocks = (static_cast<size_t>(R) + blk - 1) / blk;
     p.n_blocks = static_cast<int>(nblocks);
     // tiles of a block <= its entries / tile + one ragged tile per list; a block's tokens see the chunks up to its end
     const size_t tt = static_cast<size_t>(attend_tc_tile_tokens());
     size_t all_tiles = 0, max_blk = 0;
     for (size_t b = 0; b < nblocks; ++b) {
-        const size_t toks = (b + 1) * blk <= static_cast<size_t>(s.R) ? blk : static_cast<size_t>(s.R) - b * blk;
-        const size_t vis = ((s.pos0 + b * blk + toks) + kS - 1) / kS;
+        const size_t toks = (b + 1) * blk <= static_cast<size_t>(R) ? blk : static_cast<size_t>(R) - b * blk;
+        const size_t vis = ((s.pos0 + t0 + b * blk + toks) + kS - 1) / kS;
         // (and never more than its entries: a list that exists holds at least one)
         const size_t ents = pairs * toks * (s.K + max_local_slots(s.W));
         const size_t ragged = pairs * (toks * (s.K + max_local_slots(s.W)) / tt + (vis < nc ? vis : nc));
@@ -668,7 +670,19 @@ int build_inverse_index(const Shape& s, const int32_t* sel, void* scratch, size_
 }
 
 int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
-    const Plan p = make_plan(s);
+    // the first n_qm tokens of every sequence see few chunks and go query-major (with q_route their mixing logits would not
+    // be what that kernel's score tile holds)
+    const int n_qm = t.q_route ? 0 : prefill_query_tokens(s);
+    const int last_cand = local_lo(s.pos0 + s.R - 1, s.W, kS) / kS;
+    if (n_qm == s.R && last_cand <= s.K) {
+        // nothing to select either: one launch
+        const int rc = launch_prefill_query_tc(s, t, n_qm, 1, stream);
+        if (rc < 0) return rc;
+        trace_mark("prefill_query", stream);
+        return rc;
+    }
+    const int t0 = n_qm;
+    const Plan p = make_plan(s, 0, t0 < s.R ? t0 : 0);
     if (t.scratch_bytes < p.total) return HILS_ERR_WORKSPACE;
     const int pairs = s.B * s.Hkv;
     char* sc = static_cast<char*>(t.scratch);
@@ -698,6 +712,7 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
     a.qb = p.qb;
     a.nc = p.nc;
     a.tile_tok = attend_tc_tile_tokens();
+    a.t0 = t0;
     a.i0 = 0;
     a.i1 = 0;
     a.whole = p.whole;
@@ -723,10 +738,11 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
     int launches = 0;
     const int tiles_per_seq = (s.R + kS - 1) / kS;
     // counters of the inverse index start at zero; the tcgen05 selection kernel fills the per-chunk entry counts itself
-    if (cudaMemsetAsync(sc + p.off_cnt, 0, p.zero_bytes, stream) != cudaSuccess) return HILS_ERR_CUDA;
+    if (t0 < s.R && cudaMemsetAsync(sc + p.off_cnt, 0, p.zero_bytes, stream) != cudaSuccess) return HILS_ERR_CUDA;
     bool counted = false;
     if (prefill_select_tc_supports(s) && !g_force_mma_select) {
-        const int rc = launch_prefill_select_tc(s, a.q, t.landmarks, t.bias, t.sel_idx, t.status, a.cnt, a.qb, a.nc, stream);
+        const int rc = launch_prefill_select_tc(s, a.q, t.landmarks, t.bias, t.sel_idx, t.status, t0 < s.R ? a.cnt : nullptr, a.qb, a.nc, t0,
+                                                stream);
         if (rc < 0) return rc;
         counted = rc == 2;
     } else {
@@ -735,11 +751,18 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
     }
     trace_mark("prefill_select", stream);
     ++launches;
+    if (n_qm > 0) {
+        const int rc = launch_prefill_query_tc(s, t, n_qm, 0, stream);
+        if (rc < 0) return rc;
+        trace_mark("prefill_query", stream);
+        launches += rc;
+        if (n_qm == s.R) return launches;
+    }
 
     // inverse index for every query block at once: per-(block, pair, chunk) lists of (token, slot) entries
     // and the table of attend tiles, grouped by block
     {
-        const long long elems = static_cast<long long>(pairs) * s.R * (s.K + max_local_slots(s.W));
+        const long long elems = static_cast<long long>(pairs) * (s.R - t0) * (s.K + max_local_slots(s.W));
         const long long want = (elems + 255) / 256;
         const unsigned eb = static_cast<unsigned>(want < sm_count() * 16 ? want : sm_count() * 16);
         if (!counted) {
@@ -757,7 +780,7 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
         trace_mark("prefill_invert", stream);
         launches += 3;
     }
-    for (int i0 = 0, blk = 0; i0 < s.R; i0 += a.qb, ++blk) {
+    for (int i0 = t0, blk = 0; i0 < s.R; i0 += a.qb, ++blk) {
         a.i0 = i0;
         a.i1 = s.R < i0 + a.qb ? s.R : i0 + a.qb;
         a.blk = blk;
@@ -781,7 +804,7 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
         if (a.whole) {
             // one fusion launch after the last block's attend, over every token of the call
             if (a.i1 < s.R) continue;
-            a.i0 = 0;
+            a.i0 = t0;
         }
         const long long fuse_warps = static_cast<long long>(pairs) * (a.i1 - a.i0);
         if (launch_pdl(prefill_fuse_kernel, dim3(static_cast<unsigned>((fuse_warps + kFuseWarps - 1) / kFuseWarps)),

@@ -1,0 +1,492 @@
+// Query-major prefill on tcgen05 tensor cores (bf16, d = 128, S = 64, G = 4, one landmark per KV head) for the tokens
+// that see few chunks.
+//
+// Where the candidates of a token are not many more than top_k, neighbouring tokens attend mostly the same chunks: a tile of
+// 32 tokens x 4 heads (128 MMA rows) walks the union of its tokens' chunks, and the mix of Eq. (HiLS weights) stays in
+// tensor memory until `out` is written once.  The chunk-major kernels (prefill_attend_tc.cu) move a query row in and a
+// partial output row out and in again per (token, chunk) pair; here a chunk costs a tile one score and one value product,
+// whoever of its tokens selected it (the others meet probabilities of zero).
+//
+// A CTA works on units of 64 adjacent tokens of one (sequence, KV head): two tiles that share the K / V stream, each with
+// its own scores, probabilities and output accumulator in tensor memory (256 columns).
+//   warps 0-3, 4-7   softmax of tile 0 / 1 (warp = head, lane = token): the chunk's own softmax, its mixing logit (the
+//                    landmark is key 64 of the score tile; the exact log mass for a chunk of the local window), normalised
+//                    probabilities times the mixing weight as bf16 into tensor memory.  The weights refer to a running
+//                    reference logit per row that is raised, and the accumulator scaled, only when a logit exceeds it by
+//                    kRaise: rare, and bf16 / fp32 keep their relative precision in between.  At the end of a unit the same
+//                    warps write the tile's rows.
+//   warps 8, 9       issue the MMAs of tile 0 / 1 (the next chunk's scores before this chunk's value product)
+//   warp 10          loads K, V, landmark rows and queries by TMA
+//   warp 11          builds the unit's list of chunks (and which tile needs them, with a bit per token), one unit ahead
+// Bound: the exponentials (64 per row and chunk; 512 cycles per tile and chunk on 16 units) and the softmax warps' issue.
+#include "internal.h"
+#include "tma.cuh"
+
+namespace hils {
+namespace {
+
+constexpr int kD = 128;
+constexpr int kS = 64;
+constexpr int kG = 4;
+constexpr int kTok = 32;                        // tokens per tile
+constexpr int kUnitTok = 64;                    // tokens per unit
+constexpr int kRows = kTok * kG;
+constexpr int kNS = 80;                         // score columns: 64 keys + landmark (+ 15 zero rows)
+constexpr int kKBytes = kNS * kD * 2;
+constexpr int kVBytes = kS * kD * 2;
+constexpr int kQBytes = kRows * kD * 2;
+constexpr int kStages = 4;
+constexpr int kMaxC = 160;                      // chunks a unit may see
+constexpr int kPCol = 96;                       // columns of a tile: scores 0..79, probabilities 96..127, output 128..255
+constexpr int kOCol = 128;
+constexpr int kMmaWarp = 8, kLoadWarp = 10, kListWarp = 11;
+constexpr int kThreads = 12 * 32;
+constexpr float kLog2e = 1.4426950408889634f;
+constexpr float kRaise = 16.f;
+
+struct QmArgs {
+    Shape s;
+    const __nv_bfloat16* lm;
+    const float* bias;
+    int32_t* sel;
+    __nv_bfloat16* out;
+    float* lse;
+    int* status;
+    int n_tok;         // tokens 0 .. n_tok - 1 of every sequence
+    int write_sel;     // 1: no token has more candidates than top_k, the selection is written here
+};
+
+struct QmSmem {
+    uint64_t kv_full[kStages], kv_empty[kStages];
+    uint64_t q_full[2], q_empty[2];
+    uint64_t s_full[2], s_empty[2], p_full[2], o_done[2];
+    uint64_t list_full[2], list_empty[2];
+    uint32_t tmem_base;
+    int abort_flag;
+    int n_items[2];                             // items of the unit's list
+    int parts[2];                               // bit t: tile t has items
+    int list[2][kMaxC];                         // chunk | tile 0 needs it << 16 | tile 1 needs it << 17
+    uint32_t mask[2][2][kMaxC];                 // [list][tile][chunk]: tokens that selected it
+};
+static_assert(kStages * (kKBytes + kVBytes) + 2 * kQBytes + sizeof(QmSmem) + 1024 <= 232448, "shared memory of the query-major kernel");
+
+__device__ __forceinline__ float ex2_approx(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, uint32_t bytes, uint64_t* bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(smem_u32(sdst)), "l"(gsrc), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+
+__global__ void __launch_bounds__(kThreads, 1)
+prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
+                        const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_out, const QmArgs a) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* kbuf = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t* vbuf = kbuf + kStages * kKBytes;
+    uint8_t* qbuf = vbuf + kStages * kVBytes;
+    QmSmem& sm = *reinterpret_cast<QmSmem*>(qbuf + 2 * kQBytes);
+    const Shape& s = a.s;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int pairs = s.B * s.Hkv, n_blk = (a.n_tok + kUnitTok - 1) / kUnitTok, n_units = pairs * n_blk;
+
+    if (tid == 0) {
+        for (int i = 0; i < kStages; ++i) { mbar_init(&sm.kv_full[i], 1); mbar_init(&sm.kv_empty[i], 2); }
+        for (int t = 0; t < 2; ++t) {
+            mbar_init(&sm.q_full[t], 1); mbar_init(&sm.q_empty[t], 4);
+            mbar_init(&sm.s_full[t], 1); mbar_init(&sm.s_empty[t], 4);
+            mbar_init(&sm.p_full[t], 4); mbar_init(&sm.o_done[t], 1);
+            mbar_init(&sm.list_full[t], 1); mbar_init(&sm.list_empty[t], 11);
+        }
+        mbar_fence_init();
+        sm.abort_flag = 0;
+        tma_prefetch_desc(&map_q);
+        tma_prefetch_desc(&map_k);
+        tma_prefetch_desc(&map_v);
+        tma_prefetch_desc(&map_out);
+    }
+    // rows 64 .. 79 of every K buffer: the landmark row and zeros (TMA writes rows 0 .. 63)
+    for (int x = tid; x < kStages * 2 * 16 * 8; x += kThreads) {
+        const int st = x >> 8, kb = (x >> 7) & 1, row = 64 + ((x >> 3) & 15), pc = x & 7;
+        *reinterpret_cast<uint4*>(kbuf + st * kKBytes + kb * (kNS * 128) + swz128(row, pc)) = make_uint4(0u, 0u, 0u, 0u);
+    }
+    if (warp == kMmaWarp) tmem_alloc(&sm.tmem_base, 512);
+    fence_proxy_async_smem();
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    const uint32_t tmem_base = sm.tmem_base;
+    pdl_wait();                                  // the selection
+
+    // unit idx: (block of 64 tokens, pair), the blocks with the most chunks first; ln: its list buffer
+    auto unit_of = [&](int idx, int& blk, int& pair) { blk = n_blk - 1 - idx / pairs; pair = idx % pairs; };
+    bool ok = true;
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+        if (ok && !mbar_wait(bar, parity)) ok = false;
+        if (ok && *reinterpret_cast<volatile int*>(&sm.abort_flag)) ok = false;
+        return ok;
+    };
+
+    if (warp < kMmaWarp) {
+        // ================================================================ softmax: warp = head, lane = token
+        const int t = warp >> 2, h = warp & 3;
+        const uint32_t t_lane = tmem_base + (static_cast<uint32_t>(h * 32) << 16) + t * 256;
+        const float sl2 = s.scale * kLog2e;
+        uint32_t n_s = 0, n_u = 0;               // items of this tile / units so far
+        for (int idx = blockIdx.x; idx < n_units && ok; idx += gridDim.x, ++n_u) {
+            int blk, pair;
+            unit_of(idx, blk, pair);
+            const int ln = n_u & 1;
+            if (!wait(&sm.list_full[ln], (n_u >> 1) & 1)) break;
+            const int n = sm.n_items[ln];
+            const int b = pair / s.Hkv, gk = pair % s.Hkv;
+            const int tok = blk * kUnitTok + t * kTok + lane;
+            const bool live = tok < a.n_tok;
+            const int pos = s.pos0 + tok, lc = local_lo(pos, s.W, kS) / kS, ci = pos / kS;
+            const float* bias = a.bias ? a.bias + (static_cast<long long>(b) * s.Hl + gk) * s.C : nullptr;
+            float ref = -INFINITY, den = 0.f;
+            bool first = true;
+            for (int i = 0; i < n; ++i) {
+                const int e = sm.list[ln][i], c = e & 0xffff;
+                if (!((e >> (16 + t)) & 1)) continue;
+                const float bb = (bias && c < lc) ? bias[c] : 0.f;
+                const bool local = c >= lc;
+                const bool act = live && (local ? c <= ci : ((sm.mask[ln][t][c] >> lane) & 1u) != 0u);
+                if (!wait(&sm.s_full[t], n_s & 1)) break;
+                tc_fence_after_sync();
+                float v[64], lm4[4];
+                tmem_ld64_4(t_lane, t_lane + 64, v, lm4);
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sm.s_empty[t]);
+                const int lim = local ? pos - c * kS : kS - 1;           // last visible key
+                if (__any_sync(kFullMask, lim < kS - 1)) {
+#pragma unroll
+                    for (int j = 0; j < 64; ++j)
+                        if (j > lim) v[j] = -INFINITY;
+                }
+                float mx[4] = {v[0], v[1], v[2], v[3]};
+#pragma unroll
+                for (int j = 4; j < 60; j += 8) {
+                    mx[0] = fmax3(mx[0], v[j], v[j + 1]);
+                    mx[1] = fmax3(mx[1], v[j + 2], v[j + 3]);
+                    mx[2] = fmax3(mx[2], v[j + 4], v[j + 5]);
+                    mx[3] = fmax3(mx[3], v[j + 6], v[j + 7]);
+                }
+                mx[0] = fmax3(mx[0], v[60], v[61]);
+                mx[1] = fmax3(mx[1], v[62], v[63]);
+                float m = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+                if (m == -INFINITY) m = 0.f;                             // no visible key (the row gets weight zero)
+                const float2 sl22 = make_float2(sl2, sl2), nms2 = make_float2(-m * sl2, -m * sl2);
+                float2 zp[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    const float2 x = __ffma2_rn(make_float2(v[2 * j], v[2 * j + 1]), sl22, nms2);
+                    v[2 * j] = ex2_approx(x.x);
+                    v[2 * j + 1] = ex2_approx(x.y);
+                    zp[j & 3] = __fadd2_rn(zp[j & 3], make_float2(v[2 * j], v[2 * j + 1]));
+                }
+                const float2 z2 = __fadd2_rn(__fadd2_rn(zp[0], zp[1]), __fadd2_rn(zp[2], zp[3]));
+                const float z = z2.x + z2.y;
+                const float lam = local ? m * s.scale + __logf(z) : lm4[0] * s.scale + bb;
+                // mixing weight relative to the row's reference
+                float grow = 1.f;
+                if (act && lam > ref + kRaise) {
+                    grow = __expf(ref - lam);                            // (0 for the row's first chunk)
+                    den *= grow;
+                    ref = lam;
+                }
+                const float w = act ? __expf(lam - ref) : 0.f;
+                den += w;
+                const float pw = act ? w / z : 0.f;
+                const float2 pw2 = make_float2(pw, pw);
+                // the previous chunk's value product has read its probabilities and left the accumulator
+                if (!first) {
+                    if (!wait(&sm.o_done[t], (n_s - 1) & 1)) break;
+                    if (__any_sync(kFullMask, grow != 1.f)) {
+                        tc_fence_after_sync();
+#pragma unroll 1
+                        for (int cc = 0; cc < kD; cc += 16) {
+                            float o[16];
+                            tmem_ld16(t_lane + kOCol + cc, o);
+                            uint32_t r0[8], r1[8];
+#pragma unroll
+                            for (int x = 0; x < 8; ++x) { r0[x] = __float_as_uint(o[x] * grow); r1[x] = __float_as_uint(o[8 + x] * grow); }
+                            tmem_st8(t_lane + kOCol + cc, r0);
+                            tmem_st8(t_lane + kOCol + cc + 8, r1);
+                        }
+                    }
+                }
+                first = false;
+#pragma unroll
+                for (int pc = 0; pc < 4; ++pc) {
+                    uint32_t pk[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const float2 p = __fmul2_rn(make_float2(v[pc * 16 + 2 * j], v[pc * 16 + 2 * j + 1]), pw2);
+                        pk[j] = pack_bf16(p.x, p.y);
+                    }
+                    tmem_st8(t_lane + kPCol + pc * 8, pk);
+                }
+                tmem_wait_st();
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sm.p_full[t]);
+                ++n_s;
+            }
+            if (!ok) break;
+            if ((sm.parts[ln] >> t) & 1) {
+                // ---- the tile's output rows
+                if (!wait(&sm.o_done[t], (n_s - 1) & 1)) break;
+                tc_fence_after_sync();
+                const float inv = live ? 1.f / den : 0.f;
+                const long long orow = (static_cast<long long>(b) * s.Hq + gk * kG + h) * s.R + tok;
+                const bool whole = blk * kUnitTok + t * kTok + kTok <= a.n_tok;
+                uint8_t* stg = qbuf + t * kQBytes + h * 4096;            // this head's rows of the (no longer needed) query tile
+#pragma unroll
+                for (int half = 0; half < 4; ++half) {
+                    uint32_t v[32];
+                    tmem_ld32_issue(t_lane + kOCol + half * 32, v);
+                    tmem_ld_wait32(v);
+#pragma unroll
+                    for (int pc = 0; pc < 4; ++pc) {
+                        uint4 w;
+                        w.x = pack_bf16(__uint_as_float(v[8 * pc]) * inv, __uint_as_float(v[8 * pc + 1]) * inv);
+                        w.y = pack_bf16(__uint_as_float(v[8 * pc + 2]) * inv, __uint_as_float(v[8 * pc + 3]) * inv);
+                        w.z = pack_bf16(__uint_as_float(v[8 * pc + 4]) * inv, __uint_as_float(v[8 * pc + 5]) * inv);
+                        w.w = pack_bf16(__uint_as_float(v[8 * pc + 6]) * inv, __uint_as_float(v[8 * pc + 7]) * inv);
+                        if (whole) *reinterpret_cast<uint4*>(stg + (half >> 1) * 16384 + swz128(lane, (half & 1) * 4 + pc)) = w;
+                        else if (live) *reinterpret_cast<uint4*>(a.out + orow * kD + half * 32 + pc * 8) = w;
+                    }
+                }
+                tc_fence_before_sync();
+                if (live) a.lse[orow] = ref + __logf(den);
+                if (whole) {
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane < 2) {
+                        tma_store_2d(&map_out, stg + lane * 16384, lane * 64, static_cast<int>(orow) - lane, l2_policy_evict_first());
+                        bulk_commit();
+                        bulk_wait_read<0>();
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sm.q_empty[t]);
+            }
+            if (a.write_sel && h == 0 && live) {
+                int32_t* sel = a.sel + (static_cast<long long>(pair) * s.R + tok) * s.K;
+                for (int x = 0; x < s.K; ++x) sel[x] = x < lc ? x : -1;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.list_empty[ln]);
+        }
+    } else if (warp < kLoadWarp) {
+        // ================================================================ MMA issuer of tile t (one thread)
+        if (lane == 0) {
+            const int t = warp - kMmaWarp;
+            constexpr uint32_t idesc_s = umma_idesc_bf16(kRows, kNS);
+            constexpr uint32_t idesc_o = umma_idesc_bf16(kRows, kD) | kUmmaBMnMajor;
+            const uint32_t qa = smem_u32(qbuf + t * kQBytes), s_tm = tmem_base + t * 256;
+            uint32_t g0 = 0, n_s = 0, n_p = 0, n_q = 0, n_u = 0;         // first item of the unit; scores, products, query tiles so far
+            for (int idx = blockIdx.x; idx < n_units && ok; idx += gridDim.x, ++n_u) {
+                const int ln = n_u & 1;
+                if (!wait(&sm.list_full[ln], (n_u >> 1) & 1)) break;
+                const int n = sm.n_items[ln];
+                bool have_q = false, first = true;
+                int issued = -1;                                         // last item whose scores were issued
+                auto issue_s = [&](int i) {
+                    const uint32_t st = (g0 + i) % kStages;
+                    if (!have_q) { wait(&sm.q_full[t], n_q & 1); ++n_q; have_q = true; }
+                    wait(&sm.kv_full[st], ((g0 + i) / kStages) & 1);
+                    if (n_s > 0) wait(&sm.s_empty[t], (n_s - 1) & 1);
+                    if (!ok) return;
+                    tc_fence_after_sync();
+                    const uint32_t ka = smem_u32(kbuf + st * kKBytes);
+#pragma unroll
+                    for (int ks = 0; ks < 8; ++ks)
+                        umma_bf16(s_tm, umma_desc_k128(qa + (ks >> 2) * 16384 + (ks & 3) * 32),
+                                  umma_desc_k128(ka + (ks >> 2) * (kNS * 128) + (ks & 3) * 32), idesc_s, ks > 0 ? 1u : 0u);
+                    umma_commit(&sm.s_full[t]);
+                    ++n_s;
+                    issued = i;
+                };
+                for (int i = 0; i < n && ok; ++i) {
+                    const uint32_t st = (g0 + i) % kStages;
+                    if (!((sm.list[ln][i] >> (16 + t)) & 1)) {
+                        // not this tile's: hand the buffers back (once they are there: the barrier's phase is theirs then)
+                        if (wait(&sm.kv_full[st], ((g0 + i) / kStages) & 1)) mbar_arrive(&sm.kv_empty[st]);
+                        continue;
+                    }
+                    if (issued < i) issue_s(i);
+                    if (ok && i + 1 < n && ((sm.list[ln][i + 1] >> (16 + t)) & 1)) issue_s(i + 1);
+                    if (!ok || !wait(&sm.p_full[t], n_p & 1)) break;
+                    tc_fence_after_sync();
+                    const uint32_t va = smem_u32(vbuf + st * kVBytes);
+#pragma unroll
+                    for (int ks = 0; ks < 4; ++ks)
+                        umma_bf16_ts(s_tm + kOCol, s_tm + kPCol + ks * 8, umma_desc_mn128(va + ks * 2048, 8192u, 1024u), idesc_o,
+                                     (ks > 0 || !first) ? 1u : 0u);
+                    umma_commit(&sm.kv_empty[st]);
+                    umma_commit(&sm.o_done[t]);
+                    first = false;
+                    ++n_p;
+                }
+                g0 += static_cast<uint32_t>(n);
+                mbar_arrive(&sm.list_empty[ln]);
+            }
+        }
+    } else if (warp == kLoadWarp) {
+        // ================================================================ loader (one thread)
+        if (lane == 0) {
+            uint32_t g = 0, n_u = 0, n_q[2] = {0, 0};
+            for (int idx = blockIdx.x; idx < n_units && ok; idx += gridDim.x, ++n_u) {
+                int blk, pair;
+                unit_of(idx, blk, pair);
+                const int ln = n_u & 1;
+                if (!wait(&sm.list_full[ln], (n_u >> 1) & 1)) break;
+                const int n = sm.n_items[ln], parts = sm.parts[ln];
+                const int b = pair / s.Hkv, gk = pair % s.Hkv;
+                auto load_item = [&](int i) {
+                    const uint32_t st = g % kStages;
+                    const int c = sm.list[ln][i] & 0xffff;
+                    if (g >= kStages && !wait(&sm.kv_empty[st], ((g / kStages) - 1) & 1)) return;
+                    const int row = pair * s.T + c * kS;
+                    // chunks left of every token's window have a landmark row (the others' score column is not used)
+                    const bool lm = c < s.C;
+                    uint8_t* kd = kbuf + st * kKBytes;
+                    mbar_expect_tx(&sm.kv_full[st], 16384 + kVBytes + (lm ? 256 : 0));
+                    tma_load_2d(kd, &map_k, &sm.kv_full[st], 0, row);
+                    tma_load_2d(kd + kNS * 128, &map_k, &sm.kv_full[st], 64, row);
+                    if (lm) {
+                        // row 64: its 16-byte pieces stay in place under the swizzle (64 mod 8 = 0)
+                        const __nv_bfloat16* src = a.lm + ((static_cast<long long>(b) * s.Hl + gk) * s.C + c) * kD;
+                        bulk_load(kd + 64 * 128, src, 128, &sm.kv_full[st]);
+                        bulk_load(kd + kNS * 128 + 64 * 128, src + 64, 128, &sm.kv_full[st]);
+                    }
+                    tma_load_2d(vbuf + st * kVBytes, &map_v, &sm.kv_full[st], 0, row);
+                    tma_load_2d(vbuf + st * kVBytes + 8192, &map_v, &sm.kv_full[st], 64, row);
+                    ++g;
+                };
+                // the first chunks before the queries: their buffers are free before the last unit's rows have been written
+                int i = 0;
+                for (; i < n && i < kStages && ok; ++i) load_item(i);
+                for (int t = 0; t < 2 && ok; ++t) {
+                    if (!((parts >> t) & 1)) continue;
+                    if (n_q[t] > 0 && !wait(&sm.q_empty[t], (n_q[t] - 1) & 1)) break;
+                    mbar_expect_tx(&sm.q_full[t], kQBytes);
+                    for (int h = 0; h < kG; ++h) {
+                        const int row = (b * s.Hq + gk * kG + h) * s.R + blk * kUnitTok + t * kTok;
+                        tma_load_2d(qbuf + t * kQBytes + h * 4096, &map_q, &sm.q_full[t], 0, row);
+                        tma_load_2d(qbuf + t * kQBytes + 16384 + h * 4096, &map_q, &sm.q_full[t], 64, row);
+                    }
+                    ++n_q[t];
+                }
+                for (; i < n && ok; ++i) load_item(i);
+                mbar_arrive(&sm.list_empty[ln]);
+            }
+            // own copies in flight must have landed before the CTA leaves
+            for (uint32_t k = g > kStages ? g - kStages : 0; k < g; ++k) mbar_wait(&sm.kv_full[k % kStages], (k / kStages) & 1);
+        }
+    } else {
+        // ================================================================ the unit's chunk list, one unit ahead
+        uint32_t n_u = 0;
+        for (int idx = blockIdx.x; idx < n_units && ok; idx += gridDim.x, ++n_u) {
+            int blk, pair;
+            unit_of(idx, blk, pair);
+            const int ln = n_u & 1;
+            if (n_u >= 2 && !wait(&sm.list_empty[ln], ((n_u >> 1) - 1) & 1)) break;
+            const int tok0 = blk * kUnitTok;
+            const int last = s.pos0 + min(a.n_tok, tok0 + kUnitTok) - 1, n_vis = last / kS + 1;
+            for (int c = lane; c < n_vis; c += 32) { sm.mask[ln][0][c] = 0u; sm.mask[ln][1][c] = 0u; }
+            __syncwarp();
+            for (int t = 0; t < 2; ++t) {
+                const int tok = tok0 + t * kTok + lane, pos = s.pos0 + tok;
+                const bool live = tok < a.n_tok;
+                const int lc = live ? local_lo(pos, s.W, kS) / kS : 0;
+                const uint32_t bit = 1u << lane;
+                if (__all_sync(kFullMask, !live || lc <= s.K)) {
+                    // every token takes all its candidates
+                    const int most = __reduce_max_sync(kFullMask, lc);
+                    for (int c = 0; c < most; ++c) {
+                        const unsigned who = __ballot_sync(kFullMask, live && c < lc);
+                        if (lane == 0) sm.mask[ln][t][c] = who;
+                    }
+                } else if (live) {
+                    const int32_t* sel = a.sel + (static_cast<long long>(pair) * s.R + tok) * s.K;
+#pragma unroll 8
+                    for (int x = 0; x < s.K; ++x) {
+                        const int c = sel[x];
+                        if (c >= 0 && c < n_vis) atomicOr(&sm.mask[ln][t][c], bit);
+                    }
+                }
+                __syncwarp();
+                // chunks of the local windows
+                if (live)
+                    for (int c = lc; c <= pos / kS; ++c) atomicOr(&sm.mask[ln][t][c], bit);
+                __syncwarp();
+            }
+            int n = 0, parts = 0;
+            for (int c0 = 0; c0 < n_vis; c0 += 32) {
+                const int c = c0 + lane;
+                const bool m0 = c < n_vis && sm.mask[ln][0][c] != 0u, m1 = c < n_vis && sm.mask[ln][1][c] != 0u;
+                const unsigned v = __ballot_sync(kFullMask, m0 || m1);
+                if (m0 || m1) sm.list[ln][n + __popc(v & ((1u << lane) - 1u))] = c | (m0 ? 1 << 16 : 0) | (m1 ? 1 << 17 : 0);
+                parts |= (__any_sync(kFullMask, m0) ? 1 : 0) | (__any_sync(kFullMask, m1) ? 2 : 0);
+                n += __popc(v);
+            }
+            if (lane == 0) { sm.n_items[ln] = n; sm.parts[ln] = parts; }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.list_full[ln]);
+        }
+    }
+    if (!ok && lane == 0) { set_status(a.status, kDevTimeout); atomicExch(&sm.abort_flag, 1); }
+    __syncwarp();
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    if (warp == kMmaWarp) tmem_dealloc(tmem_base, 512);
+}
+
+}  // namespace
+
+// Tokens of a call (from its first on) that go this way; a multiple of 128 below the call's length, or all of them.
+// A tile of 32 tokens costs about 850 cycles per chunk it visits here, at most every visible one; chunk-major, a (token,
+// chunk) pair's share of tile, partial output and mix is about 3800 / 32 cycles per token: the line lies where the
+// visible chunks outnumber the attended ones 4 : 1.
+int prefill_query_tokens(const Shape& s) {
+    if (s.Hl != s.Hkv || s.K > 64) return 0;
+    const int nl = (s.W - 1 + kS - 1) / kS + 1;                          // chunks of a local window
+    int most = 4 * (s.K + nl);
+    if (most > kMaxC - 2) most = kMaxC - 2;
+    // tokens whose chunk is below `most`
+    const long long n = static_cast<long long>(most) * kS - s.pos0;
+    if (n <= 0) return 0;
+    if (n >= s.R) return s.R;
+    return static_cast<int>(n / 128 * 128);
+}
+
+int launch_prefill_query_tc(const Shape& s, const Tensors& t, int n_tok, int write_sel, cudaStream_t stream) {
+    const uint64_t kv_rows = static_cast<uint64_t>(s.B) * s.Hkv * s.T, q_rows = static_cast<uint64_t>(s.B) * s.Hq * s.R;
+    CUtensorMap map_q, map_k, map_v, map_out;
+    if (!make_bf16_2d_map(&map_q, t.q, q_rows, kD, 64, kTok) || !make_bf16_2d_map(&map_k, t.k, kv_rows, kD, 64, kS) ||
+        !make_bf16_2d_map(&map_v, t.v, kv_rows, kD, 64, kS) || !make_bf16_2d_map(&map_out, t.out, q_rows, kD, 64, kTok))
+        return HILS_ERR_CUDA;
+    const size_t smem = kStages * (kKBytes + kVBytes) + 2 * kQBytes + sizeof(QmSmem) + 1024;
+    static PerDeviceOnce once;
+    if (once.pending()) {
+        if (cudaFuncSetAttribute(prefill_query_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+            return HILS_ERR_CUDA;
+        once.done();
+    }
+    QmArgs a{s, static_cast<const __nv_bfloat16*>(t.landmarks), t.bias, t.sel_idx, static_cast<__nv_bfloat16*>(t.out), t.lse, t.status,
+             n_tok, write_sel};
+    const long long units = static_cast<long long>(s.B) * s.Hkv * ((n_tok + kUnitTok - 1) / kUnitTok);
+    const unsigned grid = static_cast<unsigned>(units < sm_count() ? units : sm_count());
+    if (launch_pdl(prefill_query_tc_kernel, dim3(grid), dim3(kThreads), smem, stream, map_q, map_k, map_v, map_out, a) != cudaSuccess)
+        return HILS_ERR_CUDA;
+    return 1;
+}
+
+}  // namespace hils

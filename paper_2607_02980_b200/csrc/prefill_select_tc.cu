@@ -40,7 +40,7 @@ struct TcArgs {
     // optional: per-(query block, pair, chunk) counts of the (token, slot) entries that attend each chunk -- the
     // first step of the inverse index, taken here because the selections are at hand (NULL: not wanted)
     int* cnt;
-    int qb, nc;        // tokens per query block (a multiple of the 128-token tile), chunk slots per pair in cnt
+    int qb, nc, t0;    // tokens per query block (a multiple of the 128-token tile), chunk slots per pair in cnt, first token counted
 };
 
 struct TcSmem {
@@ -127,7 +127,7 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         // candidates of a token = the chunks left of its local window (Sec. 2.1); the tile's last token has the most
         const int last_tok = min(s.R, (ti + 1) * kTileTok) - 1;
         const int ncand_max = local_lo(s.pos0 + last_tok, s.W, kS) / kS;
-        nsteps = (ncand_max + kS - 1) / kS;
+        nsteps = ncand_max <= K ? 0 : (ncand_max + kS - 1) / kS;        // (up to K candidates: all of them, no scores needed)
     };
 
     if (tid == 0) {
@@ -375,19 +375,19 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         // the survivors are the selection, already in ascending chunk order; -1 padded
         int ids[N];
 #pragma unroll
-        for (int e = 0; e < N; ++e) ids[e] = e < cnt ? static_cast<int>(pool[e * kTileTok] & 0xffffffffull) : -1;
+        for (int e = 0; e < N; ++e) ids[e] = nsteps == 0 ? (e < min(K, my_ncand) ? e : -1) : e < cnt ? static_cast<int>(pool[e * kTileTok] & 0xffffffffull) : -1;
         if (tok < s.R) {
             int32_t* sel = a.sel + (static_cast<long long>(pair) * s.R + tok) * K;
 #pragma unroll
             for (int e = 0; e < N; ++e)
                 if (e < K) sel[e] = ids[e];
         }
-        if (a.cnt) {
+        if (a.cnt && ti * kTileTok >= a.t0) {
             // chunk histogram of this tile's entries (selected chunks + the chunks of each token's local window) in the
             // pools' shared memory (every thread holds its ids in registers by now), then one global add per used bin
             int* hist = reinterpret_cast<int*>(lists);
             const bool in_smem = a.nc * sizeof(int) <= sizeof(unsigned long long) * 2 * kMaxK * kTileTok;
-            int* gcnt = a.cnt + (static_cast<long long>(ti * kTileTok / a.qb) * pairs + pair) * a.nc;
+            int* gcnt = a.cnt + (static_cast<long long>((ti * kTileTok - a.t0) / a.qb) * pairs + pair) * a.nc;
             asm volatile("bar.sync 1, 128;" ::: "memory");
             if (in_smem) {
                 for (int x = tid; x < a.nc; x += kTileTok) hist[x] = 0;
@@ -426,7 +426,7 @@ bool prefill_select_tc_supports(const Shape& s) {
 }
 
 int launch_prefill_select_tc(const Shape& s, const void* q, const void* landmarks, const float* bias, int32_t* sel,
-                             int* status, int* cnt, int qb, int nc, cudaStream_t stream) {
+                             int* status, int* cnt, int qb, int nc, int t0, cudaStream_t stream) {
     const int pairs = s.B * s.Hkv;
     CUtensorMap map_q, map_lm;
     if (!make_bf16_2d_map(&map_q, q, static_cast<uint64_t>(s.B) * s.Hq * s.R, kD, 64, kTileTok) ||
@@ -447,7 +447,7 @@ int launch_prefill_select_tc(const Shape& s, const void* q, const void* landmark
             return HILS_ERR_CUDA;
         attr_once.done();
     }
-    TcArgs a{s, bias, sel, status, (cnt && qb % kTileTok == 0) ? cnt : nullptr, qb, nc};
+    TcArgs a{s, bias, sel, status, (cnt && qb % kTileTok == 0) ? cnt : nullptr, qb, nc, t0};
     const int tiles = (s.R + kTileTok - 1) / kTileTok;
     const unsigned all_tiles = static_cast<unsigned>(pairs) * tiles;
     const unsigned nsm = static_cast<unsigned>(sm_count());
