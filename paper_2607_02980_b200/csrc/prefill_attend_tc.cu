@@ -84,6 +84,7 @@ struct AtcArgs {
     const int* entries;
     const int4* tiles;
     const int* n_tiles;
+    int segs;         // segments of a query block that are walked one after the other (n_tiles holds the first tile of each)
     float* lam;
     int* status;
     int i0;
@@ -156,17 +157,18 @@ prefill_attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
     // this kernel overwrites, or the inverse-index kernels).  From here on their results are needed.
     pdl_wait();
 
-    // Every role walks the same batches of tiles.  a.n_tiles[blk], a.n_tiles[blk + 1]: first tile of query block blk
-    // and of the next one; a launch that walks several blocks takes them in order, so that the CTAs stay on the same
+    // Every role walks the same batches of tiles.  a.n_tiles[x], a.n_tiles[x + 1]: first tile of segment x (a query block, or
+    // one pair of it) and of the next one; a launch that walks several blocks takes them in order, so that the CTAs stay on the same
     // block (its gathered Q rows stay in L2).  The walk is instantiated once per role.
     // body(nb, tcount, ccount, t_begin, i0): nb tiles cached in sm.recs, the CTA's running tile and chunk-run counters.
     auto walk = [&](auto&& body) {
         uint32_t tcount = 0, ccount = 0;
-        for (int blk = 0; blk < a.n_run; ++blk) {
-            const int t_begin = a.n_tiles[blk], n_tiles = a.n_tiles[blk + 1] - t_begin;
+        for (int sg = 0; sg < a.n_run * a.segs; ++sg) {
+            const int blk = sg / a.segs, t_begin = a.n_tiles[blk * a.segs];            // first tile of the query block
+            const int s_begin = a.n_tiles[sg], n_tiles = a.n_tiles[sg + 1] - s_begin;
             const int i0 = a.i0 + blk * a.qb;
-            const long long lo = t_begin + static_cast<long long>(blockIdx.x) * n_tiles / gridDim.x;
-            const long long hi = t_begin + static_cast<long long>(blockIdx.x + 1) * n_tiles / gridDim.x;
+            const long long lo = s_begin + static_cast<long long>(blockIdx.x) * n_tiles / gridDim.x;
+            const long long hi = s_begin + static_cast<long long>(blockIdx.x + 1) * n_tiles / gridDim.x;
             for (long long b0 = lo; b0 < hi; b0 += kBatch) {
                 const int nb = static_cast<int>(min(static_cast<long long>(kBatch), hi - b0));
                 for (int x = tid; x < nb; x += kThreads) sm.recs[x] = a.tiles[b0 + x];
@@ -604,7 +606,7 @@ prefill_attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
 int attend_tc_tile_tokens() { return kTok; }
 
 int launch_prefill_attend_tc(const Shape& s, const void* q, const void* maps, const void* landmarks,
-                             const float* bias, const int* entries, const void* tiles, const int* n_tiles, float* lam,
+                             const float* bias, const int* entries, const void* tiles, const int* n_tiles, int segs, float* lam,
                              int* status, int i0, int whole, int n_run, int qb, cudaStream_t stream) {
     const CUtensorMap* m = static_cast<const CUtensorMap*>(maps);
     const size_t smem = 2 * kKBytes + kVBufs * kVBytes + kQSlots * kQBytes + 2 * kPBytes + sizeof(AtcSmem) + 1024;
@@ -616,7 +618,7 @@ int launch_prefill_attend_tc(const Shape& s, const void* q, const void* maps, co
         attr_once.done();
     }
     AtcArgs a{s, static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(landmarks), bias, entries,
-              static_cast<const int4*>(tiles), n_tiles, lam, status, i0, whole, n_run, qb};
+              static_cast<const int4*>(tiles), n_tiles, segs, lam, status, i0, whole, n_run, qb};
     if (launch_pdl(prefill_attend_tc_kernel, dim3(sm_count()), dim3(kThreads), smem, stream, m[0], m[1], m[2], a) != cudaSuccess)
         return HILS_ERR_CUDA;
     if (cudaGetLastError() != cudaSuccess) return HILS_ERR_CUDA;

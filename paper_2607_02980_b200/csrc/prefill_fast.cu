@@ -44,6 +44,7 @@ struct PArgs {
     int* cnt;               // [n_blocks*pairs*nc] rows of each (block, pair, chunk): selectors + own tokens
     int* cursor;            // [pairs*C]
     int* blk_toff;          // [n_blocks + 1] first tile of every query block (tiles are grouped by block)
+    int* pair_toff;         // [n_blocks * pairs + 1] first tile of every (block, pair)
     int* seg_tiles;         // [ceil(lists / 1024)] tiles of each segment of 1024 lists
     int* off;               // [n_blocks*pairs*nc] first entry of each list; every list starts on a tile boundary
     int* entries;           // [max_tiles * tile_tok] (token_local << 8) | slot, grouped by (block, pair, chunk);
@@ -335,10 +336,14 @@ __global__ void __launch_bounds__(1024) invert_scan_kernel(const PArgs a) {
         a.off[x] = oe;
         const int pair = (x % per_blk) / a.nc, c = x % a.nc;
         if (x % per_blk == 0) a.blk_toff[x / per_blk] = ot;
+        if (c == 0) a.pair_toff[x / a.nc] = min(ot, a.max_tiles);
         for (int k = 0; k < ct; ++k)
             if (ot + k < a.max_tiles)
                 a.tiles[ot + k] = make_int4(pair, c, oe + k * a.tile_tok, min(a.tile_tok, ce - k * a.tile_tok));
-        if (x == n - 1) a.blk_toff[a.n_blocks] = min(ot + ct, a.max_tiles);
+        if (x == n - 1) {
+            a.blk_toff[a.n_blocks] = min(ot + ct, a.max_tiles);
+            a.pair_toff[n / a.nc] = min(ot + ct, a.max_tiles);
+        }
     }
 }
 
@@ -551,7 +556,7 @@ int pick_query_block(const Shape& s) {
 }
 struct Plan {
     int qb, nc, n_blocks, max_tiles, max_blk_tiles, whole;
-    size_t off_cnt, off_cursor, off_ntiles, zero_bytes, off_seg, off_off, off_entries, off_epos, off_tiles, off_obuf, off_lam,
+    size_t off_cnt, off_cursor, off_ntiles, off_ptiles, zero_bytes, off_seg, off_off, off_entries, off_epos, off_tiles, off_obuf, off_lam,
         total, obuf_tiles;
 };
 
@@ -588,6 +593,7 @@ Plan make_plan(const Shape& s, int qb_fixed = 0, int t0 = 0) {
     p.off_cursor = take(sizeof(int) * nblocks * pairs * nc);
     p.off_ntiles = take(sizeof(int) * (nblocks + 1));
     p.zero_bytes = off;                         // cnt, cursor, blk_toff are cleared together once per call
+    p.off_ptiles = take(sizeof(int) * (nblocks * pairs + 1));
     p.off_seg = take(sizeof(int) * ((nblocks * pairs * nc + 1023) / 1024));
     p.off_off = take(sizeof(int) * nblocks * pairs * nc);
     p.off_entries = take(sizeof(int) * all_tiles * tt);
@@ -637,6 +643,7 @@ int build_inverse_index(const Shape& s, const int32_t* sel, void* scratch, size_
     a.cnt = reinterpret_cast<int*>(sc + p.off_cnt);
     a.cursor = reinterpret_cast<int*>(sc + p.off_cursor);
     a.blk_toff = reinterpret_cast<int*>(sc + p.off_ntiles);
+    a.pair_toff = reinterpret_cast<int*>(sc + p.off_ptiles);
     a.n_blocks = p.n_blocks;
     a.seg_tiles = reinterpret_cast<int*>(sc + p.off_seg);
     a.off = reinterpret_cast<int*>(sc + p.off_off);
@@ -699,6 +706,7 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
     a.cnt = reinterpret_cast<int*>(sc + p.off_cnt);
     a.cursor = reinterpret_cast<int*>(sc + p.off_cursor);
     a.blk_toff = reinterpret_cast<int*>(sc + p.off_ntiles);
+    a.pair_toff = reinterpret_cast<int*>(sc + p.off_ptiles);
     a.n_blocks = p.n_blocks;
     a.blk = 0;
     a.seg_tiles = reinterpret_cast<int*>(sc + p.off_seg);
@@ -787,9 +795,13 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
         if (!a.whole || blk == 0) {
             // one launch per query block, or a single launch that walks all of them (whole-call output buffers)
             const CUtensorMap maps[3] = {map_k, map_v, map_o};
+            // With many tiles per (block, pair) the launch walks the pairs one after the other: all CTAs then gather the
+            // query rows of one KV head at a time (8 MB instead of 67 MB at 8192 tokens and 8 KV heads, which L2 keeps).
+            // Below some 40 tiles per CTA and pair the additional ends of chunk runs cost more.
+            const bool by_pair = static_cast<long long>(a.qb) * (s.K + max_local_slots(s.W)) >= 40ll * a.tile_tok * sm_count();
             const int rc = launch_prefill_attend_tc(s, t.q, maps, t.landmarks, t.bias, a.entries, a.tiles,
-                                                    a.blk_toff + blk, a.lam, t.status, a.i0, a.whole,
-                                                    a.whole ? p.n_blocks : 1, a.qb, stream);
+                                                    by_pair ? a.pair_toff + blk * pairs : a.blk_toff + blk, by_pair ? pairs : 1, a.lam,
+                                                    t.status, a.i0, a.whole, a.whole ? p.n_blocks : 1, a.qb, stream);
             if (rc < 0) return rc;
             trace_mark("prefill_attend", stream);
             ++launches;

@@ -62,11 +62,12 @@ struct QmSmem {
     uint64_t s_full[2], s_empty[2], p_full[2], o_done[2];
     uint64_t list_full[2], list_empty[2];
     uint32_t tmem_base;
-    int abort_flag;
     int n_items[2];                             // items of the unit's list
     int parts[2];                               // bit t: tile t has items
     int list[2][kMaxC];                         // chunk | tile 0 needs it << 16 | tile 1 needs it << 17
-    uint32_t mask[2][2][kMaxC];                 // [list][tile][chunk]: tokens that selected it
+    uint32_t mask[2][kMaxC];                    // (list builder) [tile][chunk]: tokens that attend it
+    int n_tile[2][2];                           // [list][tile]: items of the tile
+    int2 titem[2][2][kMaxC];                    // [list][tile][item]: chunk, tokens that attend it
 };
 static_assert(kStages * (kKBytes + kVBytes) + 2 * kQBytes + sizeof(QmSmem) + 1024 <= 232448, "shared memory of the query-major kernel");
 
@@ -74,6 +75,23 @@ __device__ __forceinline__ float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+// 2^x of two values on the FMA pipes: x = n + f with f in [-1/2, 1/2] (Cody-Waite), a polynomial of degree 5 in f fitted
+// to the smallest relative error (1e-7), n added to the exponent.  A quarter of a row's exponentials goes this way: the
+// special-function unit takes 8 cycles per warp and exponential and is the busiest unit of the softmax warps.
+__device__ __forceinline__ float2 ex2_fma(float2 x) {
+    x.x = fmaxf(x.x, -126.f);
+    x.y = fmaxf(x.y, -126.f);
+    const float2 t = __fadd2_rn(x, make_float2(12582912.f, 12582912.f));            // 1.5 * 2^23: rounds to an integer
+    const float2 n = __fadd2_rn(t, make_float2(-12582912.f, -12582912.f));
+    const float2 f = __ffma2_rn(n, make_float2(-1.f, -1.f), x);
+    float2 p = __ffma2_rn(make_float2(0.00132765f, 0.00132765f), f, make_float2(0.00967554f, 0.00967554f));
+    p = __ffma2_rn(p, f, make_float2(0.05550713f, 0.05550713f));
+    p = __ffma2_rn(p, f, make_float2(0.24022120f, 0.24022120f));
+    p = __ffma2_rn(p, f, make_float2(0.69314697f, 0.69314697f));
+    p = __ffma2_rn(p, f, make_float2(1.00000007f, 1.00000007f));
+    return make_float2(__int_as_float(__float_as_int(p.x) + (__float_as_int(t.x) << 23)),
+                       __int_as_float(__float_as_int(p.y) + (__float_as_int(t.y) << 23)));
 }
 __device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, uint32_t bytes, uint64_t* bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
@@ -101,7 +119,6 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             mbar_init(&sm.list_full[t], 1); mbar_init(&sm.list_empty[t], 11);
         }
         mbar_fence_init();
-        sm.abort_flag = 0;
         tma_prefetch_desc(&map_q);
         tma_prefetch_desc(&map_k);
         tma_prefetch_desc(&map_v);
@@ -121,11 +138,21 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
     pdl_wait();                                  // the selection
 
     // unit idx: (block of 64 tokens, pair), the blocks with the most chunks first; ln: its list buffer
-    auto unit_of = [&](int idx, int& blk, int& pair) { blk = n_blk - 1 - idx / pairs; pair = idx % pairs; };
+    // (every other round of the walk runs backwards: the units get lighter along it, and a CTA that was early in one round
+    // is late in the next)
+    auto unit_of = [&](int idx, int& blk, int& pair) {
+        const int rnd = idx / static_cast<int>(gridDim.x);
+        if (rnd & 1) {
+            const int end = min(n_units, (rnd + 1) * static_cast<int>(gridDim.x)) - 1;
+            idx = end - (idx - rnd * static_cast<int>(gridDim.x));
+        }
+        blk = n_blk - 1 - idx / pairs;
+        pair = idx % pairs;
+    };
     bool ok = true;
+    // (a test first: where the phase is over, as it mostly is, a test costs about half of a try_wait)
     auto wait = [&](uint64_t* bar, uint32_t parity) {
-        if (ok && !mbar_wait(bar, parity)) ok = false;
-        if (ok && *reinterpret_cast<volatile int*>(&sm.abort_flag)) ok = false;
+        if (ok && !mbar_test_wait(bar, parity) && !mbar_wait(bar, parity)) ok = false;
         return ok;
     };
 
@@ -140,20 +167,21 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             unit_of(idx, blk, pair);
             const int ln = n_u & 1;
             if (!wait(&sm.list_full[ln], (n_u >> 1) & 1)) break;
-            const int n = sm.n_items[ln];
+            const int n = sm.n_tile[ln][t];
             const int b = pair / s.Hkv, gk = pair % s.Hkv;
             const int tok = blk * kUnitTok + t * kTok + lane;
             const bool live = tok < a.n_tok;
             const int pos = s.pos0 + tok, lc = local_lo(pos, s.W, kS) / kS, ci = pos / kS;
             const float* bias = a.bias ? a.bias + (static_cast<long long>(b) * s.Hl + gk) * s.C : nullptr;
             float ref = -INFINITY, den = 0.f;
-            bool first = true;
+            int2 next = n > 0 ? sm.titem[ln][t][0] : make_int2(0, 0);
             for (int i = 0; i < n; ++i) {
-                const int e = sm.list[ln][i], c = e & 0xffff;
-                if (!((e >> (16 + t)) & 1)) continue;
+                const int c = next.x;
+                const uint32_t who = static_cast<uint32_t>(next.y);
+                if (i + 1 < n) next = sm.titem[ln][t][i + 1];
                 const float bb = (bias && c < lc) ? bias[c] : 0.f;
                 const bool local = c >= lc;
-                const bool act = live && (local ? c <= ci : ((sm.mask[ln][t][c] >> lane) & 1u) != 0u);
+                const bool act = ((who >> lane) & 1u) != 0u;
                 if (!wait(&sm.s_full[t], n_s & 1)) break;
                 tc_fence_after_sync();
                 float v[64], lm4[4];
@@ -184,10 +212,18 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
                     const float2 x = __ffma2_rn(make_float2(v[2 * j], v[2 * j + 1]), sl22, nms2);
-                    v[2 * j] = ex2_approx(x.x);
-                    v[2 * j + 1] = ex2_approx(x.y);
+                    if ((j & 3) == 3) {
+                        const float2 y = ex2_fma(x);
+                        v[2 * j] = y.x;
+                        v[2 * j + 1] = y.y;
+                    } else {
+                        v[2 * j] = ex2_approx(x.x);
+                        v[2 * j + 1] = ex2_approx(x.y);
+                    }
                     zp[j & 3] = __fadd2_rn(zp[j & 3], make_float2(v[2 * j], v[2 * j + 1]));
                 }
+                // (asked here, needed below: the answer arrives under the arithmetic)
+                const bool o_ready = i == 0 || mbar_test_wait(&sm.o_done[t], (n_s - 1) & 1);
                 const float2 z2 = __fadd2_rn(__fadd2_rn(zp[0], zp[1]), __fadd2_rn(zp[2], zp[3]));
                 const float z = z2.x + z2.y;
                 const float lam = local ? m * s.scale + __logf(z) : lm4[0] * s.scale + bb;
@@ -203,8 +239,8 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                 const float pw = act ? w / z : 0.f;
                 const float2 pw2 = make_float2(pw, pw);
                 // the previous chunk's value product has read its probabilities and left the accumulator
-                if (!first) {
-                    if (!wait(&sm.o_done[t], (n_s - 1) & 1)) break;
+                if (i > 0) {
+                    if (!o_ready && !wait(&sm.o_done[t], (n_s - 1) & 1)) break;
                     if (__any_sync(kFullMask, grow != 1.f)) {
                         tc_fence_after_sync();
 #pragma unroll 1
@@ -219,7 +255,6 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                         }
                     }
                 }
-                first = false;
 #pragma unroll
                 for (int pc = 0; pc < 4; ++pc) {
                     uint32_t pk[8];
@@ -237,7 +272,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                 ++n_s;
             }
             if (!ok) break;
-            if ((sm.parts[ln] >> t) & 1) {
+            if (n > 0) {
                 // ---- the tile's output rows
                 if (!wait(&sm.o_done[t], (n_s - 1) & 1)) break;
                 tc_fence_after_sync();
@@ -399,7 +434,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             if (n_u >= 2 && !wait(&sm.list_empty[ln], ((n_u >> 1) - 1) & 1)) break;
             const int tok0 = blk * kUnitTok;
             const int last = s.pos0 + min(a.n_tok, tok0 + kUnitTok) - 1, n_vis = last / kS + 1;
-            for (int c = lane; c < n_vis; c += 32) { sm.mask[ln][0][c] = 0u; sm.mask[ln][1][c] = 0u; }
+            for (int c = lane; c < n_vis; c += 32) { sm.mask[0][c] = 0u; sm.mask[1][c] = 0u; }
             __syncwarp();
             for (int t = 0; t < 2; ++t) {
                 const int tok = tok0 + t * kTok + lane, pos = s.pos0 + tok;
@@ -411,37 +446,49 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                     const int most = __reduce_max_sync(kFullMask, lc);
                     for (int c = 0; c < most; ++c) {
                         const unsigned who = __ballot_sync(kFullMask, live && c < lc);
-                        if (lane == 0) sm.mask[ln][t][c] = who;
+                        if (lane == 0) sm.mask[t][c] = who;
                     }
                 } else if (live) {
                     const int32_t* sel = a.sel + (static_cast<long long>(pair) * s.R + tok) * s.K;
 #pragma unroll 8
                     for (int x = 0; x < s.K; ++x) {
                         const int c = sel[x];
-                        if (c >= 0 && c < n_vis) atomicOr(&sm.mask[ln][t][c], bit);
+                        if (c >= 0 && c < n_vis) atomicOr(&sm.mask[t][c], bit);
                     }
                 }
                 __syncwarp();
                 // chunks of the local windows
                 if (live)
-                    for (int c = lc; c <= pos / kS; ++c) atomicOr(&sm.mask[ln][t][c], bit);
+                    for (int c = lc; c <= pos / kS; ++c) atomicOr(&sm.mask[t][c], bit);
                 __syncwarp();
             }
-            int n = 0, parts = 0;
+            int n = 0, nt[2] = {0, 0};
             for (int c0 = 0; c0 < n_vis; c0 += 32) {
                 const int c = c0 + lane;
-                const bool m0 = c < n_vis && sm.mask[ln][0][c] != 0u, m1 = c < n_vis && sm.mask[ln][1][c] != 0u;
-                const unsigned v = __ballot_sync(kFullMask, m0 || m1);
-                if (m0 || m1) sm.list[ln][n + __popc(v & ((1u << lane) - 1u))] = c | (m0 ? 1 << 16 : 0) | (m1 ? 1 << 17 : 0);
-                parts |= (__any_sync(kFullMask, m0) ? 1 : 0) | (__any_sync(kFullMask, m1) ? 2 : 0);
+                const uint32_t below = (1u << lane) - 1u;
+                uint32_t m[2];
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                    m[t] = c < n_vis ? sm.mask[t][c] : 0u;
+                    const unsigned v = __ballot_sync(kFullMask, m[t] != 0u);
+                    if (m[t]) sm.titem[ln][t][nt[t] + __popc(v & below)] = make_int2(c, static_cast<int>(m[t]));
+                    nt[t] += __popc(v);
+                }
+                const unsigned v = __ballot_sync(kFullMask, (m[0] | m[1]) != 0u);
+                if (m[0] | m[1]) sm.list[ln][n + __popc(v & below)] = c | (m[0] ? 1 << 16 : 0) | (m[1] ? 1 << 17 : 0);
                 n += __popc(v);
             }
-            if (lane == 0) { sm.n_items[ln] = n; sm.parts[ln] = parts; }
+            if (lane == 0) {
+                sm.n_items[ln] = n;
+                sm.n_tile[ln][0] = nt[0];
+                sm.n_tile[ln][1] = nt[1];
+                sm.parts[ln] = (nt[0] > 0 ? 1 : 0) | (nt[1] > 0 ? 2 : 0);
+            }
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.list_full[ln]);
         }
     }
-    if (!ok && lane == 0) { set_status(a.status, kDevTimeout); atomicExch(&sm.abort_flag, 1); }
+    if (!ok && lane == 0) set_status(a.status, kDevTimeout);
     __syncwarp();
     tc_fence_before_sync();
     __syncthreads();
@@ -452,13 +499,13 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
 }  // namespace
 
 // Tokens of a call (from its first on) that go this way; a multiple of 128 below the call's length, or all of them.
-// A tile of 32 tokens costs about 850 cycles per chunk it visits here, at most every visible one; chunk-major, a (token,
-// chunk) pair's share of tile, partial output and mix is about 3800 / 32 cycles per token: the line lies where the
-// visible chunks outnumber the attended ones 4 : 1.
+// A tile of 32 tokens costs about 1850 cycles per chunk it visits here, at most every visible one; chunk-major (index, attend
+// and fuse kernels), 32 tokens cost 4600 cycles per chunk they attend: the line lies where the visible chunks outnumber the
+// attended ones 5 : 2.
 int prefill_query_tokens(const Shape& s) {
     if (s.Hl != s.Hkv || s.K > 64) return 0;
     const int nl = (s.W - 1 + kS - 1) / kS + 1;                          // chunks of a local window
-    int most = 4 * (s.K + nl);
+    int most = 5 * (s.K + nl) / 2;
     if (most > kMaxC - 2) most = kMaxC - 2;
     // tokens whose chunk is below `most`
     const long long n = static_cast<long long>(most) * kS - s.pos0;

@@ -121,7 +121,10 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     // A CTA walks the tiles blockIdx.x, blockIdx.x + gridDim.x, ... (heavy tiles first): the query tile and the first
     // scores of the next tile are fetched and computed while the epilogue still finishes the previous one.  Every
     // role derives the same tile sequence; tiles without candidates touch no barrier.
+    // (Every other round of the walk runs backwards, so that a CTA early in one round, with heavy tiles, is late in the next.)
     auto tile_of = [&](int idx, int& ti, int& pair, int& nsteps) {
+        const int rnd = idx / static_cast<int>(gridDim.x);
+        if (rnd & 1) idx = min(n_tiles, (rnd + 1) * static_cast<int>(gridDim.x)) - 1 - (idx - rnd * static_cast<int>(gridDim.x));
         ti = tiles_per_seq - 1 - idx / pairs;
         pair = idx % pairs;
         // candidates of a token = the chunks left of its local window (Sec. 2.1); the tile's last token has the most
