@@ -147,128 +147,184 @@ __global__ void landmark_summary_kernel(const LArgs a) {
 }
 
 // ---- bf16, d = 128, S = 64, at most 8 landmark heads per KV head: both contractions on mma.sync ----
-// One warp per (sequence, KV head, chunk): the chunk's keys arrive as two TMA boxes (128B swizzle) in the warp's
-// own 16 KB tile; scores of all landmark heads of the KV head in one pass (the heads are the MMA rows), then
-// k' = P K with P split into two bf16 terms (p = hi + lo), so that the weights keep 16 bits of mantissa.
-constexpr int kTcWarps = 4;
+// Persistent: one CTA of 14 warps per SM.  A warp owns a 16 KB stage and takes every 14th (sequence, KV head, chunk) item of
+// the CTA: the keys arrive by TMA, and the next item's are requested as soon as this one's have been read.
+// S^T = K q'^T with the keys in the MMA rows and the landmark heads of the KV head in its columns, then k'^T = K^T P^T
+// with P split into two bf16 terms (p = hi + lo), so that the weights keep 16 bits of mantissa.
+// Bound: HBM, reached by the number of warps (an item takes a warp 2 us of dependent steps): 8 x 64K ragged tokens, 8 KV
+// heads: 168 us with a CTA per four chunks (load, compute, leave), 155 with 7 warps of two stages, 122 (6.1 TB/s) with 14.
+constexpr int kTcWarps = 14;
 constexpr int kTcTileBytes = 64 * 128 * 2;
 
-struct TcSmemW {
-    uint64_t bar;
-};
+__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t x) {
+    uint32_t y;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
+    return y;
+}
 
-__global__ void __launch_bounds__(kTcWarps * 32)
-landmark_summary_tc_kernel(const __grid_constant__ CUtensorMap map_k, const LArgs a, int* timeout_flag) {
+__global__ void __launch_bounds__(kTcWarps * 32, 1)
+landmark_summary_tc_kernel(const __grid_constant__ CUtensorMap map_k, const LArgs a) {
     extern __shared__ uint8_t lsm_raw[];
-    uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(lsm_raw) + 1023) & ~uintptr_t(1023));
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint8_t* tile = base + warp * kTcTileBytes;
-    TcSmemW& sw = reinterpret_cast<TcSmemW*>(base + kTcWarps * kTcTileBytes)[warp];
-    const int per = a.Hl / a.Hkv;                              // landmark heads per KV head (MMA rows), <= 8
-    const long long item = static_cast<long long>(blockIdx.x) * kTcWarps + warp;
-    const long long total = static_cast<long long>(a.B) * a.Hkv * a.cn;
-    if (item >= total) return;
-    const int c = a.c0 + static_cast<int>(item % a.cn);
-    const int hkv = static_cast<int>((item / a.cn) % a.Hkv);
-    const int b = static_cast<int>(item / (static_cast<long long>(a.cn) * a.Hkv));
-    long long len = a.seq ? a.seq[b] : a.T;
-    len = len < 0 ? 0 : (len > a.T ? a.T : len);
-    const long long j0 = static_cast<long long>(c) * 64;
-    const int n = static_cast<int>(len - j0 < 0 ? 0 : (len - j0 > 64 ? 64 : len - j0));
-    const int gq = lane >> 2, t = lane & 3;
-    const long long orow0 = (static_cast<long long>(b) * a.Hl + hkv * per) * a.C + c;      // head 0 of this KV head
+    __shared__ uint64_t full[kTcWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    uint8_t* tile = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(lsm_raw) + 1023) & ~uintptr_t(1023)) + warp * kTcTileBytes;
+    const uint32_t addr = smem_u32(tile);
+    uint64_t* bar = &full[warp];
+    const int per = a.Hl / a.Hkv;                              // landmark heads per KV head (MMA columns), <= 8
+    const int total = a.B * a.Hkv * a.cn;
     __nv_bfloat16* lm = static_cast<__nv_bfloat16*>(a.lm);
-    if (n == 0) {
-        for (int x = lane; x < per * 64; x += 32)
-            *reinterpret_cast<uint32_t*>(lm + (orow0 + static_cast<long long>(x >> 6) * a.C) * 128 + (x & 63) * 2) = 0u;
-        if (lane < per) a.bias[orow0 + static_cast<long long>(lane) * a.C] = 0.f;
-        return;
-    }
+    struct Item { int b, hkv, c, n; };
+    auto item_of = [&](int k) {                                // item k of this CTA
+        Item it;
+        const int x = blockIdx.x + k * static_cast<int>(gridDim.x), u = x / a.cn;
+        it.c = a.c0 + (x - u * a.cn);
+        it.b = u / a.Hkv;
+        it.hkv = u - it.b * a.Hkv;
+        long long len = a.seq ? a.seq[it.b] : a.T;
+        len = len < 0 ? 0 : (len > a.T ? a.T : len);
+        const long long left = len - static_cast<long long>(it.c) * 64;
+        it.n = static_cast<int>(left < 0 ? 0 : (left > 64 ? 64 : left));
+        return it;
+    };
+    auto out_row = [&](const Item& it) { return (static_cast<long long>(it.b) * a.Hl + it.hkv * per) * a.C + it.c; };    // head 0
+    auto request = [&](const Item& it) {                       // one lane
+        if (it.n == 0) return;
+        const int row = static_cast<int>((static_cast<long long>(it.b) * a.Hkv + it.hkv) * a.T + static_cast<long long>(it.c) * 64);
+        mbar_expect_tx(bar, kTcTileBytes);
+        tma_load_2d(tile, &map_k, bar, 0, row);
+        tma_load_2d(tile + 8192, &map_k, bar, 64, row);
+    };
+    const int n_items = (total - static_cast<int>(blockIdx.x) + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x);
+    if (warp >= n_items) return;
+    Item cur = item_of(warp);
     if (lane == 0) {
-        mbar_init(&sw.bar, 1);
+        mbar_init(bar, 1);
         mbar_fence_init();
-        const int row = static_cast<int>((static_cast<long long>(b) * a.Hkv + hkv) * a.T + j0);
-        mbar_expect_tx(&sw.bar, kTcTileBytes);
-        tma_load_2d(tile, &map_k, &sw.bar, 0, row);
-        tma_load_2d(tile + 8192, &map_k, &sw.bar, 64, row);
-    }
-    // A operand: the `per` learnable queries of this KV head in rows 0..per-1 (loaded while the keys travel)
-    uint32_t aq[8][2];
-#pragma unroll
-    for (int ks = 0; ks < 8; ++ks) { aq[ks][0] = 0u; aq[ks][1] = 0u; }
-    if (gq < per) {
-        const __nv_bfloat16* qrow = static_cast<const __nv_bfloat16*>(a.lq) + (orow0 + static_cast<long long>(gq) * a.C) * 128;
-#pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
-            aq[ks][0] = *reinterpret_cast<const uint32_t*>(qrow + ks * 16 + 2 * t);
-            aq[ks][1] = *reinterpret_cast<const uint32_t*>(qrow + ks * 16 + 8 + 2 * t);
-        }
+        request(cur);
     }
     __syncwarp();
-    if (!mbar_wait(&sw.bar, 0)) {
-        // the bounded wait ran out (never seen: the copy has a valid map): mark the chunk's bias NaN and leave
-        if (lane == 0 && timeout_flag) atomicExch(timeout_flag, 1);
-        if (lane < per) a.bias[orow0 + static_cast<long long>(lane) * a.C] = __int_as_float(0x7fc00000);
-        return;
-    }
-    if (n < 64) {
-        // rows past the sequence end may hold anything: zero them before they meet probabilities of 0
-        for (int x = lane; x < (64 - n) * 16; x += 32) {
-            const int row = n + (x >> 4), piece = x & 15;
-            *reinterpret_cast<uint4*>(tile + (piece >> 3) * 8192 + swz128(row, piece & 7)) = make_uint4(0u, 0u, 0u, 0u);
+    uint32_t phase = 0u;
+    for (int k = warp; k < n_items; k += kTcWarps) {
+        const Item next = k + kTcWarps < n_items ? item_of(k + kTcWarps) : Item{0, 0, 0, 0};
+        const long long orow0 = out_row(cur);
+        uint32_t q[8][2];                                      // column g: landmark head g of the KV head
+        {
+            const bool ok = cur.n > 0 && g < per;
+            const __nv_bfloat16* row = static_cast<const __nv_bfloat16*>(a.lq) + (orow0 + static_cast<long long>(ok ? g : 0) * a.C) * 128;
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks) {
+                q[ks][0] = ok ? *reinterpret_cast<const uint32_t*>(row + ks * 16 + 2 * t) : 0u;
+                q[ks][1] = ok ? *reinterpret_cast<const uint32_t*>(row + ks * 16 + 8 + 2 * t) : 0u;
+            }
         }
-        __syncwarp();
-    }
-    const uint32_t ks_addr = smem_u32(tile);
-    float sc[8][4];
-    qk_tile(aq, ks_addr, lane, sc);                             // sc[nt][0..1]: row gq, keys nt*8 + 2t, +1
-    const float sl = a.scale;
-    float m = -INFINITY;
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-        const int key = nt * 8 + 2 * t;
-        sc[nt][0] = key < n ? sc[nt][0] * sl : -INFINITY;
-        sc[nt][1] = key + 1 < n ? sc[nt][1] * sl : -INFINITY;
-        m = fmaxf(m, fmaxf(sc[nt][0], sc[nt][1]));
-    }
-    m = fmaxf(m, __shfl_xor_sync(kFullMask, m, 1));
-    m = fmaxf(m, __shfl_xor_sync(kFullMask, m, 2));
-    float z = 0.f, ps = 0.f, e[8][2];
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-        e[nt][0] = sc[nt][0] == -INFINITY ? 0.f : __expf(sc[nt][0] - m);
-        e[nt][1] = sc[nt][1] == -INFINITY ? 0.f : __expf(sc[nt][1] - m);
-        z += e[nt][0] + e[nt][1];
-    }
-    z += __shfl_xor_sync(kFullMask, z, 1);
-    z += __shfl_xor_sync(kFullMask, z, 2);
-    const float zi = 1.f / z;
-    float phi[8][4], plo[8][4];
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-#pragma unroll
-        for (int x = 0; x < 2; ++x) {
-            const float p = e[nt][x] * zi;
-            if (p > 0.f) ps = fmaf(p, sc[nt][x] - m, ps);
-            const float hi = __bfloat162float(__float2bfloat16_rn(p));
-            phi[nt][x] = hi;
-            plo[nt][x] = p - hi;
+        if (cur.n == 0) {
+            for (int y = lane; y < per * 64; y += 32)
+                *reinterpret_cast<uint32_t*>(lm + (orow0 + static_cast<long long>(y >> 6) * a.C) * 128 + (y & 63) * 2) = 0u;
+            if (lane < per) a.bias[orow0 + static_cast<long long>(lane) * a.C] = 0.f;
         }
-        phi[nt][2] = phi[nt][3] = plo[nt][2] = plo[nt][3] = 0.f;
-    }
-    ps += __shfl_xor_sync(kFullMask, ps, 1);
-    ps += __shfl_xor_sync(kFullMask, ps, 2);
-    float o[16][4];
+        float o[8][4], bias[2] = {0.f, 0.f};
+        if (cur.n > 0) {
+            if (!mbar_wait(bar, phase)) {
+                // the bounded wait ran out (never seen: the copy has a valid map): mark the chunk's bias NaN and leave
+                if (lane < per) a.bias[orow0 + static_cast<long long>(lane) * a.C] = __int_as_float(0x7fc00000);
+                return;
+            }
+            phase ^= 1u;
+            const int n = cur.n;
+            if (n < 64) {
+                // rows past the sequence end may hold anything: zero them before they meet probabilities of 0
+                for (int y = lane; y < (64 - n) * 16; y += 32) {
+                    const int row = n + (y >> 4), piece = y & 15;
+                    *reinterpret_cast<uint4*>(tile + (piece >> 3) * 8192 + swz128(row, piece & 7)) = make_uint4(0u, 0u, 0u, 0u);
+                }
+                __syncwarp();
+                fence_proxy_async_smem();                      // (the stage is overwritten by a bulk copy later)
+            }
+            float sc[4][4];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
-    pv_tile(phi, ks_addr, lane, o);                             // the keys are the "values" of Attn(q', K, K)
-    pv_tile(plo, ks_addr, lane, o);
-    if (gq < per) {
-        __nv_bfloat16* dst = lm + (orow0 + static_cast<long long>(gq) * a.C) * 128;
+            for (int mt = 0; mt < 4; ++mt) sc[mt][0] = sc[mt][1] = sc[mt][2] = sc[mt][3] = 0.f;
 #pragma unroll
-        for (int i = 0; i < 16; ++i)
-            *reinterpret_cast<uint32_t*>(dst + i * 8 + 2 * t) = pack_bf16(o[i][0], o[i][1]);
-        if (t == 0) a.bias[orow0 + static_cast<long long>(gq) * a.C] = __logf(z) - ps;
+            for (int ks = 0; ks < 8; ++ks)
+#pragma unroll
+                for (int mt = 0; mt < 4; ++mt) {
+                    const int row = mt * 16 + (lane & 7) + ((lane >> 3) & 1) * 8, dim = ks * 16 + (lane >> 4) * 8;
+                    uint32_t fr[4];
+                    ldmatrix_x4(addr + (dim >> 6) * 8192 + swz128(row, (dim & 63) >> 3), fr[0], fr[1], fr[2], fr[3]);
+                    mma_bf16_16816(sc[mt], fr, q[ks][0], q[ks][1]);
+                }
+            // columns 2 t, 2 t + 1; rows (keys) 16 mt + g, + 8
+            uint32_t hi[4][2], lo[4][2];
+            float p[4][4];
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+                float m = -INFINITY;
+#pragma unroll
+                for (int mt = 0; mt < 4; ++mt) {
+                    sc[mt][y] = mt * 16 + g < n ? sc[mt][y] * a.scale : -INFINITY;
+                    sc[mt][2 + y] = mt * 16 + 8 + g < n ? sc[mt][2 + y] * a.scale : -INFINITY;
+                    m = fmaxf(m, fmaxf(sc[mt][y], sc[mt][2 + y]));
+                }
+#pragma unroll
+                for (int x = 4; x < 32; x <<= 1) m = fmaxf(m, __shfl_xor_sync(kFullMask, m, x));
+                float z = 0.f, ps = 0.f;                       // ps = sum e (s - m)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    float& s_ = sc[i >> 1][(i & 1) * 2 + y];
+                    const float e = __expf(s_ - m);
+                    z += e;
+                    if (e > 0.f) ps = fmaf(e, s_ - m, ps);
+                    p[i >> 1][(i & 1) * 2 + y] = e;
+                }
+#pragma unroll
+                for (int x = 4; x < 32; x <<= 1) {
+                    z += __shfl_xor_sync(kFullMask, z, x);
+                    ps += __shfl_xor_sync(kFullMask, ps, x);
+                }
+                const float zi = 1.f / z;
+#pragma unroll
+                for (int mt = 0; mt < 4; ++mt) { p[mt][y] *= zi; p[mt][2 + y] *= zi; }
+                bias[y] = __logf(z) - ps * zi;
+            }
+#pragma unroll
+            for (int mt = 0; mt < 4; ++mt)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const __nv_bfloat16 h0 = __float2bfloat16_rn(p[mt][2 * h]), h1 = __float2bfloat16_rn(p[mt][2 * h + 1]);
+                    const float f0 = __bfloat162float(h0), f1 = __bfloat162float(h1);
+                    hi[mt][h] = movmatrix_trans(pack_bf16(f0, f1));
+                    lo[mt][h] = movmatrix_trans(pack_bf16(p[mt][2 * h] - f0, p[mt][2 * h + 1] - f1));
+                }
+#pragma unroll
+            for (int mt = 0; mt < 8; ++mt) o[mt][0] = o[mt][1] = o[mt][2] = o[mt][3] = 0.f;
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+                for (int mt = 0; mt < 8; ++mt) {
+                    const int row = kk * 16 + (lane >> 4) * 8 + (lane & 7), dim = mt * 16 + ((lane >> 3) & 1) * 8;
+                    uint32_t fr[4];
+                    ldmatrix_x4_trans(addr + (dim >> 6) * 8192 + swz128(row, (dim & 63) >> 3), fr[0], fr[1], fr[2], fr[3]);
+                    mma_bf16_16816(o[mt], fr, hi[kk][0], hi[kk][1]);
+                    mma_bf16_16816(o[mt], fr, lo[kk][0], lo[kk][1]);
+                }
+        }
+        __syncwarp();                                          // every lane has read the stage
+        if (lane == 0) request(next);
+        if (cur.n > 0) {
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+                const int h = 2 * t + y;
+                if (h < per) {
+                    const long long row = orow0 + static_cast<long long>(h) * a.C;
+#pragma unroll
+                    for (int mt = 0; mt < 8; ++mt) {
+                        lm[row * 128 + mt * 16 + g] = __float2bfloat16_rn(o[mt][y]);
+                        lm[row * 128 + mt * 16 + 8 + g] = __float2bfloat16_rn(o[mt][2 + y]);
+                    }
+                    if (g == 0) a.bias[row] = bias[y];
+                }
+            }
+        }
+        cur = next;
     }
 }
 
@@ -315,12 +371,13 @@ int launch_landmark_summary(int dtype, int B, int Hkv, int Hl, int C, int d, int
     LArgs a{B, Hkv, Hl, C, S, T, scale, lq, k, seq_lens, landmarks, bias, c0, cn};
     static const bool no_tc = [] { const char* e = getenv("HILS_LANDMARK_NO_MMA"); return e && e[0] == '1'; }();
     const long long rows = static_cast<long long>(B) * Hkv * T;
-    if (!no_tc && dtype == HILS_BF16 && d == 128 && S == 64 && Hl / Hkv <= 8 && rows < (1ll << 31)) {
+    if (!no_tc && dtype == HILS_BF16 && d == 128 && S == 64 && Hl / Hkv <= 8 && rows < (1ll << 31) &&
+        static_cast<long long>(B) * Hkv * cn < (1ll << 31)) {
         const long long total = static_cast<long long>(B) * Hkv * cn;
         if (total == 0) return 0;
         CUtensorMap map_k;
         if (!make_bf16_2d_map(&map_k, k, static_cast<uint64_t>(rows), 128, 64, 64)) return HILS_ERR_CUDA;
-        const size_t smem = kTcWarps * kTcTileBytes + kTcWarps * sizeof(TcSmemW) + 1024;
+        const size_t smem = kTcWarps * kTcTileBytes + 1024;
         static PerDeviceOnce attr_once;
         if (attr_once.pending()) {
             if (cudaFuncSetAttribute(landmark_summary_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -328,9 +385,8 @@ int launch_landmark_summary(int dtype, int B, int Hkv, int Hl, int C, int d, int
                 return HILS_ERR_CUDA;
             attr_once.done();
         }
-        const long long blocks = (total + kTcWarps - 1) / kTcWarps;
-        if (blocks > 0x7fffffffll) return HILS_ERR_UNSUPPORTED;
-        landmark_summary_tc_kernel<<<static_cast<unsigned>(blocks), kTcWarps * 32, smem, stream>>>(map_k, a, nullptr);
+        const unsigned blocks = static_cast<unsigned>(total < sm_count() ? total : sm_count());
+        landmark_summary_tc_kernel<<<blocks, kTcWarps * 32, smem, stream>>>(map_k, a);
         return cudaGetLastError() == cudaSuccess ? 1 : HILS_ERR_CUDA;
     }
     return dtype == HILS_F32 ? launch_typed<float>(a, d, stream) : launch_typed<__nv_bfloat16>(a, d, stream);
