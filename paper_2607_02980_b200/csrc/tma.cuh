@@ -55,9 +55,12 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
 }
 // Bounded wait.  Returns false if the phase never completed.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+    // (not unrolled: a wait is inlined some thirty times in a warp-specialised kernel, and four copies of its body in each
+    // filled half of the instruction cache)
+#pragma unroll 1
     for (uint32_t i = 0; i < kSpinLimit; ++i) {
         if (mbar_try_wait(bar, parity)) return true;
-        if (i > 64) __nanosleep(i > 4096 ? 256 : 32);
+        if (i > 64) __nanosleep(256);
     }
     return false;
 }
