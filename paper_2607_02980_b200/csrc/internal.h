@@ -107,6 +107,7 @@ struct InverseIndex {
     const int* entries;
     const int4* tiles;
     const int* blk_toff;
+    const int* pair_toff;      // [n_blocks * pairs + 1] first tile of every (query block, pair)
 };
 size_t inverse_index_bytes(const Shape& s);
 int build_inverse_index(const Shape& s, const int32_t* sel, void* scratch, size_t bytes, InverseIndex* ix,
@@ -133,7 +134,7 @@ struct BackwardTensors {
     size_t scratch_bytes;
 };
 int launch_backward_generic(const Shape& s, int dtype, const BackwardTensors& t, cudaStream_t stream);
-// chunk-major mma.sync path for the benchmark shapes (bf16, d = 128, S = 64, G = 4, Hl = Hkv)
+// chunk-major tcgen05 path for the benchmark shapes (bf16, d = 128, S = 64, G = 4, Hl = Hkv)
 bool prefill_backward_fast_supports(const Shape& s, int dtype);
 size_t prefill_backward_fast_scratch_bytes(const Shape& s);
 int launch_prefill_backward_fast(const Shape& s, const BackwardTensors& t, cudaStream_t stream);

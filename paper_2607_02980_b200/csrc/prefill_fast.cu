@@ -628,12 +628,14 @@ size_t prefill_fast_scratch_bytes(const Shape& s) { return make_plan(s).total; }
 
 // The inverse index on its own (the backward pass walks the same chunk-major tiles): per-(query block, pair, chunk)
 // entry lists and the tile table, built from a selection that is already in memory.
-// (query blocks of kQBDefault tokens: the fp32 dq rows a block accumulates into have to stay in L2)
-size_t inverse_index_bytes(const Shape& s) { return make_plan(s, kQBEnv ? kQBEnv : kQBDefault).off_obuf; }
+// (query blocks of 16384 tokens: of one KV head they take 33 MB of queries and output gradients and as much of fp32 dq,
+// which L2 holds while the head is walked; and a chunk's list is long, so that its dk and dv are added up rarely)
+constexpr int kQBIndex = 16384;
+size_t inverse_index_bytes(const Shape& s) { return make_plan(s, kQBEnv ? kQBEnv : kQBIndex).off_obuf; }
 
 int build_inverse_index(const Shape& s, const int32_t* sel, void* scratch, size_t bytes, InverseIndex* ix,
                         cudaStream_t stream) {
-    const Plan p = make_plan(s, kQBEnv ? kQBEnv : kQBDefault);
+    const Plan p = make_plan(s, kQBEnv ? kQBEnv : kQBIndex);
     if (bytes < p.off_obuf) return HILS_ERR_WORKSPACE;
     const int pairs = s.B * s.Hkv;
     char* sc = static_cast<char*>(scratch);
@@ -673,6 +675,7 @@ int build_inverse_index(const Shape& s, const int32_t* sel, void* scratch, size_
     ix->entries = a.entries;
     ix->tiles = a.tiles;
     ix->blk_toff = a.blk_toff;
+    ix->pair_toff = a.pair_toff;
     return 4;
 }
 
