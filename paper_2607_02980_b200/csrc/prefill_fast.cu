@@ -62,6 +62,7 @@ struct PArgs {
     int nc;                 // chunk slots per pair in cnt/off/...: max(C, ceil(L / S))
     int tile_tok;           // entries per attend tile
     int max_tiles;
+    int inv_parts, inv_tok; // parts of a query block's tokens that the inversion's CTAs take, tokens of a part
     int whole;              // obuf / lam cover all query blocks (indexed by global entry): one fuse launch per call
 };
 
@@ -268,17 +269,75 @@ __device__ __forceinline__ int slot_chunk(const PArgs& a, int pair, int tok, int
     return a.sel[(static_cast<long long>(pair) * a.s.R + tok) * a.s.K + slot];
 }
 
-__global__ void invert_count_kernel(const PArgs a) {
-    const Shape& s = a.s;
-    const int K1 = s.K + max_local_slots(s.W), pairs = s.B * s.Hkv;
-    const long long total = static_cast<long long>(pairs) * (s.R - a.t0) * K1;
-    for (long long x = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; x < total;
-         x += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const int slot = static_cast<int>(x % K1);
-        const int tok = a.t0 + static_cast<int>((x / K1) % (s.R - a.t0));
-        const int pair = static_cast<int>(x / (static_cast<long long>(K1) * (s.R - a.t0)));
-        const int c = slot_chunk(a, pair, tok, slot);
-        if (c >= 0) atomicAdd(&a.cnt[(static_cast<long long>((tok - a.t0) / a.qb) * pairs + pair) * a.nc + c], 1);
+// Counting and filling go through shared memory: a CTA takes a range of one pair's tokens inside one query block, counts
+// its entries per chunk there and adds each chunk's count to the global one at once.  (With an add in global memory per
+// entry the long lists serialise: a chunk that every token of a block selects takes one add per token.)  Neighbouring
+// lanes take neighbouring slots, so that selection and entry indexes are read and written in order and the lanes of a
+// warp rarely meet at a counter.  More chunks than counters: the range is walked once per kInvCounters of them.
+constexpr int kInvThreads = 512;
+constexpr int kInvCounters = 8192;
+constexpr int kInvBatch = 4;              // entries per thread whose loads are in flight together
+
+struct InvPart {
+    int pair, lo, hi, i0;                 // tokens [lo, hi) of the query block that starts at i0
+    long long list0;                      // first list of (query block, pair)
+};
+__device__ __forceinline__ InvPart invert_part(const PArgs& a) {
+    const int pairs = a.s.B * a.s.Hkv, x = static_cast<int>(blockIdx.x) / a.inv_parts;
+    const int blk = x / pairs;
+    InvPart p;
+    p.pair = x % pairs;
+    p.i0 = a.t0 + blk * a.qb;
+    p.lo = p.i0 + static_cast<int>(blockIdx.x) % a.inv_parts * a.inv_tok;
+    p.hi = min(min(p.lo + a.inv_tok, p.i0 + a.qb), a.s.R);
+    p.list0 = static_cast<long long>(x) * a.nc;
+    return p;
+}
+// f(token, slot, chunk or -1) for every (token, slot) of the part
+template <class F>
+__device__ __forceinline__ void invert_walk(const PArgs& a, const InvPart& p, F f) {
+    const int K1 = a.s.K + max_local_slots(a.s.W);
+    const int dt = kInvThreads / K1, ds = kInvThreads % K1;
+    int tok = p.lo + static_cast<int>(threadIdx.x) / K1, slot = static_cast<int>(threadIdx.x) % K1;
+    while (tok < p.hi) {
+        int tk[kInvBatch], sl[kInvBatch], c[kInvBatch];
+#pragma unroll
+        for (int i = 0; i < kInvBatch; ++i) {
+            tk[i] = tok;
+            sl[i] = slot;
+            c[i] = tok < p.hi ? slot_chunk(a, p.pair, tok, slot) : -1;
+            tok += dt;
+            slot += ds;
+            if (slot >= K1) {
+                slot -= K1;
+                ++tok;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < kInvBatch; ++i)
+            if (tk[i] < p.hi) f(tk[i], sl[i], c[i]);
+    }
+}
+// counts of the chunks [c0, c0 + n) of the part
+__device__ __forceinline__ void invert_histogram(const PArgs& a, const InvPart& p, int* ctr, int c0, int n) {
+    for (int i = threadIdx.x; i < n; i += kInvThreads) ctr[i] = 0;
+    __syncthreads();
+    invert_walk(a, p, [&](int, int, int c) {
+        if (c >= c0 && c - c0 < n) atomicAdd(&ctr[c - c0], 1);
+    });
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(kInvThreads, 3) invert_count_kernel(const PArgs a) {
+    extern __shared__ int ctr[];
+    pdl_wait();
+    const InvPart p = invert_part(a);
+    for (int c0 = 0; c0 < a.nc; c0 += kInvCounters) {
+        const int n = min(kInvCounters, a.nc - c0);
+        invert_histogram(a, p, ctr, c0, n);
+        for (int i = threadIdx.x; i < n; i += kInvThreads)
+            if (ctr[i] > 0) atomicAdd(&a.cnt[p.list0 + c0 + i], ctr[i]);
+        __syncthreads();
     }
 }
 
@@ -347,37 +406,34 @@ __global__ void __launch_bounds__(1024) invert_scan_kernel(const PArgs a) {
     }
 }
 
-// A warp takes one slot of 32 consecutive tokens: neighbouring tokens mostly hold the same chunk in a slot (the
-// local window's chunks always, the selected ones whenever adjacent queries agree), so the lanes that target the
-// same list are served by ONE add on its cursor: the lowest such lane reserves room for all of them.
-__global__ void invert_fill_kernel(const PArgs a) {
+// The part's entries per chunk once more, room for them in each list, then a cursor per chunk in shared memory.
+// Whole inversion, 16K tokens, K = 16, 8 KV heads, one query block: 204 -> 71 us; 128K tokens, K = 32, counts given:
+// 694 -> 385 us, most of it the scattered 4-byte stores of the entries.
+__global__ void __launch_bounds__(kInvThreads, 3) invert_fill_kernel(const PArgs a) {
+    extern __shared__ int ctr[];
     pdl_wait();
-    const Shape& s = a.s;
-    const int K1 = s.K + max_local_slots(s.W), pairs = s.B * s.Hkv;
-    const int lane = threadIdx.x & 31;
-    const int tblocks = (s.R - a.t0 + 31) / 32;                  // (t0 is a multiple of 32)
-    const long long total = static_cast<long long>(pairs) * tblocks * K1;
-    const long long nwarps = static_cast<long long>(gridDim.x) * (blockDim.x >> 5);
-    for (long long w = static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); w < total; w += nwarps) {
-        const int slot = static_cast<int>(w % K1);
-        const int tb = static_cast<int>((w / K1) % tblocks);
-        const int pair = static_cast<int>(w / (static_cast<long long>(K1) * tblocks));
-        const int tok = a.t0 + tb * 32 + lane;
-        const int c = tok < s.R ? slot_chunk(a, pair, tok, slot) : -1;
-        const long long idx = c >= 0 ? (static_cast<long long>((tok - a.t0) / a.qb) * pairs + pair) * a.nc + c : -1 - lane;
-        const unsigned same = __match_any_sync(kFullMask, idx);
-        const int leader = __ffs(same) - 1;
-        int base = 0;
-        if (c >= 0 && lane == leader) base = a.off[idx] + atomicAdd(&a.cursor[idx], __popc(same));
-        base = __shfl_sync(kFullMask, base, leader);
-        if (tok < s.R) {
-            int pos = -1;
-            if (c >= 0) {
-                pos = base + __popc(same & ((1u << lane) - 1u));
-                if (pos < a.max_tiles * a.tile_tok) a.entries[pos] = (((tok - a.t0) % a.qb) << 8) | slot;
-            }
-            a.epos[(static_cast<long long>(pair) * s.R + tok) * K1 + slot] = pos;
+    const InvPart p = invert_part(a);
+    const int K1 = a.s.K + max_local_slots(a.s.W);
+    int* epos = a.epos + static_cast<long long>(p.pair) * a.s.R * K1;
+    for (int c0 = 0; c0 < a.nc; c0 += kInvCounters) {
+        const int n = min(kInvCounters, a.nc - c0);
+        invert_histogram(a, p, ctr, c0, n);
+        for (int i = threadIdx.x; i < n; i += kInvThreads) {
+            const long long list = p.list0 + c0 + i;
+            if (ctr[i] > 0) ctr[i] = a.off[list] + atomicAdd(&a.cursor[list], ctr[i]);
         }
+        __syncthreads();
+        invert_walk(a, p, [&](int tok, int slot, int c) {
+            int pos = -1;
+            if (c >= c0 && c - c0 < n) {
+                pos = atomicAdd(&ctr[c - c0], 1);
+                if (pos < a.max_tiles * a.tile_tok) a.entries[pos] = ((tok - p.i0) << 8) | slot;
+            } else if (c >= 0 || c0 > 0) {
+                return;                   // another pass's chunk
+            }
+            epos[static_cast<long long>(tok) * K1 + slot] = pos;
+        });
+        __syncthreads();
     }
 }
 
@@ -626,6 +682,19 @@ bool prefill_fast_supports(const Shape& s, int dtype) {
 
 size_t prefill_fast_scratch_bytes(const Shape& s) { return make_plan(s).total; }
 
+// Parts of a query block that the inversion's CTAs take: some 8 CTAs per SM, none with fewer entries than its threads hold
+// in one batch.  Returns the CTAs.
+static unsigned invert_split(PArgs& a, const Plan& p) {
+    const long long groups = static_cast<long long>(p.n_blocks) * a.s.B * a.s.Hkv;
+    const int toks = a.s.R - a.t0 < a.qb ? a.s.R - a.t0 : a.qb, K1 = a.s.K + max_local_slots(a.s.W);
+    const long long most = (static_cast<long long>(toks) * K1 + kInvThreads * kInvBatch - 1) / (kInvThreads * kInvBatch);
+    const long long want = 8ll * sm_count() / groups;
+    a.inv_parts = static_cast<int>(want < 1 ? 1 : want < most ? want : most);
+    a.inv_tok = (toks + a.inv_parts - 1) / a.inv_parts;
+    return static_cast<unsigned>(groups * a.inv_parts);
+}
+static size_t invert_smem(const PArgs& a) { return sizeof(int) * (a.nc < kInvCounters ? a.nc : kInvCounters); }
+
 // The inverse index on its own (the backward pass walks the same chunk-major tiles): per-(query block, pair, chunk)
 // entry lists and the tile table, built from a selection that is already in memory.
 // (query blocks of 16384 tokens: of one KV head they take 33 MB of queries and output gradients and as much of fp32 dq,
@@ -657,15 +726,13 @@ int build_inverse_index(const Shape& s, const int32_t* sel, void* scratch, size_
     a.nc = p.nc;
     a.tile_tok = attend_tc_tile_tokens();
     if (cudaMemsetAsync(sc + p.off_cnt, 0, p.zero_bytes, stream) != cudaSuccess) return HILS_ERR_CUDA;
-    const long long elems = static_cast<long long>(pairs) * s.R * (s.K + max_local_slots(s.W));
-    const long long want = (elems + 255) / 256;
-    const unsigned eb = static_cast<unsigned>(want < sm_count() * 16 ? want : sm_count() * 16);
+    const unsigned eb = invert_split(a, p);
     const unsigned nseg = static_cast<unsigned>((static_cast<long long>(p.n_blocks) * pairs * p.nc + 1023) / 1024);
-    invert_count_kernel<<<eb, 256, 0, stream>>>(a);
-    invert_segsum_kernel<<<nseg, 1024, 0, stream>>>(a);
-    invert_scan_kernel<<<nseg, 1024, 0, stream>>>(a);
-    invert_fill_kernel<<<eb, 256, 0, stream>>>(a);
-    if (cudaGetLastError() != cudaSuccess) return HILS_ERR_CUDA;
+    if (launch_pdl(invert_count_kernel, dim3(eb), dim3(kInvThreads), invert_smem(a), stream, a) != cudaSuccess ||
+        launch_pdl(invert_segsum_kernel, dim3(nseg), dim3(1024), 0, stream, a) != cudaSuccess ||
+        launch_pdl(invert_scan_kernel, dim3(nseg), dim3(1024), 0, stream, a) != cudaSuccess ||
+        launch_pdl(invert_fill_kernel, dim3(eb), dim3(kInvThreads), invert_smem(a), stream, a) != cudaSuccess)
+        return HILS_ERR_CUDA;
     trace_mark("backward_invert", stream);
     ix->qb = p.qb;
     ix->nc = p.nc;
@@ -773,11 +840,9 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
     // inverse index for every query block at once: per-(block, pair, chunk) lists of (token, slot) entries
     // and the table of attend tiles, grouped by block
     {
-        const long long elems = static_cast<long long>(pairs) * (s.R - t0) * (s.K + max_local_slots(s.W));
-        const long long want = (elems + 255) / 256;
-        const unsigned eb = static_cast<unsigned>(want < sm_count() * 16 ? want : sm_count() * 16);
+        const unsigned eb = invert_split(a, p);
         if (!counted) {
-            invert_count_kernel<<<eb, 256, 0, stream>>>(a);
+            invert_count_kernel<<<eb, kInvThreads, invert_smem(a), stream>>>(a);
             ++launches;
         }
         const unsigned nseg = static_cast<unsigned>((static_cast<long long>(p.n_blocks) * pairs * p.nc + 1023) / 1024);
@@ -786,7 +851,7 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
         // triggers its dependents early: CTAs of the next kernel parked beside a running attend kernel cost 5 %.
         if (launch_pdl(invert_segsum_kernel, dim3(nseg), dim3(1024), 0, stream, a) != cudaSuccess ||
             launch_pdl(invert_scan_kernel, dim3(nseg), dim3(1024), 0, stream, a) != cudaSuccess ||
-            launch_pdl(invert_fill_kernel, dim3(eb), dim3(256), 0, stream, a) != cudaSuccess)
+            launch_pdl(invert_fill_kernel, dim3(eb), dim3(kInvThreads), invert_smem(a), stream, a) != cudaSuccess)
             return HILS_ERR_CUDA;
         trace_mark("prefill_invert", stream);
         launches += 3;
