@@ -11,7 +11,8 @@
 //            local branch) go to the buffers that prefill_fuse mixes, in entry order: a tile's 128 rows
 //            are contiguous there, so every output warp hands its 32 rows to one TMA store per half.
 // Warp roles: 0-3 and 4-7 two softmax groups (tiles alternate between them; a warp reads the TMEM lane quarter
-// warp % 4), 8-11 output group, 12-15 query gather, 16 K/V loader, 17 MMA issue.
+// warp % 4), 8-11 output group, 12-15 query gather, 16 K/V loader, 17-18 MMA issue (a warp per tile parity), 19 feeds the tile
+// records and entries through a ring.
 // The gather: a warp's cp.async requests complete at the latency of a loaded L2 and a warp keeps only so many in
 // flight, so the rate grows with the number of gathering warps (measured alone: 1 warp 1500 cycles per 32 KB tile, 2
 // warps 840, 4 and more 480; inside this kernel about three times that).  TMA boxes of one entry (512 B) cost about
@@ -35,23 +36,30 @@ constexpr int kVBytes = kS * kD * 2;            // two boxes of 64 keys x 64 dim
 constexpr int kQBytes = kRows * kD * 2;         // 32 KB
 constexpr int kPBytes = kRows * 128;            // 16 KB
 constexpr int kPCol = 96;                       // probabilities (bf16 pairs, 32 columns) behind the slot's 80 score columns
-constexpr int kBatch = 64;                      // tiles whose records and entries are cached in shared memory at a time
-                                                // (every batch ends with a drained pipeline: 32 -> 0.701 ms, 48 -> 0.674, 64 -> 0.664
-                                                // on the 16K-token benchmark shape; 64 is what fits)
 constexpr int kQSlots = 3;                      // gathered Q tiles in flight
 constexpr int kVBufs = 3;                       // V tiles in flight (K: 2)
-constexpr int kMetaSlots = 16;                  // ring of tile descriptors.  The gather of tile t starts once S(t-3) is done, which
-                                                // needs softmax(t-5) under way, hence softmax(t-7) finished, hence P V(t-9) done,
-                                                // hence the output of tile t-11 finished: the output group is at most 10 tiles behind
+constexpr int kMeta = 16;                       // tiles whose records and entries are in shared memory at a time.  The gather of
+                                                // tile t starts once S(t-3) is done, which needs softmax(t-5) under way, hence
+                                                // softmax(t-7) finished, hence P V(t-9) done, hence the output of tile t-11
+                                                // finished: the output group is at most 10 tiles behind
 constexpr int kSoftThreads = 256;               // two softmax groups of 128 threads
 constexpr int kOutWarp0 = kSoftThreads / 32;    // 8
 constexpr int kGatherWarps = 4;
 constexpr int kGatherWarp0 = kOutWarp0 + 4;     // 12 .. 15
 constexpr int kLoadWarp = kGatherWarp0 + kGatherWarps;   // 16
 constexpr int kMmaWarp = kLoadWarp + 1;         // 17, 18: one MMA issuer per tile parity
-constexpr int kThreads = (kMmaWarp + 2) * 32;   // 608
+constexpr int kFeedWarp = kMmaWarp + 2;         // 19
+constexpr int kThreads = (kFeedWarp + 1) * 32;  // 640
 constexpr float kLog2e = 1.4426950408889634f;
 
+struct AtcTile {
+    int pair, chunk;
+    int flags;                // tokens (0: no more tiles) | first tile of its chunk run << 8 | last << 9 | arrivals on k_empty << 12
+    uint32_t run;             // number of the chunk run (its K buffer: % 2, its V buffer: % kVBufs)
+    int orow0;                // first row in the output buffers
+    int i0;                   // first token of the query block
+    int ent[kTok];            // (token - i0) << 8 | slot
+};
 struct AtcSmem {
     // K tiles live in a ring of 2 (free again after the chunk's last S MMA), V tiles in a ring of kVBufs (free after
     // its last P V MMA, about one epilogue phase later)
@@ -66,14 +74,9 @@ struct AtcSmem {
     uint64_t p_full[2];       // P written to tensor memory
     uint64_t o_full[2];       // O = P V in tensor memory
     uint64_t o_empty[2];      // the output group has read O
+    uint64_t meta_full[kMeta], meta_empty[kMeta];
     uint32_t tmem_base;
-    int abort_flag;
-    int tile_meta[kMetaSlots][4];     // pair, chunk, tokens | last tile of its chunk run << 8 | K buffer << 9 | V buffer << 10,
-                                      // first entry relative to the query block
-    int4 recs[kBatch];
-    int ent_s[kBatch * kTok];         // entries of the batch's tiles: (token - block start) << 8 | slot
-    int nchunks;                      // distinct (pair, chunk) runs in the current batch
-    uint8_t cfirst[kBatch + 4];       // first tile (batch index) of each run; cfirst[nchunks] = tiles in the batch
+    alignas(16) AtcTile tile[kMeta];
 };
 
 struct AtcArgs {
@@ -121,9 +124,9 @@ prefill_attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
     AtcSmem& sm = *reinterpret_cast<AtcSmem*>(obuf + 2 * kPBytes);
 
     const Shape& s = a.s;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(kFullMask, tid >> 5, 0), lane = tid & 31;
     if (tid == 0) {
-        for (int i = 0; i < kQSlots; ++i) { mbar_init(&sm.q_full[i], kGatherWarps * 32 + kGatherWarps); mbar_init(&sm.q_empty[i], 1); }
+        for (int i = 0; i < kQSlots; ++i) { mbar_init(&sm.q_full[i], kGatherWarps * 32); mbar_init(&sm.q_empty[i], 1); }
         for (int i = 0; i < kVBufs; ++i) { mbar_init(&sm.v_ready[i], 1); mbar_init(&sm.v_empty[i], 1); }
         for (int i = 0; i < 2; ++i) {
             mbar_init(&sm.k_ready[i], 2);           // the TMA issuer's arrive.expect_tx + the landmark writer
@@ -134,8 +137,9 @@ prefill_attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
             mbar_init(&sm.o_full[i], 1);
             mbar_init(&sm.o_empty[i], 4);
         }
+        // (readers of a tile's record: four warps each of softmax, output and gather, the loader, one MMA issuer)
+        for (int i = 0; i < kMeta; ++i) { mbar_init(&sm.meta_full[i], 1); mbar_init(&sm.meta_empty[i], 14); }
         mbar_fence_init();
-        sm.abort_flag = 0;
         tma_prefetch_desc(&map_k);
         tma_prefetch_desc(&map_v);
         tma_prefetch_desc(&map_o);
@@ -150,129 +154,27 @@ prefill_attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem_base = sm.tmem_base;
+    const uint32_t tmem_base = __shfl_sync(kFullMask, sm.tmem_base, 0);
 
     // Everything above touched only this CTA's own shared and tensor memory, so it may overlap the tail of the
     // previous kernel of the stream (the fusion of the previous query block, which still reads the partial outputs
     // this kernel overwrites, or the inverse-index kernels).  From here on their results are needed.
     pdl_wait();
 
-    // Every role walks the same batches of tiles.  a.n_tiles[x], a.n_tiles[x + 1]: first tile of segment x (a query block, or
-    // one pair of it) and of the next one; a launch that walks several blocks takes them in order, so that the CTAs stay on the same
-    // block (its gathered Q rows stay in L2).  The walk is instantiated once per role.
-    // body(nb, tcount, ccount, t_begin, i0): nb tiles cached in sm.recs, the CTA's running tile and chunk-run counters.
-    auto walk = [&](auto&& body) {
-        uint32_t tcount = 0, ccount = 0;
-        for (int sg = 0; sg < a.n_run * a.segs; ++sg) {
-            const int blk = sg / a.segs, t_begin = a.n_tiles[blk * a.segs];            // first tile of the query block
-            const int s_begin = a.n_tiles[sg], n_tiles = a.n_tiles[sg + 1] - s_begin;
-            const int i0 = a.i0 + blk * a.qb;
-            const long long lo = s_begin + static_cast<long long>(blockIdx.x) * n_tiles / gridDim.x;
-            const long long hi = s_begin + static_cast<long long>(blockIdx.x + 1) * n_tiles / gridDim.x;
-            for (long long b0 = lo; b0 < hi; b0 += kBatch) {
-                const int nb = static_cast<int>(min(static_cast<long long>(kBatch), hi - b0));
-                for (int x = tid; x < nb; x += kThreads) sm.recs[x] = a.tiles[b0 + x];
-                // A list starts on a tile boundary of the global entry space, so the entries of tile t are
-                // entries[32 t .. 32 t + 31]: the batch's entries are one contiguous run, fetched now, all at once (a
-                // load per tile inside the gather loop waited several thousand cycles under the partial-output stores).
-                for (int x = tid; x < nb * kTok; x += kThreads) sm.ent_s[x] = a.entries[b0 * kTok + x];
-                __syncthreads();
-                if (sm.abort_flag) return;
-                if (warp == 0) {
-                    // table of chunk runs: where each run of tiles of one (pair, chunk) starts
-                    int basec = 0;
-                    for (int w = 0; w < (kBatch + 31) / 32; ++w) {
-                        const int x = w * 32 + lane;
-                        const bool nw = x < nb && (x == 0 || sm.recs[x].x != sm.recs[x - 1].x || sm.recs[x].y != sm.recs[x - 1].y);
-                        const unsigned m = __ballot_sync(kFullMask, nw);
-                        if (nw) sm.cfirst[basec + __popc(m & ((1u << lane) - 1u))] = static_cast<uint8_t>(x);
-                        basec += __popc(m);
-                    }
-                    if (lane == 0) { sm.cfirst[basec] = static_cast<uint8_t>(nb); sm.nchunks = basec; }
-                }
-                __syncthreads();
-                body(nb, tcount, ccount, t_begin, i0);
-                // every role advances the shared counters identically
-                tcount += static_cast<uint32_t>(nb);
-                ccount += static_cast<uint32_t>(sm.nchunks);
-                __syncthreads();
-                if (sm.abort_flag) return;
-            }
-        }
+    bool ok = true;
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+        if (ok && !mbar_wait(bar, parity)) ok = false;
+        return ok;
     };
-
-    auto gather_role = [&]() {
-        // ================================================================ Q gather (four warps)
-        // The tile's 128 rows (entry-major, head-minor) are 64 cp.async instructions of two 256-byte rows (a half-warp
-        // each, both of one entry); warp gw issues numbers 16 gw .. 16 gw + 15.  Lane l < 8 holds entry 8 gw + l and
-        // hands its token to the warp by a uniform shuffle: no address table, no barrier between the gather warps.
-        const int gw = warp - kGatherWarp0;
-        constexpr int kPerWarp = 64 / kGatherWarps;
-        const int j0 = gw * kPerWarp, j1 = j0 + kPerWarp;
-        const int e0 = j0 >> 1;                                      // first entry this warp touches
-        const int el = min(e0 + (lane & 7), kTok - 1);
-        const int p16 = lane & 15, hh = lane >> 4;
-        const long long hstride = static_cast<long long>(s.R) * kD;
-        walk([&](int nb, uint32_t tcount, uint32_t ccount, int t_begin, int i0) {
-            uint32_t tc = tcount;
-            bool dead = false;
-            int ck = 0;                        // chunk run (ordinal within the batch) of the current tile
-            for (int ti = 0; ti < nb; ++ti) {
-                const int4 rec = sm.recs[ti];
-                const int pair = rec.x, ntok = rec.w;
-                // this lane's entry (rows past a ragged tile's last entry repeat that entry)
-                const int e = sm.ent_s[ti * kTok + min(el, ntok - 1)];
-                const uint32_t qs = tc % kQSlots, ms = tc % kMetaSlots;
-                if (tc >= kQSlots && !mbar_wait(&sm.q_empty[qs], ((tc / kQSlots) - 1) & 1)) { dead = true; break; }
-                if (*reinterpret_cast<volatile int*>(&sm.abort_flag)) { dead = true; break; }
-                if (gw == 0 && lane == 0) {
-                    // A tcgen05.commit costs the issuing thread about a hundred cycles, so only the two the epilogue
-                    // groups wait on are issued; those groups pass "this Q slot / K buffer / V buffer is free" on.
-                    if (ti >= sm.cfirst[ck + 1]) ++ck;
-                    const bool last = ti + 1 >= sm.cfirst[ck + 1];
-                    // The K buffer of a chunk run is free when the score MMAs of the run's last tile of EITHER parity are
-                    // done (the two parities have an issuing thread each, and a thread's MMAs complete in order): those
-                    // two tiles arrive once each on k_empty, a run of a single tile twice.
-                    const int karr = (ti + 2 >= sm.cfirst[ck + 1] ? 1 : 0) + (sm.cfirst[ck + 1] - sm.cfirst[ck] == 1 ? 1 : 0);
-                    const uint32_t cc = ccount + static_cast<uint32_t>(ck);
-                    sm.tile_meta[ms][0] = pair; sm.tile_meta[ms][1] = rec.y;
-                    sm.tile_meta[ms][2] = ntok | (last ? 256 : 0) | static_cast<int>((cc & 1u) << 9) | static_cast<int>((cc % kVBufs) << 10) | (karr << 12);
-                    sm.tile_meta[ms][3] = rec.z - (a.whole ? 0 : t_begin * kTok);
-                }
-                {
-                    const uint32_t qaddr = smem_u32(qbuf + qs * kQBytes) + (p16 >> 3) * 16384;
-                    const __nv_bfloat16* qb0 = a.q + (static_cast<long long>(pair / s.Hkv) * s.Hq + (pair % s.Hkv) * kG + hh) * hstride +
-                                               static_cast<long long>(i0) * kD + p16 * 8;
-                    // the tokens of the warp's entries first (shuffles and copies are both ordered operations: interleaved
-                    // they would run strictly one after the other)
-                    int tokv[kPerWarp / 2];
-#pragma unroll
-                    for (int k = 0; k < kPerWarp / 2; ++k) tokv[k] = __shfl_sync(kFullMask, e, k) >> 8;
-#pragma unroll
-                    for (int jj = 0; jj < kPerWarp; ++jj) {
-                        const int j = j0 + jj;
-                        const int row = 2 * j + hh;
-                        const __nv_bfloat16* src = qb0 + (2 * j & 3) * hstride + static_cast<long long>(tokv[jj >> 1]) * kD;
-                        cp_async16(qaddr + swz128(row, p16 & 7), src);
-                    }
-                }
-                // The tile's barrier hears from every gather thread when that thread's copies have landed (no thread
-                // waits for them), and from one lane per warp for the tile's descriptor written above.
-                asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&sm.q_full[qs])) : "memory");
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sm.q_full[qs]);
-                ++tc;
-            }
-            if (dead && lane == 0) { set_status(a.status, kDevTimeout); atomicExch(&sm.abort_flag, 1); }
-        });
+    // record of tile n of this CTA (false: there is none)
+    auto tile_of = [&](uint32_t n) {
+        if (!wait(&sm.meta_full[n % kMeta], (n / kMeta) & 1)) return false;
+        return (sm.tile[n % kMeta].flags & 255) != 0;
     };
-
-    // (called at the end of every role)
-    auto finish = [&]() {
-        tc_fence_before_sync();
-        __syncthreads();
-        tc_fence_after_sync();
-        if (warp == kMmaWarp) tmem_dealloc(tmem_base, 512);
+    // this warp needs the record no more
+    auto tile_done = [&](uint32_t n) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.meta_empty[n % kMeta]);
     };
 
     if (warp < kOutWarp0) {
@@ -285,27 +187,24 @@ prefill_attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
         const int tk = row >> 2, hd = row & 3;
         const float sl2 = s.scale * kLog2e;
         const int lh = (s.Hl == s.Hkv) ? 0 : hd;
-        walk([&](int nb, uint32_t tcount, uint32_t, int, int i0) {
-            bool ok = true;
-            for (int ti = static_cast<int>((grp ^ tcount) & 1u); ti < nb && ok; ti += 2) {
-                const uint32_t tcv = tcount + ti;                      // (tcv & 1) == grp
-                ok = mbar_wait(&sm.s_full[grp], (tcv >> 1) & 1);
-                if (!ok) break;
+        for (uint32_t n = grp; tile_of(n); n += 2) {
+                const AtcTile& tl = sm.tile[n % kMeta];
+                const int pair = tl.pair, c = tl.chunk, flags = tl.flags, e = tl.ent[min(tk, (flags & 255) - 1)];
+                const uint32_t run = tl.run;
+                const int il = tl.i0 + (e >> 8), orow0 = tl.orow0;
+                tile_done(n);
+                const bool local = (e & 255) >= s.K;                       // a chunk of the local window: mass = its exact log-sum-exp
+                const int lim = local ? s.pos0 + il - c * kS : kS - 1;     // last visible key of the chunk
+                const float bb = (a.bias && c < s.C)
+                    ? __ldg(a.bias + (static_cast<long long>(pair / s.Hkv) * s.Hl + (pair % s.Hkv) * (s.Hl / s.Hkv) + lh) * s.C + c) : 0.f;
+                if (!wait(&sm.s_full[grp], (n >> 1) & 1)) break;
                 tc_fence_after_sync();
-                const uint32_t ms = tcv % kMetaSlots;
-                const int pair = sm.tile_meta[ms][0], c = sm.tile_meta[ms][1];
                 // the tile's score MMAs are done: its gathered rows, and its chunk's K tile after the chunk's last tile,
                 // may be overwritten
                 if ((warp & 3) == 0 && lane == 0) {
-                    const int flags = sm.tile_meta[ms][2];
-                    mbar_arrive(&sm.q_empty[tcv % kQSlots]);
-                    for (int x = (flags >> 12) & 3; x > 0; --x) mbar_arrive(&sm.k_empty[(flags >> 9) & 1]);
+                    mbar_arrive(&sm.q_empty[n % kQSlots]);
+                    for (int x = (flags >> 12) & 3; x > 0; --x) mbar_arrive(&sm.k_empty[run & 1]);
                 }
-                const int orow0 = sm.tile_meta[ms][3] * kG;          // first row of the tile in the output buffers
-                const int e = sm.ent_s[ti * kTok + min(tk, (sm.tile_meta[ms][2] & 255) - 1)];
-                const int il = e >> 8, slot = e & 255;
-                const bool local = slot >= s.K;                            // a chunk of the local window: mass = its exact log-sum-exp
-                const int lim = local ? s.pos0 + i0 + il - c * kS : kS - 1;   // last visible key of the chunk
                 // the 64 key scores and the surrogate score columns: the landmark of this row's head (key 64 + hd)
                 // or the shared one (key 64); warp-uniform addresses, the lane picks its column
                 float v[64];
@@ -348,10 +247,7 @@ prefill_attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
                 const float zi = 1.f / z;
                 const float2 zi2 = make_float2(zi, zi);
                 // the P V product of this slot's previous tile must have read its probabilities
-                if (tcv >= 2) {
-                    ok = mbar_wait(&sm.o_full[grp], ((tcv >> 1) - 1) & 1);
-                    if (!ok) break;
-                }
+                if (n >= 2 && !wait(&sm.o_full[grp], ((n >> 1) - 1) & 1)) break;
 #pragma unroll
                 for (int pc = 0; pc < 4; ++pc) {
                     uint32_t pk[8];
@@ -363,17 +259,12 @@ prefill_attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
                     tmem_st8(t_lane + kPCol + pc * 8, pk);
                 }
                 // chunk mass of the row (rows of a ragged tile's padding land in the list's padding)
-                const float bb = (a.bias && c < s.C)
-                    ? a.bias[(static_cast<long long>(pair / s.Hkv) * s.Hl + (pair % s.Hkv) * (s.Hl / s.Hkv) + lh) * s.C + c] : 0.f;
                 a.lam[orow0 + row] = local ? m * s.scale + __logf(z) : lmk * s.scale + bb;
                 tmem_wait_st();
                 tc_fence_before_sync();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sm.p_full[grp]);
-            }
-            if (!ok && lane == 0) { set_status(a.status, kDevTimeout); atomicExch(&sm.abort_flag, 1); }
-        });
-        finish();
+        }
     } else if (warp < kGatherWarp0) {
         // ================================================================ output group: O = P V -> bf16 rows
         // The warp's 32 rows of the staging buffer (4 KB, swizzled as the output map expects) take 64 columns at a
@@ -383,19 +274,14 @@ prefill_attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
         const uint32_t t_lane = tmem_base + (static_cast<uint32_t>(ow * 32) << 16);
         const uint64_t pol = l2_policy_evict_first();
         uint8_t* wstg = obuf + ow * 4096;            // columns 0..63; + kPBytes: columns 64..127
-        walk([&](int nb, uint32_t tcount, uint32_t, int, int) {
-            bool ok = true;
-            for (int ti = 0; ti < nb && ok; ++ti) {
-                const uint32_t tcv = tcount + ti, sl = tcv & 1u;
-                ok = mbar_wait(&sm.o_full[sl], (tcv >> 1) & 1);
-                if (!ok) break;
+        for (uint32_t n = 0; tile_of(n); ++n) {
+                const uint32_t sl = n & 1u, run = sm.tile[n % kMeta].run;
+                const int orow0 = sm.tile[n % kMeta].orow0, flags = sm.tile[n % kMeta].flags;
+                tile_done(n);
+                if (!wait(&sm.o_full[sl], (n >> 1) & 1)) break;
                 tc_fence_after_sync();
-                const int orow0 = sm.tile_meta[tcv % kMetaSlots][3] * kG;
-                if (ow == 0 && lane == 0) {
-                    // the tile's P V MMAs are done: after the chunk's last tile its V tile may be overwritten
-                    const int flags = sm.tile_meta[tcv % kMetaSlots][2];
-                    if (flags & 256) mbar_arrive(&sm.v_empty[(flags >> 10) & 3]);
-                }
+                // the tile's P V MMAs are done: after the chunk's last tile its V tile may be overwritten
+                if (ow == 0 && lane == 0 && (flags & 512)) mbar_arrive(&sm.v_empty[run % kVBufs]);
                 // The accumulator leaves tensor memory in four quarters of 32 columns; the load of the next quarter runs
                 // under the packing and staging of the current one.
                 uint32_t va[32], vb[32];
@@ -437,15 +323,46 @@ prefill_attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
                     tma_store_2d(&map_o, wstg + lane * kPBytes, lane * 64, orow0 + ow * 32, pol);
                     bulk_commit();
                 }
-            }
-            if (!ok && lane == 0) { set_status(a.status, kDevTimeout); atomicExch(&sm.abort_flag, 1); }
-        });
-        finish();
+        }
+        if (lane < 2) bulk_wait_read<0>();
     } else if (warp < kLoadWarp) {
-        gather_role();
-        finish();
-    } else {
-        if (warp == kLoadWarp) {
+        // ================================================================ Q gather (four warps)
+        // The tile's 128 rows (entry-major, head-minor) are 64 cp.async instructions of two 256-byte rows (a half-warp
+        // each, both of one entry); warp gw issues numbers 16 gw .. 16 gw + 15.  Lane l < 8 holds entry 8 gw + l and
+        // hands its token to the warp by a uniform shuffle: no address table, no barrier between the gather warps.
+        const int gw = warp - kGatherWarp0;
+        constexpr int kPerWarp = 64 / kGatherWarps;
+        const int j0 = gw * kPerWarp;
+        const int el = (j0 >> 1) + (lane & 7);
+        const int p16 = lane & 15, hh = lane >> 4;
+        const long long hstride = static_cast<long long>(s.R) * kD;
+        for (uint32_t n = 0; tile_of(n); ++n) {
+            const AtcTile& tl = sm.tile[n % kMeta];
+            const int pair = tl.pair, i0 = tl.i0;
+            // this lane's entry (rows past a ragged tile's last entry repeat that entry)
+            const int e = tl.ent[min(el, (tl.flags & 255) - 1)];
+            tile_done(n);
+            const uint32_t qs = n % kQSlots;
+            if (n >= kQSlots && !wait(&sm.q_empty[qs], ((n / kQSlots) - 1) & 1)) break;
+            const uint32_t qaddr = smem_u32(qbuf + qs * kQBytes) + (p16 >> 3) * 16384;
+            const __nv_bfloat16* qb0 = a.q + (static_cast<long long>(pair / s.Hkv) * s.Hq + (pair % s.Hkv) * kG + hh) * hstride +
+                                       static_cast<long long>(i0) * kD + p16 * 8;
+            // the tokens of the warp's entries first (shuffles and copies are both ordered operations: interleaved
+            // they would run strictly one after the other)
+            int tokv[kPerWarp / 2];
+#pragma unroll
+            for (int k = 0; k < kPerWarp / 2; ++k) tokv[k] = __shfl_sync(kFullMask, e, k) >> 8;
+#pragma unroll
+            for (int jj = 0; jj < kPerWarp; ++jj) {
+                const int j = j0 + jj;
+                const int row = 2 * j + hh;
+                const __nv_bfloat16* src = qb0 + (2 * j & 3) * hstride + static_cast<long long>(tokv[jj >> 1]) * kD;
+                cp_async16(qaddr + swz128(row, p16 & 7), src);
+            }
+            // the tile's barrier hears from every gather thread when that thread's copies have landed (no thread waits for them)
+            asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&sm.q_full[qs])) : "memory");
+        }
+    } else if (warp == kLoadWarp) {
             // ================================================================ K/V loader (one warp)
             // One chunk run after the other: wait until the run's K and V buffers are free, request the tiles (they
             // complete on k_ready / v_ready, which only the MMA warp waits for), write the landmark row(s).
@@ -459,146 +376,177 @@ prefill_attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
                 }
                 return v;
             };
-            walk([&](int, uint32_t, uint32_t ccount, int, int) {
-                const int nch = sm.nchunks;
-                bool dead = false;
-                // landmark pieces of the current run (piece x = lane + 32 r of the `per` rows, 16 pieces each),
-                // fetched a run ahead
-                uint4 lm_cur[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
-                if (nch > 0) {
-                    const int4 r0 = sm.recs[0];
+            uint32_t runs = 0;
+            for (uint32_t n = 0; tile_of(n); ++n) {
+                const int pair = sm.tile[n % kMeta].pair, c = sm.tile[n % kMeta].chunk, flags = sm.tile[n % kMeta].flags;
+                tile_done(n);
+                if (!(flags & 256)) continue;
+                const uint32_t cc = runs++, cbuf = cc & 1u, vb = cc % kVBufs;
+                // landmark pieces (piece x = lane + 32 r of the `per` rows, 16 pieces each), requested before the wait
+                uint4 lmv[2];
 #pragma unroll
-                    for (int r = 0; r < 2; ++r)
-                        if (lane + 32 * r < per * 16) lm_cur[r] = lm_piece(r0.x, r0.y, lane + 32 * r);
+                for (int r = 0; r < 2; ++r)
+                    if (lane + 32 * r < per * 16) lmv[r] = lm_piece(pair, c, lane + 32 * r);
+                if (cc >= 2 && !wait(&sm.k_empty[cbuf], ((cc >> 1) - 1) & 1)) break;
+                if (cc >= kVBufs && !wait(&sm.v_empty[vb], ((cc / kVBufs) - 1) & 1)) break;
+                if (lane == 0) {
+                    const int row = pair * s.T + c * kS;
+                    mbar_expect_tx(&sm.k_ready[cbuf], 2 * 8192);
+                    tma_load_2d(kbuf + cbuf * kKBytes, &map_k, &sm.k_ready[cbuf], 0, row);
+                    tma_load_2d(kbuf + cbuf * kKBytes + kNS * 128, &map_k, &sm.k_ready[cbuf], 64, row);
+                    mbar_expect_tx(&sm.v_ready[vb], kVBytes);
+                    tma_load_2d(vbuf + vb * kVBytes, &map_v, &sm.v_ready[vb], 0, row);
+                    tma_load_2d(vbuf + vb * kVBytes + 8192, &map_v, &sm.v_ready[vb], 64, row);
                 }
-                for (int ck = 0; ck < nch; ++ck) {
-                    const uint32_t cc = ccount + static_cast<uint32_t>(ck);
-                    const int4 rec = sm.recs[sm.cfirst[ck]];
-                    const int pair = rec.x, c = rec.y;
-                    const uint32_t cbuf = cc & 1u, vb = cc % kVBufs;
-                    if (lane == 0) {
-                        if (cc >= 2 && !mbar_wait(&sm.k_empty[cbuf], ((cc >> 1) - 1) & 1)) dead = true;
-                        if (!dead && cc >= kVBufs && !mbar_wait(&sm.v_empty[vb], ((cc / kVBufs) - 1) & 1)) dead = true;
-                        if (!dead) {
-                            const int row = pair * s.T + c * kS;
-                            mbar_expect_tx(&sm.k_ready[cbuf], 2 * 8192);
-                            tma_load_2d(kbuf + cbuf * kKBytes, &map_k, &sm.k_ready[cbuf], 0, row);
-                            tma_load_2d(kbuf + cbuf * kKBytes + kNS * 128, &map_k, &sm.k_ready[cbuf], 64, row);
-                            mbar_expect_tx(&sm.v_ready[vb], kVBytes);
-                            tma_load_2d(vbuf + vb * kVBytes, &map_v, &sm.v_ready[vb], 0, row);
-                            tma_load_2d(vbuf + vb * kVBytes + 8192, &map_v, &sm.v_ready[vb], 64, row);
-                            // warm L2 with the K/V rows of the run after the next one
-                            if (ck + 2 < nch) {
-                                const int4 r2 = sm.recs[sm.cfirst[ck + 2]];
-                                const int row2 = r2.x * s.T + r2.y * kS;
-                                tma_prefetch_l2_2d(&map_k, 0, row2);
-                                tma_prefetch_l2_2d(&map_k, 64, row2);
-                                tma_prefetch_l2_2d(&map_v, 0, row2);
-                                tma_prefetch_l2_2d(&map_v, 64, row2);
-                            }
-                        }
-                    }
-                    dead = __shfl_sync(kFullMask, dead ? 1 : 0, 0) != 0;
-                    if (dead || *reinterpret_cast<volatile int*>(&sm.abort_flag)) { dead = true; break; }
-                    // landmark row(s) (keys 64 .. 64 + per - 1) of both K-blocks: the buffer is free (its previous
-                    // user's MMAs are done) and TMA never writes these rows.  V stays as TMA writes it (keys x dims):
-                    // the second MMA reads it as an MN-major operand; keys past the end of the sequence hold other
-                    // rows' data (or TMA zero fill) and meet probabilities of 0.
-                    const bool have_next = ck + 1 < nch;
-                    const int4 r1 = have_next ? sm.recs[sm.cfirst[ck + 1]] : make_int4(0, 0, 0, 0);
+                // landmark row(s) (keys 64 .. 64 + per - 1) of both K-blocks: the buffer is free (its previous
+                // user's MMAs are done) and TMA never writes these rows.  V stays as TMA writes it (keys x dims):
+                // the second MMA reads it as an MN-major operand; keys past the end of the sequence hold other
+                // rows' data (or TMA zero fill) and meet probabilities of 0.
 #pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        const int x = lane + 32 * r;
-                        if (x < per * 16) {
-                            const int pc = x & 15;
-                            *reinterpret_cast<uint4*>(kbuf + cbuf * kKBytes + (pc >> 3) * (kNS * 128) + swz128(64 + (x >> 4), pc & 7)) = lm_cur[r];
-                            if (have_next) lm_cur[r] = lm_piece(r1.x, r1.y, x);
-                        }
-                    }
-                    fence_proxy_async_smem();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&sm.k_ready[cbuf]);
+                for (int r = 0; r < 2; ++r) {
+                    const int x = lane + 32 * r, pc = x & 15;
+                    if (x < per * 16)
+                        *reinterpret_cast<uint4*>(kbuf + cbuf * kKBytes + (pc >> 3) * (kNS * 128) + swz128(64 + (x >> 4), pc & 7)) = lmv[r];
                 }
-                if (dead && lane == 0) { set_status(a.status, kDevTimeout); atomicExch(&sm.abort_flag, 1); }
-            });
-        } else {
-            // ================================================================ MMA issuers (one thread per tile parity)
-            // The issuing thread is the critical path of a tile (it is blocked while the tensor pipe takes its MMAs and
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sm.k_ready[cbuf]);
+            }
+        } else if (warp < kFeedWarp) {
+            // ================================================================ MMA issuers (one warp per tile parity)
+            // The issuer is the critical path of a tile (it is blocked while the tensor pipe takes its MMAs and
             // every barrier test is a shared-memory round trip), so the tiles are split between two of them: warp 17
-            // serves the tiles in S/P/O slot 0, warp 18 those in slot 1.  Each commits its own s_full / o_full; a
-            // thread's MMAs complete in order, which is what the K-buffer hand-back above relies on.
-            const uint32_t par = static_cast<uint32_t>(warp - kMmaWarp);
-            walk([&](int nb, uint32_t tcount, uint32_t ccount, int, int) {
-                if (lane != 0) return;
-                constexpr uint32_t idesc_s = umma_idesc_bf16(kRows, kNS);
-                constexpr uint32_t idesc_o = umma_idesc_bf16(kRows, kD) | kUmmaBMnMajor;
-                const uint32_t sl = par;
-                bool ok = true;
-                // Two in-order queues (S MMAs, O MMAs) over this thread's tiles, served by polling: an O MMA whose
-                // probabilities are ready is never held up by a Q tile that has not arrived yet, and vice versa.  The
-                // chunk run of a tile (its K / V buffers) is looked up in the batch's run table.
-                int ns = static_cast<int>((par ^ tcount) & 1u), no = ns;       // next tile (batch index) for S / O
-                int ck_s = 0, ck_o = 0, run_s = -1, run_o = -1;                 // run of that tile; last run waited for
-                uint32_t idle = 0;
-                while (no < nb && ok) {
-                    bool progressed = false;
-                    if (ns < nb) {
-                        const uint32_t tcv = tcount + ns, qs = tcv % kQSlots;
-                        while (ns >= sm.cfirst[ck_s + 1]) ++ck_s;
-                        const uint32_t cc = ccount + static_cast<uint32_t>(ck_s);
-                        bool ready = mbar_test_wait(&sm.q_full[qs], (tcv / kQSlots) & 1);
-                        if (ready && run_s != ck_s) ready = mbar_test_wait(&sm.k_ready[cc & 1u], (cc >> 1) & 1);
-                        if (ready && tcv >= 2) ready = mbar_test_wait(&sm.s_empty[sl], ((tcv >> 1) - 1) & 1);
-                        if (ready) {
-                            run_s = ck_s;
-                            // the gathered rows were written by cp.async (generic proxy), the MMA reads them through
-                            // the async proxy
-                            fence_proxy_async_smem();
-                            tc_fence_after_sync();
-                            const uint32_t qa = smem_u32(qbuf + qs * kQBytes), ka = smem_u32(kbuf + (cc & 1u) * kKBytes);
-#pragma unroll
-                            for (int ks = 0; ks < 8; ++ks)
-                                umma_bf16(tmem_base + sl * 128, umma_desc_k128(qa + (ks >> 2) * 16384 + (ks & 3) * 32),
-                                          umma_desc_k128(ka + (ks >> 2) * (kNS * 128) + (ks & 3) * 32), idesc_s, ks > 0 ? 1u : 0u);
-                            umma_commit(&sm.s_full[sl]);
-                            ns += 2;
-                            progressed = true;
+            // serves the tiles in S/P/O slot 0, warp 18 those in slot 1.  Each commits its own s_full / o_full; an
+            // issuer's MMAs complete in order, which is what the K-buffer hand-back above relies on.
+            constexpr uint32_t idesc_s = umma_idesc_bf16(kRows, kNS);
+            constexpr uint32_t idesc_o = umma_idesc_bf16(kRows, kD) | kUmmaBMnMajor;
+            const uint32_t sl = static_cast<uint32_t>(warp - kMmaWarp);
+            // Two in-order queues (S MMAs, O MMAs) over this issuer's tiles, served by polling: an O MMA whose
+            // probabilities are ready is never held up by a Q tile that has not arrived yet, and vice versa.
+            uint32_t ns = sl, no = sl;                                     // next tile for S / O
+            uint32_t run_s = ~0u, run_o = ~0u;                              // last runs waited for
+            bool more = true;                                               // there may be another tile for S
+            uint32_t idle = 0;
+            while ((more || no < ns) && ok) {
+                bool progressed = false;
+                if (more) {
+                    const uint32_t qs = ns % kQSlots, m = ns % kMeta;
+                    bool ready = mbar_test_wait(&sm.meta_full[m], (ns / kMeta) & 1);
+                    uint32_t cc = 0;
+                    if (__all_sync(kFullMask, ready)) {
+                        cc = sm.tile[m].run;
+                        if ((sm.tile[m].flags & 255) == 0) {
+                            more = false;
+                            continue;
                         }
+                        ready = mbar_test_wait(&sm.q_full[qs], (ns / kQSlots) & 1);
+                        if (ready && run_s != cc) ready = mbar_test_wait(&sm.k_ready[cc & 1u], (cc >> 1) & 1);
+                        if (ready && ns >= 2) ready = mbar_test_wait(&sm.s_empty[sl], ((ns >> 1) - 1) & 1);
                     }
-                    if (no < ns) {
-                        const uint32_t tcv = tcount + no;
-                        while (no >= sm.cfirst[ck_o + 1]) ++ck_o;
-                        const uint32_t cco = ccount + static_cast<uint32_t>(ck_o);
-                        bool ready = mbar_test_wait(&sm.p_full[sl], (tcv >> 1) & 1);
-                        if (ready && run_o != ck_o) ready = mbar_test_wait(&sm.v_ready[cco % kVBufs], (cco / kVBufs) & 1);
-                        if (ready && tcv >= 2) ready = mbar_test_wait(&sm.o_empty[sl], ((tcv >> 1) - 1) & 1);
-                        if (ready) {
-                            run_o = ck_o;
-                            tc_fence_after_sync();
-                            const uint32_t va = smem_u32(vbuf + (cco % kVBufs) * kVBytes);
-                            // P from tensor memory (columns kPCol.. of the slot: 8 columns = 16 keys per step), V from
-                            // shared memory, 16 keys per step = two 8-row groups
+                    if (__all_sync(kFullMask, ready)) {                     // (the whole warp issues or none of it)
+                        run_s = cc;
+                        // the gathered rows were written by cp.async (generic proxy), the MMA reads them through
+                        // the async proxy
+                        fence_proxy_async_smem();
+                        tc_fence_after_sync();
+                        const uint32_t qa = smem_u32(qbuf + qs * kQBytes), ka = smem_u32(kbuf + (cc & 1u) * kKBytes);
 #pragma unroll
-                            for (int ks = 0; ks < 4; ++ks)
-                                umma_bf16_ts(tmem_base + 256 + sl * 128, tmem_base + sl * 128 + kPCol + ks * 8,
-                                             umma_desc_mn128(va + ks * 2048, 8192u, 1024u), idesc_o, ks > 0 ? 1u : 0u);
-                            umma_commit(&sm.o_full[sl]);
-                            no += 2;
-                            progressed = true;
-                        }
-                    }
-                    if (progressed) {
-                        idle = 0;
-                    } else {
-                        if (++idle > kSpinLimit) ok = false;          // bounded: give up instead of hanging
-                        if (idle > 64) __nanosleep(idle > 4096 ? 256 : 32);
+                        for (int ks = 0; ks < 8; ++ks)
+                            umma_bf16_w(tmem_base + sl * 128, umma_desc_k128(qa + (ks >> 2) * 16384 + (ks & 3) * 32),
+                                        umma_desc_k128(ka + (ks >> 2) * (kNS * 128) + (ks & 3) * 32), idesc_s, ks > 0 ? 1u : 0u);
+                        umma_commit_w(&sm.s_full[sl]);
+                        ns += 2;
+                        progressed = true;
                     }
                 }
-                if (!ok) { set_status(a.status, kDevTimeout); atomicExch(&sm.abort_flag, 1); }
-            });
+                if (no < ns) {
+                    const uint32_t cc = sm.tile[no % kMeta].run;
+                    bool ready = mbar_test_wait(&sm.p_full[sl], (no >> 1) & 1);
+                    if (ready && run_o != cc) ready = mbar_test_wait(&sm.v_ready[cc % kVBufs], (cc / kVBufs) & 1);
+                    if (ready && no >= 2) ready = mbar_test_wait(&sm.o_empty[sl], ((no >> 1) - 1) & 1);
+                    if (__all_sync(kFullMask, ready)) {
+                        run_o = cc;
+                        tc_fence_after_sync();
+                        const uint32_t va = smem_u32(vbuf + (cc % kVBufs) * kVBytes);
+                        // P from tensor memory (columns kPCol.. of the slot: 8 columns = 16 keys per step), V from
+                        // shared memory, 16 keys per step = two 8-row groups
+#pragma unroll
+                        for (int ks = 0; ks < 4; ++ks)
+                            umma_bf16_ts_w(tmem_base + 256 + sl * 128, tmem_base + sl * 128 + kPCol + ks * 8,
+                                           umma_desc_mn128(va + ks * 2048, 8192u, 1024u), idesc_o, ks > 0 ? 1u : 0u);
+                        umma_commit_w(&sm.o_full[sl]);
+                        tile_done(no);
+                        no += 2;
+                        progressed = true;
+                    }
+                }
+                if (progressed) {
+                    idle = 0;
+                } else {
+                    if (++idle > kSpinLimit) ok = false;                    // bounded: give up instead of hanging
+                    if (idle > 64) __nanosleep(256);
+                }
+            }
+    } else {
+        // ================================================================ tile records and entries
+        // a.n_tiles[x], a.n_tiles[x + 1]: first tile of segment x (a query block, or one pair of it) and of the next one; a
+        // launch that walks several blocks takes them in order, the CTA's share of each, so that the CTAs stay on the same
+        // block (its gathered Q rows stay in L2).  A run is a stretch of the share's tiles on one (pair, chunk).  A list
+        // starts on a tile boundary of the global entry space, so the entries of tile t are entries[32 t .. 32 t + 31].
+        // Four tiles are fetched while the ones before them are handed on.  (Batches of 64 tiles between CTA barriers
+        // instead of this ring: 538 us instead of FIG on 16K tokens, K = 16, 32 heads.)
+        uint32_t n = 0, run = 0;
+        auto put = [&](int4 rec, int ent, int flags, int orow0, int first_tok) {
+            AtcTile& tl = sm.tile[n % kMeta];
+            if (n >= kMeta && !wait(&sm.meta_empty[n % kMeta], ((n / kMeta) - 1) & 1)) return;
+            tl.ent[lane] = ent;
+            if (lane == 0) { tl.pair = rec.x; tl.chunk = rec.y; tl.flags = flags; tl.run = run; tl.orow0 = orow0; tl.i0 = first_tok; }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.meta_full[n % kMeta]);
+            ++n;
+        };
+        for (int sg = 0; sg < a.n_run * a.segs && ok; ++sg) {
+            const int blk = sg / a.segs, row0 = a.whole ? 0 : a.n_tiles[blk * a.segs] * kTok;
+            const int s_begin = a.n_tiles[sg], n_tiles = a.n_tiles[sg + 1] - s_begin, i0 = a.i0 + blk * a.qb;
+            const long long lo = s_begin + static_cast<long long>(blockIdx.x) * n_tiles / gridDim.x;
+            const long long hi = s_begin + static_cast<long long>(blockIdx.x + 1) * n_tiles / gridDim.x;
+            int4 prev = make_int4(-1, -1, 0, 0), rec[6];
+            int ent[4];
+            auto same = [](const int4& x, const int4& y) { return x.x == y.x && x.y == y.y; };
+            for (long long t = lo; t < hi && ok; t += 4) {
+#pragma unroll
+                for (int x = 0; x < 6; ++x) rec[x] = t + x < hi ? a.tiles[t + x] : make_int4(-1, -1, 0, 0);
+#pragma unroll
+                for (int x = 0; x < 4; ++x) ent[x] = t + x < hi ? a.entries[(t + x) * kTok + lane] : 0;
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    if (t + x >= hi || !ok) break;
+                    const bool first = !same(rec[x], prev), last = !same(rec[x], rec[x + 1]);
+                    if (first && lane == 0) {                              // some ten tiles ahead of their use: K and V into L2
+                        const int row = rec[x].x * s.T + rec[x].y * kS;
+                        tma_prefetch_l2_2d(&map_k, 0, row);
+                        tma_prefetch_l2_2d(&map_k, 64, row);
+                        tma_prefetch_l2_2d(&map_v, 0, row);
+                        tma_prefetch_l2_2d(&map_v, 64, row);
+                    }
+                    // The K buffer of a run is free when the score MMAs of the run's last tile of EITHER parity are done (the
+                    // two parities have an issuer each): those two tiles arrive once each on k_empty, a run of one tile twice.
+                    const int karr = (last || !same(rec[x], rec[x + 2]) ? 1 : 0) + (first && last ? 1 : 0);
+                    put(rec[x], ent[x], rec[x].w | (first ? 256 : 0) | (last ? 512 : 0) | (karr << 12), (rec[x].z - row0) * kG, i0);
+                    if (last) ++run;
+                    prev = rec[x];
+                }
+            }
         }
-        finish();
+        for (int x = 0; x < 2; ++x)                                        // (one for either parity)
+            if (ok) put(make_int4(0, 0, 0, 0), 0, 0, 0, 0);
     }
+    if (!ok && lane == 0) set_status(a.status, kDevTimeout);
+    __syncwarp();
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    if (warp == kMmaWarp) tmem_dealloc(tmem_base, 512);
 }
 
 }  // namespace
