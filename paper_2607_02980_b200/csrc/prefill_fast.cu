@@ -24,9 +24,8 @@ namespace {
 constexpr int kD = 128;
 constexpr int kS = 64;
 constexpr int kG = 4;
-constexpr int kQBDefault = 4096;             // tokens per pass of the invert/attend/fuse phases: the block's
-                                             // queries (QB x 32 heads x 256 B = 32 MB) stay L2-resident while
-                                             // they are gathered once per selected chunk
+constexpr int kQBMin = 4096, kQBMax = 16384;  // tokens per pass of the invert/attend/fuse phases
+constexpr size_t kObufBytes = 5ull << 30;    // partial outputs that a call keeps at a time (at least those of kQBMin tokens)
 constexpr int kSelStages = 3;
 constexpr int kSelStageBytes = kS * kD * 2;  // 64 landmark rows
 constexpr float kLog2e = 1.4426950408889634f;
@@ -599,15 +598,15 @@ const int kQBEnv = [] {
     const int v = e ? atoi(e) : 0;
     return (v >= 64 && v % 64 == 0 && v <= (1 << 20)) ? v : 0;
 }();
-// Tokens per query block.  A block's tokens that selected a chunk form that chunk's list; lists of about 500 entries
-// (16 tiles) amortise the chunk's K/V load and the ragged last tile, and a list holds about block * K / (visible
-// chunks ~ L / 2S) entries: block ~ 4 L / K, between 4096 (the gathered Q rows of a block stay in L2) and 8192
-// (16384 gains another 0.7 % on 128K tokens for twice the partial-output buffer).
+// Tokens per query block: the longer a block, the longer the lists of its chunks (fewer K/V loads and ragged last tiles), and
+// the attend kernel's walk over one KV head at a time keeps the head's query rows in L2 (16 MB at 16384 tokens).  The
+// partial outputs set the limit: attend + fuse at 16384 against 8192 and 4096 tokens, us:
+// 32K tokens, K = 16: 1698, 1747, -;  64K tokens, K = 32: 6384, 6564, -;  16K tokens, K = 16: 763, 772, 811;  32768 gains nothing.
 int pick_query_block(const Shape& s) {
     if (kQBEnv) return kQBEnv;
-    const long long want = 4ll * (static_cast<long long>(s.pos0) + s.R) / (s.K > 0 ? s.K : 1);
-    int qb = kQBDefault;
-    while (qb < want && qb < 2 * kQBDefault) qb *= 2;
+    const size_t per_tok = static_cast<size_t>(s.B) * s.Hkv * (s.K + max_local_slots(s.W)) * kG * kD * sizeof(__nv_bfloat16);
+    int qb = kQBMax;
+    while (qb > kQBMin && qb * per_tok > kObufBytes) qb /= 2;
     return qb;
 }
 struct Plan {
@@ -655,9 +654,9 @@ Plan make_plan(const Shape& s, int qb_fixed = 0, int t0 = 0) {
     p.off_entries = take(sizeof(int) * all_tiles * tt);
     p.off_epos = take(sizeof(int) * pairs * s.R * (s.K + max_local_slots(s.W)));
     p.off_tiles = take(sizeof(int4) * all_tiles);
-    // Partial outputs of all query blocks at once while that stays under 4 GB: the fusion then runs as one launch
+    // Partial outputs of all query blocks at once where they fit: the fusion then runs as one launch
     // over the whole call instead of one per block (each launch pays its ramp and its last wave).
-    p.whole = (nblocks > 1 && all_tiles * tt * kG * kD * sizeof(__nv_bfloat16) <= (4ull << 30)) ? 1 : 0;
+    p.whole = (nblocks > 1 && all_tiles * tt * kG * kD * sizeof(__nv_bfloat16) <= kObufBytes) ? 1 : 0;
     const size_t obuf_tiles = p.whole ? all_tiles : max_blk;
     p.obuf_tiles = obuf_tiles;
     p.off_obuf = take(sizeof(__nv_bfloat16) * obuf_tiles * tt * kG * kD);
@@ -680,7 +679,13 @@ bool prefill_fast_supports(const Shape& s, int dtype) {
            static_cast<long long>(s.B) * s.Hkv * s.R * (s.K + max_local_slots(s.W)) < (1ll << 31);
 }
 
-size_t prefill_fast_scratch_bytes(const Shape& s) { return make_plan(s).total; }
+size_t prefill_fast_scratch_bytes(const Shape& s) {
+    // (with a routing query no token goes query-major; and fewer tokens may take more scratch, where they just fit at once)
+    const size_t all = make_plan(s).total;
+    const int t0 = prefill_query_tokens(s);
+    const size_t rest = t0 < s.R ? make_plan(s, 0, t0).total : 0;
+    return all > rest ? all : rest;
+}
 
 // Parts of a query block that the inversion's CTAs take: some 8 CTAs per SM, none with fewer entries than its threads hold
 // in one batch.  Returns the CTAs.
@@ -864,9 +869,9 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
             // one launch per query block, or a single launch that walks all of them (whole-call output buffers)
             const CUtensorMap maps[3] = {map_k, map_v, map_o};
             // With many tiles per (block, pair) the launch walks the pairs one after the other: all CTAs then gather the
-            // query rows of one KV head at a time (8 MB instead of 67 MB at 8192 tokens and 8 KV heads, which L2 keeps).
-            // Below some 40 tiles per CTA and pair the additional ends of chunk runs cost more.
-            const bool by_pair = static_cast<long long>(a.qb) * (s.K + max_local_slots(s.W)) >= 40ll * a.tile_tok * sm_count();
+            // query rows of one KV head at a time, which L2 keeps.  With few tiles the additional ends of chunk runs cost more:
+            // at 29 tiles per CTA and pair 1202 -> 1026 us, at 20 200 -> 191, at 4 102 -> 115.
+            const bool by_pair = static_cast<long long>(a.qb) * (s.K + max_local_slots(s.W)) >= 12ll * a.tile_tok * sm_count();
             const int rc = launch_prefill_attend_tc(s, t.q, maps, t.landmarks, t.bias, a.entries, a.tiles,
                                                     by_pair ? a.pair_toff + blk * pairs : a.blk_toff + blk, by_pair ? pairs : 1, a.lam,
                                                     t.status, a.i0, a.whole, a.whole ? p.n_blocks : 1, a.qb, stream);
