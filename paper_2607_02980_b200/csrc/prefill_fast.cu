@@ -44,7 +44,7 @@ struct PArgs {
     int* cursor;            // [pairs*C]
     int* blk_toff;          // [n_blocks + 1] first tile of every query block (tiles are grouped by block)
     int* pair_toff;         // [n_blocks * pairs + 1] first tile of every (block, pair)
-    int* seg_tiles;         // [ceil(lists / 1024)] tiles of each segment of 1024 lists
+    int* seg_tiles;         // [ceil(lists / kSegLists)] tiles of each segment of lists
     int* off;               // [n_blocks*pairs*nc] first entry of each list; every list starts on a tile boundary
     int* entries;           // [max_tiles * tile_tok] (token_local << 8) | slot, grouped by (block, pair, chunk);
                             // slot K marks the token's own chunk (local branch); list tails up to the next tile
@@ -340,31 +340,32 @@ __global__ void __launch_bounds__(kInvThreads, 3) invert_count_kernel(const PArg
     }
 }
 
-// Exclusive prefix sum of the tiles per list, ceil(cnt / tile_tok), in two launches of one CTA per 1024 lists:
+// Exclusive prefix sum of the tiles per list, ceil(cnt / tile_tok), in two launches of one CTA per kSegLists lists:
 // segment sums first, then every CTA adds up the sums of the segments before its own and scans its segment.
 // A list's first entry is its first tile x tile_tok, so the tiles of a query block cover one contiguous,
-// tile-aligned range of entries.
-__global__ void __launch_bounds__(1024) invert_segsum_kernel(const PArgs a) {
-    __shared__ int wsum[32];
+// tile-aligned range of entries.  (Small segments: the scan also writes the tile records, and 1024 lists can have 30,000 of
+// them; 16K tokens, K = 16: inversion 48 -> 38 us with 256 lists and a warp per list.)
+constexpr int kSegLists = 256;
+__global__ void __launch_bounds__(kSegLists) invert_segsum_kernel(const PArgs a) {
+    __shared__ int wsum[kSegLists / 32];
     pdl_wait();
     const int n = a.s.B * a.s.Hkv * a.nc * a.n_blocks;
-    const int x = blockIdx.x * 1024 + threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int x = blockIdx.x * kSegLists + threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int ct = x < n ? (a.cnt[x] + a.tile_tok - 1) / a.tile_tok : 0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ct += __shfl_xor_sync(kFullMask, ct, o);
     if (lane == 0) wsum[warp] = ct;
     __syncthreads();
-    if (warp == 0) {
-        int v = wsum[lane];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFullMask, v, o);
-        if (lane == 0) a.seg_tiles[blockIdx.x] = v;
+    if (threadIdx.x == 0) {
+        int v = 0;
+        for (int w = 0; w < kSegLists / 32; ++w) v += wsum[w];
+        a.seg_tiles[blockIdx.x] = v;
     }
 }
 
-__global__ void __launch_bounds__(1024) invert_scan_kernel(const PArgs a) {
-    __shared__ int wsum_t[32];
-    __shared__ int wpre[32];
+__global__ void __launch_bounds__(kSegLists) invert_scan_kernel(const PArgs a) {
+    __shared__ int wsum_t[kSegLists / 32];
+    __shared__ int wpre[kSegLists / 32];
     pdl_wait();
     const Shape& s = a.s;
     const int per_blk = s.B * s.Hkv * a.nc;
@@ -372,11 +373,11 @@ __global__ void __launch_bounds__(1024) invert_scan_kernel(const PArgs a) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // tiles of all earlier segments
     int pre = 0;
-    for (int sg = tid; sg < static_cast<int>(blockIdx.x); sg += 1024) pre += a.seg_tiles[sg];
+    for (int sg = tid; sg < static_cast<int>(blockIdx.x); sg += kSegLists) pre += a.seg_tiles[sg];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) pre += __shfl_xor_sync(kFullMask, pre, o);
     if (lane == 0) wpre[warp] = pre;
-    const int x = blockIdx.x * 1024 + tid;
+    const int x = blockIdx.x * kSegLists + tid;
     const int ce = x < n ? a.cnt[x] : 0;
     const int ct = (ce + a.tile_tok - 1) / a.tile_tok;
     int it = ct;
@@ -388,20 +389,24 @@ __global__ void __launch_bounds__(1024) invert_scan_kernel(const PArgs a) {
     if (lane == 31) wsum_t[warp] = it;
     __syncthreads();
     int bt = 0;
-    for (int w = 0; w < 32; ++w) bt += wpre[w] + (w < warp ? wsum_t[w] : 0);
+    for (int w = 0; w < kSegLists / 32; ++w) bt += wpre[w] + (w < warp ? wsum_t[w] : 0);
     const int ot = bt + it - ct, oe = ot * a.tile_tok;
     if (x < n) {
         a.off[x] = oe;
-        const int pair = (x % per_blk) / a.nc, c = x % a.nc;
         if (x % per_blk == 0) a.blk_toff[x / per_blk] = ot;
-        if (c == 0) a.pair_toff[x / a.nc] = min(ot, a.max_tiles);
-        for (int k = 0; k < ct; ++k)
-            if (ot + k < a.max_tiles)
-                a.tiles[ot + k] = make_int4(pair, c, oe + k * a.tile_tok, min(a.tile_tok, ce - k * a.tile_tok));
+        if (x % a.nc == 0) a.pair_toff[x / a.nc] = min(ot, a.max_tiles);
         if (x == n - 1) {
             a.blk_toff[a.n_blocks] = min(ot + ct, a.max_tiles);
             a.pair_toff[n / a.nc] = min(ot + ct, a.max_tiles);
         }
+    }
+    // the tile records, a list at a time
+    for (int l = 0; l < 32; ++l) {
+        const int lct = __shfl_sync(kFullMask, ct, l), lot = __shfl_sync(kFullMask, ot, l), lce = __shfl_sync(kFullMask, ce, l);
+        const int lx = x - lane + l, pair = (lx % per_blk) / a.nc, c = lx % a.nc;
+        for (int k = lane; k < lct; k += 32)
+            if (lot + k < a.max_tiles)
+                a.tiles[lot + k] = make_int4(pair, c, (lot + k) * a.tile_tok, min(a.tile_tok, lce - k * a.tile_tok));
     }
 }
 
@@ -649,7 +654,7 @@ Plan make_plan(const Shape& s, int qb_fixed = 0, int t0 = 0) {
     p.off_ntiles = take(sizeof(int) * (nblocks + 1));
     p.zero_bytes = off;                         // cnt, cursor, blk_toff are cleared together once per call
     p.off_ptiles = take(sizeof(int) * (nblocks * pairs + 1));
-    p.off_seg = take(sizeof(int) * ((nblocks * pairs * nc + 1023) / 1024));
+    p.off_seg = take(sizeof(int) * ((nblocks * pairs * nc + kSegLists - 1) / kSegLists));
     p.off_off = take(sizeof(int) * nblocks * pairs * nc);
     p.off_entries = take(sizeof(int) * all_tiles * tt);
     p.off_epos = take(sizeof(int) * pairs * s.R * (s.K + max_local_slots(s.W)));
@@ -732,10 +737,10 @@ int build_inverse_index(const Shape& s, const int32_t* sel, void* scratch, size_
     a.tile_tok = attend_tc_tile_tokens();
     if (cudaMemsetAsync(sc + p.off_cnt, 0, p.zero_bytes, stream) != cudaSuccess) return HILS_ERR_CUDA;
     const unsigned eb = invert_split(a, p);
-    const unsigned nseg = static_cast<unsigned>((static_cast<long long>(p.n_blocks) * pairs * p.nc + 1023) / 1024);
+    const unsigned nseg = static_cast<unsigned>((static_cast<long long>(p.n_blocks) * pairs * p.nc + kSegLists - 1) / kSegLists);
     if (launch_pdl(invert_count_kernel, dim3(eb), dim3(kInvThreads), invert_smem(a), stream, a) != cudaSuccess ||
-        launch_pdl(invert_segsum_kernel, dim3(nseg), dim3(1024), 0, stream, a) != cudaSuccess ||
-        launch_pdl(invert_scan_kernel, dim3(nseg), dim3(1024), 0, stream, a) != cudaSuccess ||
+        launch_pdl(invert_segsum_kernel, dim3(nseg), dim3(kSegLists), 0, stream, a) != cudaSuccess ||
+        launch_pdl(invert_scan_kernel, dim3(nseg), dim3(kSegLists), 0, stream, a) != cudaSuccess ||
         launch_pdl(invert_fill_kernel, dim3(eb), dim3(kInvThreads), invert_smem(a), stream, a) != cudaSuccess)
         return HILS_ERR_CUDA;
     trace_mark("backward_invert", stream);
@@ -850,12 +855,12 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
             invert_count_kernel<<<eb, kInvThreads, invert_smem(a), stream>>>(a);
             ++launches;
         }
-        const unsigned nseg = static_cast<unsigned>((static_cast<long long>(p.n_blocks) * pairs * p.nc + 1023) / 1024);
+        const unsigned nseg = static_cast<unsigned>((static_cast<long long>(p.n_blocks) * pairs * p.nc + kSegLists - 1) / kSegLists);
         // From here on every kernel of the call is launched so that its launch and prologue overlap the previous
         // kernel's tail; each of them waits for its predecessors' results before its first dependent access.  None
         // triggers its dependents early: CTAs of the next kernel parked beside a running attend kernel cost 5 %.
-        if (launch_pdl(invert_segsum_kernel, dim3(nseg), dim3(1024), 0, stream, a) != cudaSuccess ||
-            launch_pdl(invert_scan_kernel, dim3(nseg), dim3(1024), 0, stream, a) != cudaSuccess ||
+        if (launch_pdl(invert_segsum_kernel, dim3(nseg), dim3(kSegLists), 0, stream, a) != cudaSuccess ||
+            launch_pdl(invert_scan_kernel, dim3(nseg), dim3(kSegLists), 0, stream, a) != cudaSuccess ||
             launch_pdl(invert_fill_kernel, dim3(eb), dim3(kInvThreads), invert_smem(a), stream, a) != cudaSuccess)
             return HILS_ERR_CUDA;
         trace_mark("prefill_invert", stream);
