@@ -312,7 +312,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
             if (lane == 0) tile_done(n);
             if (!wait(&sm.dq_full, n & 1)) break;
             tc_fence_after_sync();
-            uint32_t va[32], vb[32];
+            uint32_t va[32];
             // 32 columns at a time, the borrowed ones first (the first for the even tiles, the last for the odd ones)
             const uint32_t q_tm = t_lane + dq_col(sl);
             const int x0 = sl ? 3 : 0, dx = sl ? -1 : 1;
@@ -320,11 +320,20 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
             const float dl = sm.dlam[sl][row];
             float* dst0 = a.dq + (lane & 7) * 4;
             // through shared memory: a request then adds whole 128-byte runs of four rows
-            auto add = [&](const uint32_t (&v)[32], int x) {
-                const float4 l = *reinterpret_cast<const float4*>(&sm.lmf[rw][32 * x + (lane & 7) * 4]);
+#pragma unroll 1
+            for (int p = 0; p < 4; ++p) {
+                const int x = x0 + dx * p;
+                tmem_ld_wait32(va);
+                if (p == 0 || p == 3) {
+                    tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(p == 0 ? &sm.slot_empty[sl] : &sm.dq_empty);
+                }
 #pragma unroll
                 for (int i = 0; i < 8; ++i)
-                    *reinterpret_cast<uint4*>(&stg[lane][4 * i]) = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                    *reinterpret_cast<uint4*>(&stg[lane][4 * i]) = make_uint4(va[4 * i], va[4 * i + 1], va[4 * i + 2], va[4 * i + 3]);
+                if (p < 3) tmem_ld32_issue(q_tm + 32 * (x + dx), va);
+                const float4 l = *reinterpret_cast<const float4*>(&sm.lmf[rw][32 * x + (lane & 7) * 4]);
                 __syncwarp();
 #pragma unroll
                 for (int i0 = 0; i0 < 8; i0 += 4) {
@@ -341,26 +350,6 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                     }
                 }
                 __syncwarp();
-            };
-#pragma unroll 1
-            for (int x = 0; x < 4; x += 2) {
-                tmem_ld_wait32(va);
-                if (x == 0) {
-                    tc_fence_before_sync();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&sm.slot_empty[sl]);
-                }
-                tmem_ld32_issue(q_tm + 32 * (x0 + dx * (x + 1)), vb);
-                add(va, x0 + dx * x);
-                tmem_ld_wait32(vb);
-                if (x == 0) {
-                    tmem_ld32_issue(q_tm + 32 * (x0 + dx * 2), va);
-                } else {
-                    tc_fence_before_sync();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&sm.dq_empty);
-                }
-                add(vb, x0 + dx * (x + 1));
             }
             if (flags & 512) {
                 // ---- the run's last tile: d K^T and d V^T leave tensor memory, a lane per dimension
@@ -426,20 +415,21 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 bacc = 0.f;
             }
         };
-        uint32_t n = 0;
-        for (; tile_of(n); ++n) {
-            const Tile& tl = sm.tile[n % kMeta];
+        uint32_t end = ~0u;                                              // number of tiles, once known; the sums run two behind
+        for (uint32_t n = 0; ok; ++n) {
+            if (n < end && !tile_of(n)) end = n;
+            if (!ok || (end != ~0u && n >= end + 2)) break;
             const uint32_t sl = n & 1u;
+            if (n >= 2) landmark_sums(n - 2, fl1, lr1);
+            fl1 = fl0;
+            lr1 = lr0;
+            if (n >= end) continue;
+            const Tile& tl = sm.tile[n % kMeta];
             const int tok = tl.ent[min(8 * gw + (lane & 7), (tl.flags & 255) - 1)] >> 8;
             const int b = tl.pair / s.Hkv, gk = tl.pair - b * s.Hkv, c = tl.chunk, i0 = tl.i0, flags = tl.flags;
             __syncwarp();
             if (lane == 0) tile_done(n);
-            if (n >= 2) {
-                landmark_sums(n - 2, fl1, lr1);
-                if (!wait(&sm.done[sl], ((n >> 1) - 1) & 1)) break;
-            }
-            fl1 = fl0;
-            lr1 = lr0;
+            if (n >= 2 && !wait(&sm.done[sl], ((n >> 1) - 1) & 1)) break;
             fl0 = flags;
             lr0 = c < s.C ? (b * s.Hl + gk) * s.C + c : -1;              // (B Hkv C < 2^24)
             __syncwarp();
@@ -464,8 +454,6 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.q_full[sl]);
         }
-        if (n >= 2) landmark_sums(n - 2, fl1, lr1);
-        if (n >= 1) landmark_sums(n - 1, fl0, lr0);
         asm volatile("cp.async.wait_all;" ::: "memory");
     } else if (warp == kLoadWarp) {
         // ================================================================ K, V and landmark of the runs
@@ -521,15 +509,18 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 tc_fence_after_sync();
                 const uint64_t dq0 = umma_desc_k128(smem_u32(qbuf) + sl * kQBytes), do0 = umma_desc_k128(smem_u32(obuf) + sl * kQBytes);
                 const uint32_t d = tmem_base + slot_col(sl);
+                if (elect_one()) {
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks)
-                    umma_bf16_w(d, dq0 + (((ks >> 2) * 16384 + (ks & 3) * 32) >> 4), dk0 + (((ks >> 2) * (kNS * 128) + (ks & 3) * 32) >> 4),
-                              idesc_s, ks > 0 ? 1u : 0u);
+                    for (int ks = 0; ks < 8; ++ks)
+                        umma_bf16(d, dq0 + (((ks >> 2) * 16384 + (ks & 3) * 32) >> 4), dk0 + (((ks >> 2) * (kNS * 128) + (ks & 3) * 32) >> 4),
+                                  idesc_s, ks > 0 ? 1u : 0u);
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks)
-                    umma_bf16_w(d + kTCol, do0 + (((ks >> 2) * 16384 + (ks & 3) * 32) >> 4), dv0 + (((ks >> 2) * 8192 + (ks & 3) * 32) >> 4),
-                              idesc_t, ks > 0 ? 1u : 0u);
-                umma_commit_w(&sm.st_full[sl]);
+                    for (int ks = 0; ks < 8; ++ks)
+                        umma_bf16(d + kTCol, do0 + (((ks >> 2) * 16384 + (ks & 3) * 32) >> 4), dv0 + (((ks >> 2) * 8192 + (ks & 3) * 32) >> 4),
+                                  idesc_t, ks > 0 ? 1u : 0u);
+                    umma_commit(&sm.st_full[sl]);
+                }
+                __syncwarp();
             }
         }
     } else if (warp == kBackWarp) {
@@ -551,11 +542,14 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 if (n > 0) wait(&sm.dq_empty, (n - 1) & 1);
                 if (!wait(&sm.ds_full[sl], (n >> 1) & 1)) break;
                 tc_fence_after_sync();
+                if (elect_one()) {
 #pragma unroll
-                for (int ks = 0; ks < 4; ++ks)
-                    umma_bf16_w(tmem_base + dq_col(sl), dsk + ((ks * 32) >> 4), kmn + ((ks * 2048) >> 4), idesc_q, ks > 0 ? 1u : 0u);
-                umma_commit_w(&sm.dq_full);
-                if (flags & 512) umma_commit_w(&sm.k_empty);
+                    for (int ks = 0; ks < 4; ++ks)
+                        umma_bf16(tmem_base + dq_col(sl), dsk + ((ks * 32) >> 4), kmn + ((ks * 2048) >> 4), idesc_q, ks > 0 ? 1u : 0u);
+                    umma_commit(&sm.dq_full);
+                    if (flags & 512) umma_commit(&sm.k_empty);
+                }
+                __syncwarp();
                 // the previous run's accumulators have been read
                 if (first && run > 1) {
                     if (!wait(&sm.acc_empty, (run - 2) & 1)) break;
@@ -563,13 +557,16 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 }
                 const uint64_t qmn = umma_desc_mn128(smem_u32(qbuf) + sl * kQBytes, 16384u, 1024u);
                 const uint64_t omn = umma_desc_mn128(smem_u32(obuf) + sl * kQBytes, 16384u, 1024u);
+                if (elect_one()) {
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {
-                    const uint32_t accf = (!first || ks > 0) ? 1u : 0u;
-                    umma_bf16_w(tmem_base + kDkCol, qmn + ((ks * 2048) >> 4), dsmn + ((ks * 2048) >> 4), idesc_kv, accf);
-                    umma_bf16_w(tmem_base + kDvCol, omn + ((ks * 2048) >> 4), wmn + ((ks * 2048) >> 4), idesc_kv, accf);
+                    for (int ks = 0; ks < 8; ++ks) {
+                        const uint32_t accf = (!first || ks > 0) ? 1u : 0u;
+                        umma_bf16(tmem_base + kDkCol, qmn + ((ks * 2048) >> 4), dsmn + ((ks * 2048) >> 4), idesc_kv, accf);
+                        umma_bf16(tmem_base + kDvCol, omn + ((ks * 2048) >> 4), wmn + ((ks * 2048) >> 4), idesc_kv, accf);
+                    }
+                    umma_commit(&sm.done[sl]);
                 }
-                umma_commit_w(&sm.done[sl]);
+                __syncwarp();
             }
             // every product has completed before tensor memory is freed
             if (n > 0 && ok) wait(&sm.done[(n - 1) & 1], ((n - 1) >> 1) & 1);
@@ -577,16 +574,16 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     } else {
         // ================================================================ tile records and entries
         // The segments (query blocks, or one pair of each) one after the other, the CTA's share of each; a run is a stretch
-        // of the share's tiles on one (pair, chunk).  Four tiles are fetched while the four before them are handed on.
+        // of the share's tiles on one (pair, chunk).  A lane holds a tile's record; the entries are fetched two tiles ahead.
         uint32_t n = 0;
         int sg = -1;
         long long t = 0, hi = 0;
         int i0 = 0;
-        auto put = [&](int4 rec, int ent, int flags, int first_tok) {
+        auto put = [&](int pair, int chunk, int flags, int ent, int first_tok) {
             Tile& tl = sm.tile[n % kMeta];
             if (n >= kMeta && !wait(&sm.meta_empty[n % kMeta], ((n / kMeta) - 1) & 1)) return;
             tl.ent[lane] = ent;
-            if (lane == 0) { tl.pair = rec.x; tl.chunk = rec.y; tl.flags = flags; tl.i0 = first_tok; }
+            if (lane == 0) { tl.pair = pair; tl.chunk = chunk; tl.flags = flags; tl.i0 = first_tok; }
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.meta_full[n % kMeta]);
             ++n;
@@ -599,27 +596,33 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 hi = t_begin + static_cast<long long>(blockIdx.x + 1) * n_tiles / gridDim.x;
             }
             if (t >= hi) break;
-            const long long lo = t;
-            int4 prev = make_int4(-1, -1, 0, 0), rec[5];
-            int ent[4];
-            for (; t < hi && ok; t += 4) {
-#pragma unroll
-                for (int x = 0; x < 5; ++x) rec[x] = t + x < hi ? a.tiles[t + x] : make_int4(-1, -1, 0, 0);
-#pragma unroll
-                for (int x = 0; x < 4; ++x) ent[x] = t + x < hi ? a.entries[(t + x) * kTok + lane] : 0;
-#pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    if (t + x >= hi || !ok) break;
-                    const bool first = t + x == lo || rec[x].x != prev.x || rec[x].y != prev.y;
-                    const bool last = rec[x].x != rec[x + 1].x || rec[x].y != rec[x + 1].y;
-                    put(rec[x], ent[x], rec[x].w | (first ? 256 : 0) | (last ? 512 : 0), i0);
-                    prev = rec[x];
+            int4 prev = make_int4(-1, -1, 0, 0);
+            for (; t < hi && ok; t += 32) {
+                // lane x: record and flags of tile t + x
+                const int nb = static_cast<int>(hi - t < 32 ? hi - t : 32);
+                const int4 rec = lane < nb ? a.tiles[t + lane] : make_int4(-1, -1, 0, 0);
+                const int4 after = t + 32 < hi ? a.tiles[t + 32] : make_int4(-1, -1, 0, 0);
+                int px = __shfl_up_sync(kFullMask, rec.x, 1), py = __shfl_up_sync(kFullMask, rec.y, 1);
+                int nx = __shfl_down_sync(kFullMask, rec.x, 1), ny = __shfl_down_sync(kFullMask, rec.y, 1);
+                if (lane == 0) { px = prev.x; py = prev.y; }
+                if (lane == 31) { nx = after.x; ny = after.y; }
+                const int flags = rec.w | (rec.x != px || rec.y != py ? 256 : 0) | (rec.x != nx || rec.y != ny ? 512 : 0);
+                int e0 = a.entries[t * kTok + lane], e1 = nb > 1 ? a.entries[(t + 1) * kTok + lane] : 0;
+#pragma unroll 1
+                for (int x = 0; x < nb && ok; ++x) {
+                    const int e2 = x + 2 < nb ? a.entries[(t + x + 2) * kTok + lane] : 0;
+                    put(__shfl_sync(kFullMask, rec.x, x), __shfl_sync(kFullMask, rec.y, x), __shfl_sync(kFullMask, flags, x), e0, i0);
+                    e0 = e1;
+                    e1 = e2;
                 }
+                prev.x = __shfl_sync(kFullMask, rec.x, 31);
+                prev.y = __shfl_sync(kFullMask, rec.y, 31);
             }
             t = hi;
         }
+#pragma unroll 1
         for (int x = 0; x < 2; ++x)                                     // (one for either statistics group)
-            if (ok) put(make_int4(0, 0, 0, 0), 0, 0, 0);
+            if (ok) put(0, 0, 0, 0, 0);
     }
     if (!ok && lane == 0) set_status(a.status, kDevTimeout);
     __syncwarp();

@@ -450,11 +450,14 @@ prefill_attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
                         fence_proxy_async_smem();
                         tc_fence_after_sync();
                         const uint32_t qa = smem_u32(qbuf + qs * kQBytes), ka = smem_u32(kbuf + (cc & 1u) * kKBytes);
+                        if (elect_one()) {
 #pragma unroll
-                        for (int ks = 0; ks < 8; ++ks)
-                            umma_bf16_w(tmem_base + sl * 128, umma_desc_k128(qa + (ks >> 2) * 16384 + (ks & 3) * 32),
-                                        umma_desc_k128(ka + (ks >> 2) * (kNS * 128) + (ks & 3) * 32), idesc_s, ks > 0 ? 1u : 0u);
-                        umma_commit_w(&sm.s_full[sl]);
+                            for (int ks = 0; ks < 8; ++ks)
+                                umma_bf16(tmem_base + sl * 128, umma_desc_k128(qa + (ks >> 2) * 16384 + (ks & 3) * 32),
+                                          umma_desc_k128(ka + (ks >> 2) * (kNS * 128) + (ks & 3) * 32), idesc_s, ks > 0 ? 1u : 0u);
+                            umma_commit(&sm.s_full[sl]);
+                        }
+                        __syncwarp();
                         ns += 2;
                         progressed = true;
                     }
@@ -470,11 +473,14 @@ prefill_attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
                         const uint32_t va = smem_u32(vbuf + (cc % kVBufs) * kVBytes);
                         // P from tensor memory (columns kPCol.. of the slot: 8 columns = 16 keys per step), V from
                         // shared memory, 16 keys per step = two 8-row groups
+                        if (elect_one()) {
 #pragma unroll
-                        for (int ks = 0; ks < 4; ++ks)
-                            umma_bf16_ts_w(tmem_base + 256 + sl * 128, tmem_base + sl * 128 + kPCol + ks * 8,
-                                           umma_desc_mn128(va + ks * 2048, 8192u, 1024u), idesc_o, ks > 0 ? 1u : 0u);
-                        umma_commit_w(&sm.o_full[sl]);
+                            for (int ks = 0; ks < 4; ++ks)
+                                umma_bf16_ts(tmem_base + 256 + sl * 128, tmem_base + sl * 128 + kPCol + ks * 8,
+                                             umma_desc_mn128(va + ks * 2048, 8192u, 1024u), idesc_o, ks > 0 ? 1u : 0u);
+                            umma_commit(&sm.o_full[sl]);
+                        }
+                        __syncwarp();
                         tile_done(no);
                         no += 2;
                         progressed = true;
