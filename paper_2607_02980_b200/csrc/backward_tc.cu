@@ -320,6 +320,13 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
             const float dl = sm.dlam[sl][row];
             float* dst0 = a.dq + (lane & 7) * 4;
             // through shared memory: a request then adds whole 128-byte runs of four rows
+            int ro[8];
+            float rd[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                ro[i] = __shfl_sync(kFullMask, orow, i * 4 + (lane >> 3));
+                rd[i] = __shfl_sync(kFullMask, dl, i * 4 + (lane >> 3));
+            }
 #pragma unroll 1
             for (int p = 0; p < 4; ++p) {
                 const int x = x0 + dx * p;
@@ -342,8 +349,8 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                     for (int i = 0; i < 4; ++i) g[i] = *reinterpret_cast<const float4*>(&stg[(i0 + i) * 4 + (lane >> 3)][(lane & 7) * 4]);
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        const int rr = (i0 + i) * 4 + (lane >> 3), o = __shfl_sync(kFullMask, orow, rr);
-                        const float d = __shfl_sync(kFullMask, dl, rr);
+                        const int o = ro[i0 + i];
+                        const float d = rd[i0 + i];
                         if (o >= 0)
                             red_add_v4(dst0 + static_cast<long long>(o) * kD + 32 * x, fmaf(d, l.x, g[i].x), fmaf(d, l.y, g[i].y),
                                        fmaf(d, l.z, g[i].z), fmaf(d, l.w, g[i].w));
