@@ -62,10 +62,12 @@ struct BArgs {
 };
 
 struct Tile {
-    int pair, chunk;
-    int flags;                                  // entries (0: no more tiles) | first tile of its run << 8 | last << 9
-    int i0;                                     // first token of the query block
-    int ent[kTok];                              // (token - i0) << 8 | slot
+    int flags;                                  // entries (0: no more tiles) | first tile of its run << 8 | last << 9 | keys << 16
+    int row0;                                   // q, dO, dq row of the query block's first token, head 0 of the KV head
+    int kv;                                     // first k, v row of the chunk
+    int lm;                                     // landmark row of the chunk (-1: none)
+    int vis;                                    // last visible key of a local row: this + the token
+    int ent[kTok];                              // (token of the query block) << 8 | slot
 };
 struct BSmem {
     alignas(16) float stg[4][32][36];           // read-out of d Q: a warp's 32 rows x 32 columns (padded rows)
@@ -163,14 +165,13 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         const float c2 = s.scale * kLog2e;
         for (uint32_t n = grp; tile_of(n); n += 2) {
             const Tile& tl = sm.tile[n % kMeta];
-            const int n_ent = tl.flags & 255, ent = tl.ent[min(e_row, n_ent - 1)], tok = tl.i0 + (ent >> 8);
-            const int b = tl.pair / s.Hkv, gk = tl.pair - b * s.Hkv, c = tl.chunk;
+            const int n_ent = tl.flags & 255, ent = tl.ent[min(e_row, n_ent - 1)], lmr = tl.lm;
             const bool local = (ent & 255) >= s.K;
             // last visible key of the row; -1 for the rows of a ragged tile's padding
-            const int limit = e_row >= n_ent ? -1 : local ? min(kS - 1, s.pos0 + tok - c * kS) : kS - 1;
-            const int orow = (b * s.Hq + gk * kG + hd) * hs + tok;
+            const int limit = e_row >= n_ent ? -1 : local ? min(kS - 1, tl.vis + (ent >> 8)) : kS - 1;
+            const int orow = tl.row0 + hd * hs + (ent >> 8);
             const float lse = __ldg(a.lse + orow), dsum = a.dsum[orow];
-            const float bb = (a.bias && c < s.C) ? __ldg(a.bias + (static_cast<long long>(b) * s.Hl + gk) * s.C + c) : 0.f;
+            const float bb = (a.bias && lmr >= 0) ? __ldg(a.bias + lmr) : 0.f;
             const bool masked = __any_sync(kFullMask, limit < kS - 1);
             if (lane == 0) tile_done(n);
             if (!wait(&sm.st_full[grp], (n >> 1) & 1)) break;
@@ -296,18 +297,17 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         for (uint32_t n = 0; tile_of(n); ++n) {
             const Tile& tl = sm.tile[n % kMeta];
             const uint32_t sl = n & 1u;
-            const int flags = tl.flags, pair = tl.pair, c = tl.chunk;
-            const int b = pair / s.Hkv, gk = pair - b * s.Hkv;
+            const int flags = tl.flags, kv = tl.kv;
             if (flags & 256) {
                 float4 l = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (c < s.C) {
-                    const uint2 raw = *reinterpret_cast<const uint2*>(a.lm + ((static_cast<long long>(b) * s.Hl + gk) * s.C + c) * kD + 4 * lane);
+                if (tl.lm >= 0) {
+                    const uint2 raw = *reinterpret_cast<const uint2*>(a.lm + static_cast<long long>(tl.lm) * kD + 4 * lane);
                     l = make_float4(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u),
                                     __uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u));
                 }
                 *reinterpret_cast<float4*>(&sm.lmf[rw][4 * lane]) = l;
             }
-            const int orow = e_row < (flags & 255) ? (b * s.Hq + gk * kG + (row & 3)) * hs + tl.i0 + (tl.ent[e_row] >> 8) : -1;
+            const int orow = e_row < (flags & 255) ? tl.row0 + (row & 3) * hs + (tl.ent[e_row] >> 8) : -1;
             __syncwarp();
             if (lane == 0) tile_done(n);
             if (!wait(&sm.dq_full, n & 1)) break;
@@ -362,8 +362,8 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 // ---- the run's last tile: d K^T and d V^T leave tensor memory, a lane per dimension
                 if (!wait(&sm.done[sl], (n >> 1) & 1)) break;
                 tc_fence_after_sync();
-                const long long at = (static_cast<long long>(pair) * s.T + static_cast<long long>(c) * kS) * kD + rw * 32 + lane;
-                const int keys = min(kS, s.T - c * kS);
+                const long long at = static_cast<long long>(kv) * kD + rw * 32 + lane;
+                const int keys = (flags >> 16) & 127;
 #pragma unroll 1
                 for (int h = 0; h < 4; ++h) {
                     tmem_ld32_issue(t_lane + kDkCol + 32 * h, va);
@@ -385,30 +385,35 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         // (entry-major, head-minor; an instruction copies two 256-byte rows of one entry, see the forward's gather; a warp
         // fills rows 32 gw .. 32 gw + 31 of the tile and sums the same rows for d landmark before it overwrites them)
         const int gw = warp - kGatherWarp, p16 = lane & 15, hh = lane >> 4;
-        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, bacc = 0.f;       // dims 8 p16 .. + 7, rows of parity hh
+        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, bacc = 0.f;       // dims 8 p16 .. + 7, rows of half hh
         int fl0 = 0, fl1 = 0;                                                       // flags of the last tile and the one before
         int lr0 = 0, lr1 = 0;                                                       // their landmark rows (-1: none)
         auto landmark_sums = [&](uint32_t n, int fl, int lr) {                                      // tile n: + sum over its rows of (scale d lambda) q
             const uint32_t sl = n & 1u;
             if (!wait(&sm.ds_full[sl], (n >> 1) & 1)) return;
-            const float dl = sm.dlam[sl][gw * 32 + lane];
+            // (half a warp sums 16 neighbouring rows)
+            const float4* dl = reinterpret_cast<const float4*>(&sm.dlam[sl][gw * 32 + hh * 16]);
             const uint8_t* qt = qbuf + sl * kQBytes + (p16 >> 3) * 16384;
-#pragma unroll 4
-            for (int r = 0; r < 16; ++r) {
-                const float d = __shfl_sync(kFullMask, dl, 2 * r + hh);
-                const uint4 raw = *reinterpret_cast<const uint4*>(qt + swz128(gw * 32 + 2 * r + hh, p16 & 7));
-                const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll 1
+            for (int r = 0; r < 4; ++r) {
+                const float4 d4 = dl[r];
+                const float d[4] = {d4.x, d4.y, d4.z, d4.w};
 #pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    acc[2 * x] = fmaf(d, __uint_as_float(w[x] << 16), acc[2 * x]);
-                    acc[2 * x + 1] = fmaf(d, __uint_as_float(w[x] & 0xffff0000u), acc[2 * x + 1]);
+                for (int i = 0; i < 4; ++i) {
+                    const uint4 raw = *reinterpret_cast<const uint4*>(qt + swz128(gw * 32 + hh * 16 + 4 * r + i, p16 & 7));
+                    const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) {
+                        acc[2 * x] = fmaf(d[i], __uint_as_float(w[x] << 16), acc[2 * x]);
+                        acc[2 * x + 1] = fmaf(d[i], __uint_as_float(w[x] & 0xffff0000u), acc[2 * x + 1]);
+                    }
+                    bacc += d[i];
                 }
             }
-            bacc += dl;
             if (fl & 512) {
 #pragma unroll
                 for (int x = 0; x < 8; ++x) acc[x] += __shfl_xor_sync(kFullMask, acc[x], 16);
-                bacc = warp_sum(bacc);
+                bacc += __shfl_xor_sync(kFullMask, bacc, 16);
                 if (lr >= 0) {
                     if (hh == 0) {
                         float* dst = a.dlm + static_cast<long long>(lr) * kD + 8 * p16;
@@ -432,17 +437,16 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
             lr1 = lr0;
             if (n >= end) continue;
             const Tile& tl = sm.tile[n % kMeta];
-            const int tok = tl.ent[min(8 * gw + (lane & 7), (tl.flags & 255) - 1)] >> 8;
-            const int b = tl.pair / s.Hkv, gk = tl.pair - b * s.Hkv, c = tl.chunk, i0 = tl.i0, flags = tl.flags;
+            const int tok = tl.ent[min(8 * gw + (lane & 7), (tl.flags & 255) - 1)] >> 8, row0 = tl.row0;
+            fl0 = tl.flags;
+            lr0 = tl.lm;
             __syncwarp();
             if (lane == 0) tile_done(n);
             if (n >= 2 && !wait(&sm.done[sl], ((n >> 1) - 1) & 1)) break;
-            fl0 = flags;
-            lr0 = c < s.C ? (b * s.Hl + gk) * s.C + c : -1;              // (B Hkv C < 2^24)
             __syncwarp();
             const uint32_t off = sl * kQBytes + (p16 >> 3) * 16384;
             const uint32_t qa = smem_u32(qbuf) + off, oa = smem_u32(obuf) + off;
-            const long long src0 = (static_cast<long long>(b * s.Hq + gk * kG + hh) * hs + i0) * kD + p16 * 8;
+            const long long src0 = static_cast<long long>(row0 + hh * hs) * kD + p16 * 8;
 #pragma unroll 1
             for (int k0 = 0; k0 < 8; k0 += 4) {
                 int tokv[4];
@@ -467,11 +471,10 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         uint32_t run = 0;
         for (uint32_t n = 0; tile_of(n); ++n) {
             const Tile& tl = sm.tile[n % kMeta];
-            const int flags = tl.flags, pair = tl.pair, c = tl.chunk;
+            const int flags = tl.flags, row = tl.kv, lmr = tl.lm;
             __syncwarp();
             if (lane == 0) tile_done(n);
             if (!(flags & 256)) continue;
-            const int row = pair * s.T + c * kS;
             if (lane == 0) {                                            // (mostly a few tiles ahead: into L2 already)
                 tma_prefetch_l2_2d(&map_k, 0, row);
                 tma_prefetch_l2_2d(&map_k, 64, row);
@@ -479,10 +482,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 tma_prefetch_l2_2d(&map_v, 64, row);
             }
             uint4 lmp = make_uint4(0u, 0u, 0u, 0u);
-            if (lane < 16 && c < s.C) {
-                const int b = pair / s.Hkv;
-                lmp = *reinterpret_cast<const uint4*>(a.lm + ((static_cast<long long>(b) * s.Hl + pair - b * s.Hkv) * s.C + c) * kD + lane * 8);
-            }
+            if (lane < 16 && lmr >= 0) lmp = *reinterpret_cast<const uint4*>(a.lm + static_cast<long long>(lmr) * kD + lane * 8);
             if (run > 0 && !wait(&sm.k_empty, (run - 1) & 1)) break;
             ++run;
             if (lane == 0) {
@@ -586,11 +586,11 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         int sg = -1;
         long long t = 0, hi = 0;
         int i0 = 0;
-        auto put = [&](int pair, int chunk, int flags, int ent, int first_tok) {
+        auto put = [&](int flags, int row0, int kv, int lmr, int vis, int ent) {
             Tile& tl = sm.tile[n % kMeta];
             if (n >= kMeta && !wait(&sm.meta_empty[n % kMeta], ((n / kMeta) - 1) & 1)) return;
             tl.ent[lane] = ent;
-            if (lane == 0) { tl.pair = pair; tl.chunk = chunk; tl.flags = flags; tl.i0 = first_tok; }
+            if (lane == 0) { tl.flags = flags; tl.row0 = row0; tl.kv = kv; tl.lm = lmr; tl.vis = vis; }
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.meta_full[n % kMeta]);
             ++n;
@@ -613,12 +613,16 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 int nx = __shfl_down_sync(kFullMask, rec.x, 1), ny = __shfl_down_sync(kFullMask, rec.y, 1);
                 if (lane == 0) { px = prev.x; py = prev.y; }
                 if (lane == 31) { nx = after.x; ny = after.y; }
-                const int flags = rec.w | (rec.x != px || rec.y != py ? 256 : 0) | (rec.x != nx || rec.y != ny ? 512 : 0);
+                const int b = rec.x / s.Hkv, gk = rec.x - b * s.Hkv, c = rec.y;
+                const int row0 = (b * s.Hq + gk * kG) * hs + i0, kv = rec.x * s.T + c * kS;
+                const int lmr = c < s.C ? (b * s.Hl + gk) * s.C + c : -1, vis = s.pos0 + i0 - c * kS;     // (B Hkv C < 2^24)
+                const int flags = min(kS, s.T - c * kS) << 16 | rec.w | (rec.x != px || rec.y != py ? 256 : 0) | (rec.x != nx || rec.y != ny ? 512 : 0);
                 int e0 = a.entries[t * kTok + lane], e1 = nb > 1 ? a.entries[(t + 1) * kTok + lane] : 0;
 #pragma unroll 1
                 for (int x = 0; x < nb && ok; ++x) {
                     const int e2 = x + 2 < nb ? a.entries[(t + x + 2) * kTok + lane] : 0;
-                    put(__shfl_sync(kFullMask, rec.x, x), __shfl_sync(kFullMask, rec.y, x), __shfl_sync(kFullMask, flags, x), e0, i0);
+                    put(__shfl_sync(kFullMask, flags, x), __shfl_sync(kFullMask, row0, x), __shfl_sync(kFullMask, kv, x),
+                        __shfl_sync(kFullMask, lmr, x), __shfl_sync(kFullMask, vis, x), e0);
                     e0 = e1;
                     e1 = e2;
                 }
@@ -629,7 +633,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         }
 #pragma unroll 1
         for (int x = 0; x < 2; ++x)                                     // (one for either statistics group)
-            if (ok) put(0, 0, 0, 0, 0);
+            if (ok) put(0, 0, 0, 0, 0, 0);
     }
     if (!ok && lane == 0) set_status(a.status, kDevTimeout);
     __syncwarp();
