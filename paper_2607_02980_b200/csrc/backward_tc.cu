@@ -511,7 +511,8 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 if (lane == 0) tile_done(n);
                 if (flags & 256) { wait(&sm.k_ready, run & 1); ++run; }
                 if (n >= 2) wait(&sm.slot_empty[sl], ((n >> 1) - 1) & 1);
-                if (!wait(&sm.q_full[sl], (n >> 1) & 1)) break;
+                wait(&sm.q_full[sl], (n >> 1) & 1);
+                if (!(ok = __all_sync(kFullMask, ok))) break;           // (one answer per warp: an election follows)
                 fence_proxy_async_smem();
                 tc_fence_after_sync();
                 const uint64_t dq0 = umma_desc_k128(smem_u32(qbuf) + sl * kQBytes), do0 = umma_desc_k128(smem_u32(obuf) + sl * kQBytes);
@@ -547,7 +548,8 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 if (lane == 0) tile_done(n);
                 if (first) { wait(&sm.k_ready, run & 1); ++run; }
                 if (n > 0) wait(&sm.dq_empty, (n - 1) & 1);
-                if (!wait(&sm.ds_full[sl], (n >> 1) & 1)) break;
+                wait(&sm.ds_full[sl], (n >> 1) & 1);
+                if (!(ok = __all_sync(kFullMask, ok))) break;
                 tc_fence_after_sync();
                 if (elect_one()) {
 #pragma unroll
@@ -559,7 +561,8 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 __syncwarp();
                 // the previous run's accumulators have been read
                 if (first && run > 1) {
-                    if (!wait(&sm.acc_empty, (run - 2) & 1)) break;
+                    wait(&sm.acc_empty, (run - 2) & 1);
+                    if (!(ok = __all_sync(kFullMask, ok))) break;
                     tc_fence_after_sync();
                 }
                 const uint64_t qmn = umma_desc_mn128(smem_u32(qbuf) + sl * kQBytes, 16384u, 1024u);

@@ -318,9 +318,14 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             if (lane == 0) mbar_arrive(&sm.list_empty[ln]);
         }
     } else if (warp < kLoadWarp) {
-        // ================================================================ MMA issuer of tile t (one thread)
-        if (lane == 0) {
+        // ================================================================ MMA issuer of tile t
+        {
             const int t = warp - kMmaWarp;
+            // (one answer per warp: elections follow)
+            auto wait = [&](uint64_t* bar, uint32_t parity) {
+                if (ok && !__all_sync(kFullMask, mbar_wait(bar, parity))) ok = false;
+                return ok;
+            };
             constexpr uint32_t idesc_s = umma_idesc_bf16(kRows, kNS);
             constexpr uint32_t idesc_o = umma_idesc_bf16(kRows, kD) | kUmmaBMnMajor;
             const uint32_t qa = smem_u32(qbuf + t * kQBytes), s_tm = tmem_base + t * 256;
@@ -339,11 +344,14 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                     if (!ok) return;
                     tc_fence_after_sync();
                     const uint32_t ka = smem_u32(kbuf + st * kKBytes);
+                    if (elect_one()) {
 #pragma unroll
-                    for (int ks = 0; ks < 8; ++ks)
-                        umma_bf16(s_tm, umma_desc_k128(qa + (ks >> 2) * 16384 + (ks & 3) * 32),
-                                  umma_desc_k128(ka + (ks >> 2) * (kNS * 128) + (ks & 3) * 32), idesc_s, ks > 0 ? 1u : 0u);
-                    umma_commit(&sm.s_full[t]);
+                        for (int ks = 0; ks < 8; ++ks)
+                            umma_bf16(s_tm, umma_desc_k128(qa + (ks >> 2) * 16384 + (ks & 3) * 32),
+                                      umma_desc_k128(ka + (ks >> 2) * (kNS * 128) + (ks & 3) * 32), idesc_s, ks > 0 ? 1u : 0u);
+                        umma_commit(&sm.s_full[t]);
+                    }
+                    __syncwarp();
                     ++n_s;
                     issued = i;
                 };
@@ -351,7 +359,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                     const uint32_t st = (g0 + i) % kStages;
                     if (!((sm.list[ln][i] >> (16 + t)) & 1)) {
                         // not this tile's: hand the buffers back (once they are there: the barrier's phase is theirs then)
-                        if (wait(&sm.kv_full[st], ((g0 + i) / kStages) & 1)) mbar_arrive(&sm.kv_empty[st]);
+                        if (wait(&sm.kv_full[st], ((g0 + i) / kStages) & 1) && lane == 0) mbar_arrive(&sm.kv_empty[st]);
                         continue;
                     }
                     if (issued < i) issue_s(i);
@@ -359,17 +367,21 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                     if (!ok || !wait(&sm.p_full[t], n_p & 1)) break;
                     tc_fence_after_sync();
                     const uint32_t va = smem_u32(vbuf + st * kVBytes);
+                    if (elect_one()) {
 #pragma unroll
-                    for (int ks = 0; ks < 4; ++ks)
-                        umma_bf16_ts(s_tm + kOCol, s_tm + kPCol + ks * 8, umma_desc_mn128(va + ks * 2048, 8192u, 1024u), idesc_o,
-                                     (ks > 0 || !first) ? 1u : 0u);
-                    umma_commit(&sm.kv_empty[st]);
-                    umma_commit(&sm.o_done[t]);
+                        for (int ks = 0; ks < 4; ++ks)
+                            umma_bf16_ts(s_tm + kOCol, s_tm + kPCol + ks * 8, umma_desc_mn128(va + ks * 2048, 8192u, 1024u), idesc_o,
+                                         (ks > 0 || !first) ? 1u : 0u);
+                        umma_commit(&sm.kv_empty[st]);
+                        umma_commit(&sm.o_done[t]);
+                    }
+                    __syncwarp();
                     first = false;
                     ++n_p;
                 }
                 g0 += static_cast<uint32_t>(n);
-                mbar_arrive(&sm.list_empty[ln]);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sm.list_empty[ln]);
             }
         }
     } else if (warp == kLoadWarp) {

@@ -191,7 +191,9 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         }
     } else if (warp == 5) {
         // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        {
+            // (one answer per warp: elections follow)
+            auto wait = [](uint64_t* bar, uint32_t parity) { return __all_sync(kFullMask, mbar_wait(bar, parity)) != 0; };
             constexpr uint32_t idesc = umma_idesc_bf16(kTileTok, kS);
             // S_h = Q_h x landmark tile^T (M = 128 tokens, N = 64 chunks, K = 128) into head h's 64 columns
             auto issue_head = [&](uint32_t d_tmem, uint32_t q_addr, uint32_t lm_addr) {
@@ -210,43 +212,51 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                 int ti, pair, nsteps;
                 tile_of(idx, ti, pair, nsteps);
                 if (nsteps == 0) continue;
-                ok = mbar_wait(&sm.q_full, tn & 1);
+                ok = wait(&sm.q_full, tn & 1);
                 for (int it = 0; it < nsteps && ok; ++it, ++n_step) {
                     const uint32_t buf = n_step & 1u;
-                    if (n_step >= 2) ok = mbar_wait(&sm.tmem_empty[buf], ((n_step >> 1) - 1) & 1);
+                    if (n_step >= 2) ok = wait(&sm.tmem_empty[buf], ((n_step >> 1) - 1) & 1);
                     if (!ok) break;
                     if (per == 1) {
                         // one landmark tile for the four query heads
                         const uint32_t st = n_lm % kLmStages;
-                        ok = mbar_wait(&sm.full[st], (n_lm / kLmStages) & 1);
+                        ok = wait(&sm.full[st], (n_lm / kLmStages) & 1);
                         if (!ok) break;
                         tc_fence_after_sync();
                         const uint32_t lm_addr = smem_u32(lms + st * kLmStageBytes);
+                        if (elect_one()) {
 #pragma unroll
-                        for (int h = 0; h < kG; ++h) issue_head(tmem_base + buf * 256 + h * kS, q0 + h * 32768, lm_addr);
-                        umma_commit(&sm.empty[st]);        // landmark stage reusable once these MMAs are done
+                            for (int h = 0; h < kG; ++h) issue_head(tmem_base + buf * 256 + h * kS, q0 + h * 32768, lm_addr);
+                            umma_commit(&sm.empty[st]);        // landmark stage reusable once these MMAs are done
+                            umma_commit(&sm.tmem_full[buf]);   // scores of this step readable
+                        }
+                        __syncwarp();
                         ++n_lm;
                     } else {
                         // one landmark tile per query head (App. C), in ring order
 #pragma unroll
                         for (int h = 0; h < kG; ++h) {
                             const uint32_t st = n_lm % kLmStages;
-                            if (ok) ok = mbar_wait(&sm.full[st], (n_lm / kLmStages) & 1);
+                            if (ok) ok = wait(&sm.full[st], (n_lm / kLmStages) & 1);
                             if (ok) {
                                 tc_fence_after_sync();
-                                issue_head(tmem_base + buf * 256 + h * kS, q0 + h * 32768, smem_u32(lms + st * kLmStageBytes));
-                                umma_commit(&sm.empty[st]);
+                                if (elect_one()) {
+                                    issue_head(tmem_base + buf * 256 + h * kS, q0 + h * 32768, smem_u32(lms + st * kLmStageBytes));
+                                    umma_commit(&sm.empty[st]);
+                                    if (h == kG - 1) umma_commit(&sm.tmem_full[buf]);
+                                }
+                                __syncwarp();
                                 ++n_lm;
                             }
                         }
                         if (!ok) break;
                     }
-                    umma_commit(&sm.tmem_full[buf]);       // scores of this step readable
                 }
-                if (ok) umma_commit(&sm.q_empty);          // the query tile may be replaced once all of these are done
+                if (ok && elect_one()) umma_commit(&sm.q_empty);          // the query tile may be replaced once all of these are done
+                __syncwarp();
                 ++tn;
             }
-            if (!ok) set_status(a.status, kDevTimeout);
+            if (!ok && lane == 0) set_status(a.status, kDevTimeout);
         }
     } else {
         // ------------------------------------------------------------------ epilogue: one token per thread
@@ -299,7 +309,7 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                     } else {
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
-                            float u = fmaxf(fmaxf(r[0][j], r[1][j]), fmaxf(r[2][j], r[3][j])) * s.scale;
+                            float u = fmaxf(fmax3(r[0][j], r[1][j], r[2][j]), r[3][j]) * s.scale;
                             if (bias) u += bias[min(cbase + j, s.C - 1)];
                             u16[j] = u + 0.0f;                 // -0 folds into +0: scores compare as numbers
                         }
@@ -381,9 +391,15 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         for (int e = 0; e < N; ++e) ids[e] = nsteps == 0 ? (e < min(K, my_ncand) ? e : -1) : e < cnt ? static_cast<int>(pool[e * kTileTok] & 0xffffffffull) : -1;
         if (tok < s.R) {
             int32_t* sel = a.sel + (static_cast<long long>(pair) * s.R + tok) * K;
+            if (((reinterpret_cast<uintptr_t>(sel) | static_cast<uintptr_t>(4 * K)) & 15) == 0) {     // rows of whole 16-byte pieces
 #pragma unroll
-            for (int e = 0; e < N; ++e)
-                if (e < K) sel[e] = ids[e];
+                for (int e = 0; e < N; e += 4)
+                    if (e < K) *reinterpret_cast<int4*>(sel + e) = make_int4(ids[e], ids[e + 1], ids[e + 2], ids[e + 3]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < N; ++e)
+                    if (e < K) sel[e] = ids[e];
+            }
         }
         if (a.cnt && ti * kTileTok >= a.t0) {
             // chunk histogram of this tile's entries (selected chunks + the chunks of each token's local window) in the
