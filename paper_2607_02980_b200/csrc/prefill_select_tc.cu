@@ -54,25 +54,25 @@ struct TcSmem {
     int abort;                 // a bounded wait of an epilogue thread ran out: every epilogue warp leaves after the tile
 };
 
-// Sorts N scores in registers, largest first (bitonic network, fully unrolled: static register indices; a
-// compare-exchange is one max and one min).
-template <int N>
-__device__ __forceinline__ void bitonic_sort_desc(float (&a)[N]) {
+// Sorts N scores from a[o] on in registers, largest first (Batcher's odd-even merge sort, fully unrolled: static register
+// indices; a compare-exchange is one max and one min; 191 of them for 32 scores, a bitonic network takes 240).
+template <int N, int M>
+__device__ __forceinline__ void oddeven_sort_desc(float (&a)[M], int o) {
     constexpr int kLog = N == 32 ? 5 : 4;
 #pragma unroll
-    for (int ks = 1; ks <= kLog; ++ks) {
+    for (int ps = 0; ps < kLog; ++ps) {
 #pragma unroll
-        for (int js = kLog - 1; js >= 0; --js) {
-            if (js >= ks) continue;
-            const int k = 1 << ks, j = 1 << js;
+        for (int ks = kLog - 1; ks >= 0; --ks) {
+            if (ks > ps) continue;
+            const int p = 1 << ps, k = 1 << ks;
 #pragma unroll
             for (int i = 0; i < N; ++i) {
-                const int l = i ^ j;
-                if (l > i) {
-                    const bool desc = (i & k) == 0;
-                    const float hi = fmaxf(a[i], a[l]), lo = fminf(a[i], a[l]);
-                    a[i] = desc ? hi : lo;
-                    a[l] = desc ? lo : hi;
+                // pairs (i, i + k) with i - k % p in the lower half of a block of 2 k, both in one block of 2 p
+                const int r = i - k % p;
+                if (r >= 0 && (r & k) == 0 && i + k < N && i / (2 * p) == (i + k) / (2 * p)) {
+                    const float hi = fmaxf(a[o + i], a[o + i + k]), lo = fminf(a[o + i], a[o + i + k]);
+                    a[o + i] = hi;
+                    a[o + i + k] = lo;
                 }
             }
         }
@@ -95,6 +95,27 @@ __device__ __forceinline__ void bitonic_merge_desc(float (&a)[N]) {
             }
         }
     }
+}
+
+// Entry (score, chunk) to the shared-memory address `at` if the score beats `tau`, and `at` to the next entry.
+__device__ __forceinline__ void append_if(uint32_t& at, float score, float tau, int chunk) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.gt.f32 p, %1, %2;\n\t"
+        "@p st.shared.v2.b32 [%0], {%3, %4};\n\t"
+        "@p add.u32 %0, %0, %5;\n\t}"
+        : "+r"(at) : "f"(score), "f"(tau), "r"(chunk), "r"(__float_as_uint(score)), "n"(8 * kTileTok) : "memory");
+}
+// The entry to `at` if its score is at least `tau` and `valid`, and `at` to the next entry.
+__device__ __forceinline__ void keep_if(uint32_t& at, unsigned long long raw, float tau, bool valid) {
+    asm volatile(
+        "{\n\t.reg .pred p, v;\n\t"
+        "setp.ne.b32 v, %4, 0;\n\t"
+        "setp.ge.and.f32 p, %2, %3, v;\n\t"
+        "@p st.shared.b64 [%0], %1;\n\t"
+        "@p add.u32 %0, %0, %5;\n\t}"
+        : "+r"(at) : "l"(raw), "f"(__uint_as_float(static_cast<uint32_t>(raw >> 32))), "f"(tau), "r"(static_cast<int>(valid)), "n"(8 * kTileTok)
+        : "memory");
 }
 
 // N = length of the per-token sorted score list: 16 for K <= 16, else 32; a pool has room for kRoom = 32 candidates
@@ -274,6 +295,7 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         // pool[e * 128]; the first `kept` entries survived the last compaction (at most K), the rest were appended
         // since (at most kRoom).
         unsigned long long* pool = lists + tid;
+        const uint32_t pool_at = smem_u32(pool);
         // bias rows of this KV head's landmark heads (per = 1: one row, shared by the four query heads)
         const float* bias = a.bias ? a.bias + (static_cast<long long>(b) * s.Hl + gk * per) * s.C : nullptr;
         float tau_f = -INFINITY;           // score of the K-th best candidate so far: the filter of the scan
@@ -308,25 +330,33 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                         }
                     } else {
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            float u = fmaxf(fmax3(r[0][j], r[1][j], r[2][j]), r[3][j]) * s.scale;
-                            if (bias) u += bias[min(cbase + j, s.C - 1)];
-                            u16[j] = u + 0.0f;                 // -0 folds into +0: scores compare as numbers
+                        for (int j = 0; j < 16; ++j) u16[j] = fmaxf(fmax3(r[0][j], r[1][j], r[2][j]), r[3][j]) * s.scale;
+                        if (bias) {
+                            const float* bp = bias + cbase;
+                            if (cbase + 16 <= s.C) {
+#pragma unroll
+                                for (int j = 0; j < 16; ++j) u16[j] += __ldg(bp + j);
+                            } else {
+#pragma unroll
+                                for (int j = 0; j < 16; ++j) u16[j] += __ldg(bias + min(cbase + j, s.C - 1));
+                            }
                         }
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) u16[j] += 0.0f;       // -0 folds into +0: scores compare as numbers
+                    }
+                    if (tail) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            if (cbase + j >= my_ncand) u16[j] = -INFINITY;
                     }
                 }
                 const int c0 = it * kS + cb * 8;
                 // Filter on the score: a candidate that only EQUALS the K-th best score so far loses to the K
-                // candidates at or above it, which all have lower chunk ids.  Branch-free append: the slot is
-                // written always and kept only when the candidate passes.
+                // candidates at or above it, which all have lower chunk ids.
+                uint32_t at = pool_at + cnt * (8 * kTileTok);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const float u = (cb & 1) ? u16[8 + j] : u16[j];
-                    const int c = c0 + j;
-                    const bool pass = u > tau_f && (!tail || c < my_ncand);
-                    pool[cnt * kTileTok] = (static_cast<unsigned long long>(__float_as_uint(u)) << 32) | static_cast<uint32_t>(c);
-                    cnt += pass ? 1 : 0;
-                }
+                for (int j = 0; j < 8; ++j) append_if(at, (cb & 1) ? u16[8 + j] : u16[j], tau_f, c0 + j);
+                cnt = static_cast<int>(at - pool_at) / (8 * kTileTok);
                 // Compaction (one call site: the code is large): when a row of the warp may overflow on the next
                 // round (at most 8 appends between checks), and once after the last round.
                 const bool last_round = it + 1 == nsteps && cb == 7;
@@ -339,9 +369,21 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                         const unsigned long long raw = pool[(kept + e) * kTileTok];
                         nw[e] = kept + e < cnt ? __uint_as_float(static_cast<uint32_t>(raw >> 32)) : -INFINITY;
                     }
-                    bitonic_sort_desc<kRoom>(nw);
+                    if constexpr (N == kRoom) {
+                        oddeven_sort_desc<N>(nw, 0);
 #pragma unroll
-                    for (int e = 0; e < N; ++e) best[e] = fmaxf(best[e], nw[N - 1 - e]);
+                        for (int e = 0; e < N; ++e) best[e] = fmaxf(best[e], nw[N - 1 - e]);
+                    } else {
+                        // (only the N best of the new ones matter: two sorted halves, merged)
+                        oddeven_sort_desc<N>(nw, 0);
+                        oddeven_sort_desc<N>(nw, N);
+                        float mid[N];
+#pragma unroll
+                        for (int e = 0; e < N; ++e) mid[e] = fmaxf(nw[e], nw[kRoom - 1 - e]);
+                        bitonic_merge_desc<N>(mid);
+#pragma unroll
+                        for (int e = 0; e < N; ++e) best[e] = fmaxf(best[e], mid[N - 1 - e]);
+                    }
                     bitonic_merge_desc<N>(best);
                     // the K-th best = the smallest of the first K (written so that the list stays in registers:
                     // picking entry K - 1 would index it dynamically)
@@ -349,30 +391,33 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
 #pragma unroll
                     for (int e = 0; e < N; ++e) tau = fminf(tau, e < K ? best[e] : INFINITY);
                     if (tau > -INFINITY) {
-                        // exactly K survive: every score above tau, and the earliest of those equal to it
-                        int above = 0;
-#pragma unroll
-                        for (int e = 0; e < N; ++e) above += (e < K && best[e] > tau) ? 1 : 0;
-                        int ties = K - above, w = 0;
-                        // eight entries per round: their loads go out together (slots past cnt hold old entries or
-                        // nothing that matters: their stores land at or behind w and are overwritten or ignored)
+                        // Exactly K survive: every score above tau, and the earliest of those equal to it.  All at or
+                        // above it first; that leaves more than K only where scores beyond the K-th equal it.
+                        // (eight entries per round: their loads go out together)
+                        uint32_t to = pool_at;
 #pragma unroll 1
                         for (int e0 = 0; e0 < cnt; e0 += 8) {
                             unsigned long long raw[8];
 #pragma unroll
                             for (int j = 0; j < 8; ++j) raw[j] = pool[(e0 + j) * kTileTok];
 #pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                const float sc = __uint_as_float(static_cast<uint32_t>(raw[j] >> 32));
-                                const bool valid = e0 + j < cnt;
-                                const bool tie = valid && sc == tau && ties > 0;
-                                const bool keep = valid && (sc > tau || tie);
-                                ties -= tie ? 1 : 0;
-                                if (valid) pool[w * kTileTok] = raw[j];   // w <= e: in place, order preserved
-                                w += keep ? 1 : 0;
-                            }
+                            for (int j = 0; j < 8; ++j) keep_if(to, raw[j], tau, e0 + j < cnt);     // to <= the entry: in place, in order
                         }
-                        cnt = w;
+                        cnt = static_cast<int>(to - pool_at) / (8 * kTileTok);
+                        if (cnt > K) {
+                            int above = 0;
+#pragma unroll
+                            for (int e = 0; e < N; ++e) above += (e < K && best[e] > tau) ? 1 : 0;
+                            int ties = K - above, w = 0;
+#pragma unroll 1
+                            for (int e = 0; e < cnt; ++e) {
+                                const unsigned long long raw = pool[e * kTileTok];
+                                const bool tie = __uint_as_float(static_cast<uint32_t>(raw >> 32)) == tau;
+                                if (!tie || ties > 0) pool[w++ * kTileTok] = raw;
+                                ties -= tie ? 1 : 0;
+                            }
+                            cnt = w;
+                        }
                     }
                     kept = cnt;
                     tau_f = tau;
