@@ -1,0 +1,47 @@
+"""hils_prefill where its tokens are split between the query-major and the chunk-major kernels, and where the chunk-major
+walk changes: all tokens query-major with ragged last tiles, a split inside the sequence, slices, KV heads walked together and
+one after the other, selection rows of odd length, a workspace whose plan depends on the split."""
+import pytest
+import torch
+
+import paper_2607_02980_b200 as hils
+from paper_2607_02980_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,Hkv,L,K,W,bias_scale,pos0", [
+    (1, 1, 65, 4, 1, 0.0, 0),          # one unit, one token past a chunk
+    (3, 1, 129, 16, 1, 0.5, 0),        # every token takes all its candidates: one launch writes the selection
+    (2, 2, 1000, 8, 65, 0.0, 0),       # query-major to the end of a ragged tile
+    (1, 2, 1025, 4, 1, 60.0, 0),       # split at 768 tokens; logits that raise the running reference and hide chunks
+    (2, 1, 3000, 5, 130, 0.5, 0),      # split; selection rows of 20 bytes
+    (1, 2, 4200, 16, 1, 0.0, 0),       # KV heads together
+    (1, 1, 16384, 16, 1, 0.0, 0),      # one KV head at a time, several query blocks' worth of lists
+    (1, 2, 1500, 8, 64, 0.5, 300),     # a slice that begins among the query-major tokens
+    (1, 2, 900, 8, 1, 0.0, 7777),      # a slice past them
+])
+def test_fast_and_generic_agree(B, Hkv, L, K, W, bias_scale, pos0):
+    gen = torch.Generator(device="cuda").manual_seed(L + K)
+    T = pos0 + L
+    rnd = lambda h, n: torch.randn((B, h, n, 128), device="cuda", generator=gen).to(torch.bfloat16)
+    q, k, v, lm = rnd(4 * Hkv, L), rnd(Hkv, T), rnd(Hkv, T), rnd(Hkv, T // 64)
+    bias = torch.randn((B, Hkv, T // 64), device="cuda", generator=gen) * bias_scale if bias_scale else None
+    run = lambda impl: (hils.hils_prefill_at(q, k, v, lm, 64, K, pos0, bias=bias, window=W, impl=impl) if pos0 else
+                        hils.hils_prefill(q, k, v, lm, 64, K, bias=bias, window=W, impl=impl))
+    (o1, l1, s1), (o2, l2, s2) = run("fast"), run("generic")
+    torch.cuda.synchronize()
+    same = (s1 == s2).all(dim=-1).repeat_interleave(4, dim=1)       # (scores that tie in bf16 accumulation order may swap)
+    assert same.float().mean().item() >= 0.99
+    assert (o1.float() - o2.float()).abs().amax(dim=-1)[same].max().item() <= 3.2e-2
+    assert (l1 - l2).abs()[same].max().item() <= 2e-2
+
+
+def test_workspace_covers_the_plan_without_the_query_major_tokens():
+    """All tokens' partial outputs exceed what a call keeps at a time, those of the chunk-major tokens alone do not: the call
+    then holds them all, and the reported size has to say so."""
+    cfg = wl.HilsConfig("ws", "prefill", 1, 32, 8, 16384, 128, 64, 32, "bf16", 5, window=512)
+    t = wl.make_prefill_inputs(cfg, "cuda")
+    out, lse, sel = hils.hils_prefill(t["q"], t["k"], t["v"], t["landmarks"], 64, 32, window=512)
+    torch.cuda.synchronize()
+    assert torch.isfinite(out).all() and torch.isfinite(lse).all()
