@@ -1,19 +1,19 @@
 // Landmark scoring + exact top-K for prefill on the 5th-generation tensor cores (tcgen05 + TMEM).
 //
-// One persistent CTA per SM walks (sequence, KV head, 128-token tile) triples, heavy tiles first; the next tile's
-// queries and first scores are fetched and computed while the epilogue finishes the previous tile.  The tile's queries (4 heads x 128 tokens x 128 d)
-// stay in shared memory; landmark tiles of 64 chunks stream through a TMA ring.  One thread issues
-// tcgen05.mma (M = 128 tokens, N = 64 chunks, K = 128) once per head into tensor memory, double
-// buffered; the four epilogue warps own one token per thread (token = TMEM lane), read the four
-// heads' scores, take the group max (App. C) and keep the token's exact running top-K
-// (Eq. surrogate top-k; equal scores go to the lower chunk id).  A token's candidates that beat its current
-// K-th best score are appended, in arrival order = ascending chunk id, to its pool in shared memory; the N best
-// SCORES so far stay sorted in registers.  When a pool of the warp may fill up, every thread sorts the scores
-// appended since the last time (register bitonic network on 32-bit values: one max and one min per
-// compare-exchange), merges them into its sorted list, reads the new K-th best score off it and filters its pool
-// in place: everything above that score and the earliest of those equal to it, exactly K entries, still in
-// ascending chunk order -- which is the order the selection is written in.  The number of such compactions grows
-// with log(candidates / K), not with the candidates.
+// One persistent CTA per SM walks (sequence, KV head, 128-token tile) triples, heavy tiles first.  The tile's queries
+// (4 heads x 128 tokens x 128 d) stay in shared memory; landmark tiles of 64 chunks stream through a TMA ring.  One warp
+// issues tcgen05.mma (M = 128 tokens, N = 64 chunks, K = 128) once per head into tensor memory, double buffered.
+// Scan warps own one token per thread (token = TMEM lane): they read the four heads' scores, take the group max (App. C)
+// and append the candidates that beat the token's K-th best score known so far to a buffer in shared memory, in arrival
+// order = ascending chunk id.  When a buffer of the warp may fill up it goes to the warp's partner among the sort warps,
+// and the scan goes on with the other buffer.  The sort warp keeps the token's exact running top-K (Eq. surrogate top-k;
+// equal scores go to the lower chunk id): the N best SCORES so far stay sorted in registers; it sorts the new ones
+// (register network on 32-bit values: one max and one min per compare-exchange), merges them in, reads the new K-th best
+// score off the list, and filters the kept entries in place: everything above that score and the earliest of those equal
+// to it, exactly K, still in ascending chunk order -- the order in which it writes the selection at the end of the tile,
+// while the scan works on the next one.  The number of buffers grows with log(candidates / K), not with the candidates.
+// Bound: the latencies of the sort warps' code (one per scheduler; with scan and sort in one warp 16K tokens, K = 16 took
+// 101.5 us instead of 95, a 2048-token slice at 48K, K = 32, 74 instead of 68).
 #include "internal.h"
 #include "tma.cuh"
 
@@ -28,8 +28,9 @@ constexpr int kLmStages = 2;
 constexpr int kLmStageBytes = kS * kD * 2;          // 64 landmark rows = two 8 KB K-blocks
 constexpr int kQBytes = kG * kTileTok * kD * 2;     // 128 KB
 constexpr int kMaxK = 32;
-constexpr int kRoom = 32;                           // candidates a pool takes between two compactions
-constexpr int kThreads = 192;                       // 4 epilogue warps, 1 TMA warp, 1 MMA warp
+constexpr int kRoom = 16;                           // candidates that a thread hands over at a time
+constexpr int kTmaWarp = 4, kMmaWarp = 5, kSortWarp = 6;
+constexpr int kThreads = 320;                       // 4 scan warps, 1 TMA warp, 1 MMA warp, 4 sort warps
 constexpr uint32_t kTmemCols = 512;                 // 2 buffers x 4 heads x 64 columns
 
 struct TcArgs {
@@ -51,13 +52,17 @@ struct TcSmem {
     uint64_t tmem_full[2];
     uint64_t tmem_empty[2];
     uint32_t tmem_base;
-    int abort;                 // a bounded wait of an epilogue thread ran out: every epilogue warp leaves after the tile
+    int abort;                 // a bounded wait of a sort warp ran out: every sort warp leaves after the tile
+    uint64_t new_full[4][2], new_empty[4][2];   // [scan warp][buffer] candidates handed over / read
+    int last[2][4];                             // the buffer is its tile's last
+    uint8_t n_new[2][kTileTok];                 // candidates of each thread
+    float tau[2][kTileTok];                     // [tile parity] each token's K-th best score so far
 };
 
-// Sorts N scores from a[o] on in registers, largest first (Batcher's odd-even merge sort, fully unrolled: static register
+// Sorts N scores in registers, largest first (Batcher's odd-even merge sort, fully unrolled: static register
 // indices; a compare-exchange is one max and one min; 191 of them for 32 scores, a bitonic network takes 240).
-template <int N, int M>
-__device__ __forceinline__ void oddeven_sort_desc(float (&a)[M], int o) {
+template <int N>
+__device__ __forceinline__ void oddeven_sort_desc(float (&a)[N]) {
     constexpr int kLog = N == 32 ? 5 : 4;
 #pragma unroll
     for (int ps = 0; ps < kLog; ++ps) {
@@ -70,9 +75,9 @@ __device__ __forceinline__ void oddeven_sort_desc(float (&a)[M], int o) {
                 // pairs (i, i + k) with i - k % p in the lower half of a block of 2 k, both in one block of 2 p
                 const int r = i - k % p;
                 if (r >= 0 && (r & k) == 0 && i + k < N && i / (2 * p) == (i + k) / (2 * p)) {
-                    const float hi = fmaxf(a[o + i], a[o + i + k]), lo = fminf(a[o + i], a[o + i + k]);
-                    a[o + i] = hi;
-                    a[o + i + k] = lo;
+                    const float hi = fmaxf(a[i], a[i + k]), lo = fminf(a[i], a[i + k]);
+                    a[i] = hi;
+                    a[i + k] = lo;
                 }
             }
         }
@@ -118,8 +123,7 @@ __device__ __forceinline__ void keep_if(uint32_t& at, unsigned long long raw, fl
         : "memory");
 }
 
-// N = length of the per-token sorted score list: 16 for K <= 16, else 32; a pool has room for kRoom = 32 candidates
-// appended between two compactions (fewer, larger compactions are cheaper than more, smaller ones).
+// N = length of the per-token sorted score list: 16 for K <= 16, else 32.
 // PERHEAD: one landmark row (and bias) per query head (App. C) instead of one per KV head.  A template parameter, not
 // a run-time branch: the scan loop's code has to stay small (the kernel is sensitive to instruction fetch).
 template <int N, bool PERHEAD>
@@ -140,7 +144,7 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     const int K = s.K;
     constexpr int per = PERHEAD ? kG : 1;     // landmark rows per chunk
     // A CTA walks the tiles blockIdx.x, blockIdx.x + gridDim.x, ... (heavy tiles first): the query tile and the first
-    // scores of the next tile are fetched and computed while the epilogue still finishes the previous one.  Every
+    // scores of the next tile are fetched and computed while the sort warps still finish the previous one.  Every
     // role derives the same tile sequence; tiles without candidates touch no barrier.
     // (Every other round of the walk runs backwards, so that a CTA early in one round, with heavy tiles, is late in the next.)
     auto tile_of = [&](int idx, int& ti, int& pair, int& nsteps) {
@@ -159,18 +163,22 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         mbar_init(&sm.q_empty, 1);
         sm.abort = 0;
         for (int i = 0; i < kLmStages; ++i) { mbar_init(&sm.full[i], 1); mbar_init(&sm.empty[i], 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(&sm.tmem_full[i], 1); mbar_init(&sm.tmem_empty[i], 4); }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&sm.tmem_full[i], 1);
+            mbar_init(&sm.tmem_empty[i], 4);
+            for (int w = 0; w < 4; ++w) { mbar_init(&sm.new_full[w][i], 1); mbar_init(&sm.new_empty[w][i], 1); }
+        }
         mbar_fence_init();
         tma_prefetch_desc(&map_q);
         tma_prefetch_desc(&map_lm);
     }
-    if (warp == 5) tmem_alloc(&sm.tmem_base, kTmemCols);
+    if (warp == kMmaWarp) tmem_alloc(&sm.tmem_base, kTmemCols);
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = sm.tmem_base;
 
-    if (warp == 4) {
+    if (warp == kTmaWarp) {
         // ------------------------------------------------------------------ TMA producer
         if (lane == 0) {
             uint32_t n_lm = 0;            // landmark tiles requested so far, over all tiles of this CTA
@@ -210,7 +218,7 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
             for (uint32_t n = n_lm > kLmStages ? n_lm - kLmStages : 0; n < n_lm; ++n)
                 mbar_wait(&sm.full[n % kLmStages], (n / kLmStages) & 1);
         }
-    } else if (warp == 5) {
+    } else if (warp == kMmaWarp) {
         // ------------------------------------------------------------------ MMA issuer
         {
             // (one answer per warp: elections follow)
@@ -279,47 +287,49 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
             }
             if (!ok && lane == 0) set_status(a.status, kDevTimeout);
         }
-    } else {
-        // ------------------------------------------------------------------ epilogue: one token per thread
-        const int row = warp * 32 + lane;
+    } else if (warp < kTmaWarp) {
+        // ------------------------------------------------------------------ scan: one token per thread
         const uint32_t t_lane = tmem_base + (static_cast<uint32_t>(warp * 32) << 16);
-        uint32_t n_step = 0;               // steps so far, over all tiles of this CTA
+        const uint32_t room_at = smem_u32(lists) + tid * 8;      // [buffer][kRoom][128] entries
+        uint32_t n_step = 0, n_buf = 0;                          // steps / buffers so far, over all tiles of this CTA
+        int tn = 0;                                              // tiles with candidates so far
         bool ok = true;
-        for (int idx = blockIdx.x; idx < n_tiles; idx += gridDim.x) {
-        int ti, pair, nsteps;
-        tile_of(idx, ti, pair, nsteps);
-        const int b = pair / s.Hkv, gk = pair % s.Hkv;
-        const int tok = ti * kTileTok + row;
-        const int my_ncand = local_lo(s.pos0 + tok, s.W, kS) / kS;
-        // The token's pool of raw (score bits, chunk id) pairs in arrival order = ascending chunk id: entry e at
-        // pool[e * 128]; the first `kept` entries survived the last compaction (at most K), the rest were appended
-        // since (at most kRoom).
-        unsigned long long* pool = lists + tid;
-        const uint32_t pool_at = smem_u32(pool);
-        // bias rows of this KV head's landmark heads (per = 1: one row, shared by the four query heads)
-        const float* bias = a.bias ? a.bias + (static_cast<long long>(b) * s.Hl + gk * per) * s.C : nullptr;
-        float tau_f = -INFINITY;           // score of the K-th best candidate so far: the filter of the scan
-        float best[N];                     // the N best scores so far, largest first (-inf = none)
-#pragma unroll
-        for (int e = 0; e < N; ++e) best[e] = -INFINITY;
-        int cnt = 0, kept = 0;
-
-        for (int it = 0; it < nsteps && ok; ++it, ++n_step) {
-            const uint32_t buf = n_step & 1u;
-            ok = mbar_wait(&sm.tmem_full[buf], (n_step >> 1) & 1);
-            if (!ok) break;
-            tc_fence_after_sync();
-            const bool tail = (it + 1) * kS > my_ncand;     // only the last step holds chunks this token may not see
-            // 8 candidates per round (a short loop body: the code has to stay resident close to the core); the group
-            // scores of 16 candidates are read from tensor memory and reduced over the heads every other round
-            float u16[16];
+        for (int idx = blockIdx.x; idx < n_tiles && ok; idx += gridDim.x) {
+            int ti, pair, nsteps;
+            tile_of(idx, ti, pair, nsteps);
+            if (nsteps == 0) continue;
+            const int b = pair / s.Hkv, gk = pair % s.Hkv;
+            const int my_ncand = local_lo(s.pos0 + ti * kTileTok + tid, s.W, kS) / kS;
+            // bias rows of this KV head's landmark heads (per = 1: one row, shared by the four query heads)
+            const float* bias = a.bias ? a.bias + (static_cast<long long>(b) * s.Hl + gk * per) * s.C : nullptr;
+            uint32_t at0 = 0, at = 0;
+            auto acquire = [&]() {
+                if (n_buf >= 2 && !__all_sync(kFullMask, mbar_wait(&sm.new_empty[warp][n_buf & 1], ((n_buf >> 1) - 1) & 1))) ok = false;
+                at = at0 = room_at + (n_buf & 1) * (kRoom * 8 * kTileTok);
+            };
+            auto hand_over = [&](bool last) {
+                sm.n_new[n_buf & 1][tid] = static_cast<uint8_t>((at - at0) / (8 * kTileTok));
+                if (lane == 0) sm.last[n_buf & 1][warp] = last;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sm.new_full[warp][n_buf & 1]);
+                ++n_buf;
+            };
+            // (the sort warp has read the last buffer of the tile two before, so it writes this slot no more)
+            acquire();
+            volatile float* tau_sm = &sm.tau[tn & 1][tid];
+            *tau_sm = -INFINITY;
+            for (int it = 0; it < nsteps && ok; ++it, ++n_step) {
+                const uint32_t buf = n_step & 1u;
+                if (!__all_sync(kFullMask, mbar_wait(&sm.tmem_full[buf], (n_step >> 1) & 1))) { ok = false; break; }
+                tc_fence_after_sync();
+                const bool tail = (it + 1) * kS > my_ncand;     // only the last step holds chunks this token may not see
 #pragma unroll 1
-            for (int cb = 0; cb < 8; ++cb) {
-                if ((cb & 1) == 0) {
+                for (int cb = 0; cb < 4; ++cb) {
+                    float u16[16];
                     float r[4][16];
-                    const uint32_t col = t_lane + buf * 256 + cb * 8;
+                    const uint32_t col = t_lane + buf * 256 + cb * 16;
                     tmem_ld16x4(col, col + kS, col + 2 * kS, col + 3 * kS, r);
-                    const int cbase = it * kS + cb * 8;
+                    const int cbase = it * kS + cb * 16;
                     if (PERHEAD && bias != nullptr) {
                         // every head adds its own bias before the maximum over the group (App. C)
 #pragma unroll
@@ -349,84 +359,116 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                         for (int j = 0; j < 16; ++j)
                             if (cbase + j >= my_ncand) u16[j] = -INFINITY;
                     }
-                }
-                const int c0 = it * kS + cb * 8;
-                // Filter on the score: a candidate that only EQUALS the K-th best score so far loses to the K
-                // candidates at or above it, which all have lower chunk ids.
-                uint32_t at = pool_at + cnt * (8 * kTileTok);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) append_if(at, (cb & 1) ? u16[8 + j] : u16[j], tau_f, c0 + j);
-                cnt = static_cast<int>(at - pool_at) / (8 * kTileTok);
-                // Compaction (one call site: the code is large): when a row of the warp may overflow on the next
-                // round (at most 8 appends between checks), and once after the last round.
-                const bool last_round = it + 1 == nsteps && cb == 7;
-                if (__any_sync(kFullMask, cnt - kept > kRoom - 8) || last_round) {
-                    // the N best scores of (best so far) + (appended since): sort the new ones, take the larger of
-                    // the i-th best old and the i-th worst new, sort that bitonic sequence
-                    float nw[kRoom];
-#pragma unroll
-                    for (int e = 0; e < kRoom; ++e) {
-                        const unsigned long long raw = pool[(kept + e) * kTileTok];
-                        nw[e] = kept + e < cnt ? __uint_as_float(static_cast<uint32_t>(raw >> 32)) : -INFINITY;
+                    if (cb == 3) {
+                        tc_fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&sm.tmem_empty[buf]);
                     }
-                    if constexpr (N == kRoom) {
-                        oddeven_sort_desc<N>(nw, 0);
+                    // Filter on the score: a candidate that only EQUALS the K-th best score so far loses to the K
+                    // candidates at or above it, which all have lower chunk ids.  (The threshold may be some buffers old.)
+                    const int c0 = it * kS + cb * 16;
 #pragma unroll
-                        for (int e = 0; e < N; ++e) best[e] = fmaxf(best[e], nw[N - 1 - e]);
-                    } else {
-                        // (only the N best of the new ones matter: two sorted halves, merged)
-                        oddeven_sort_desc<N>(nw, 0);
-                        oddeven_sort_desc<N>(nw, N);
-                        float mid[N];
-#pragma unroll
-                        for (int e = 0; e < N; ++e) mid[e] = fmaxf(nw[e], nw[kRoom - 1 - e]);
-                        bitonic_merge_desc<N>(mid);
-#pragma unroll
-                        for (int e = 0; e < N; ++e) best[e] = fmaxf(best[e], mid[N - 1 - e]);
-                    }
-                    bitonic_merge_desc<N>(best);
-                    // the K-th best = the smallest of the first K (written so that the list stays in registers:
-                    // picking entry K - 1 would index it dynamically)
-                    float tau = INFINITY;
-#pragma unroll
-                    for (int e = 0; e < N; ++e) tau = fminf(tau, e < K ? best[e] : INFINITY);
-                    if (tau > -INFINITY) {
-                        // Exactly K survive: every score above tau, and the earliest of those equal to it.  All at or
-                        // above it first; that leaves more than K only where scores beyond the K-th equal it.
-                        // (eight entries per round: their loads go out together)
-                        uint32_t to = pool_at;
-#pragma unroll 1
-                        for (int e0 = 0; e0 < cnt; e0 += 8) {
-                            unsigned long long raw[8];
-#pragma unroll
-                            for (int j = 0; j < 8; ++j) raw[j] = pool[(e0 + j) * kTileTok];
-#pragma unroll
-                            for (int j = 0; j < 8; ++j) keep_if(to, raw[j], tau, e0 + j < cnt);     // to <= the entry: in place, in order
+                    for (int h = 0; h < 2; ++h) {
+                        if (__any_sync(kFullMask, at - at0 > (kRoom - 8) * 8 * kTileTok)) {
+                            hand_over(false);
+                            acquire();
                         }
-                        cnt = static_cast<int>(to - pool_at) / (8 * kTileTok);
-                        if (cnt > K) {
-                            int above = 0;
+                        const float tau = *tau_sm;
 #pragma unroll
-                            for (int e = 0; e < N; ++e) above += (e < K && best[e] > tau) ? 1 : 0;
-                            int ties = K - above, w = 0;
-#pragma unroll 1
-                            for (int e = 0; e < cnt; ++e) {
-                                const unsigned long long raw = pool[e * kTileTok];
-                                const bool tie = __uint_as_float(static_cast<uint32_t>(raw >> 32)) == tau;
-                                if (!tie || ties > 0) pool[w++ * kTileTok] = raw;
-                                ties -= tie ? 1 : 0;
-                            }
-                            cnt = w;
-                        }
+                        for (int j = 0; j < 8; ++j) append_if(at, u16[8 * h + j], tau, c0 + 8 * h + j);
                     }
-                    kept = cnt;
-                    tau_f = tau;
                 }
             }
-            tc_fence_before_sync();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&sm.tmem_empty[buf]);
+            if (ok) hand_over(true);
+            ++tn;
         }
+        if (!ok && lane == 0) set_status(a.status, kDevTimeout);
+    } else {
+        // ------------------------------------------------------------------ sort: one token per thread
+        const int sw = warp - kSortWarp, row = sw * 32 + lane;
+        unsigned long long* pool = lists + 2 * kRoom * kTileTok + row;       // the token's kept entries: entry e at pool[e * 128]
+        const uint32_t pool_at = smem_u32(pool);
+        uint32_t n_buf = 0;
+        int tn = 0;
+        bool ok = true;
+        for (int idx = blockIdx.x; idx < n_tiles; idx += gridDim.x) {
+        int ti, pair, nsteps;
+        tile_of(idx, ti, pair, nsteps);
+        const int tok = ti * kTileTok + row;
+        const int my_ncand = local_lo(s.pos0 + tok, s.W, kS) / kS;
+        float best[N];                     // the N best scores so far, largest first (-inf = none)
+#pragma unroll
+        for (int e = 0; e < N; ++e) best[e] = -INFINITY;
+        int cnt = 0;
+        for (bool last = nsteps == 0; !last && ok; ++n_buf) {
+            const uint32_t bf = n_buf & 1u;
+            if (!__all_sync(kFullMask, mbar_wait(&sm.new_full[sw][bf], (n_buf >> 1) & 1))) { ok = false; break; }
+            const int n_new = sm.n_new[bf][row];
+            last = sm.last[bf][sw] != 0;
+            unsigned long long raw[kRoom];
+            const unsigned long long* src = lists + bf * (kRoom * kTileTok) + row;
+#pragma unroll
+            for (int e = 0; e < kRoom; ++e) raw[e] = src[e * kTileTok];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.new_empty[sw][bf]);
+            // the N best scores of (best so far) + (new): sort the new ones, take the larger of the i-th best old and the
+            // i-th worst new, sort that bitonic sequence
+            float nw[kRoom];
+            auto score = [&](int e) { return __uint_as_float(static_cast<uint32_t>(raw[e] >> 32)); };
+#pragma unroll
+            for (int e = 0; e < kRoom; ++e) nw[e] = e < n_new ? score(e) : -INFINITY;
+            oddeven_sort_desc<kRoom>(nw);
+#pragma unroll
+            for (int e = 0; e < kRoom; ++e) best[N - 1 - e] = fmaxf(best[N - 1 - e], nw[e]);
+            bitonic_merge_desc<N>(best);
+            // the K-th best = the smallest of the first K (written so that the list stays in registers:
+            // picking entry K - 1 would index it dynamically)
+            float tau = INFINITY;
+#pragma unroll
+            for (int e = 0; e < N; ++e) tau = fminf(tau, e < K ? best[e] : INFINITY);
+            if (!last) *const_cast<volatile float*>(&sm.tau[tn & 1][row]) = tau;
+            // Exactly K survive: every score above tau, and the earliest of those equal to it.  All at or above it first;
+            // that leaves more than K only where scores beyond the K-th equal it.
+            // (eight entries per round: their loads go out together)
+            uint32_t to = pool_at;
+#pragma unroll 1
+            for (int e0 = 0; e0 < cnt; e0 += 8) {
+                unsigned long long old[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) old[j] = pool[(e0 + j) * kTileTok];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) keep_if(to, old[j], tau, e0 + j < cnt);     // to <= the entry: in place, in order
+            }
+            cnt = static_cast<int>(to - pool_at) / (8 * kTileTok);
+            uint32_t live = 0;                                  // new entries that stay
+#pragma unroll
+            for (int e = 0; e < kRoom; ++e) live |= (e < n_new && score(e) >= tau) ? 1u << e : 0u;
+            if (cnt + __popc(live) > K) {
+                int above = 0;
+#pragma unroll
+                for (int e = 0; e < N; ++e) above += (e < K && best[e] > tau) ? 1 : 0;
+                int ties = K - above, w = 0;
+#pragma unroll 1
+                for (int e = 0; e < cnt; ++e) {
+                    const unsigned long long x = pool[e * kTileTok];
+                    const bool tie = __uint_as_float(static_cast<uint32_t>(x >> 32)) == tau;
+                    if (!tie || ties > 0) pool[w++ * kTileTok] = x;
+                    ties -= tie ? 1 : 0;
+                }
+                cnt = w;
+#pragma unroll
+                for (int e = 0; e < kRoom; ++e)
+                    if (((live >> e) & 1u) && score(e) == tau) {
+                        if (ties <= 0) live &= ~(1u << e);
+                        --ties;
+                    }
+            }
+            to = pool_at + cnt * (8 * kTileTok);
+#pragma unroll
+            for (int e = 0; e < kRoom; ++e) keep_if(to, raw[e], -INFINITY, ((live >> e) & 1u) != 0);
+            cnt = static_cast<int>(to - pool_at) / (8 * kTileTok);
+        }
+        tn += nsteps > 0 ? 1 : 0;
         // (after a timeout the thread still walks through the tile's barriers; every warp leaves together below)
         if (!ok) { set_status(a.status, kDevTimeout); *reinterpret_cast<volatile int*>(&sm.abort) = 1; }
 
@@ -449,12 +491,12 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         if (a.cnt && ti * kTileTok >= a.t0) {
             // chunk histogram of this tile's entries (selected chunks + the chunks of each token's local window) in the
             // pools' shared memory (every thread holds its ids in registers by now), then one global add per used bin
-            int* hist = reinterpret_cast<int*>(lists);
-            const bool in_smem = a.nc * sizeof(int) <= sizeof(unsigned long long) * 2 * kMaxK * kTileTok;
+            int* hist = reinterpret_cast<int*>(lists + 2 * kRoom * kTileTok);
+            const bool in_smem = a.nc * sizeof(int) <= sizeof(unsigned long long) * kMaxK * kTileTok;
             int* gcnt = a.cnt + (static_cast<long long>((ti * kTileTok - a.t0) / a.qb) * pairs + pair) * a.nc;
             asm volatile("bar.sync 1, 128;" ::: "memory");
             if (in_smem) {
-                for (int x = tid; x < a.nc; x += kTileTok) hist[x] = 0;
+                for (int x = row; x < a.nc; x += kTileTok) hist[x] = 0;
                 asm volatile("bar.sync 1, 128;" ::: "memory");
             }
             if (tok < s.R) {
@@ -467,7 +509,7 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
             }
             if (in_smem) {
                 asm volatile("bar.sync 1, 128;" ::: "memory");
-                for (int x = tid; x < a.nc; x += kTileTok)
+                for (int x = row; x < a.nc; x += kTileTok)
                     if (hist[x]) atomicAdd(gcnt + x, hist[x]);
             }
         }
@@ -480,7 +522,7 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    if (warp == 5) tmem_dealloc(tmem_base, kTmemCols);
+    if (warp == kMmaWarp) tmem_dealloc(tmem_base, kTmemCols);
 }
 
 }  // namespace
