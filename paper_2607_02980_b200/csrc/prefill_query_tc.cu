@@ -510,20 +510,38 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
 
 }  // namespace
 
-// Tokens of a call (from its first on) that go this way; a multiple of 128 below the call's length, or all of them.
-// A tile of 32 tokens costs about 1850 cycles per chunk it visits here, at most every visible one; chunk-major (index, attend
-// and fuse kernels), 32 tokens cost 4600 cycles per chunk they attend: the line lies where the visible chunks outnumber the
-// attended ones 5 : 2.
+// Tokens of a call (from its first on) that go this way: a multiple of 128 below the call's length, or all of them.  The
+// split with the largest gain by these costs (SM cycles; fitted to 16K, 2 x 6000 and 3 x 1000 tokens):
+//   here, a unit of 64 tokens: 2500 per chunk it visits (at most every visible one) + 18000, the last unit at least in full;
+//   chunk-major (index, attend and fuse kernels): 3830 per 32 tokens and chunk they attend, and 55000 for the launches.
+// With units for every SM the line lies near visible : attended = 5 : 2.  With few (sequence, KV head) pairs the units are a
+// serial chain on some of the SMs, and everything goes chunk-major unless that saves its launches (2 KV heads, a slice of
+// 2190 tokens at 4395, K = 32: 107 us chunk-major, 193 with the first 768 tokens here).  The parts of a call that the library
+// itself cuts into slices keep the whole call's split (Shape::qsplit): the same bits either way.
 int prefill_query_tokens(const Shape& s) {
     if (s.Hl != s.Hkv || s.K > 64) return 0;
+    if (s.qsplit >= 0) {
+        const int n = s.qsplit - s.pos0;
+        return n <= 0 ? 0 : n >= s.R ? s.R : n / 128 * 128;
+    }
     const int nl = (s.W - 1 + kS - 1) / kS + 1;                          // chunks of a local window
-    int most = 5 * (s.K + nl) / 2;
-    if (most > kMaxC - 2) most = kMaxC - 2;
-    // tokens whose chunk is below `most`
-    const long long n = static_cast<long long>(most) * kS - s.pos0;
-    if (n <= 0) return 0;
-    if (n >= s.R) return s.R;
-    return static_cast<int>(n / 128 * 128);
+    const long long pairs = static_cast<long long>(s.B) * s.Hkv, sms = sm_count();
+    long long here = 0, there = 0, most = 0;
+    int best = 0;
+    for (int n = 0; n < s.R;) {
+        const int end = n + kUnitTok < s.R ? n + kUnitTok : s.R;
+        const long long vis = (s.pos0 + end - 1) / kS + 1, att = vis < s.K + nl ? vis : s.K + nl, unit = 2500 * vis + 18000;
+        if (vis > kMaxC) break;
+        here += pairs * unit;
+        there += pairs * (end - n) * att * 3830 / 32;
+        n = end;
+        const long long t = here / sms > unit ? here / sms : unit, gain = there / sms + (n == s.R ? 55000 : 0) - t;
+        if (gain > most && (n == s.R || n % 128 == 0)) {
+            most = gain;
+            best = n;
+        }
+    }
+    return best;
 }
 
 int launch_prefill_query_tc(const Shape& s, const Tensors& t, int n_tok, int write_sel, cudaStream_t stream) {

@@ -14,11 +14,12 @@ pytestmark = pytest.mark.gpu
     (1, 1, 65, 4, 1, 0.0, 0),          # one unit, one token past a chunk
     (3, 1, 129, 16, 1, 0.5, 0),        # every token takes all its candidates: one launch writes the selection
     (2, 2, 1000, 8, 65, 0.0, 0),       # query-major to the end of a ragged tile
-    (1, 2, 1025, 4, 1, 60.0, 0),       # split at 768 tokens; logits that raise the running reference and hide chunks
-    (2, 1, 3000, 5, 130, 0.5, 0),      # split; selection rows of 20 bytes
+    (16, 4, 2500, 8, 1, 60.0, 0),      # split; logits that raise the running reference and hide chunks
+    (4, 8, 2500, 5, 130, 0.5, 0),      # split; selection rows of 20 bytes
+    (2, 1, 3000, 5, 130, 0.5, 0),      # too few KV heads to split
     (1, 2, 4200, 16, 1, 0.0, 0),       # KV heads together
     (1, 1, 16384, 16, 1, 0.0, 0),      # one KV head at a time, several query blocks' worth of lists
-    (1, 2, 1500, 8, 64, 0.5, 300),     # a slice that begins among the query-major tokens
+    (4, 8, 1500, 8, 64, 0.5, 300),     # a slice that begins among the query-major tokens
     (1, 2, 900, 8, 1, 0.0, 7777),      # a slice past them
 ])
 def test_fast_and_generic_agree(B, Hkv, L, K, W, bias_scale, pos0):
