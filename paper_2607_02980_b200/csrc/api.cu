@@ -75,6 +75,7 @@ int make_shape(const hils_params* p, int is_decode, Shape* s, long long pos0 = 0
     s->pos0 = 0;
     s->qps = 1;
     s->qsplit = -1;
+    s->lsplit = -1;
     if (is_decode) {
         if (p->T_max < 1) return HILS_ERR_INVALID_ARG;
         s->R = 1;
@@ -129,12 +130,13 @@ size_t scratch_bytes(const Shape& s, Path path, int dtype) {
 int run(const hils_params* p, int is_decode, const void* q, const void* k, const void* v, const void* lm,
         const float* bias, const int32_t* seq_lens, void* out, float* lse, int32_t* sel, void* ws,
         size_t ws_bytes, void* stream_v, const int32_t* block_table = nullptr, int num_pages = 0, long long pos0 = 0,
-        const void* q_route = nullptr, int qps = 1, int qsplit = -1) {
+        const void* q_route = nullptr, int qps = 1, int qsplit = -1, int lsplit = -1) {
     g_last_launches = 0;
     Shape s;
     int rc = make_shape(p, is_decode, &s, pos0);
     if (rc != HILS_OK) return rc;
     s.qsplit = qsplit;
+    s.lsplit = lsplit;
     if (qps != 1) {
         // multi-token decode: qps queries per sequence, run as B * qps decode queries over shared caches
         if (!is_decode || qps < 1 || static_cast<long long>(s.B) * qps > (1 << 24)) return HILS_ERR_INVALID_ARG;
@@ -278,6 +280,7 @@ int run_host_prefill_pipelined(const hils_params* p, const ArenaLayout& full, co
     bp.T_max = L;
     Path path;
     const int qsplit = pick_path(s, p, &path) == HILS_OK && path == Path::PrefillFast ? prefill_query_tokens(s) : -1;
+    const int lsplit = qsplit >= 0 ? prefill_local_query(s, qsplit) : -1;
     size_t ws_b = 0;
     for (int b = 0; b < nb; ++b) {
         bp.L = blk_len[b];
@@ -328,7 +331,7 @@ int run_host_prefill_pipelined(const hils_params* p, const ArenaLayout& full, co
         const int rc = run(&bp, 0, base + a_q[sl], base + a_k, base + a_v, base + a_lm,
                            bias ? reinterpret_cast<const float*>(base + a_bias) : nullptr, nullptr, base + a_out[sl],
                            reinterpret_cast<float*>(base + a_lse[sl]), reinterpret_cast<int32_t*>(base + a_sel[sl]),
-                           base + a_ws, ws_b, hp->cmp, nullptr, 0, i0, nullptr, 1, qsplit);
+                           base + a_ws, ws_b, hp->cmp, nullptr, 0, i0, nullptr, 1, qsplit, lsplit);
         if (rc != HILS_OK) return rc;
         launches += g_last_launches;
         ok = ok && cudaEventRecord(hp->cmp_done[sl], hp->cmp) == cudaSuccess;

@@ -29,6 +29,7 @@ struct Shape {
     int qps;        // decode: queries per sequence (multi-token decode).  B then counts queries: query b belongs to
                     // cache sequence b / qps and is its token number b % qps of the qps newest ones; 1 otherwise
     int qsplit;     // prefill: first position that is not computed query-major (-1: chosen for the call)
+    int lsplit;     // prefill: the other positions' local windows are (1), are not (0), -1: chosen for the call
 };
 
 __host__ __device__ inline int floordiv_i(int a, int b) {

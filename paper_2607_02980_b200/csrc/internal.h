@@ -74,12 +74,13 @@ bool prefill_select_tc_supports(const Shape& s);
 // cnt (optional): [query blocks][pairs][nc] entry counts per chunk, accumulated by the kernel (zeroed by the
 // caller) for the tokens from t0 on when qb and t0 are multiples of 128; returns 2 instead of 1 when it did so.
 int launch_prefill_select_tc(const Shape& s, const void* q, const void* landmarks, const float* bias, int32_t* sel,
-                             int* status, int* cnt, int qb, int nc, int t0, cudaStream_t stream);
+                             int* status, int* cnt, int qb, int nc, int t0, int local_counted, cudaStream_t stream);
 
 // Query-major attention on tcgen05 for the first tokens of a call, whose visible chunks are not many more than the ones
 // they attend: how many, and the kernel (write_sel = 1: no token has more candidates than top_k; it writes sel_idx too).
 int prefill_query_tokens(const Shape& s);
-int launch_prefill_query_tc(const Shape& s, const Tensors& t, int n_tok, int write_sel, cudaStream_t stream);
+int launch_prefill_query_tc(const Shape& s, const Tensors& t, int first, int n_tok, int local, int write_sel, cudaStream_t stream);
+bool prefill_local_query(const Shape& s, int first);
 
 // tcgen05 chunk-major attention over the tile table built by the invert kernels (32-token tiles).
 int attend_tc_tile_tokens();

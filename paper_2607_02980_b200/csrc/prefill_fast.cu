@@ -61,6 +61,7 @@ struct PArgs {
     int nc;                 // chunk slots per pair in cnt/off/...: max(C, ceil(L / S))
     int tile_tok;           // entries per attend tile
     int max_tiles;
+    int nl;                 // slots of a token's local window: max_local_slots(W), 0 where `out` and `lse` hold that branch
     int inv_parts, inv_tok; // parts of a query block's tokens that the inversion's CTAs take, tokens of a part
     int whole;              // obuf / lam cover all query blocks (indexed by global entry): one fuse launch per call
 };
@@ -295,7 +296,7 @@ __device__ __forceinline__ InvPart invert_part(const PArgs& a) {
 // f(token, slot, chunk or -1) for every (token, slot) of the part
 template <class F>
 __device__ __forceinline__ void invert_walk(const PArgs& a, const InvPart& p, F f) {
-    const int K1 = a.s.K + max_local_slots(a.s.W);
+    const int K1 = a.s.K + a.nl;
     const int dt = kInvThreads / K1, ds = kInvThreads % K1;
     int tok = p.lo + static_cast<int>(threadIdx.x) / K1, slot = static_cast<int>(threadIdx.x) % K1;
     while (tok < p.hi) {
@@ -417,7 +418,7 @@ __global__ void __launch_bounds__(kInvThreads, 3) invert_fill_kernel(const PArgs
     extern __shared__ int ctr[];
     pdl_wait();
     const InvPart p = invert_part(a);
-    const int K1 = a.s.K + max_local_slots(a.s.W);
+    const int K1 = a.s.K + a.nl;
     int* epos = a.epos + static_cast<long long>(p.pair) * a.s.R * K1;
     for (int c0 = 0; c0 < a.nc; c0 += kInvCounters) {
         const int n = min(kInvCounters, a.nc - c0);
@@ -485,13 +486,16 @@ __global__ void __launch_bounds__(128) prefill_route_scores_kernel(const PArgs a
 constexpr int kFuseWarps = 4;
 constexpr int kFuseRows = 96;             // rows mixed per token: K <= 64 selected + up to 16 local chunks, 3 x 32 lanes
 
+// LOCAL_ROW: the local branch is one more row, in `out` and `lse` (a template parameter: its registers cost the other form
+// resident warps).
+template <bool LOCAL_ROW>
 __global__ void __launch_bounds__(kFuseWarps * 32) prefill_fuse_kernel(const PArgs a) {
     __shared__ float wsm[kFuseWarps][kG][kFuseRows];
     __shared__ int esm[kFuseWarps][kFuseRows];
     pdl_wait();
     const Shape& s = a.s;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int K = s.K, K1 = K + max_local_slots(s.W), nblk = a.i1 - a.i0;
+    const int K = s.K, K1 = K + a.nl, nblk = a.i1 - a.i0;
     const long long total = static_cast<long long>(s.B) * s.Hkv * nblk;
     const long long w = static_cast<long long>(blockIdx.x) * kFuseWarps + wib;
     if (w >= total) return;
@@ -503,7 +507,7 @@ __global__ void __launch_bounds__(kFuseWarps * 32) prefill_fuse_kernel(const PAr
     const int pos = s.pos0 + tok;                    // sequence position of this query row
     const int lc = local_lo(pos, s.W, kS) / kS;      // first local chunk = number of candidate chunks
     const int nsel = min(K, lc);
-    const int nl = pos / kS - lc + 1;
+    const int nl = LOCAL_ROW ? 0 : pos / kS - lc + 1;
     const int nrows = nsel + nl;
     const int e0 = a.whole ? 0 : a.blk_toff[a.blk] * a.tile_tok;   // first entry of this query block
     const int* ep = a.epos + (static_cast<long long>(pair) * s.R + tok) * K1;
@@ -523,32 +527,47 @@ __global__ void __launch_bounds__(kFuseWarps * 32) prefill_fuse_kernel(const PAr
         }
         lam[st][0] = v.x; lam[st][1] = v.y; lam[st][2] = v.z; lam[st][3] = v.w;
     }
+    if (LOCAL_ROW && nrows == 0 && lane == 0) ev[0] = 0;          // (local branch alone: the loads below read a row that nobody uses)
     // the first four rows are requested before the weights are worked out (their addresses need only the entries)
     __syncwarp();
     uint4 ra[4], rb[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-        const int r = min(u, nrows - 1);
+        const int r = max(min(u, nrows - 1), 0);
         const __nv_bfloat16* row = a.obuf + static_cast<long long>(ev[r]) * kG * kD;
         ra[u] = obuf_load(reinterpret_cast<const uint4*>(row + lane * 8));
         rb[u] = obuf_load(reinterpret_cast<const uint4*>(row + 256 + lane * 8));
     }
+    const int hA = lane >> 4, hB = 2 + (lane >> 4), piece = lane & 15;
+    const long long rowA = (static_cast<long long>(b) * s.Hq + gk * kG + hA) * s.R + tok;
+    const long long rowB = (static_cast<long long>(b) * s.Hq + gk * kG + hB) * s.R + tok;
+    // the local branch where the query-major kernel left it: one more row, in this token's rows of `out` and `lse`
+    float lam_l[kG], w_l[kG] = {0.f, 0.f, 0.f, 0.f};
+    uint4 la = make_uint4(0u, 0u, 0u, 0u), lb = la;
+#pragma unroll
+    for (int h = 0; h < kG; ++h) lam_l[h] = LOCAL_ROW ? a.lse[(static_cast<long long>(b) * s.Hq + gk * kG + h) * s.R + tok] : -INFINITY;
+    if (LOCAL_ROW) {
+        la = *reinterpret_cast<const uint4*>(a.out + rowA * kD + piece * 8);
+        lb = *reinterpret_cast<const uint4*>(a.out + rowB * kD + piece * 8);
+    }
     float lse_h = 0.f;
 #pragma unroll
     for (int h = 0; h < kG; ++h) {
-        const float Mx = warp_max(fmaxf(fmaxf(lam[0][h], lam[1][h]), lam[2][h]));
+        float Mx = warp_max(fmaxf(fmaxf(lam[0][h], lam[1][h]), lam[2][h]));
+        if (LOCAL_ROW) Mx = fmaxf(Mx, lam_l[h]);
         float ex[3];
 #pragma unroll
         for (int st = 0; st < 3; ++st) ex[st] = __expf(lam[st][h] - Mx);
-        const float D = warp_sum(ex[0] + ex[1] + ex[2]);
+        const float ex_l = LOCAL_ROW ? __expf(lam_l[h] - Mx) : 0.f;
+        const float D = warp_sum(ex[0] + ex[1] + ex[2]) + ex_l;
         const float inv = 1.f / D;
+        w_l[h] = ex_l * inv;
 #pragma unroll
         for (int st = 0; st < 3; ++st)
             if (lane + 32 * st < nrows) wv[h][lane + 32 * st] = ex[st] * inv;
         if (lane == h) lse_h = Mx + __logf(D);
     }
     __syncwarp();
-    const int hA = lane >> 4, hB = 2 + (lane >> 4), piece = lane & 15;
     float accA[8], accB[8];
 #pragma unroll
     for (int x = 0; x < 8; ++x) { accA[x] = 0.f; accB[x] = 0.f; }
@@ -560,6 +579,10 @@ __global__ void __launch_bounds__(kFuseWarps * 32) prefill_fuse_kernel(const PAr
             acc[2 * x + 1] = fmaf(wgt, __uint_as_float(wd[x] & 0xffff0000u), acc[2 * x + 1]);
         }
     };
+    if (LOCAL_ROW) {
+        fma8(accA, la, hA ? w_l[1] : w_l[0]);
+        fma8(accB, lb, hA ? w_l[3] : w_l[2]);
+    }
     // four rows at a time (8 loads in flight per lane)
     for (int r0 = 0; r0 < nrows; r0 += 4) {
         if (r0 > 0) {
@@ -579,8 +602,6 @@ __global__ void __launch_bounds__(kFuseWarps * 32) prefill_fuse_kernel(const PAr
             }
         }
     }
-    const long long rowA = (static_cast<long long>(b) * s.Hq + gk * kG + hA) * s.R + tok;
-    const long long rowB = (static_cast<long long>(b) * s.Hq + gk * kG + hB) * s.R + tok;
     uint4 pa, pb;
     pa.x = pack_bf16(accA[0], accA[1]); pa.y = pack_bf16(accA[2], accA[3]);
     pa.z = pack_bf16(accA[4], accA[5]); pa.w = pack_bf16(accA[6], accA[7]);
@@ -607,9 +628,9 @@ const int kQBEnv = [] {
 // the attend kernel's walk over one KV head at a time keeps the head's query rows in L2 (16 MB at 16384 tokens).  The
 // partial outputs set the limit: attend + fuse at 16384 against 8192 and 4096 tokens, us:
 // 32K tokens, K = 16: 1698, 1747, -;  64K tokens, K = 32: 6384, 6564, -;  16K tokens, K = 16: 763, 772, 811;  32768 gains nothing.
-int pick_query_block(const Shape& s) {
+int pick_query_block(const Shape& s, int nl) {
     if (kQBEnv) return kQBEnv;
-    const size_t per_tok = static_cast<size_t>(s.B) * s.Hkv * (s.K + max_local_slots(s.W)) * kG * kD * sizeof(__nv_bfloat16);
+    const size_t per_tok = static_cast<size_t>(s.B) * s.Hkv * (s.K + nl) * kG * kD * sizeof(__nv_bfloat16);
     int qb = kQBMax;
     while (qb > kQBMin && qb * per_tok > kObufBytes) qb /= 2;
     return qb;
@@ -620,11 +641,12 @@ struct Plan {
         total, obuf_tiles;
 };
 
-Plan make_plan(const Shape& s, int qb_fixed = 0, int t0 = 0) {
+// (nl: slots of a token's local window, 0 where it goes query-major)
+Plan make_plan(const Shape& s, int qb_fixed, int t0, int nl) {
     Plan p;
     const int R = s.R - t0;                      // tokens of the chunk-major part
     const size_t pairs = static_cast<size_t>(s.B) * s.Hkv;
-    const int QB = qb_fixed > 0 ? qb_fixed : pick_query_block(s);
+    const int QB = qb_fixed > 0 ? qb_fixed : pick_query_block(s, nl);
     const size_t blk = static_cast<size_t>(R < QB ? (R + 127) / 128 * 128 : QB);
     p.qb = static_cast<int>(blk);
     const size_t nchunks = (static_cast<size_t>(s.pos0) + s.R + kS - 1) / kS;     // chunks the queries can touch
@@ -639,8 +661,8 @@ Plan make_plan(const Shape& s, int qb_fixed = 0, int t0 = 0) {
         const size_t toks = (b + 1) * blk <= static_cast<size_t>(R) ? blk : static_cast<size_t>(R) - b * blk;
         const size_t vis = ((s.pos0 + t0 + b * blk + toks) + kS - 1) / kS;
         // (and never more than its entries: a list that exists holds at least one)
-        const size_t ents = pairs * toks * (s.K + max_local_slots(s.W));
-        const size_t ragged = pairs * (toks * (s.K + max_local_slots(s.W)) / tt + (vis < nc ? vis : nc));
+        const size_t ents = pairs * toks * (s.K + nl);
+        const size_t ragged = pairs * (toks * (s.K + nl) / tt + (vis < nc ? vis : nc));
         const size_t tiles = (ents < ragged ? ents : ragged) + 1;
         all_tiles += tiles;
         max_blk = tiles > max_blk ? tiles : max_blk;
@@ -657,7 +679,7 @@ Plan make_plan(const Shape& s, int qb_fixed = 0, int t0 = 0) {
     p.off_seg = take(sizeof(int) * ((nblocks * pairs * nc + kSegLists - 1) / kSegLists));
     p.off_off = take(sizeof(int) * nblocks * pairs * nc);
     p.off_entries = take(sizeof(int) * all_tiles * tt);
-    p.off_epos = take(sizeof(int) * pairs * s.R * (s.K + max_local_slots(s.W)));
+    p.off_epos = take(sizeof(int) * pairs * s.R * (s.K + nl));
     p.off_tiles = take(sizeof(int4) * all_tiles);
     // Partial outputs of all query blocks at once where they fit: the fusion then runs as one launch
     // over the whole call instead of one per block (each launch pays its ramp and its last wave).
@@ -685,10 +707,10 @@ bool prefill_fast_supports(const Shape& s, int dtype) {
 }
 
 size_t prefill_fast_scratch_bytes(const Shape& s) {
-    // (with a routing query no token goes query-major; and fewer tokens may take more scratch, where they just fit at once)
-    const size_t all = make_plan(s).total;
-    const int t0 = prefill_query_tokens(s);
-    const size_t rest = t0 < s.R ? make_plan(s, 0, t0).total : 0;
+    // (with a routing query nothing goes query-major; and fewer entries may take more scratch, where they just fit at once)
+    const int t0 = prefill_query_tokens(s), nl = max_local_slots(s.W);
+    const size_t all = make_plan(s, 0, 0, nl).total;
+    const size_t rest = t0 < s.R ? make_plan(s, 0, t0, prefill_local_query(s, t0) ? 0 : nl).total : 0;
     return all > rest ? all : rest;
 }
 
@@ -696,7 +718,7 @@ size_t prefill_fast_scratch_bytes(const Shape& s) {
 // in one batch.  Returns the CTAs.
 static unsigned invert_split(PArgs& a, const Plan& p) {
     const long long groups = static_cast<long long>(p.n_blocks) * a.s.B * a.s.Hkv;
-    const int toks = a.s.R - a.t0 < a.qb ? a.s.R - a.t0 : a.qb, K1 = a.s.K + max_local_slots(a.s.W);
+    const int toks = a.s.R - a.t0 < a.qb ? a.s.R - a.t0 : a.qb, K1 = a.s.K + a.nl;
     const long long most = (static_cast<long long>(toks) * K1 + kInvThreads * kInvBatch - 1) / (kInvThreads * kInvBatch);
     const long long want = 8ll * sm_count() / groups;
     a.inv_parts = static_cast<int>(want < 1 ? 1 : want < most ? want : most);
@@ -710,11 +732,11 @@ static size_t invert_smem(const PArgs& a) { return sizeof(int) * (a.nc < kInvCou
 // (query blocks of 16384 tokens: of one KV head they take 33 MB of queries and output gradients and as much of fp32 dq,
 // which L2 holds while the head is walked; and a chunk's list is long, so that its dk and dv are added up rarely)
 constexpr int kQBIndex = 16384;
-size_t inverse_index_bytes(const Shape& s) { return make_plan(s, kQBEnv ? kQBEnv : kQBIndex).off_obuf; }
+size_t inverse_index_bytes(const Shape& s) { return make_plan(s, kQBEnv ? kQBEnv : kQBIndex, 0, max_local_slots(s.W)).off_obuf; }
 
 int build_inverse_index(const Shape& s, const int32_t* sel, void* scratch, size_t bytes, InverseIndex* ix,
                         cudaStream_t stream) {
-    const Plan p = make_plan(s, kQBEnv ? kQBEnv : kQBIndex);
+    const Plan p = make_plan(s, kQBEnv ? kQBEnv : kQBIndex, 0, max_local_slots(s.W));
     if (bytes < p.off_obuf) return HILS_ERR_WORKSPACE;
     const int pairs = s.B * s.Hkv;
     char* sc = static_cast<char*>(scratch);
@@ -735,6 +757,7 @@ int build_inverse_index(const Shape& s, const int32_t* sel, void* scratch, size_
     a.qb = p.qb;
     a.nc = p.nc;
     a.tile_tok = attend_tc_tile_tokens();
+    a.nl = max_local_slots(s.W);
     if (cudaMemsetAsync(sc + p.off_cnt, 0, p.zero_bytes, stream) != cudaSuccess) return HILS_ERR_CUDA;
     const unsigned eb = invert_split(a, p);
     const unsigned nseg = static_cast<unsigned>((static_cast<long long>(p.n_blocks) * pairs * p.nc + kSegLists - 1) / kSegLists);
@@ -763,13 +786,15 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
     const int last_cand = local_lo(s.pos0 + s.R - 1, s.W, kS) / kS;
     if (n_qm == s.R && last_cand <= s.K) {
         // nothing to select either: one launch
-        const int rc = launch_prefill_query_tc(s, t, n_qm, 1, stream);
+        const int rc = launch_prefill_query_tc(s, t, 0, n_qm, 0, 1, stream);
         if (rc < 0) return rc;
         trace_mark("prefill_query", stream);
         return rc;
     }
     const int t0 = n_qm;
-    const Plan p = make_plan(s, 0, t0 < s.R ? t0 : 0);
+    const bool local_qm = !t.q_route && t0 < s.R && prefill_local_query(s, t0);
+    const int nl = local_qm ? 0 : max_local_slots(s.W);
+    const Plan p = make_plan(s, 0, t0 < s.R ? t0 : 0, nl);
     if (t.scratch_bytes < p.total) return HILS_ERR_WORKSPACE;
     const int pairs = s.B * s.Hkv;
     char* sc = static_cast<char*>(t.scratch);
@@ -801,6 +826,7 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
     a.nc = p.nc;
     a.tile_tok = attend_tc_tile_tokens();
     a.t0 = t0;
+    a.nl = nl;
     a.i0 = 0;
     a.i1 = 0;
     a.whole = p.whole;
@@ -829,7 +855,7 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
     if (t0 < s.R && cudaMemsetAsync(sc + p.off_cnt, 0, p.zero_bytes, stream) != cudaSuccess) return HILS_ERR_CUDA;
     bool counted = false;
     if (prefill_select_tc_supports(s) && !g_force_mma_select) {
-        const int rc = launch_prefill_select_tc(s, a.q, t.landmarks, t.bias, t.sel_idx, t.status, t0 < s.R ? a.cnt : nullptr, a.qb, a.nc, t0,
+        const int rc = launch_prefill_select_tc(s, a.q, t.landmarks, t.bias, t.sel_idx, t.status, t0 < s.R ? a.cnt : nullptr, a.qb, a.nc, t0, !local_qm,
                                                 stream);
         if (rc < 0) return rc;
         counted = rc == 2;
@@ -840,11 +866,17 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
     trace_mark("prefill_select", stream);
     ++launches;
     if (n_qm > 0) {
-        const int rc = launch_prefill_query_tc(s, t, n_qm, 0, stream);
+        const int rc = launch_prefill_query_tc(s, t, 0, n_qm, 0, 0, stream);
         if (rc < 0) return rc;
         trace_mark("prefill_query", stream);
         launches += rc;
         if (n_qm == s.R) return launches;
+    }
+    if (local_qm) {
+        const int rc = launch_prefill_query_tc(s, t, t0, s.R, 1, 0, stream);
+        if (rc < 0) return rc;
+        trace_mark("prefill_local", stream);
+        launches += rc;
     }
 
     // inverse index for every query block at once: per-(block, pair, chunk) lists of (token, slot) entries
@@ -876,7 +908,7 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
             // With many tiles per (block, pair) the launch walks the pairs one after the other: all CTAs then gather the
             // query rows of one KV head at a time, which L2 keeps.  With few tiles the additional ends of chunk runs cost more:
             // at 29 tiles per CTA and pair 1202 -> 1026 us, at 20 200 -> 191, at 4 102 -> 115.
-            const bool by_pair = static_cast<long long>(a.qb) * (s.K + max_local_slots(s.W)) >= 12ll * a.tile_tok * sm_count();
+            const bool by_pair = static_cast<long long>(a.qb) * (s.K + nl) >= 12ll * a.tile_tok * sm_count();
             const int rc = launch_prefill_attend_tc(s, t.q, maps, t.landmarks, t.bias, a.entries, a.tiles,
                                                     by_pair ? a.pair_toff + blk * pairs : a.blk_toff + blk, by_pair ? pairs : 1, a.lam,
                                                     t.status, a.i0, a.whole, a.whole ? p.n_blocks : 1, a.qb, stream);
@@ -897,7 +929,7 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
             a.i0 = t0;
         }
         const long long fuse_warps = static_cast<long long>(pairs) * (a.i1 - a.i0);
-        if (launch_pdl(prefill_fuse_kernel, dim3(static_cast<unsigned>((fuse_warps + kFuseWarps - 1) / kFuseWarps)),
+        if (launch_pdl(a.nl == 0 ? prefill_fuse_kernel<true> : prefill_fuse_kernel<false>, dim3(static_cast<unsigned>((fuse_warps + kFuseWarps - 1) / kFuseWarps)),
                        dim3(kFuseWarps * 32), 0, stream, a) != cudaSuccess)
             return HILS_ERR_CUDA;
         trace_mark("prefill_fuse", stream);

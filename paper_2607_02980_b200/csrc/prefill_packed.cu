@@ -354,7 +354,7 @@ int launch_prefill_packed(const Shape& s, const Tensors& t, cudaStream_t stream)
     const int pairs = s.B * s.Hkv;
     if (t.q_route) return HILS_ERR_UNSUPPORTED;      // (the mixing logits would need the routing query's scores)
     // selection: the tcgen05 scoring + top-K kernel
-    const int rc = launch_prefill_select_tc(s, t.q, t.landmarks, t.bias, t.sel_idx, t.status, nullptr, 0, 0, 0, stream);
+    const int rc = launch_prefill_select_tc(s, t.q, t.landmarks, t.bias, t.sel_idx, t.status, nullptr, 0, 0, 0, 1, stream);
     if (rc < 0) return rc;
     trace_mark("prefill_select", stream);
     CUtensorMap map_k, map_v;

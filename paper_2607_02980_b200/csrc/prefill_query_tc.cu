@@ -1,6 +1,8 @@
 // Query-major prefill on tcgen05 tensor cores (bf16, d = 128, S = 64, G = 4, one landmark per KV head) for the tokens
 // that see few chunks.
 //
+// (And, for the other tokens, the chunks of wide local windows, which neighbours share too: prefill_local_query.)
+//
 // Where the candidates of a token are not many more than top_k, neighbouring tokens attend mostly the same chunks: a tile of
 // 32 tokens x 4 heads (128 MMA rows) walks the union of its tokens' chunks, and the mix of Eq. (HiLS weights) stays in
 // tensor memory until `out` is written once.  The chunk-major kernels (prefill_attend_tc.cu) move a query row in and a
@@ -52,7 +54,8 @@ struct QmArgs {
     __nv_bfloat16* out;
     float* lse;
     int* status;
-    int n_tok;         // tokens 0 .. n_tok - 1 of every sequence
+    int first, n_tok;  // tokens first .. n_tok - 1 of every sequence (first: a multiple of 64)
+    int local;         // 1: the chunks of the local windows alone; out and lse are then that branch's output and log mass
     int write_sel;     // 1: no token has more candidates than top_k, the selection is written here
 };
 
@@ -63,6 +66,7 @@ struct QmSmem {
     uint64_t list_full[2], list_empty[2];
     uint32_t tmem_base;
     int n_items[2];                             // items of the unit's list
+    int base[2];                                // first chunk of the unit (lists and masks count from it)
     int parts[2];                               // bit t: tile t has items
     int list[2][kMaxC];                         // chunk | tile 0 needs it << 16 | tile 1 needs it << 17
     uint32_t mask[2][kMaxC];                    // (list builder) [tile][chunk]: tokens that attend it
@@ -108,7 +112,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
     QmSmem& sm = *reinterpret_cast<QmSmem*>(qbuf + 2 * kQBytes);
     const Shape& s = a.s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int pairs = s.B * s.Hkv, n_blk = (a.n_tok + kUnitTok - 1) / kUnitTok, n_units = pairs * n_blk;
+    const int pairs = s.B * s.Hkv, blk0 = a.first / kUnitTok, n_blk = (a.n_tok - a.first + kUnitTok - 1) / kUnitTok, n_units = pairs * n_blk;
 
     if (tid == 0) {
         for (int i = 0; i < kStages; ++i) { mbar_init(&sm.kv_full[i], 1); mbar_init(&sm.kv_empty[i], 2); }
@@ -146,7 +150,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             const int end = min(n_units, (rnd + 1) * static_cast<int>(gridDim.x)) - 1;
             idx = end - (idx - rnd * static_cast<int>(gridDim.x));
         }
-        blk = n_blk - 1 - idx / pairs;
+        blk = blk0 + n_blk - 1 - idx / pairs;
         pair = idx % pairs;
     };
     bool ok = true;
@@ -393,11 +397,11 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                 unit_of(idx, blk, pair);
                 const int ln = n_u & 1;
                 if (!wait(&sm.list_full[ln], (n_u >> 1) & 1)) break;
-                const int n = sm.n_items[ln], parts = sm.parts[ln];
+                const int n = sm.n_items[ln], parts = sm.parts[ln], base = sm.base[ln];
                 const int b = pair / s.Hkv, gk = pair % s.Hkv;
                 auto load_item = [&](int i) {
                     const uint32_t st = g % kStages;
-                    const int c = sm.list[ln][i] & 0xffff;
+                    const int c = base + (sm.list[ln][i] & 0xffff);
                     if (g >= kStages && !wait(&sm.kv_empty[st], ((g / kStages) - 1) & 1)) return;
                     const int row = pair * s.T + c * kS;
                     // chunks left of every token's window have a landmark row (the others' score column is not used)
@@ -445,7 +449,8 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             const int ln = n_u & 1;
             if (n_u >= 2 && !wait(&sm.list_empty[ln], ((n_u >> 1) - 1) & 1)) break;
             const int tok0 = blk * kUnitTok;
-            const int last = s.pos0 + min(a.n_tok, tok0 + kUnitTok) - 1, n_vis = last / kS + 1;
+            const int last = s.pos0 + min(a.n_tok, tok0 + kUnitTok) - 1;
+            const int base = a.local ? local_lo(s.pos0 + tok0, s.W, kS) / kS : 0, n_vis = last / kS + 1 - base;
             for (int c = lane; c < n_vis; c += 32) { sm.mask[0][c] = 0u; sm.mask[1][c] = 0u; }
             __syncwarp();
             for (int t = 0; t < 2; ++t) {
@@ -453,7 +458,9 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                 const bool live = tok < a.n_tok;
                 const int lc = live ? local_lo(pos, s.W, kS) / kS : 0;
                 const uint32_t bit = 1u << lane;
-                if (__all_sync(kFullMask, !live || lc <= s.K)) {
+                if (a.local) {
+                    // (nothing to select)
+                } else if (__all_sync(kFullMask, !live || lc <= s.K)) {
                     // every token takes all its candidates
                     const int most = __reduce_max_sync(kFullMask, lc);
                     for (int c = 0; c < most; ++c) {
@@ -471,7 +478,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                 __syncwarp();
                 // chunks of the local windows
                 if (live)
-                    for (int c = lc; c <= pos / kS; ++c) atomicOr(&sm.mask[t][c], bit);
+                    for (int c = lc; c <= pos / kS; ++c) atomicOr(&sm.mask[t][c - base], bit);
                 __syncwarp();
             }
             int n = 0, nt[2] = {0, 0};
@@ -483,7 +490,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                 for (int t = 0; t < 2; ++t) {
                     m[t] = c < n_vis ? sm.mask[t][c] : 0u;
                     const unsigned v = __ballot_sync(kFullMask, m[t] != 0u);
-                    if (m[t]) sm.titem[ln][t][nt[t] + __popc(v & below)] = make_int2(c, static_cast<int>(m[t]));
+                    if (m[t]) sm.titem[ln][t][nt[t] + __popc(v & below)] = make_int2(base + c, static_cast<int>(m[t]));
                     nt[t] += __popc(v);
                 }
                 const unsigned v = __ballot_sync(kFullMask, (m[0] | m[1]) != 0u);
@@ -492,6 +499,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             }
             if (lane == 0) {
                 sm.n_items[ln] = n;
+                sm.base[ln] = base;
                 sm.n_tile[ln][0] = nt[0];
                 sm.n_tile[ln][1] = nt[1];
                 sm.parts[ln] = (nt[0] > 0 ? 1 : 0) | (nt[1] > 0 ? 2 : 0);
@@ -544,7 +552,21 @@ int prefill_query_tokens(const Shape& s) {
     return best;
 }
 
-int launch_prefill_query_tc(const Shape& s, const Tensors& t, int n_tok, int write_sel, cudaStream_t stream) {
+// Whether the local windows of the chunk-major tokens (from `first` on) go this way too, as one partial output row per token
+// and head (in out and lse, for the fuse kernel) instead of one per window chunk.  A unit visits the nl chunks of a window and
+// one more; costs as above, with a margin that keeps windows of up to five chunks chunk-major, where nothing is gained
+// (W = 256, 8192 tokens, K = 16: 541 us, 544 this way).  W = 512: 60,000 tokens, K = 16: 5.47 -> 4.98 ms; 16K 1.29 -> 1.19 ms; a
+// slice of 2048 tokens at 48K, K = 32: the kernels after the selection 320 -> 297 us.
+bool prefill_local_query(const Shape& s, int first) {
+    if (s.Hl != s.Hkv) return false;
+    if (s.lsplit >= 0) return s.lsplit != 0;
+    const int nl = (s.W - 1 + kS - 1) / kS + 1;
+    const long long pairs = static_cast<long long>(s.B) * s.Hkv, sms = sm_count(), toks = s.R - first, unit = 3000 * (nl + 1) + 18000;
+    const long long here = pairs * ((toks + kUnitTok - 1) / kUnitTok) * unit / sms, there = pairs * toks * nl * 3830 / 32 / sms;
+    return (here > unit ? here : unit) * 11 / 10 + 5000 < there;
+}
+
+int launch_prefill_query_tc(const Shape& s, const Tensors& t, int first, int n_tok, int local, int write_sel, cudaStream_t stream) {
     const uint64_t kv_rows = static_cast<uint64_t>(s.B) * s.Hkv * s.T, q_rows = static_cast<uint64_t>(s.B) * s.Hq * s.R;
     CUtensorMap map_q, map_k, map_v, map_out;
     if (!make_bf16_2d_map(&map_q, t.q, q_rows, kD, 64, kTok) || !make_bf16_2d_map(&map_k, t.k, kv_rows, kD, 64, kS) ||
@@ -558,8 +580,8 @@ int launch_prefill_query_tc(const Shape& s, const Tensors& t, int n_tok, int wri
         once.done();
     }
     QmArgs a{s, static_cast<const __nv_bfloat16*>(t.landmarks), t.bias, t.sel_idx, static_cast<__nv_bfloat16*>(t.out), t.lse, t.status,
-             n_tok, write_sel};
-    const long long units = static_cast<long long>(s.B) * s.Hkv * ((n_tok + kUnitTok - 1) / kUnitTok);
+             first, n_tok, local, write_sel};
+    const long long units = static_cast<long long>(s.B) * s.Hkv * ((n_tok - first + kUnitTok - 1) / kUnitTok);
     const unsigned grid = static_cast<unsigned>(units < sm_count() ? units : sm_count());
     if (launch_pdl(prefill_query_tc_kernel, dim3(grid), dim3(kThreads), smem, stream, map_q, map_k, map_v, map_out, a) != cudaSuccess)
         return HILS_ERR_CUDA;

@@ -42,6 +42,7 @@ struct TcArgs {
     // first step of the inverse index, taken here because the selections are at hand (NULL: not wanted)
     int* cnt;
     int qb, nc, t0;    // tokens per query block (a multiple of the 128-token tile), chunk slots per pair in cnt, first token counted
+    int local;         // 1: the chunks of the local windows are counted too
 };
 
 struct TcSmem {
@@ -505,7 +506,8 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                 for (int e = 0; e < N; ++e)
                     if (ids[e] >= 0) atomicAdd(dst + ids[e], 1);
                 const int pos = s.pos0 + tok;
-                for (int c = local_lo(pos, s.W, kS) / kS; c <= pos / kS; ++c) atomicAdd(dst + c, 1);
+                if (a.local)
+                    for (int c = local_lo(pos, s.W, kS) / kS; c <= pos / kS; ++c) atomicAdd(dst + c, 1);
             }
             if (in_smem) {
                 asm volatile("bar.sync 1, 128;" ::: "memory");
@@ -532,7 +534,7 @@ bool prefill_select_tc_supports(const Shape& s) {
 }
 
 int launch_prefill_select_tc(const Shape& s, const void* q, const void* landmarks, const float* bias, int32_t* sel,
-                             int* status, int* cnt, int qb, int nc, int t0, cudaStream_t stream) {
+                             int* status, int* cnt, int qb, int nc, int t0, int local_counted, cudaStream_t stream) {
     const int pairs = s.B * s.Hkv;
     CUtensorMap map_q, map_lm;
     if (!make_bf16_2d_map(&map_q, q, static_cast<uint64_t>(s.B) * s.Hq * s.R, kD, 64, kTileTok) ||
@@ -553,7 +555,7 @@ int launch_prefill_select_tc(const Shape& s, const void* q, const void* landmark
             return HILS_ERR_CUDA;
         attr_once.done();
     }
-    TcArgs a{s, bias, sel, status, (cnt && qb % kTileTok == 0) ? cnt : nullptr, qb, nc, t0};
+    TcArgs a{s, bias, sel, status, (cnt && qb % kTileTok == 0) ? cnt : nullptr, qb, nc, t0, local_counted};
     const int tiles = (s.R + kTileTok - 1) / kTileTok;
     const unsigned all_tiles = static_cast<unsigned>(pairs) * tiles;
     const unsigned nsm = static_cast<unsigned>(sm_count());

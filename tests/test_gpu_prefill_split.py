@@ -17,6 +17,9 @@ pytestmark = pytest.mark.gpu
     (16, 4, 2500, 8, 1, 60.0, 0),      # split; logits that raise the running reference and hide chunks
     (4, 8, 2500, 5, 130, 0.5, 0),      # split; selection rows of 20 bytes
     (2, 1, 3000, 5, 130, 0.5, 0),      # too few KV heads to split
+    (2, 4, 5000, 4, 512, 0.5, 0),      # the others' local windows query-major too
+    (1, 8, 2100, 8, 512, 0.5, 9001),   # a slice at an odd position, windows query-major
+    (2, 2, 6001, 5, 897, 0.0, 0),      # the widest window, a ragged last unit
     (1, 2, 4200, 16, 1, 0.0, 0),       # KV heads together
     (1, 1, 16384, 16, 1, 0.0, 0),      # one KV head at a time, several query blocks' worth of lists
     (4, 8, 1500, 8, 64, 0.5, 300),     # a slice that begins among the query-major tokens
