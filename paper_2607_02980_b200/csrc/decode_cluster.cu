@@ -709,7 +709,9 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                 const int m = ctok[nt][x];
                 const bool loc = m < TG && ((it.flags >> m) & 1u), sel = m < TG && ((it.flags >> (8 + m)) & 1u);
                 if (any_loc) {
-                    const int lim = loc ? sm.len[m] - 1 - it.chunk * kS : kS - 1;      // last visible key of the column
+                    // last visible key of the column; in a column whose token does not see the chunk, the last one that exists
+                    // (rows past the unit's last token may hold anything, and a NaN outlives the weight of 0)
+                    const int lim = (loc ? sm.len[m] : len_max) - 1 - it.chunk * kS;
 #pragma unroll
                     for (int mt = 0; mt < 4; ++mt) {
                         if (mt * 16 + g > lim) sc[mt][nt][x] = -INFINITY;
