@@ -87,6 +87,10 @@ __device__ inline int key_chunk(unsigned long long key) {
     return static_cast<int>(0xffffffffu - static_cast<uint32_t>(key & 0xffffffffull));
 }
 
+// Where a running maximum of mixing logits starts.  Finite: the logit of a chunk that the bias masks is -inf, and
+// exp(-inf - lowest) is the weight of 0 that it has to get, where exp(-inf + inf) is NaN.
+constexpr float kLowestLogit = -3.402823466e+38f;
+
 __device__ inline float warp_max(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(kFullMask, v, o));

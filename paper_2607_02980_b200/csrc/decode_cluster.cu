@@ -641,7 +641,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
         for (int x = 0; x < 2; ++x) {
-            Mx[nt][x] = -INFINITY;
+            Mx[nt][x] = kLowestLogit;
             Dn[nt][x] = 0.f;
             const int col = nt * 8 + 2 * t + x;
             ctok[nt][x] = col % Gp < G ? col / Gp : TG;           // token of the column (TG: none)

@@ -1,0 +1,62 @@
+"""A bias of minus infinity takes a chunk out of a sequence: it may still fill a place of the selection (where fewer than
+top_k others are left: the lowest ids among equals, like any tie) and then has weight zero.  Every kernel that mixes chunks,
+against the CPU oracle, with some, most and all chunks masked."""
+import pytest
+import torch
+
+import paper_2607_02980_b200 as hils
+from paper_2607_02980_b200 import workloads as wl
+from parity import check_decode
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+def masked_bias(cfg, share, heads=None):
+    """bias [B, Hl, C] with `share` of the chunks masked, chunk 0 among them."""
+    g = torch.Generator().manual_seed(cfg.seed)
+    bias = torch.randn((cfg.B, heads or cfg.Hkv, cfg.C), generator=g)
+    bias[torch.rand(bias.shape, generator=g) < share] = float("-inf")
+    bias[:, :, 0] = float("-inf")
+    return bias
+
+
+def decode(cfg, share, seq=None, impl="auto", per_head=False):
+    seq = torch.tensor(seq or [cfg.L - 97 * b for b in range(cfg.B)], dtype=torch.int32)
+    inp = wl.make_decode_inputs(cfg, "cpu", seq_lens=seq)
+    if per_head:
+        inp["landmarks"] = inp["landmarks"].repeat_interleave(cfg.G, dim=1).contiguous()
+    bias = masked_bias(cfg, share, cfg.Hq if per_head else None)
+    g = {n: t.to(DEV) for n, t in inp.items()}
+    got = hils.hils_decode(g["q"], g["k"], g["v"], g["landmarks"], g["seq_lens"], 64, cfg.K, window=cfg.window,
+                           bias=bias.to(DEV), impl=impl)
+    torch.cuda.synchronize()
+    check_decode(cfg, inp, *got, bias=bias, W=cfg.window)
+
+
+@pytest.mark.parametrize("share", [0.5, 0.97, 1.0])
+@pytest.mark.parametrize("B,Hkv,T,K,W", [
+    (2, 2, 64 * 20, 16, 1),            # every token takes nearly all its candidates
+    (3, 2, 64 * 130, 16, 65),          # every candidate is ranked
+    (2, 8, 64 * 400, 32, 512),         # lists longer than what is ranked
+    (40, 8, 64 * 70, 16, 1),           # two CTAs per SM
+])
+def test_decode_in_clusters(B, Hkv, T, K, W, share):
+    cfg = wl.HilsConfig("masked", "decode", B, 4 * Hkv, Hkv, T, 128, 64, K, "bf16", 1100 + B + K, window=W)
+    decode(cfg, share)
+
+
+@pytest.mark.parametrize("share", [0.5, 1.0])
+def test_draft_tokens(share):
+    B, M = 10, 4
+    cfg = wl.HilsConfig("masked", "decode", B, 32, 8, 64 * 40, 128, 64, 16, "bf16", 1150)
+    seq = torch.tensor([cfg.L - 61 * b for b in range(B)], dtype=torch.int32)
+    inp = wl.make_decode_inputs(cfg, "cpu", seq_lens=seq)
+    q = torch.randn((B, M, 32, 128), generator=torch.Generator().manual_seed(5)).to(torch.bfloat16)
+    bias = masked_bias(cfg, share)
+    g = {n: t.to(DEV) for n, t in inp.items()}
+    out, lse, sel = hils.hils_decode_multi(q.to(DEV), g["k"], g["v"], g["landmarks"], g["seq_lens"], 64, 16, bias=bias.to(DEV))
+    torch.cuda.synchronize()
+    for m in range(M):
+        one = dict(inp, q=q[:, m].contiguous(), seq_lens=seq - (M - 1 - m))
+        check_decode(cfg, one, out[:, m], lse[:, m], sel[:, m], bias=bias)
