@@ -333,7 +333,7 @@ generic_attend_kernel(const GArgs a) {
     const int32_t* sel = a.sel + ((static_cast<long long>(b) * s.Hkv + g) * s.R + r) * s.K;
 
     const int n_loc = (pos - lo) / 64 + 1, n_items = n_loc + min(s.K, ncand);
-    float Mx = -INFINITY, Dn = 0.f;
+    float Mx = kLowestLogit, Dn = 0.f;
     Q acc;
     acc.fill(0.f);
     for (int it = warp; it < n_items; it += nw) {

@@ -6,7 +6,7 @@ import torch
 
 import paper_2607_02980_b200 as hils
 from paper_2607_02980_b200 import workloads as wl
-from parity import check_decode
+from parity import check_decode, check_prefill
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -32,6 +32,17 @@ def decode(cfg, share, seq=None, impl="auto", per_head=False):
                            bias=bias.to(DEV), impl=impl)
     torch.cuda.synchronize()
     check_decode(cfg, inp, *got, bias=bias, W=cfg.window)
+
+
+def prefill(cfg, share, impl="auto", per_head=False):
+    inp = wl.make_prefill_inputs(cfg, "cpu")
+    if per_head:
+        inp["landmarks"] = inp["landmarks"].repeat_interleave(cfg.G, dim=1).contiguous()
+    bias = masked_bias(cfg, share, cfg.Hq if per_head else None)
+    g = {n: t.to(DEV) for n, t in inp.items()}
+    got = hils.hils_prefill(g["q"], g["k"], g["v"], g["landmarks"], 64, cfg.K, bias=bias.to(DEV), window=cfg.window, impl=impl)
+    torch.cuda.synchronize()
+    check_prefill(cfg, inp, *got, bias=bias, W=cfg.window)
 
 
 @pytest.mark.parametrize("share", [0.5, 0.97, 1.0])
@@ -60,3 +71,16 @@ def test_draft_tokens(share):
     for m in range(M):
         one = dict(inp, q=q[:, m].contiguous(), seq_lens=seq - (M - 1 - m))
         check_decode(cfg, one, out[:, m], lse[:, m], sel[:, m], bias=bias)
+
+
+@pytest.mark.parametrize("share", [0.5, 1.0])
+@pytest.mark.parametrize("mode,dtype,d,L,K,W", [
+    ("decode", "bf16", 128, 64 * 40, 16, 65),
+    ("decode", "f32", 64, 64 * 30, 4, 1),
+    ("prefill", "bf16", 128, 700, 4, 1),
+    ("prefill", "f32", 96, 500, 4, 65),        # the row kernel
+    ("prefill", "f32", 64, 700, 4, 1),         # the chunk-major kernels
+])
+def test_generic_kernels(mode, dtype, d, L, K, W, share):
+    cfg = wl.HilsConfig("masked", mode, 2, 8, 2, L, d, 64, K, dtype, 1160 + d, window=W)
+    (decode if mode == "decode" else prefill)(cfg, share, impl="generic")
