@@ -177,7 +177,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             const bool live = tok < a.n_tok;
             const int pos = s.pos0 + tok, lc = local_lo(pos, s.W, kS) / kS, ci = pos / kS;
             const float* bias = a.bias ? a.bias + (static_cast<long long>(b) * s.Hl + gk) * s.C : nullptr;
-            float ref = -INFINITY, den = 0.f;
+            float ref = kLowestLogit, den = 0.f;
             int2 next = n > 0 ? sm.titem[ln][t][0] : make_int2(0, 0);
             for (int i = 0; i < n; ++i) {
                 const int c = next.x;

@@ -84,3 +84,11 @@ def test_draft_tokens(share):
 def test_generic_kernels(mode, dtype, d, L, K, W, share):
     cfg = wl.HilsConfig("masked", mode, 2, 8, 2, L, d, 64, K, dtype, 1160 + d, window=W)
     (decode if mode == "decode" else prefill)(cfg, share, impl="generic")
+
+
+@pytest.mark.parametrize("share", [0.5, 1.0])
+def test_query_major_prefill(share):
+    """No more candidates than top_k: one launch, chunk 0 first in every token's walk."""
+    cfg = wl.HilsConfig("masked", "prefill", 3, 8, 2, 1000, 128, 64, 16, "bf16", 1170)
+    prefill(cfg, share)
+    assert hils.last_launch_count() == 1
