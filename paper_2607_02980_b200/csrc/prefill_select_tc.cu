@@ -473,6 +473,19 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         // (after a timeout the thread still walks through the tile's barriers; every warp leaves together below)
         if (!ok) { set_status(a.status, kDevTimeout); *reinterpret_cast<volatile int*>(&sm.abort) = 1; }
 
+        // Scores of -inf (chunks that the bias masks) and NaN beat no threshold, so fewer than K may have been kept: the lowest
+        // of the other ids fill the places, as ties do.  With x the last of them, that makes every id up to x.
+        const int miss = min(K, my_ncand) - cnt;
+        if (ok && nsteps > 0 && tok < s.R && miss > 0) {
+            int x = miss - 1, below = 0;
+#pragma unroll 1
+            while (below < cnt && static_cast<int>(pool[below * kTileTok] & 0xffffffffull) <= x) { ++below; ++x; }
+#pragma unroll 1
+            for (int e = cnt - 1; e >= below; --e) pool[(e + miss) * kTileTok] = pool[e * kTileTok];
+#pragma unroll 1
+            for (int e = 0; e <= x; ++e) pool[e * kTileTok] = static_cast<unsigned long long>(e);
+            cnt += miss;
+        }
         // the survivors are the selection, already in ascending chunk order; -1 padded
         int ids[N];
 #pragma unroll

@@ -92,3 +92,36 @@ def test_query_major_prefill(share):
     cfg = wl.HilsConfig("masked", "prefill", 3, 8, 2, 1000, 128, 64, 16, "bf16", 1170)
     prefill(cfg, share)
     assert hils.last_launch_count() == 1
+
+
+@pytest.mark.parametrize("share", [0.5, 0.97, 1.0])
+@pytest.mark.parametrize("B,Hkv,L,K,W,impl,per_head", [
+    (1, 1, 3000, 5, 130, "auto", False),       # everything chunk-major
+    (2, 2, 64 * 40 + 1, 16, 1, "auto", False),
+    (1, 2, 64 * 50, 32, 1, "auto", True),
+    (1, 2, 64 * 60, 40, 65, "auto", False),    # the selection kernel of top_k > 32
+    (1, 2, 64 * 30, 8, 1, "packed", False),
+])
+def test_selected_prefill(B, Hkv, L, K, W, impl, per_head, share):
+    cfg = wl.HilsConfig("masked", "prefill", B, 4 * Hkv, Hkv, L, 128, 64, K, "bf16", 1180 + K, window=W)
+    prefill(cfg, share, impl=impl, per_head=per_head)
+
+
+@pytest.mark.parametrize("L,K", [(64 * 60 + 9, 16), (64 * 60, 32), (64 * 60, 40)])
+def test_a_query_that_is_not_a_number_spoils_its_own_row_only(L, K):
+    """Its scores beat no threshold either: the selection still has to be K chunks that exist."""
+    cfg = wl.HilsConfig("nan", "prefill", 1, 4, 1, L, 128, 64, K, "bf16", 1190 + K)
+    g = wl.make_prefill_inputs(cfg, DEV)
+    clean = hils.hils_prefill(g["q"], g["k"], g["v"], g["landmarks"], 64, K)
+    rows = torch.tensor([0, 77, 64 * 50 + 3, L - 1], device=DEV)
+    g["q"][:, :, rows] = float("nan")
+    out, lse, sel = hils.hils_prefill(g["q"], g["k"], g["v"], g["landmarks"], 64, K)
+    torch.cuda.synchronize()
+    rest = torch.ones(L, dtype=torch.bool, device=DEV)
+    rest[rows] = False
+    assert torch.equal(out[:, :, rest], clean[0][:, :, rest]) and torch.equal(lse[:, :, rest], clean[1][:, :, rest])
+    assert torch.isnan(out[:, :, rows]).all()
+    for r in rows.tolist():
+        ids = sel[0, 0, r].tolist()
+        n = min(K, r // 64)
+        assert ids[n:] == [-1] * (K - n) and sorted(set(ids[:n])) == ids[:n] and all(0 <= c < r // 64 for c in ids[:n])
