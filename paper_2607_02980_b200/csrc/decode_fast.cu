@@ -484,7 +484,7 @@ __device__ void select_pair(const DArgs& a, int pair, int ncand, SelShared& sh, 
     }
     __syncthreads();
     for (int h = warp; h < G; h += nw) {
-        float mx = -INFINITY;
+        float mx = kLowestLogit;
         for (int t = lane; t < n; t += 32) mx = fmaxf(mx, sh.lam_s[h][t]);
         mx = warp_max(mx);
         float sum = 0.f;

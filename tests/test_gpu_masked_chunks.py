@@ -73,6 +73,14 @@ def test_draft_tokens(share):
         check_decode(cfg, one, out[:, m], lse[:, m], sel[:, m], bias=bias)
 
 
+@pytest.mark.parametrize("share", [0.5, 0.97, 1.0])
+@pytest.mark.parametrize("T,K,W,per_head", [(64 * 40, 8, 1, False), (64 * 60, 16, 65, True)])
+def test_decode_in_three_kernels(T, K, W, per_head, share):
+    cfg = wl.HilsConfig("masked", "decode", 2, 8, 2, T, 128, 64, K, "bf16", 1155 + K, window=W)
+    decode(cfg, share, per_head=per_head)
+    assert hils.last_launch_count() == 3
+
+
 @pytest.mark.parametrize("share", [0.5, 1.0])
 @pytest.mark.parametrize("mode,dtype,d,L,K,W", [
     ("decode", "bf16", 128, 64 * 40, 16, 65),
