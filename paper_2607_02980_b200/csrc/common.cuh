@@ -44,6 +44,12 @@ __host__ __device__ inline int local_lo(int pos, int W, int S) {
     return lo < 0 ? 0 : lo;
 }
 
+// Position of row `tok` of a prefill call whose rows end at n_tok.  The lanes of a ragged last tile that have no row stand
+// where the last row does: one further on may have a candidate chunk more, whose landmark and bias rows need not exist.
+__host__ __device__ inline int lane_position(const Shape& s, int tok, int n_tok) {
+    return s.pos0 + (tok < n_tok ? tok : n_tok - 1);
+}
+
 __device__ inline float to_f32(float x) { return x; }
 __device__ inline float to_f32(__nv_bfloat16 x) { return __bfloat162float(x); }
 

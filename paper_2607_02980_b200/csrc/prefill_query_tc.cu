@@ -175,7 +175,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             const int b = pair / s.Hkv, gk = pair % s.Hkv;
             const int tok = blk * kUnitTok + t * kTok + lane;
             const bool live = tok < a.n_tok;
-            const int pos = s.pos0 + tok, lc = local_lo(pos, s.W, kS) / kS, ci = pos / kS;
+            const int pos = lane_position(s, tok, a.n_tok), lc = local_lo(pos, s.W, kS) / kS;
             const float* bias = a.bias ? a.bias + (static_cast<long long>(b) * s.Hl + gk) * s.C : nullptr;
             float ref = kLowestLogit, den = 0.f;
             int2 next = n > 0 ? sm.titem[ln][t][0] : make_int2(0, 0);
