@@ -466,7 +466,8 @@ generic_chunk_kernel(const GArgs a, float* part, float* lam) {
     if (s.pos0 + min(s.R, r0 + kRowBlock) - 1 < c * s.S) return;            // the chunk lies after the block's last row
     const float* kc = static_cast<const float*>(a.k) + ((static_cast<long long>(b) * s.Hkv + g) * s.T + static_cast<long long>(c) * s.S) * D;
     const float* vc = static_cast<const float*>(a.v) + (kc - static_cast<const float*>(a.k));
-    const int rows_k = min(s.S, s.T - c * s.S);                             // rows of the chunk that exist
+    // rows of the chunk up to the call's last token: the ones after it may hold anything, and 0 x NaN is NaN
+    const int rows_k = min(s.S, s.pos0 + s.R - c * s.S);
     for (int x = tid; x < rows_k * (D / 4); x += blockDim.x)
         cp_async16(smem_u32(&sm.k[x / (D / 4)][(x % (D / 4)) * 4]), kc + x * 4);
     for (int x = tid; x < rows_k * (D / 4); x += blockDim.x)

@@ -47,3 +47,27 @@ def test_drafts_that_straddle_a_chunk(B, M, W, G, value):
         sl = torch.tensor([n - M + m + 1 for n in lens], dtype=torch.int32)
         ref = oracle.hils_decode(q[:, m].contiguous(), inp["k"], inp["v"], inp["landmarks"], None, sl, S=64, K=16, W=W)
         check((out[:, m], lse[:, m], sel[:, m]), ref, 16)
+
+
+@pytest.mark.parametrize("dtype,impl,S,Hkv,pos0,L,W", [
+    ("f32", "generic", 64, 1, 300, 200, 1),
+    ("f32", "generic", 48, 2, 100, 333, 100),
+    ("bf16", "generic", 64, 1, 300, 200, 1),
+])
+def test_slice_that_ends_inside_a_chunk(dtype, impl, S, Hkv, pos0, L, W):
+    cfg = wl.HilsConfig("tail", "prefill", 2, 4 * Hkv, Hkv, (pos0 + L + 2 * S) // S * S, 128, S, 4, dtype, 730 + L, window=W)
+    inp = wl.make_prefill_inputs(cfg, "cpu")
+    n = pos0 + L
+    assert n % S and cfg.L > n
+    for t in (inp["k"], inp["v"]):
+        t[:, :, n:] = float("nan")
+    inp["landmarks"][:, :, n // S:] = float("nan")
+    q = inp["q"][:, :, pos0:n].contiguous()
+    g = {x: t.to(DEV) for x, t in inp.items()}
+    out, lse, sel = hils.hils_prefill_at(q.to(DEV), g["k"], g["v"], g["landmarks"], S, 4, pos0, window=W, impl=impl)
+    torch.cuda.synchronize()
+    rows = np.arange(L)
+    for b in range(2):
+        ref = oracle.hils_rows(q, inp["k"], inp["v"], inp["landmarks"], None, S=S, K=4, W=W,
+                               row_b=np.full(L, b, np.int32), row_qi=rows.astype(np.int32), row_pos=(pos0 + rows).astype(np.int64))
+        check((out[b].transpose(0, 1), lse[b].T, sel[b].transpose(0, 1)), ref, 4, dtype)
