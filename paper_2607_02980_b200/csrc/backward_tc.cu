@@ -473,15 +473,15 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         uint32_t run = 0;
         for (uint32_t n = 0; tile_of(n); ++n) {
             const Tile& tl = sm.tile[n % kMeta];
-            const int flags = tl.flags, row = tl.kv, lmr = tl.lm;
+            const int flags = tl.flags, pair = tl.kv / s.T, row = tl.kv - pair * s.T, lmr = tl.lm;
             __syncwarp();
             if (lane == 0) tile_done(n);
             if (!(flags & 256)) continue;
             if (lane == 0) {                                            // (mostly a few tiles ahead: into L2 already)
-                tma_prefetch_l2_2d(&map_k, 0, row);
-                tma_prefetch_l2_2d(&map_k, 64, row);
-                tma_prefetch_l2_2d(&map_v, 0, row);
-                tma_prefetch_l2_2d(&map_v, 64, row);
+                tma_prefetch_l2_3d(&map_k, 0, row, pair);
+                tma_prefetch_l2_3d(&map_k, 64, row, pair);
+                tma_prefetch_l2_3d(&map_v, 0, row, pair);
+                tma_prefetch_l2_3d(&map_v, 64, row, pair);
             }
             uint4 lmp = make_uint4(0u, 0u, 0u, 0u);
             if (lane < 16 && lmr >= 0) lmp = *reinterpret_cast<const uint4*>(a.lm + static_cast<long long>(lmr) * kD + lane * 8);
@@ -489,10 +489,10 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
             ++run;
             if (lane == 0) {
                 mbar_expect_tx(&sm.k_ready, 16384 + kVBytes);
-                tma_load_2d(kbuf, &map_k, &sm.k_ready, 0, row);
-                tma_load_2d(kbuf + kNS * 128, &map_k, &sm.k_ready, 64, row);
-                tma_load_2d(vbuf, &map_v, &sm.k_ready, 0, row);
-                tma_load_2d(vbuf + 8192, &map_v, &sm.k_ready, 64, row);
+                tma_load_3d(kbuf, &map_k, &sm.k_ready, 0, row, pair);
+                tma_load_3d(kbuf + kNS * 128, &map_k, &sm.k_ready, 64, row, pair);
+                tma_load_3d(vbuf, &map_v, &sm.k_ready, 0, row, pair);
+                tma_load_3d(vbuf + 8192, &map_v, &sm.k_ready, 64, row, pair);
             }
             if (lane < 16) *reinterpret_cast<uint4*>(kbuf + (lane >> 3) * (kNS * 128) + swz128(64, lane & 7)) = lmp;
             fence_proxy_async_smem();
@@ -693,8 +693,8 @@ int launch_prefill_backward_fast(const Shape& s, const BackwardTensors& t, cudaS
     const int rc = build_inverse_index(s, t.sel_idx, sc + dsum_bytes(s), t.scratch_bytes - dsum_bytes(s), &ix, stream);
     if (rc < 0) return rc;
     CUtensorMap map_k, map_v;
-    const uint64_t kv_rows = static_cast<uint64_t>(s.B) * s.Hkv * s.T;
-    if (!make_bf16_2d_map(&map_k, t.k, kv_rows, kD, 64, kS) || !make_bf16_2d_map(&map_v, t.v, kv_rows, kD, 64, kS))
+    const uint64_t kv_pairs = static_cast<uint64_t>(s.B) * s.Hkv;
+    if (!make_kv_map(&map_k, t.k, kv_pairs, s.T, s.pos0 + s.R, kD, 64, kS) || !make_kv_map(&map_v, t.v, kv_pairs, s.T, s.pos0 + s.R, kD, 64, kS))
         return HILS_ERR_CUDA;
     static PerDeviceOnce attr_once;
     if (attr_once.pending()) {

@@ -393,18 +393,17 @@ prefill_attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
                 if (cc >= 2 && !wait(&sm.k_empty[cbuf], ((cc >> 1) - 1) & 1)) break;
                 if (cc >= kVBufs && !wait(&sm.v_empty[vb], ((cc / kVBufs) - 1) & 1)) break;
                 if (lane == 0) {
-                    const int row = pair * s.T + c * kS;
+                    const int row = c * kS;
                     mbar_expect_tx(&sm.k_ready[cbuf], 2 * 8192);
-                    tma_load_2d(kbuf + cbuf * kKBytes, &map_k, &sm.k_ready[cbuf], 0, row);
-                    tma_load_2d(kbuf + cbuf * kKBytes + kNS * 128, &map_k, &sm.k_ready[cbuf], 64, row);
+                    tma_load_3d(kbuf + cbuf * kKBytes, &map_k, &sm.k_ready[cbuf], 0, row, pair);
+                    tma_load_3d(kbuf + cbuf * kKBytes + kNS * 128, &map_k, &sm.k_ready[cbuf], 64, row, pair);
                     mbar_expect_tx(&sm.v_ready[vb], kVBytes);
-                    tma_load_2d(vbuf + vb * kVBytes, &map_v, &sm.v_ready[vb], 0, row);
-                    tma_load_2d(vbuf + vb * kVBytes + 8192, &map_v, &sm.v_ready[vb], 64, row);
+                    tma_load_3d(vbuf + vb * kVBytes, &map_v, &sm.v_ready[vb], 0, row, pair);
+                    tma_load_3d(vbuf + vb * kVBytes + 8192, &map_v, &sm.v_ready[vb], 64, row, pair);
                 }
                 // landmark row(s) (keys 64 .. 64 + per - 1) of both K-blocks: the buffer is free (its previous
                 // user's MMAs are done) and TMA never writes these rows.  V stays as TMA writes it (keys x dims):
-                // the second MMA reads it as an MN-major operand; keys past the end of the sequence hold other
-                // rows' data (or TMA zero fill) and meet probabilities of 0.
+                // the second MMA reads it as an MN-major operand; keys past the call's last token are zeros (make_kv_map).
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
                     const int x = lane + 32 * r, pc = x & 15;
@@ -532,11 +531,11 @@ prefill_attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
                     if (t + x >= hi || !ok) break;
                     const bool first = !same(rec[x], prev), last = !same(rec[x], rec[x + 1]);
                     if (first && lane == 0) {                              // some ten tiles ahead of their use: K and V into L2
-                        const int row = rec[x].x * s.T + rec[x].y * kS;
-                        tma_prefetch_l2_2d(&map_k, 0, row);
-                        tma_prefetch_l2_2d(&map_k, 64, row);
-                        tma_prefetch_l2_2d(&map_v, 0, row);
-                        tma_prefetch_l2_2d(&map_v, 64, row);
+                        const int row = rec[x].y * kS, pair = rec[x].x;
+                        tma_prefetch_l2_3d(&map_k, 0, row, pair);
+                        tma_prefetch_l2_3d(&map_k, 64, row, pair);
+                        tma_prefetch_l2_3d(&map_v, 0, row, pair);
+                        tma_prefetch_l2_3d(&map_v, 64, row, pair);
                     }
                     // The K buffer of a run is free when the score MMAs of the run's last tile of EITHER parity are done (the
                     // two parities have an issuer each): those two tiles arrive once each on k_empty, a run of one tile twice.

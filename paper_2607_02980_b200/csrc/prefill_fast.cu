@@ -833,8 +833,7 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
 
     // K, V: boxes of 64 dims x 64 keys; partial outputs: boxes of 64 dims x 32 rows (one epilogue warp's rows)
     CUtensorMap map_k, map_v, map_lm, map_o;
-    const uint64_t kv_rows = static_cast<uint64_t>(pairs) * s.T;
-    if (!make_bf16_2d_map(&map_k, t.k, kv_rows, kD, 64, kS) || !make_bf16_2d_map(&map_v, t.v, kv_rows, kD, 64, kS) ||
+    if (!make_kv_map(&map_k, t.k, pairs, s.T, s.pos0 + s.R, kD, 64, kS) || !make_kv_map(&map_v, t.v, pairs, s.T, s.pos0 + s.R, kD, 64, kS) ||
         !make_bf16_2d_map(&map_lm, t.landmarks, static_cast<uint64_t>(pairs) * s.C, kD, 64, kS) ||
         !make_bf16_2d_map(&map_o, a.obuf, static_cast<uint64_t>(p.obuf_tiles) * a.tile_tok * kG, kD, 64, 32))
         return HILS_ERR_CUDA;

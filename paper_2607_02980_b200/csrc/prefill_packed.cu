@@ -174,14 +174,14 @@ prefill_packed_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                     if (it >= kStages) ok = mbar_wait(&sm.empty[st], ((it / kStages) - 1) & 1);
                     if (!ok) break;
                     const int c = item_chunk(j);
-                    const int row = pair * s.T + c * kS;
+                    const int row = c * kS;
                     uint8_t* dst = ring + st * kStride;
                     const bool selected = j >= n_local;
                     mbar_expect_tx(&sm.full[st], 2 * kS * kD * 2 + (selected ? kLmBytes : 0));
-                    tma_load_2d(dst, &map_k, &sm.full[st], 0, row);
-                    tma_load_2d(dst + 8192, &map_k, &sm.full[st], 64, row);
-                    tma_load_2d(dst + 16384, &map_v, &sm.full[st], 0, row);
-                    tma_load_2d(dst + 24576, &map_v, &sm.full[st], 64, row);
+                    tma_load_3d(dst, &map_k, &sm.full[st], 0, row, pair);
+                    tma_load_3d(dst + 8192, &map_k, &sm.full[st], 64, row, pair);
+                    tma_load_3d(dst + 16384, &map_v, &sm.full[st], 0, row, pair);
+                    tma_load_3d(dst + 24576, &map_v, &sm.full[st], 64, row, pair);
                     if (selected)
                         bulk_load(dst + 32768, a.lm + (static_cast<long long>(pair) * s.C + c) * kD, kLmBytes, &sm.full[st]);
                 }
@@ -358,8 +358,7 @@ int launch_prefill_packed(const Shape& s, const Tensors& t, cudaStream_t stream)
     if (rc < 0) return rc;
     trace_mark("prefill_select", stream);
     CUtensorMap map_k, map_v;
-    const uint64_t kv_rows = static_cast<uint64_t>(pairs) * s.T;
-    if (!make_bf16_2d_map(&map_k, t.k, kv_rows, kD, 64, kS) || !make_bf16_2d_map(&map_v, t.v, kv_rows, kD, 64, kS))
+    if (!make_kv_map(&map_k, t.k, pairs, s.T, s.pos0 + s.R, kD, 64, kS) || !make_kv_map(&map_v, t.v, pairs, s.T, s.pos0 + s.R, kD, 64, kS))
         return HILS_ERR_CUDA;
     const size_t smem = kStages * (kStageBytes + 768) + sizeof(PkSmem) + 1024;
     static PerDeviceOnce attr_once;

@@ -403,21 +403,21 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                     const uint32_t st = g % kStages;
                     const int c = base + (sm.list[ln][i] & 0xffff);
                     if (g >= kStages && !wait(&sm.kv_empty[st], ((g / kStages) - 1) & 1)) return;
-                    const int row = pair * s.T + c * kS;
+                    const int row = c * kS;
                     // chunks left of every token's window have a landmark row (the others' score column is not used)
                     const bool lm = c < s.C;
                     uint8_t* kd = kbuf + st * kKBytes;
                     mbar_expect_tx(&sm.kv_full[st], 16384 + kVBytes + (lm ? 256 : 0));
-                    tma_load_2d(kd, &map_k, &sm.kv_full[st], 0, row);
-                    tma_load_2d(kd + kNS * 128, &map_k, &sm.kv_full[st], 64, row);
+                    tma_load_3d(kd, &map_k, &sm.kv_full[st], 0, row, pair);
+                    tma_load_3d(kd + kNS * 128, &map_k, &sm.kv_full[st], 64, row, pair);
                     if (lm) {
                         // row 64: its 16-byte pieces stay in place under the swizzle (64 mod 8 = 0)
                         const __nv_bfloat16* src = a.lm + ((static_cast<long long>(b) * s.Hl + gk) * s.C + c) * kD;
                         bulk_load(kd + 64 * 128, src, 128, &sm.kv_full[st]);
                         bulk_load(kd + kNS * 128 + 64 * 128, src + 64, 128, &sm.kv_full[st]);
                     }
-                    tma_load_2d(vbuf + st * kVBytes, &map_v, &sm.kv_full[st], 0, row);
-                    tma_load_2d(vbuf + st * kVBytes + 8192, &map_v, &sm.kv_full[st], 64, row);
+                    tma_load_3d(vbuf + st * kVBytes, &map_v, &sm.kv_full[st], 0, row, pair);
+                    tma_load_3d(vbuf + st * kVBytes + 8192, &map_v, &sm.kv_full[st], 64, row, pair);
                     ++g;
                 };
                 // the first chunks before the queries: their buffers are free before the last unit's rows have been written
@@ -567,10 +567,10 @@ bool prefill_local_query(const Shape& s, int first) {
 }
 
 int launch_prefill_query_tc(const Shape& s, const Tensors& t, int first, int n_tok, int local, int write_sel, cudaStream_t stream) {
-    const uint64_t kv_rows = static_cast<uint64_t>(s.B) * s.Hkv * s.T, q_rows = static_cast<uint64_t>(s.B) * s.Hq * s.R;
+    const uint64_t pairs = static_cast<uint64_t>(s.B) * s.Hkv, q_rows = static_cast<uint64_t>(s.B) * s.Hq * s.R;
     CUtensorMap map_q, map_k, map_v, map_out;
-    if (!make_bf16_2d_map(&map_q, t.q, q_rows, kD, 64, kTok) || !make_bf16_2d_map(&map_k, t.k, kv_rows, kD, 64, kS) ||
-        !make_bf16_2d_map(&map_v, t.v, kv_rows, kD, 64, kS) || !make_bf16_2d_map(&map_out, t.out, q_rows, kD, 64, kTok))
+    if (!make_bf16_2d_map(&map_q, t.q, q_rows, kD, 64, kTok) || !make_kv_map(&map_k, t.k, pairs, s.T, s.pos0 + s.R, kD, 64, kS) ||
+        !make_kv_map(&map_v, t.v, pairs, s.T, s.pos0 + s.R, kD, 64, kS) || !make_bf16_2d_map(&map_out, t.out, q_rows, kD, 64, kTok))
         return HILS_ERR_CUDA;
     const size_t smem = kStages * (kKBytes + kVBytes) + 2 * kQBytes + sizeof(QmSmem) + 1024;
     static PerDeviceOnce once;

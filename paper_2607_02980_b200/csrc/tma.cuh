@@ -141,8 +141,8 @@ __device__ __forceinline__ void tma_store_2d(const void* map, const void* smem_s
 }
 
 // Brings one box of a tiled tensor into L2 without touching shared memory.
-__device__ __forceinline__ void tma_prefetch_l2_2d(const void* map, int x, int y) {
-    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y) : "memory");
+__device__ __forceinline__ void tma_prefetch_l2_3d(const void* map, int x, int y, int z) {
+    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(map), "r"(x), "r"(y), "r"(z) : "memory");
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
@@ -481,17 +481,16 @@ inline bool make_bf16_2d_map(CUtensorMap* map, const void* base, uint64_t rows, 
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-
-// bf16 tensor [n2, n1, cols] (cols contiguous, pitches of cols and n1 * cols elements) -> map with box
-// {box_cols, box1, box2} and the 128-byte swizzle (box_cols * 2 bytes must be 128): the box's box1 * box2 rows land
-// as consecutive 128-byte rows in shared memory.
-inline bool make_bf16_3d_map(CUtensorMap* map, const void* base, uint64_t n2, uint64_t n1, uint64_t cols,
-                             uint32_t box_cols, uint32_t box1, uint32_t box2) {
+// K or V of every (sequence, KV head), [pairs, T, cols] bf16 -> boxes of box_cols x box_rows of one pair.  Rows from n on read as
+// zeros: a tile that reaches past a call's last token would multiply whatever the cache holds there, or the next pair's
+// rows, with probabilities of 0, and 0 x NaN is NaN.
+inline bool make_kv_map(CUtensorMap* map, const void* base, uint64_t pairs, uint64_t T, uint64_t n, uint64_t cols,
+                        uint32_t box_cols, uint32_t box_rows) {
     EncodeTiledFn fn = get_encode_tiled();
     if (!fn) return false;
-    cuuint64_t dims[3] = {cols, n1, n2};
-    cuuint64_t strides[2] = {cols * 2, n1 * cols * 2};
-    cuuint32_t box[3] = {box_cols, box1, box2};
+    cuuint64_t dims[3] = {cols, n, pairs};
+    cuuint64_t strides[2] = {cols * 2, T * cols * 2};
+    cuuint32_t box[3] = {box_cols, box_rows, 1};
     cuuint32_t estr[3] = {1, 1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,

@@ -53,6 +53,10 @@ def test_drafts_that_straddle_a_chunk(B, M, W, G, value):
     ("f32", "generic", 64, 1, 300, 200, 1),
     ("f32", "generic", 48, 2, 100, 333, 100),
     ("bf16", "generic", 64, 1, 300, 200, 1),
+    ("bf16", "fast", 64, 1, 300, 200, 1),              # query-major
+    ("bf16", "fast", 64, 8, 3000, 1300, 512),          # chunk-major, local windows query-major
+    ("bf16", "fast", 64, 1, 3000, 3300, 1),            # chunk-major
+    ("bf16", "packed", 64, 1, 304, 200, 1),
 ])
 def test_slice_that_ends_inside_a_chunk(dtype, impl, S, Hkv, pos0, L, W):
     cfg = wl.HilsConfig("tail", "prefill", 2, 4 * Hkv, Hkv, (pos0 + L + 2 * S) // S * S, 128, S, 4, dtype, 730 + L, window=W)
@@ -71,3 +75,39 @@ def test_slice_that_ends_inside_a_chunk(dtype, impl, S, Hkv, pos0, L, W):
         ref = oracle.hils_rows(q, inp["k"], inp["v"], inp["landmarks"], None, S=S, K=4, W=W,
                                row_b=np.full(L, b, np.int32), row_qi=rows.astype(np.int32), row_pos=(pos0 + rows).astype(np.int64))
         check((out[b].transpose(0, 1), lse[b].T, sel[b].transpose(0, 1)), ref, 4, dtype)
+
+
+@pytest.mark.parametrize("impl,L", [("fast", 900), ("fast", 3001), ("packed", 300), ("generic", 300)])
+def test_a_sequence_is_not_spoilt_by_the_next_one(impl, L):
+    """A tile of the first sequence's last chunk reaches into the rows of the second."""
+    cfg = wl.HilsConfig("next", "prefill", 2, 4, 1, L, 128, 64, 16, "bf16", 760 + L)
+    g = wl.make_prefill_inputs(cfg, DEV)
+    run = lambda: hils.hils_prefill(g["q"], g["k"], g["v"], g["landmarks"], 64, 16, impl=impl)
+    clean = run()
+    for n in ("q", "k", "v"):
+        g[n][1] = float("nan")
+    got = run()
+    torch.cuda.synchronize()
+    for x, y in zip(got, clean):
+        assert torch.equal(x[0], y[0])
+
+
+@pytest.mark.parametrize("L", [300, 3001])
+def test_gradients_of_a_sequence_that_ends_inside_a_chunk(L):
+    """Caches longer than the sequence: the gradients are those of caches cut to it, and zero behind it."""
+    cfg = wl.HilsConfig("tail", "prefill", 2, 8, 2, L, 128, 64, 8, "bf16", 780 + L)
+    t = wl.make_prefill_inputs(cfg, DEV)
+    dout = torch.randn(t["q"].shape, device=DEV, generator=torch.Generator(device=DEV).manual_seed(L)).to(torch.bfloat16)
+    def grads(k, v):
+        leaves = [x.clone().requires_grad_(True) for x in (t["q"], k, v, t["landmarks"])]
+        out, lse, sel = hils.hils_attention(*leaves, 64, 8)
+        return (out.detach(), lse.detach()) + torch.autograd.grad(out, leaves, dout)
+    tail = torch.full((2, 2, 100, 128), float("nan"), dtype=torch.bfloat16, device=DEV)
+    want = grads(t["k"], t["v"])
+    got = grads(torch.cat([t["k"], tail], dim=2), torch.cat([t["v"], tail], dim=2))
+    for i, (x, y) in enumerate(zip(got, want)):
+        if i in (3, 4):                                        # dk, dv
+            assert (x[:, :, L:] == 0).all()
+            x = x[:, :, :L]
+        # (sums in another order: the last bit of a bf16 gradient)
+        assert (x.float() - y.float()).norm() <= 4e-3 * y.float().norm()
