@@ -60,7 +60,7 @@ typedef enum {
     HILS_ERR_INVALID_ARG = -1,   /* null pointer, non-positive size, Hq % Hkv != 0, ...           */
     HILS_ERR_UNSUPPORTED = -2,   /* a shape or option this build has no kernel for                */
     HILS_ERR_ALIGNMENT = -3,     /* a base pointer is not 16-byte aligned                         */
-    HILS_ERR_WORKSPACE = -4,     /* workspace missing or smaller than hils_workspace_bytes()      */
+    HILS_ERR_WORKSPACE = -4,     /* workspace missing or too small (see hils_workspace_bytes)     */
     HILS_ERR_CUDA = -5,          /* a CUDA runtime call failed (launch, copy, attribute)          */
     HILS_ERR_DEVICE_TIMEOUT = -6,/* a bounded device-side wait ran out                            */
     HILS_ERR_DEVICE_INDEX = -7   /* a kernel met a chunk id outside its valid range               */
@@ -94,12 +94,16 @@ typedef struct hils_params {
     int32_t impl;        /* hils_impl                                                               */
 } hils_params;
 
-/* Bytes of device scratch hils_prefill (is_decode = 0) or hils_decode (is_decode = 1) needs for
+/* Bytes of device scratch with which hils_prefill (is_decode = 0) or hils_decode (is_decode = 1) is fastest for
  * these parameters.  Returns 0 if the parameters are invalid.  The first 256 bytes hold the
  * device status word; the caller must zero them once after allocation.
  * Prefill on the tensor-core path keeps per-(token, retrieved chunk) partial outputs in the workspace:
- * (K + window chunks) * Hq * d * 2 bytes per token, for all tokens of the call while that is at most 4 GiB
- * (2.3 GB for 16K tokens, 32 heads, K = 16), else for one block of 4096-8192 tokens at a time. */
+ * (K + window chunks) * Hq * d * 2 bytes per token (the window's chunks not where it goes query-major), for all tokens of
+ * the call while that is at most 5 GiB (2.3 GB for 16K tokens, 32 heads, K = 16), else for one block of 4096-16384 tokens at
+ * a time (5.3 GB for 128K tokens, 32 heads, K = 32).  fp32 prefill on short sequences keeps fp32 ones (up to 256 MiB).
+ * Prefill also runs in less: in a smaller workspace it takes blocks of down to 2048 tokens (fp32: kernels that need none), with
+ * the same results and more time; HILS_ERR_WORKSPACE only where that does not fit either.  The same goes for
+ * hils_prefill_at, hils_prefill_routed and the arena of hils_prefill_host; decode and backward take what is reported. */
 size_t hils_workspace_bytes(const hils_params* params, int is_decode);
 
 /* Prefill: Eq. (surrogate top-k) + Eq. (HiLS weights) (GQA form: App. C) for all L positions of

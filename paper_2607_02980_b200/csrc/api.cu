@@ -118,11 +118,19 @@ int pick_path(const Shape& s, const hils_params* p, Path* path) {
     return HILS_OK;
 }
 
+// Scratch behind the status block: what the fastest kernels take, and the least that a call runs with.
 size_t scratch_bytes(const Shape& s, Path path, int dtype) {
     switch (path) {
         case Path::DecodeFast: return decode_fast_scratch_bytes(s);
         case Path::PrefillFast: return prefill_fast_scratch_bytes(s);
         case Path::Generic: return generic_scratch_bytes(s, dtype);
+        default: return 0;
+    }
+}
+size_t least_scratch_bytes(const Shape& s, Path path) {
+    switch (path) {
+        case Path::DecodeFast: return decode_fast_scratch_bytes(s);
+        case Path::PrefillFast: return prefill_fast_scratch_bytes(s, true);
         default: return 0;
     }
 }
@@ -158,7 +166,7 @@ int run(const hils_params* p, int is_decode, const void* q, const void* k, const
         if (num_pages < 1 || static_cast<long long>(num_pages) * s.Hkv * s.S >= (1ll << 31)) return HILS_ERR_INVALID_ARG;
         if (reinterpret_cast<uintptr_t>(block_table) & 3u) return HILS_ERR_ALIGNMENT;
     }
-    const size_t need = kStatusBytes + scratch_bytes(s, path, p->dtype);
+    const size_t need = kStatusBytes + least_scratch_bytes(s, path);
     if (!ws || ws_bytes < need) return HILS_ERR_WORKSPACE;
     if (!aligned16(ws)) return HILS_ERR_ALIGNMENT;
     Tensors t{q, k, v, lm, bias, seq_lens, out, lse, sel, static_cast<int*>(ws),
@@ -186,7 +194,9 @@ struct ArenaLayout {
     size_t q_b, kv_b, lm_b, bias_b, seq_b, out_b, lse_b, sel_b, ws_b;
 };
 
-int arena_layout(const hils_params* p, int is_decode, ArenaLayout* a) {
+// (have: bytes of the caller's arena; where they are fewer than the fastest kernels' workspace asks for, the workspace shrinks as
+// far as a call can do with)
+int arena_layout(const hils_params* p, int is_decode, ArenaLayout* a, size_t have = ~static_cast<size_t>(0)) {
     Shape s;
     int rc = make_shape(p, is_decode, &s);
     if (rc != HILS_OK) return rc;
@@ -203,11 +213,23 @@ int arena_layout(const hils_params* p, int is_decode, ArenaLayout* a) {
     a->ws_b = hils_workspace_bytes(p, is_decode);
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
-    a->ws = take(a->ws_b);        // first, so that the arena's head is the status word
-    a->q = take(a->q_b); a->k = take(a->kv_b); a->v = take(a->kv_b); a->lm = take(a->lm_b);
-    a->bias = take(a->bias_b); a->seq = take(a->seq_b); a->out = take(a->out_b);
-    a->lse = take(a->lse_b); a->sel = take(a->sel_b);
-    a->total = off;
+    auto lay = [&] {
+        off = 0;
+        a->ws = take(a->ws_b);    // first, so that the arena's head is the status word
+        a->q = take(a->q_b); a->k = take(a->kv_b); a->v = take(a->kv_b); a->lm = take(a->lm_b);
+        a->bias = take(a->bias_b); a->seq = take(a->seq_b); a->out = take(a->out_b);
+        a->lse = take(a->lse_b); a->sel = take(a->sel_b);
+        a->total = off;
+    };
+    lay();
+    Path path;
+    if (a->total > have && pick_path(s, p, &path) == HILS_OK) {
+        const size_t least = kStatusBytes + align_up(least_scratch_bytes(s, path), 256), over = align_up(a->total - have, 256);
+        if (a->ws_b >= least + over) {
+            a->ws_b -= over;
+            lay();
+        }
+    }
     return HILS_OK;
 }
 
@@ -360,7 +382,7 @@ int run_host(const hils_params* p, int is_decode, const void* q, const void* k, 
              const float* bias, const int32_t* seq_lens, void* out, float* lse, int32_t* sel, void* arena,
              size_t arena_bytes, void* stream_v) {
     ArenaLayout a;
-    int rc = arena_layout(p, is_decode, &a);
+    int rc = arena_layout(p, is_decode, &a, arena_bytes);
     if (rc != HILS_OK) return rc;
     if (!q || !k || !v || !lm || !out || !lse || !sel || (is_decode && !seq_lens)) return HILS_ERR_INVALID_ARG;
     if (!arena || arena_bytes < a.total) return HILS_ERR_WORKSPACE;

@@ -676,7 +676,7 @@ int launch_chunk_major(const GArgs& a, void* scratch, cudaStream_t stream) {
 }
 
 template <typename T, int D, bool X>
-int launch_dim(const GArgs& a, int dtype, void* scratch, cudaStream_t stream) {
+int launch_dim(const GArgs& a, void* scratch, cudaStream_t stream) {
     const Shape& s = a.s;
     const long long sel_warps = static_cast<long long>(s.B) * s.Hkv * s.R;
     const long long rows = static_cast<long long>(s.B) * s.Hq * s.R;
@@ -688,7 +688,7 @@ int launch_dim(const GArgs& a, int dtype, void* scratch, cudaStream_t stream) {
     else generic_select_kernel<T, D, X, 4><<<sel_blocks, kWarpsPerBlock * 32, 0, stream>>>(a);
     if (cudaGetLastError() != cudaSuccess) return HILS_ERR_CUDA;
     trace_mark("generic_select", stream);
-    if (chunk_major(s, dtype)) return s.d == 64 ? launch_chunk_major<64>(a, scratch, stream) : launch_chunk_major<128>(a, scratch, stream);
+    if (scratch) return s.d == 64 ? launch_chunk_major<64>(a, scratch, stream) : launch_chunk_major<128>(a, scratch, stream);
     // a warp per item of the row, at most eight
     const long long items = static_cast<long long>(s.K) + (s.W + s.S - 2) / 64 + 1;
     const unsigned warps = static_cast<unsigned>(items < kAttWarps ? items : kAttWarps);
@@ -698,12 +698,13 @@ int launch_dim(const GArgs& a, int dtype, void* scratch, cudaStream_t stream) {
     return 2;
 }
 
+// (scratch: for the chunk-major kernels; none where they do not apply)
 template <typename T>
-int launch_typed(const GArgs& a, int dtype, void* scratch, cudaStream_t stream) {
-    if (a.s.d == 64) return launch_dim<T, 64, true>(a, dtype, scratch, stream);
-    if (a.s.d == 128) return launch_dim<T, 128, true>(a, dtype, scratch, stream);
-    if (a.s.d < 128) return launch_dim<T, 128, false>(a, dtype, scratch, stream);
-    return launch_dim<T, 256, false>(a, dtype, scratch, stream);
+int launch_typed(const GArgs& a, void* scratch, cudaStream_t stream) {
+    if (a.s.d == 64) return launch_dim<T, 64, true>(a, scratch, stream);
+    if (a.s.d == 128) return launch_dim<T, 128, true>(a, scratch, stream);
+    if (a.s.d < 128) return launch_dim<T, 128, false>(a, scratch, stream);
+    return launch_dim<T, 256, false>(a, scratch, stream);
 }
 
 }  // namespace
@@ -721,8 +722,10 @@ size_t generic_scratch_bytes(const Shape& s, int dtype) {
 int launch_generic(const Shape& s, int dtype, const Tensors& t, cudaStream_t stream) {
     if (!generic_supports(s)) return HILS_ERR_UNSUPPORTED;
     GArgs a{s, t.q, t.q_route ? t.q_route : t.q, t.k, t.v, t.landmarks, t.bias, t.seq_lens, t.out, t.lse, t.sel_idx, t.status};
-    if (dtype == HILS_F32) return launch_typed<float>(a, dtype, t.scratch, stream);
-    return launch_typed<__nv_bfloat16>(a, dtype, t.scratch, stream);
+    // a workspace without room for the chunk-major kernels' partial outputs: the row kernel
+    void* scratch = chunk_major(s, dtype) && t.scratch_bytes >= generic_scratch_bytes(s, dtype) ? t.scratch : nullptr;
+    if (dtype == HILS_F32) return launch_typed<float>(a, scratch, stream);
+    return launch_typed<__nv_bfloat16>(a, scratch, stream);
 }
 
 }  // namespace hils

@@ -152,6 +152,7 @@ int launch_prefill_packed(const Shape& s, const Tensors& t, cudaStream_t stream)
 
 int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream);
 bool prefill_fast_supports(const Shape& s, int dtype);
-size_t prefill_fast_scratch_bytes(const Shape& s);
+// (least: what a call has to have, with smaller query blocks than are fastest)
+size_t prefill_fast_scratch_bytes(const Shape& s, bool least = false);
 
 }  // namespace hils

@@ -25,6 +25,7 @@ constexpr int kD = 128;
 constexpr int kS = 64;
 constexpr int kG = 4;
 constexpr int kQBMin = 4096, kQBMax = 16384;  // tokens per pass of the invert/attend/fuse phases
+constexpr int kQBLeast = 2048;               // (in a workspace that holds no more)
 constexpr size_t kObufBytes = 5ull << 30;    // partial outputs that a call keeps at a time (at least those of kQBMin tokens)
 constexpr int kSelStages = 3;
 constexpr int kSelStageBytes = kS * kD * 2;  // 64 landmark rows
@@ -641,8 +642,9 @@ struct Plan {
         total, obuf_tiles;
 };
 
-// (nl: slots of a token's local window, 0 where it goes query-major)
-Plan make_plan(const Shape& s, int qb_fixed, int t0, int nl) {
+// (nl: slots of a token's local window, 0 where it goes query-major; qb_fixed: tokens per query block, 0 = the fastest;
+// at_once: whether the partial outputs of all blocks may be kept)
+Plan make_plan(const Shape& s, int qb_fixed, int t0, int nl, bool at_once = true) {
     Plan p;
     const int R = s.R - t0;                      // tokens of the chunk-major part
     const size_t pairs = static_cast<size_t>(s.B) * s.Hkv;
@@ -670,7 +672,7 @@ Plan make_plan(const Shape& s, int qb_fixed, int t0, int nl) {
     p.max_tiles = static_cast<int>(all_tiles);
     p.max_blk_tiles = static_cast<int>(max_blk);
     size_t off = 0;
-    auto take = [&](size_t bytes) { size_t o = off; off = (off + bytes + 255) / 256 * 256; return o; };
+    auto take = [&](size_t bytes, size_t align = 16) { size_t o = (off + align - 1) / align * align; off = o + bytes; return o; };
     p.off_cnt = take(sizeof(int) * nblocks * pairs * nc);
     p.off_cursor = take(sizeof(int) * nblocks * pairs * nc);
     p.off_ntiles = take(sizeof(int) * (nblocks + 1));
@@ -678,18 +680,30 @@ Plan make_plan(const Shape& s, int qb_fixed, int t0, int nl) {
     p.off_ptiles = take(sizeof(int) * (nblocks * pairs + 1));
     p.off_seg = take(sizeof(int) * ((nblocks * pairs * nc + kSegLists - 1) / kSegLists));
     p.off_off = take(sizeof(int) * nblocks * pairs * nc);
-    p.off_entries = take(sizeof(int) * all_tiles * tt);
+    p.off_entries = take(sizeof(int) * all_tiles * tt, 256);
     p.off_epos = take(sizeof(int) * pairs * s.R * (s.K + nl));
     p.off_tiles = take(sizeof(int4) * all_tiles);
     // Partial outputs of all query blocks at once where they fit: the fusion then runs as one launch
     // over the whole call instead of one per block (each launch pays its ramp and its last wave).
-    p.whole = (nblocks > 1 && all_tiles * tt * kG * kD * sizeof(__nv_bfloat16) <= kObufBytes) ? 1 : 0;
+    p.whole = (at_once && nblocks > 1 && all_tiles * tt * kG * kD * sizeof(__nv_bfloat16) <= kObufBytes) ? 1 : 0;
     const size_t obuf_tiles = p.whole ? all_tiles : max_blk;
     p.obuf_tiles = obuf_tiles;
-    p.off_obuf = take(sizeof(__nv_bfloat16) * obuf_tiles * tt * kG * kD);
+    p.off_obuf = take(sizeof(__nv_bfloat16) * obuf_tiles * tt * kG * kD, 256);
     p.off_lam = take(sizeof(float) * obuf_tiles * tt * kG);
     p.total = off;
     return p;
+}
+// The fastest plan that `bytes` of workspace hold (128K tokens, K = 32: 18.5 ms with the 5.3 GB of blocks of 16384 tokens, 19.4 with
+// the 2.8 GB of 8192, 20.0 with 1.6 GB); the smallest one if none does.
+Plan fitting_plan(const Shape& s, int t0, int nl, size_t bytes) {
+    Plan least = make_plan(s, 0, t0, nl);
+    if (least.total <= bytes) return least;
+    for (int qb = kQBMax; qb >= kQBLeast; qb /= 2) {
+        const Plan p = make_plan(s, qb, t0, nl, false);
+        if (p.total <= bytes) return p;
+        if (p.total < least.total) least = p;
+    }
+    return least;
 }
 
 }  // namespace
@@ -706,11 +720,12 @@ bool prefill_fast_supports(const Shape& s, int dtype) {
            static_cast<long long>(s.B) * s.Hkv * s.R * (s.K + max_local_slots(s.W)) < (1ll << 31);
 }
 
-size_t prefill_fast_scratch_bytes(const Shape& s) {
+size_t prefill_fast_scratch_bytes(const Shape& s, bool least) {
     // (with a routing query nothing goes query-major; and fewer entries may take more scratch, where they just fit at once)
+    const size_t bytes = least ? 0 : ~static_cast<size_t>(0);
     const int t0 = prefill_query_tokens(s), nl = max_local_slots(s.W);
-    const size_t all = make_plan(s, 0, 0, nl).total;
-    const size_t rest = t0 < s.R ? make_plan(s, 0, t0, prefill_local_query(s, t0) ? 0 : nl).total : 0;
+    const size_t all = fitting_plan(s, 0, nl, bytes).total;
+    const size_t rest = t0 < s.R ? fitting_plan(s, t0, prefill_local_query(s, t0) ? 0 : nl, bytes).total : 0;
     return all > rest ? all : rest;
 }
 
@@ -794,7 +809,7 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
     const int t0 = n_qm;
     const bool local_qm = !t.q_route && t0 < s.R && prefill_local_query(s, t0);
     const int nl = local_qm ? 0 : max_local_slots(s.W);
-    const Plan p = make_plan(s, 0, t0 < s.R ? t0 : 0, nl);
+    const Plan p = fitting_plan(s, t0 < s.R ? t0 : 0, nl, t.scratch_bytes);
     if (t.scratch_bytes < p.total) return HILS_ERR_WORKSPACE;
     const int pairs = s.B * s.Hkv;
     char* sc = static_cast<char*>(t.scratch);
