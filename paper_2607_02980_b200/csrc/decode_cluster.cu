@@ -113,7 +113,7 @@ struct CSmem {
     unsigned long long own[TG][kCand];         // this CTA's candidates (score key, ~chunk id)
     unsigned long long all[TG][kCand];         // the cluster's
     unsigned kmin, kmax;                       // span of this CTA's scores (ordered keys)
-    float edge[TG];                            // published: score that ceil(K / CTAs) of this CTA's candidates reach
+    float edge[TG];                            // published: score that this CTA's share of K of its candidates reach
     unsigned long long thr[TG];                // candidates from this key on are collected
     int cnt[TG];                               // this CTA's candidates collected
     int start[TG][kMaxCluster + 1];            // positions of the CTAs' candidates in `all`
@@ -367,11 +367,10 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
             n_rank = 1;
         } else {
             __syncthreads();
-            // A score that ceil(K / CS) of this CTA's candidates reach, off a histogram with bins of equal width in the
+            // A score that this CTA's share of K of its candidates reach, off a histogram with bins of equal width in the
             // score (the bins of a radix digit are equal in the exponent, and most scores share two or three exponents).
             const float lo = key_to_float(sm.kmin), inv = static_cast<float>(kBins) / (key_to_float(sm.kmax) - lo);
             const bool cut = inv > 0.f && inv < INFINITY;              // (no span: every candidate is collected)
-            const int want = (K + CS - 1) >> a.lcs;
 #pragma unroll 1
             for (int m = m_first; m < ntok; m += m_step) {
                 if (sm.nc[m] <= K || !cut) continue;
@@ -384,7 +383,14 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
             __syncthreads();
 #pragma unroll 1
             for (int m = warp; m < ntok; m += NW) {
-                // walk the bins from the top until the running count reaches `want`
+                // walk the bins from the top until the running count reaches `want` (all of them reach the lowest score)
+                // This CTA's share of K: equal ones where each CTA holds a full tile of candidates.  Where there are fewer, those that
+                // hold one share K (rounded up, plus one), and the others publish +inf: an empty CTA would leave no threshold, and
+                // the best of a handful is a poor one (one sequence of 17K-29K tokens, 8 CTAs and 4-7 full tiles, K = 32: 28.2 us
+                // by the radix selection below, 13.9 this way).
+                const int full = sm.nc[m] >> 6;
+                int want = (K + CS - 1) >> a.lcs;
+                if (full < CS && K <= 64 * full) want = rank < full ? static_cast<int>(__fdividef(static_cast<float>(K), static_cast<float>(full))) + 1 : 0;
                 constexpr int kPer = kBins / 32;
                 const int* h = sm.hist[m] + kBins - kPer * (lane + 1);      // this lane's bins, the top one last
                 int mine = 0;
@@ -399,7 +405,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                     const int nn = __shfl_up_sync(kFullMask, inc, o);
                     if (lane >= o) inc += nn;
                 }
-                if (lane == 0) sm.edge[m] = -INFINITY;
+                if (lane == 0) sm.edge[m] = want > 0 ? lo : INFINITY;
                 __syncwarp();
                 int cum = inc - mine;
                 if (cum < want && inc >= want) {               // at most one lane

@@ -95,3 +95,15 @@ def test_invalid_lengths_and_pages_set_the_status_and_leave_the_rest_alone():
                                            64, 16, workspace=ws)
     assert hils.poll_status(ws) == -7
     assert torch.equal(sel, good[2]) and torch.equal(out[1:], good[0][1:])
+
+
+@pytest.mark.parametrize("n,K,W", [(258, 32, 1), (300, 32, 1), (321, 64, 1), (449, 32, 1), (330, 16, 512), (150, 128, 1), (129, 127, 1)])
+def test_lists_that_leave_some_ctas_few_candidates_or_none(n, K, W):
+    """One sequence: eight CTAs per KV head, fewer full tiles of 64 candidates than that."""
+    T = 64 * (n + (W + 62) // 64) + 5
+    cfg = wl.HilsConfig("few", "decode", 1, 32, 8, T, 128, 64, K, "bf16", 980 + n, n_needles=2, window=W)
+    inp = wl.make_decode_inputs(cfg, "cpu")
+    g = {x: t.to(DEV) for x, t in inp.items()}
+    got = hils.hils_decode(g["q"], g["k"], g["v"], g["landmarks"], g["seq_lens"], 64, K, window=W)
+    torch.cuda.synchronize()
+    check_decode(cfg, inp, *got, W=W)
