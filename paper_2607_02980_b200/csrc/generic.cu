@@ -436,9 +436,6 @@ constexpr int kRowBlock = 32;                // (early chunks are attended by ev
 constexpr int kChunkWarps = 4;
 static_assert(kRowBlock <= kChunkWarps * 32, "one row per thread in the look-through");
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
 
 // Slots of a row: the selected chunks 0 .. K - 1, then the chunks of its local window.
 __host__ __device__ inline int chunk_slots(const Shape& s) { return s.K + (s.W + s.S - 2) / s.S + 1; }

@@ -35,9 +35,6 @@ __device__ __forceinline__ float elem_f32(float x) { return x; }
 __device__ __forceinline__ float elem_f32(__nv_bfloat16 x) { return __bfloat162float(x); }
 __device__ __forceinline__ void elem_set(float& dst, float x) { dst = x; }
 __device__ __forceinline__ void elem_set(__nv_bfloat16& dst, float x) { dst = __float2bfloat16_rn(x); }
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
 
 // D = head dimension (32, 64, 128, 256).  Shared memory per warp: S rows of D * sizeof(T) + 16 bytes, D floats
 // for the scaled query and kMaxS floats for the probabilities.
@@ -156,11 +153,6 @@ __global__ void landmark_summary_kernel(const LArgs a) {
 constexpr int kTcWarps = 14;
 constexpr int kTcTileBytes = 64 * 128 * 2;
 
-__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t x) {
-    uint32_t y;
-    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
-    return y;
-}
 
 __global__ void __launch_bounds__(kTcWarps * 32, 1)
 landmark_summary_tc_kernel(const __grid_constant__ CUtensorMap map_k, const LArgs a) {

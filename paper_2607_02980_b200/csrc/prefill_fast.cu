@@ -29,7 +29,6 @@ constexpr int kQBLeast = 2048;               // (in a workspace that holds no mo
 constexpr size_t kObufBytes = 5ull << 30;    // partial outputs that a call keeps at a time (at least those of kQBMin tokens)
 constexpr int kSelStages = 3;
 constexpr int kSelStageBytes = kS * kD * 2;  // 64 landmark rows
-constexpr float kLog2e = 1.4426950408889634f;
 
 struct PArgs {
     Shape s;
@@ -529,15 +528,15 @@ __global__ void __launch_bounds__(kFuseWarps * 32) prefill_fuse_kernel(const PAr
         lam[st][0] = v.x; lam[st][1] = v.y; lam[st][2] = v.z; lam[st][3] = v.w;
     }
     if (LOCAL_ROW && nrows == 0 && lane == 0) ev[0] = 0;          // (local branch alone: the loads below read a row that nobody uses)
-    // the first four rows are requested before the weights are worked out (their addresses need only the entries)
+    // (streaming loads: a partial row is read once.)  The first four rows are requested before the weights are worked out (their addresses need only the entries)
     __syncwarp();
     uint4 ra[4], rb[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         const int r = max(min(u, nrows - 1), 0);
         const __nv_bfloat16* row = a.obuf + static_cast<long long>(ev[r]) * kG * kD;
-        ra[u] = obuf_load(reinterpret_cast<const uint4*>(row + lane * 8));
-        rb[u] = obuf_load(reinterpret_cast<const uint4*>(row + 256 + lane * 8));
+        ra[u] = __ldcs(reinterpret_cast<const uint4*>(row + lane * 8));
+        rb[u] = __ldcs(reinterpret_cast<const uint4*>(row + 256 + lane * 8));
     }
     const int hA = lane >> 4, hB = 2 + (lane >> 4), piece = lane & 15;
     const long long rowA = (static_cast<long long>(b) * s.Hq + gk * kG + hA) * s.R + tok;
@@ -591,8 +590,8 @@ __global__ void __launch_bounds__(kFuseWarps * 32) prefill_fuse_kernel(const PAr
             for (int u = 0; u < 4; ++u) {
                 const int r = min(r0 + u, nrows - 1);
                 const __nv_bfloat16* row = a.obuf + static_cast<long long>(ev[r]) * kG * kD;
-                ra[u] = obuf_load(reinterpret_cast<const uint4*>(row + lane * 8));
-                rb[u] = obuf_load(reinterpret_cast<const uint4*>(row + 256 + lane * 8));
+                ra[u] = __ldcs(reinterpret_cast<const uint4*>(row + lane * 8));
+                rb[u] = __ldcs(reinterpret_cast<const uint4*>(row + 256 + lane * 8));
             }
         }
 #pragma unroll

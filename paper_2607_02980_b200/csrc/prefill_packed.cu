@@ -96,10 +96,6 @@ __device__ __forceinline__ void pv_tile16(const float (&p)[8][4], uint32_t vs_ad
     }
 }
 
-__device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, uint32_t bytes, uint64_t* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_u32(sdst)), "l"(gsrc), "r"(bytes), "r"(smem_u32(bar)) : "memory");
-}
 
 __global__ void __launch_bounds__(kThreads, 2)
 prefill_packed_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
@@ -114,7 +110,6 @@ prefill_packed_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     const int tiles_per_seq = (s.R + kM - 1) / kM;
     const int n_tiles = pairs * tiles_per_seq;
     const int K = s.K;
-    const int NL = (s.W - 1 + kS - 1) / kS + 1;         // chunks a local window can touch
 
     if (tid == 0) {
         for (int i = 0; i < kStages; ++i) { mbar_init(&sm.full[i], 1); mbar_init(&sm.empty[i], kWarps); }

@@ -41,7 +41,7 @@ constexpr int kStages = 4;
 constexpr int kMaxC = 160;                      // chunks a unit may see
 constexpr int kPCol = 96;                       // columns of a tile: scores 0..79, probabilities 96..127, output 128..255
 constexpr int kOCol = 128;
-constexpr int kMmaWarp = 8, kLoadWarp = 10, kListWarp = 11;
+constexpr int kMmaWarp = 8, kLoadWarp = 10;           // (and warp 11, the list)
 constexpr int kThreads = 12 * 32;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kRaise = 16.f;
@@ -75,11 +75,6 @@ struct QmSmem {
 };
 static_assert(kStages * (kKBytes + kVBytes) + 2 * kQBytes + sizeof(QmSmem) + 1024 <= 232448, "shared memory of the query-major kernel");
 
-__device__ __forceinline__ float ex2_approx(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 // 2^x of two values on the FMA pipes: x = n + f with f in [-1/2, 1/2] (Cody-Waite), a polynomial of degree 5 in f fitted
 // to the smallest relative error (1e-7), n added to the exponent.  A quarter of a row's exponentials goes this way: the
 // special-function unit takes 8 cycles per warp and exponential and is the busiest unit of the softmax warps.
@@ -96,10 +91,6 @@ __device__ __forceinline__ float2 ex2_fma(float2 x) {
     p = __ffma2_rn(p, f, make_float2(1.00000007f, 1.00000007f));
     return make_float2(__int_as_float(__float_as_int(p.x) + (__float_as_int(t.x) << 23)),
                        __int_as_float(__float_as_int(p.y) + (__float_as_int(t.y) << 23)));
-}
-__device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, uint32_t bytes, uint64_t* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_u32(sdst)), "l"(gsrc), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
