@@ -111,3 +111,19 @@ def test_gradients_of_a_sequence_that_ends_inside_a_chunk(L):
             x = x[:, :, :L]
         # (sums in another order: the last bit of a bf16 gradient)
         assert (x.float() - y.float()).norm() <= 4e-3 * y.float().norm()
+
+
+@pytest.mark.parametrize("K,impl,W,per_head,launches", [(16, "auto", 1, False, 1), (16, "auto", 200, False, 1), (8, "auto", 1, False, 3),
+                                                        (16, "auto", 65, True, 3), (8, "generic", 65, False, 2)])
+def test_decode_inside_a_chunk(K, impl, W, per_head, launches):
+    cfg = wl.HilsConfig("tail", "decode", 3, 8, 2, 64 * 42, 128, 64, K, "bf16", 790 + K, window=W)
+    lens = [64 * 41 + 1, 64 * 30 + 63, 17]
+    inp = wl.make_decode_inputs(cfg, "cpu", seq_lens=torch.tensor(lens, dtype=torch.int32))
+    if per_head:
+        inp["landmarks"] = inp["landmarks"].repeat_interleave(4, dim=1).contiguous()
+    poison(inp, lens, float("nan"))
+    g = {n: t.to(DEV) for n, t in inp.items()}
+    got = hils.hils_decode(g["q"], g["k"], g["v"], g["landmarks"], g["seq_lens"], 64, K, window=W, impl=impl)
+    assert hils.last_launch_count() == launches
+    torch.cuda.synchronize()
+    check(got, oracle.hils_decode(inp["q"], inp["k"], inp["v"], inp["landmarks"], None, inp["seq_lens"], S=64, K=K, W=W), K)
