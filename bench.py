@@ -289,6 +289,11 @@ def roofline_for(w, kernel_ms, peaks):
                     frac=ach / peaks["hbm_gbs"], algorithmic_bytes=algo)
     gathered, scoring = prefill_flops(w.cfg)
     algo = (scoring if ("score" in name or "select" in name) else gathered) / nl
+    if name == "prefill_attend":
+        # the gathered FLOP of a call are shared with the query-major kernel (early tokens, wide local windows)
+        together = [k for k in ("prefill_attend", "prefill_query", "prefill_local") if k in kernel_ms]
+        sec = sum(kernel_ms[k] for k in together) * 1e-3 / nl
+        common["achieved_over"] = together
     if w.cfg.dtype == "f32":
         # fp32 path on plain FMA units: 148 SMs x 128 lanes x 2 FLOP x max SM clock
         peak = 148 * 128 * 2 * peaks.get("sm_max_mhz", 1965.0) * 1e6 / 1e12

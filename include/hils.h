@@ -35,9 +35,11 @@
  *       k, v        [B, Hkv, T, d]         T = L for prefill, T_max for decode
  *       landmarks   [B, Hl, C, d]          C = params.C rows per landmark head; row c is only read
  *                                          when chunk c is complete and precedes the local window
- *       bias        [B, Hl, C] fp32 or NULL (NULL means 0)
+ *       bias        [B, Hl, C] fp32 or NULL (NULL means 0); -inf masks a chunk: it fills a place of the
+ *                   selection only where fewer than K others are left, with weight 0
  *       lse         [B, Hq, L] fp32        (decode: [B, Hq])
  *       sel_idx     [B, Hkv, L, K] int32   (decode: [B, Hkv, K]) ascending chunk ids, -1 padded
+ *       (rows of k and v behind the last token that a call sees may hold anything: they are in no result)
  *       seq_lens    [B] int32              decode: tokens in the cache INCLUDING the new one; the
  *                                          query sits at position seq_lens[b]-1, 1 <= seq_lens <= T_max
  *   - Argument errors are found on the host and returned before anything is launched.
@@ -136,9 +138,9 @@ int hils_decode(const hils_params* params, const void* q, const void* k_cache, c
  *
  *  - Nothing is allocated or freed, by CUDA or otherwise, on any call.
  *  - Limit: the decode workspace of the shape, hils_workspace_bytes(params, 1) (its 256-byte status block
- *    included), must fit in 16 MiB, otherwise HILS_ERR_WORKSPACE is returned before anything is launched (both benchmark decode shapes fit: B=64 x 64K tokens with
- *    K=32 needs about 13.7 MiB, B=4 x 1M tokens with K=64 about 10.9 MiB; most of it is the table of per-head
- *    landmark scores, B x Hq x C floats).  Shapes outside the
+ *    included), must fit in 16 MiB, otherwise HILS_ERR_WORKSPACE is returned before anything is launched (B=64 x 64K tokens
+ *    with K=32: about 13.7 MiB, B=4 x 1M tokens with K=64: about 10.9 MiB; most of it is the table of per-head landmark
+ *    scores that the three-kernel form keeps, B x Hq x C floats).  Shapes outside the
  *    bandwidth-tuned decode kernels (bf16, d=128, chunk 64, window <= 897, one landmark per KV or per query head,
  *    at most 8 query heads per KV head) return HILS_ERR_UNSUPPORTED.
  *  - The first call on each device looks up the array's device address (with that device current);

@@ -17,8 +17,8 @@
 //   combine  the warps' sums meet in shared memory, the CTAs' in distributed shared memory.
 // Bound: HBM (landmarks scanned + selected K / V), and where a call has few units the chain of dependent steps.  One
 // launch per step (decode_fast.cu) drains and ramps between short phases and leaves the memory idle during the
-// selection.  Before / now, B200, us per call back to back: 1 x 6000 tokens, K = 16: 20.8 / 12.1; 8 x 4K-16K paged,
-// K = 32, W = 512: 41.6 / 23.6; 64 x 64K, K = 32: 139 / 116 (6.0 TB/s); 4 x 1M, K = 64: 61.5 / 47.
+// selection.  Before / now, B200, us per call through the Python entry points, calls back to back: 1 x 6000 tokens, K = 16:
+// 22.7 / 12.7; 8 x 4K-16K paged, K = 32, W = 512: 49.3 / 28.1; 64 x 64K, K = 32: 142.6 / 118 (5.8 TB/s); 4 x 1M, K = 64: 65.4 / 46.7.
 // Draft tokens of one sequence retrieve mostly the same chunks: the union of their selections is loaded once, and all
 // their heads fill the MMA's columns.
 #include "internal.h"

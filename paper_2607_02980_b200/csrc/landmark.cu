@@ -8,8 +8,7 @@
 //               272-byte apart for d = 128 bf16, so a quarter warp touches all 32 banks once), no shuffles;
 //   softmax     two warp reductions; b' = log Z - sum p (s - max);
 //   k'          lane l owns d/32 output dimensions and runs over the rows.
-// The loops are rolled (a first, fully unrolled register version was bound by instruction fetch at 20 % of
-// the memory bandwidth).  The kernel is bound by HBM: algorithmic bytes = the keys of the summarised chunks.
+// The loops are rolled (a first, fully unrolled register version reached 20 % of the memory bandwidth).  The kernel is bound by HBM: algorithmic bytes = the keys of the summarised chunks.
 #include "internal.h"
 #include "tma.cuh"
 

@@ -19,9 +19,10 @@
 // 86 cycles each and 1-D bulk copies of one row 54: both slower.  More than four gather warps need per-group register
 // budgets (setmaxnreg), which measured slower (1.08 ms against 0.73 ms on the 16K-token benchmark shape).
 // S/P/O are double buffered, three gathered Q tiles are in flight, K tiles are double and V tiles triple buffered.
-// Bound: softmax groups and output group are both busy more than 85 % of a tile period of 2100 cycles (32 KB of partial
-// output per tile and SM: 4.3 TB/s).  16K tokens, K = 16, 32 heads, 59 K tiles: 0.44 ms (0.55 ms in batches between barriers and
-// with all KV heads walked together).
+// Bound: a tile period of 2100 cycles, in which softmax and output groups follow each other (32 KB of partial output per tile
+// and SM: 4.3 TB/s; the shared-memory port carries 56 % of its wavefronts in warp accesses and MMA operands, the TMA's beside
+// them).  16K tokens, K = 16, 32 heads, 59 K tiles: 0.44 ms (0.55 ms in batches between barriers and with all KV heads walked
+// together).
 #include "internal.h"
 #include "tma.cuh"
 
