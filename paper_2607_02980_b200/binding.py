@@ -336,7 +336,8 @@ def hils_prefill_at(q, k, v, landmarks, chunk_size: int, top_k: int, pos0: int, 
     lse = torch.empty((B, Hq, L), dtype=torch.float32, device=q.device) if lse is None else lse
     sel_idx = torch.empty((B, Hkv, L, top_k), dtype=torch.int32, device=q.device) if sel_idx is None else sel_idx
     rc = lib.hils_prefill_at(p, _ptr(q), _ptr(k), _ptr(v), _ptr(landmarks), _ptr(bias), int(pos0),
-                             _ptr(out), _ptr(lse), _ptr(sel_idx), _ptr(ws), nbytes, _stream_ptr(stream))
+                             _ptr(out), _ptr(lse), _ptr(sel_idx), _ptr(ws), ws.numel() * ws.element_size(),
+                             _stream_ptr(stream))
     if rc != 0:
         raise HilsError(rc, "hils_prefill_at")
     return out, lse, sel_idx

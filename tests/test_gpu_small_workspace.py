@@ -38,6 +38,22 @@ def test_query_blocks_shrink_to_the_workspace(B, Hkv, L, K, W):
         run(ws[:B * Hkv * K * 2048 * 1024])
 
 
+def test_a_slice_stays_inside_the_workspace_it_was_given():
+    cfg = wl.HilsConfig("ws", "prefill", 1, 8, 2, 12000, 128, 64, 16, "bf16", 1340)
+    g = wl.make_prefill_inputs(cfg, DEV)
+    n, q = reported(cfg)[1], g["q"][:, :, 2000:].contiguous()
+    run = lambda ws: hils.hils_prefill_at(q, g["k"], g["v"], g["landmarks"], 64, 16, 2000, workspace=ws)
+    full = run(None)
+    ws = torch.full((n,), 255, dtype=torch.uint8, device=DEV)
+    ws[:256].zero_()
+    got = run(ws[:n // 2])
+    torch.cuda.synchronize()
+    assert all(torch.equal(x, y) for x, y in zip(got, full))
+    assert (ws[n // 2:] == 255).all()
+    with pytest.raises(hils.HilsError):
+        run(ws[:n // 20])
+
+
 def test_fp32_without_scratch_takes_the_row_kernel():
     cfg = wl.HilsConfig("ws", "prefill", 1, 2, 1, 1000, 64, 64, 4, "f32", 1350)
     g = wl.make_prefill_inputs(cfg, DEV)
