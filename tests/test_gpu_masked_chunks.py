@@ -12,21 +12,21 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda"
 
 
-def masked_bias(cfg, share, heads=None):
+def masked_bias(cfg, share, heads=None, mask=float("-inf")):
     """bias [B, Hl, C] with `share` of the chunks masked, chunk 0 among them."""
     g = torch.Generator().manual_seed(cfg.seed)
     bias = torch.randn((cfg.B, heads or cfg.Hkv, cfg.C), generator=g)
-    bias[torch.rand(bias.shape, generator=g) < share] = float("-inf")
-    bias[:, :, 0] = float("-inf")
+    bias[torch.rand(bias.shape, generator=g) < share] = mask
+    bias[:, :, 0] = mask
     return bias
 
 
-def decode(cfg, share, seq=None, impl="auto", per_head=False):
+def decode(cfg, share, seq=None, impl="auto", per_head=False, mask=float("-inf")):
     seq = torch.tensor(seq or [cfg.L - 97 * b for b in range(cfg.B)], dtype=torch.int32)
     inp = wl.make_decode_inputs(cfg, "cpu", seq_lens=seq)
     if per_head:
         inp["landmarks"] = inp["landmarks"].repeat_interleave(cfg.G, dim=1).contiguous()
-    bias = masked_bias(cfg, share, cfg.Hq if per_head else None)
+    bias = masked_bias(cfg, share, cfg.Hq if per_head else None, mask)
     g = {n: t.to(DEV) for n, t in inp.items()}
     got = hils.hils_decode(g["q"], g["k"], g["v"], g["landmarks"], g["seq_lens"], 64, cfg.K, window=cfg.window,
                            bias=bias.to(DEV), impl=impl)
@@ -34,11 +34,11 @@ def decode(cfg, share, seq=None, impl="auto", per_head=False):
     check_decode(cfg, inp, *got, bias=bias, W=cfg.window)
 
 
-def prefill(cfg, share, impl="auto", per_head=False):
+def prefill(cfg, share, impl="auto", per_head=False, mask=float("-inf")):
     inp = wl.make_prefill_inputs(cfg, "cpu")
     if per_head:
         inp["landmarks"] = inp["landmarks"].repeat_interleave(cfg.G, dim=1).contiguous()
-    bias = masked_bias(cfg, share, cfg.Hq if per_head else None)
+    bias = masked_bias(cfg, share, cfg.Hq if per_head else None, mask)
     g = {n: t.to(DEV) for n, t in inp.items()}
     got = hils.hils_prefill(g["q"], g["k"], g["v"], g["landmarks"], 64, cfg.K, bias=bias.to(DEV), window=cfg.window, impl=impl)
     torch.cuda.synchronize()
@@ -133,3 +133,11 @@ def test_a_query_that_is_not_a_number_spoils_its_own_row_only(L, K):
         ids = sel[0, 0, r].tolist()
         n = min(K, r // 64)
         assert ids[n:] == [-1] * (K - n) and sorted(set(ids[:n])) == ids[:n] and all(0 <= c < r // 64 for c in ids[:n])
+
+
+@pytest.mark.parametrize("share", [0.5, 0.97])
+@pytest.mark.parametrize("mode,L,K,impl", [("decode", 64 * 400, 32, "auto"), ("decode", 64 * 40, 8, "auto"), ("decode", 64 * 40, 8, "generic"),
+                                           ("prefill", 1000, 16, "auto"), ("prefill", 3000, 5, "auto"), ("prefill", 64 * 60, 40, "auto")])
+def test_masks_of_the_lowest_finite_number(mode, L, K, impl, share):
+    cfg = wl.HilsConfig("lowest", mode, 1, 8, 2, L, 128, 64, K, "bf16", 1400 + K)
+    (decode if mode == "decode" else prefill)(cfg, share, impl=impl, mask=torch.finfo(torch.float32).min)
