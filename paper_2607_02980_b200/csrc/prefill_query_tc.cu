@@ -20,7 +20,11 @@
 //   warps 8, 9       issue the MMAs of tile 0 / 1 (the next chunk's scores before this chunk's value product)
 //   warp 10          loads K, V, landmark rows and queries by TMA
 //   warp 11          builds the unit's list of chunks (and which tile needs them, with a bit per token), one unit ahead
-// Bound: the exponentials (64 per row and chunk; 512 cycles per tile and chunk on 16 units) and the softmax warps' issue.
+// Bound: the softmax warps' serial chain per chunk, 2000 cycles: answer of the barrier 290, tensor-memory load 100, maximum 200, exponentials
+// 750 (two warps per scheduler; special-function unit 37 % busy), weight 200, accumulator's answer 170, probabilities back 190.  The
+// tensor pipe needs 1350 of them.  2 x 6000 tokens, K = 32: 661 -> 587 us with the quotient w / z by the approximate reciprocal (the
+// exactly rounded division took 300 cycles of the chain; its result is rounded to bf16 next) and the next item's barrier asked early.
+// Sixteen softmax warps, half a row's keys or every other item each: 704 and 781 us (more instructions, colder instruction cache).
 #include "internal.h"
 #include "tma.cuh"
 
@@ -169,6 +173,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             const int pos = lane_position(s, tok, a.n_tok), lc = local_lo(pos, s.W, kS) / kS;
             const float* bias = a.bias ? a.bias + (static_cast<long long>(b) * s.Hl + gk) * s.C : nullptr;
             float ref = kLowestLogit, den = 0.f;
+            bool s_ready = false;
             int2 next = n > 0 ? sm.titem[ln][t][0] : make_int2(0, 0);
             for (int i = 0; i < n; ++i) {
                 const int c = next.x;
@@ -177,7 +182,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                 const float bb = (bias && c < lc) ? bias[c] : 0.f;
                 const bool local = c >= lc;
                 const bool act = ((who >> lane) & 1u) != 0u;
-                if (!wait(&sm.s_full[t], n_s & 1)) break;
+                if (!s_ready && !wait(&sm.s_full[t], n_s & 1)) break;
                 tc_fence_after_sync();
                 float v[64], lm4[4];
                 tmem_ld64_4(t_lane, t_lane + 64, v, lm4);
@@ -231,7 +236,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                 }
                 const float w = act ? __expf(lam - ref) : 0.f;
                 den += w;
-                const float pw = act ? w / z : 0.f;
+                const float pw = act ? __fdividef(w, z) : 0.f;
                 const float2 pw2 = make_float2(pw, pw);
                 // the previous chunk's value product has read its probabilities and left the accumulator
                 if (i > 0) {
@@ -260,6 +265,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                     }
                     tmem_st8(t_lane + kPCol + pc * 8, pk);
                 }
+                s_ready = i + 1 < n && mbar_test_wait(&sm.s_full[t], (n_s + 1) & 1);
                 tmem_wait_st();
                 tc_fence_before_sync();
                 __syncwarp();
@@ -318,7 +324,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             const int t = warp - kMmaWarp;
             // (one answer per warp: elections follow)
             auto wait = [&](uint64_t* bar, uint32_t parity) {
-                if (ok && !__all_sync(kFullMask, mbar_wait(bar, parity))) ok = false;
+                if (ok && !__all_sync(kFullMask, mbar_test_wait(bar, parity)) && !__all_sync(kFullMask, mbar_wait(bar, parity))) ok = false;
                 return ok;
             };
             constexpr uint32_t idesc_s = umma_idesc_bf16(kRows, kNS);
@@ -511,7 +517,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
 
 // Tokens of a call (from its first on) that go this way: a multiple of 128 below the call's length, or all of them.  The
 // split with the largest gain by these costs (SM cycles; fitted to 16K, 2 x 6000 and 3 x 1000 tokens):
-//   here, a unit of 64 tokens: 2500 per chunk it visits (at most every visible one) + 18000, the last unit at least in full;
+//   here, a unit of 64 tokens: 2200 per chunk it visits (at most every visible one) + 18000, the last unit at least in full;
 //   chunk-major (index, attend and fuse kernels): 3830 per 32 tokens and chunk they attend, and 55000 for the launches.
 // With units for every SM the line lies near visible : attended = 5 : 2.  With few (sequence, KV head) pairs the units are a
 // serial chain on some of the SMs, and everything goes chunk-major unless that saves its launches (2 KV heads, a slice of
@@ -529,7 +535,7 @@ int prefill_query_tokens(const Shape& s) {
     int best = 0;
     for (int n = 0; n < s.R;) {
         const int end = n + kUnitTok < s.R ? n + kUnitTok : s.R;
-        const long long vis = (s.pos0 + end - 1) / kS + 1, att = vis < s.K + nl ? vis : s.K + nl, unit = 2500 * vis + 18000;
+        const long long vis = (s.pos0 + end - 1) / kS + 1, att = vis < s.K + nl ? vis : s.K + nl, unit = 2200 * vis + 18000;
         if (vis > kMaxC) break;
         here += pairs * unit;
         there += pairs * (end - n) * att * 3830 / 32;
