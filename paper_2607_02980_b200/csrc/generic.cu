@@ -427,40 +427,183 @@ generic_attend_kernel(const GArgs a) {
 
 // ---- fp32 prefill on small shapes: chunk-major ------------------------------------------------------------------
 // The row kernel above reads (K + 1) chunks per row, mostly from L2 (61 % of its requests on 2048 tokens, d = 64, K = 4;
-// 38 us).  Here a CTA takes one chunk and the rows of a block that attend it: it looks its rows' selections through,
-// keeps K and V in shared memory and scores four rows at a time (lane = key, then lane = dimension), so that a K or V
-// value read from shared memory meets four rows.  Partial outputs and masses per (row, slot) go through global memory
-// to generic_fuse_kernel.  Same shape: 38 -> 26 us for the two kernels (bound by shared-memory reads while all CTAs
-// score, by latencies at both ends).
-constexpr int kRowBlock = 32;                // (early chunks are attended by every row of a block: two groups of four per warp)
-constexpr int kChunkWarps = 4;
-static_assert(kRowBlock <= kChunkWarps * 32, "one row per thread in the look-through");
-
+// 38 us).  Here a CTA takes one chunk of one KV head and the tokens of a block that attend it: it looks their selections through,
+// keeps K and V in shared memory and scores four or eight (token, head) rows at a time per warp (lane = key, then lane = dimension),
+// so that a K or V value read from shared memory meets that many rows.  Partial outputs and masses per (row, slot) go through
+// global memory to generic_fuse_kernel.
+// Bound: shared-memory reads while all warps score (with eight rows as many cycles as the packed FMAs take, with four 1.5 times
+// as many), latencies at both ends on small shapes.  The blocks are longer on larger shapes (launch_chunk_major): with blocks of 32
+// tokens of one head the CTAs mostly loaded K and V (64 KB for six rows at 3072 tokens, d = 128, K = 4).
+constexpr int kRowBlockMax = 128;
 
 // Slots of a row: the selected chunks 0 .. K - 1, then the chunks of its local window.
 __host__ __device__ inline int chunk_slots(const Shape& s) { return s.K + (s.W + s.S - 2) / s.S + 1; }
 
-template <int D>
+// Chunks up to the last token of block r of rb tokens.
+__host__ __device__ inline int block_chunks(const Shape& s, int rb, int r) { return (s.pos0 + (s.R < (r + 1) * rb ? s.R : (r + 1) * rb) - 1) / s.S + 1; }
+
+template <int D, int NW>
 struct ChunkSmem {
     alignas(16) float k[64][D + 4];            // (padded: eight lanes reading the same piece of eight rows miss each other's banks)
     alignas(16) float v[64][D];
-    alignas(16) float q[kChunkWarps][4][D];
-    alignas(16) float4 p[kChunkWarps][64][2];  // probabilities of four rows per key, each twice (pairs of a packed multiply)
-    int row[kRowBlock];                        // rows (of the block) that attend the chunk and the slot they hold it in
-    int slot[kRowBlock];
-    int cnt[kChunkWarps];
+    union Warp {
+        float q[NW][D];
+        float4 p[64][NW / 2 + 1];                       // probabilities of a warp's rows per key, each twice (pairs of a packed multiply; padded)
+    };
+    alignas(16) Warp w[NW];
+    int row[kRowBlockMax];                     // tokens (of the block) that attend the chunk and the slot they hold it in
+    int slot[kRowBlockMax];
+    int cnt[NW];
 };
 
-template <int D>
-__global__ void __launch_bounds__(kChunkWarps * 32)
-generic_chunk_kernel(const GArgs a, float* part, float* lam) {
-    extern __shared__ uint8_t chunk_raw[];
-    ChunkSmem<D>& sm = *reinterpret_cast<ChunkSmem<D>*>(chunk_raw);
+template <int D, int NW, int NR>
+__device__ __forceinline__ void fetch_rows(const GArgs& a, const ChunkSmem<D, NW>& sm, int b, int h0, int nh, int n, int e0, float (&qv)[NR][D / 32]) {
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+        const int x = min(e0 + i, n * nh - 1), e = nh == 1 ? x : x / nh;
+        const long long row = (static_cast<long long>(b) * a.s.Hq + h0 + (x - e * nh)) * a.s.R + sm.row[e];
+#pragma unroll
+        for (int y = 0; y < D / 32; ++y) qv[i][y] = static_cast<const float*>(a.q)[row * D + (threadIdx.x & 31) + 32 * y];
+    }
+}
+
+// Rows (token, head) e0 .. e0 + NR - 1 of the n tokens x nh heads from h0 on (of KV head g), by one warp.  qv: their queries with four rows
+// at a time (fetch_rows), and on return those of the rows from e0 + step on.
+template <int D, int NW, int NR>
+__device__ __forceinline__ void chunk_rows(const GArgs& a, ChunkSmem<D, NW>& sm, int c, int b, int g, int h0, int nh, int n, int e0, int step, float (&qv)[NR][D / 32], const float (&lmv)[D / 32],
+                                           float* part, float* lam) {
     constexpr int kV = D / 32;                 // dimensions per lane in the value pass
     const Shape& s = a.s;
+    const int lane = threadIdx.x & 31, NS = chunk_slots(s);
+    typename ChunkSmem<D, NW>::Warp& w = sm.w[threadIdx.x >> 5];
+    const bool own_lm = s.Hl == s.Hq && s.G > 1;                              // a landmark row per head
+    long long orow[NR];                                                       // row of q
+    int lim[NR], slot[NR], head[NR];
+    float lm[NR];
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+        const int x = min(e0 + i, n * nh - 1), e = nh == 1 ? x : x / nh, r = sm.row[e];
+        head[i] = h0 + (x - e * nh);
+        orow[i] = (static_cast<long long>(b) * s.Hq + head[i]) * s.R + r;
+        slot[i] = sm.slot[e];
+        lim[i] = slot[i] < s.K ? s.S - 1 : min(s.S - 1, s.pos0 + r - c * s.S);
+    }
+    {
+        if (NR > 4) fetch_rows<D, NW, NR>(a, sm, b, h0, nh, n, e0, qv);
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            lm[i] = 0.f;
+            const float* lr = static_cast<const float*>(a.lm) + ((static_cast<long long>(b) * s.Hl + head[i]) * s.C + c) * D;
+#pragma unroll
+            for (int x = 0; x < kV; ++x) {
+                w.q[i][lane + 32 * x] = qv[i][x];
+                const float rv = a.q_route == a.q ? qv[i][x] : static_cast<const float*>(a.q_route)[orow[i] * D + lane + 32 * x];
+                lm[i] = fmaf(rv, own_lm && c < s.C ? lr[lane + 32 * x] : lmv[x], lm[i]);
+            }
+        }
+    }
+    __syncwarp();
+    if (NR == 4 && e0 + step < n * nh) fetch_rows<D, NW, NR>(a, sm, b, h0, nh, n, e0 + step, qv);
+    // two dimensions per instruction: a pair's halves are added at the end
+    float2 a0[NR], a1[NR];                                                    // keys lane, lane + 32
+#pragma unroll
+    for (int i = 0; i < NR; ++i) a0[i] = a1[i] = make_float2(0.f, 0.f);
+#pragma unroll 4
+    for (int x = 0; x < D; x += 4) {
+        const float4 k0 = *reinterpret_cast<const float4*>(&sm.k[lane][x]), k1 = *reinterpret_cast<const float4*>(&sm.k[lane + 32][x]);
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            const float4 qv = *reinterpret_cast<const float4*>(&w.q[i][x]);
+            const float2 ql = make_float2(qv.x, qv.y), qh = make_float2(qv.z, qv.w);
+            a0[i] = __ffma2_rn(ql, make_float2(k0.x, k0.y), a0[i]);
+            a1[i] = __ffma2_rn(ql, make_float2(k1.x, k1.y), a1[i]);
+            a0[i] = __ffma2_rn(qh, make_float2(k0.z, k0.w), a0[i]);
+            a1[i] = __ffma2_rn(qh, make_float2(k1.z, k1.w), a1[i]);
+        }
+    }
+    float mx[NR], z[NR], s0[NR], s1[NR];
+    __syncwarp();                                                             // (the probabilities overwrite the queries)
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+        s0[i] = lane <= lim[i] ? (a0[i].x + a0[i].y) * s.scale : -INFINITY;
+        s1[i] = lane + 32 <= lim[i] ? (a1[i].x + a1[i].y) * s.scale : -INFINITY;
+        mx[i] = fmaxf(s0[i], s1[i]);
+    }
+    // (the rows' reductions side by side: one after the other their shuffles would wait for one another)
+#pragma unroll
+    for (int x = 16; x > 0; x >>= 1)
+#pragma unroll
+        for (int i = 0; i < NR; ++i) mx[i] = fmaxf(mx[i], __shfl_xor_sync(kFullMask, mx[i], x));
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+        s0[i] = __expf(s0[i] - mx[i]);
+        s1[i] = __expf(s1[i] - mx[i]);
+        z[i] = s0[i] + s1[i];
+    }
+#pragma unroll
+    for (int x = 16; x > 0; x >>= 1)
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            z[i] += __shfl_xor_sync(kFullMask, z[i], x);
+            lm[i] += __shfl_xor_sync(kFullMask, lm[i], x);
+        }
+#pragma unroll
+    for (int i = 0; i < NR; i += 2) {
+        w.p[lane][i / 2] = make_float4(s0[i], s0[i], s0[i + 1], s0[i + 1]);
+        w.p[lane + 32][i / 2] = make_float4(s1[i], s1[i], s1[i + 1], s1[i + 1]);
+    }
+    __syncwarp();
+    float2 o[NR][kV / 2];
+#pragma unroll
+    for (int i = 0; i < NR; ++i)
+#pragma unroll
+        for (int x = 0; x < kV / 2; ++x) o[i][x] = make_float2(0.f, 0.f);
+#pragma unroll (NR == 4 ? 8 : 4)
+    for (int j = 0; j < 64; ++j) {
+        float4 p[NR / 2];
+#pragma unroll
+        for (int i = 0; i < NR / 2; ++i) p[i] = w.p[j][i];
+#pragma unroll
+        for (int x = 0; x < kV / 2; ++x) {
+            const float2 v = *reinterpret_cast<const float2*>(&sm.v[j][2 * lane + 64 * x]);
+#pragma unroll
+            for (int i = 0; i < NR; i += 2) {
+                o[i][x] = __ffma2_rn(make_float2(p[i / 2].x, p[i / 2].y), v, o[i][x]);
+                o[i + 1][x] = __ffma2_rn(make_float2(p[i / 2].z, p[i / 2].w), v, o[i + 1][x]);
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+        if (e0 + i >= n * nh) break;
+        const long long at = orow[i] * NS + slot[i];
+        const float zi = 1.f / z[i];
+#pragma unroll
+        for (int x = 0; x < kV / 2; ++x)
+            *reinterpret_cast<float2*>(part + at * D + 2 * lane + 64 * x) = make_float2(o[i][x].x * zi, o[i][x].y * zi);
+        if (lane == 0) {
+            const int hl = s.Hl == s.Hq ? head[i] : g;
+            lam[at] = slot[i] < s.K ? lm[i] * s.scale + (a.bias ? a.bias[(static_cast<long long>(b) * s.Hl + hl) * s.C + c] : 0.f)
+                                    : mx[i] + __logf(z[i]);
+        }
+    }
+    __syncwarp();
+}
+
+// NW: warps per CTA and most rows of a warp at a time, row_block: tokens, nh: query heads (of one KV head)
+template <int D, int NW>
+__global__ void __launch_bounds__(NW * 32, 16 / NW)
+generic_chunk_kernel(const GArgs a, int row_block, int nh, float* part, float* lam) {
+    extern __shared__ uint8_t chunk_raw[];
+    ChunkSmem<D, NW>& sm = *reinterpret_cast<ChunkSmem<D, NW>*>(chunk_raw);
+    const Shape& s = a.s;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int c = blockIdx.y, r0 = blockIdx.x * kRowBlock, bh = blockIdx.z, h = bh % s.Hq, b = bh / s.Hq, g = h / s.G;
-    if (s.pos0 + min(s.R, r0 + kRowBlock) - 1 < c * s.S) return;            // the chunk lies after the block's last row
+    // blocks of tokens y (from the last one on) and y (from the first one on) share a row of CTAs, one per chunk up to their last tokens
+    const int nb = (s.R + row_block - 1) / row_block, hi = nb - 1 - blockIdx.y, n_hi = block_chunks(s, row_block, hi);
+    const bool low = static_cast<int>(blockIdx.x) >= n_hi;
+    const int blk = low ? blockIdx.y : hi, c = low ? blockIdx.x - n_hi : blockIdx.x;
+    if (low && (blk == hi || c >= block_chunks(s, row_block, blk))) return;
+    const int r0 = blk * row_block, hg = s.Hq / nh, h0 = blockIdx.z % hg * nh, g = h0 / s.G, b = blockIdx.z / hg;
     const float* kc = static_cast<const float*>(a.k) + ((static_cast<long long>(b) * s.Hkv + g) * s.T + static_cast<long long>(c) * s.S) * D;
     const float* vc = static_cast<const float*>(a.v) + (kc - static_cast<const float*>(a.k));
     // rows of the chunk up to the call's last token: the ones after it may hold anything, and 0 x NaN is NaN
@@ -471,11 +614,15 @@ generic_chunk_kernel(const GArgs a, float* part, float* lam) {
         cp_async16(smem_u32(&sm.v[x / (D / 4)][(x % (D / 4)) * 4]), vc + x * 4);
     asm volatile("cp.async.commit_group;" ::: "memory");
     for (int x = rows_k * D + tid; x < 64 * D; x += blockDim.x) { sm.k[x / D][x % D] = 0.f; sm.v[x / D][x % D] = 0.f; }
+    float lmv[D / 32];                          // the chunk's landmark (with one per head: not used)
+#pragma unroll
+    for (int x = 0; x < D / 32; ++x)
+        lmv[x] = c < s.C ? static_cast<const float*>(a.lm)[((static_cast<long long>(b) * s.Hl + (s.Hl == s.Hq ? g * s.G : g)) * s.C + c) * D + lane + 32 * x] : 0.f;
     pdl_wait();                                 // the selection
     int slot = -1;
     {
         const int r = r0 + tid, pos = s.pos0 + r;
-        if (tid < kRowBlock && r < s.R && c * s.S <= pos) {
+        if (tid < row_block && r < s.R && c * s.S <= pos) {
             const int lc = local_lo(pos, s.W, s.S) / s.S;
             if (c >= lc) {
                 slot = s.K + c - lc;
@@ -493,111 +640,16 @@ generic_chunk_kernel(const GArgs a, float* part, float* lam) {
         if (slot >= 0) { sm.row[at] = r; sm.slot[at] = slot; }
     }
     int n = 0;
-    for (int w = 0; w < kChunkWarps; ++w) n += sm.cnt[w];
+    for (int w = 0; w < NW; ++w) n += sm.cnt[w];
     __syncthreads();
-    const int NS = chunk_slots(s), hl = (s.Hl == s.Hq) ? h : g;
-    const long long lrow = (static_cast<long long>(b) * s.Hl + hl) * s.C + c;
-    float lmv[kV];                              // the chunk's landmark
-#pragma unroll
-    for (int x = 0; x < kV; ++x) lmv[x] = c < s.C ? static_cast<const float*>(a.lm)[lrow * D + lane + 32 * x] : 0.f;
-    // query rows of a group of four, requested a group ahead
-    float qv[4][kV], rv[4][kV];
-    auto fetch = [&](int e0) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const long long at = (static_cast<long long>(bh) * s.R + sm.row[min(e0 + i, n - 1)]) * D + lane;
-#pragma unroll
-            for (int x = 0; x < kV; ++x) {
-                qv[i][x] = static_cast<const float*>(a.q)[at + 32 * x];
-                rv[i][x] = static_cast<const float*>(a.q_route)[at + 32 * x];
-            }
-        }
-    };
-    if (warp * 4 < n) fetch(warp * 4);
-    for (int e0 = warp * 4; e0 < n; e0 += kChunkWarps * 4) {
-        int row[4], lim[4];
-        bool sel[4];
-        float lm[4];
-        float (*q)[D] = sm.q[warp];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int e = min(e0 + i, n - 1);
-            row[i] = sm.row[e];
-            sel[i] = sm.slot[e] < s.K;
-            lim[i] = sel[i] ? s.S - 1 : min(s.S - 1, s.pos0 + row[i] - c * s.S);
-            lm[i] = 0.f;
-#pragma unroll
-            for (int x = 0; x < kV; ++x) {
-                q[i][lane + 32 * x] = qv[i][x];
-                lm[i] = fmaf(rv[i][x], lmv[x], lm[i]);
-            }
-        }
-        if (e0 + kChunkWarps * 4 < n) fetch(e0 + kChunkWarps * 4);
-        __syncwarp();
-        // two dimensions per instruction: a pair's halves are added at the end
-        float2 a0[4], a1[4];                                                  // keys lane, lane + 32
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a0[i] = a1[i] = make_float2(0.f, 0.f);
-#pragma unroll 4
-        for (int x = 0; x < D; x += 4) {
-            const float4 k0 = *reinterpret_cast<const float4*>(&sm.k[lane][x]), k1 = *reinterpret_cast<const float4*>(&sm.k[lane + 32][x]);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float4 qv = *reinterpret_cast<const float4*>(&q[i][x]);
-                const float2 ql = make_float2(qv.x, qv.y), qh = make_float2(qv.z, qv.w);
-                a0[i] = __ffma2_rn(ql, make_float2(k0.x, k0.y), a0[i]);
-                a1[i] = __ffma2_rn(ql, make_float2(k1.x, k1.y), a1[i]);
-                a0[i] = __ffma2_rn(qh, make_float2(k0.z, k0.w), a0[i]);
-                a1[i] = __ffma2_rn(qh, make_float2(k1.z, k1.w), a1[i]);
-            }
-        }
-        float s0[4], s1[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) { s0[i] = a0[i].x + a0[i].y; s1[i] = a1[i].x + a1[i].y; }
-        float mx[4], z[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            s0[i] = lane <= lim[i] ? s0[i] * s.scale : -INFINITY;
-            s1[i] = lane + 32 <= lim[i] ? s1[i] * s.scale : -INFINITY;
-            mx[i] = warp_max(fmaxf(s0[i], s1[i]));
-            s0[i] = __expf(s0[i] - mx[i]);
-            s1[i] = __expf(s1[i] - mx[i]);
-            z[i] = warp_sum(s0[i] + s1[i]);
-            lm[i] = warp_sum(lm[i]);
-        }
-        sm.p[warp][lane][0] = make_float4(s0[0], s0[0], s0[1], s0[1]);
-        sm.p[warp][lane][1] = make_float4(s0[2], s0[2], s0[3], s0[3]);
-        sm.p[warp][lane + 32][0] = make_float4(s1[0], s1[0], s1[1], s1[1]);
-        sm.p[warp][lane + 32][1] = make_float4(s1[2], s1[2], s1[3], s1[3]);
-        __syncwarp();
-        float2 o[4][kV / 2];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int x = 0; x < kV / 2; ++x) o[i][x] = make_float2(0.f, 0.f);
-#pragma unroll 8
-        for (int j = 0; j < 64; ++j) {
-            const float4 p0 = sm.p[warp][j][0], p1 = sm.p[warp][j][1];
-#pragma unroll
-            for (int x = 0; x < kV / 2; ++x) {
-                const float2 v = *reinterpret_cast<const float2*>(&sm.v[j][2 * lane + 64 * x]);
-                o[0][x] = __ffma2_rn(make_float2(p0.x, p0.y), v, o[0][x]);
-                o[1][x] = __ffma2_rn(make_float2(p0.z, p0.w), v, o[1][x]);
-                o[2][x] = __ffma2_rn(make_float2(p1.x, p1.y), v, o[2][x]);
-                o[3][x] = __ffma2_rn(make_float2(p1.z, p1.w), v, o[3][x]);
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (e0 + i >= n) break;
-            const long long at = (static_cast<long long>(bh) * s.R + row[i]) * NS + sm.slot[e0 + i];
-            const float zi = 1.f / z[i];
-#pragma unroll
-            for (int x = 0; x < kV / 2; ++x)
-                *reinterpret_cast<float2*>(part + at * D + 2 * lane + 64 * x) = make_float2(o[i][x].x * zi, o[i][x].y * zi);
-            if (lane == 0) lam[at] = sel[i] ? lm[i] * s.scale + (a.bias ? a.bias[lrow] : 0.f) : mx[i] + __logf(z[i]);
-        }
-        __syncwarp();
+    const int rows = n * nh;
+    if (NW == 8 && rows > NW * 4) {
+        float qv[8][D / 32];
+        for (int e0 = warp * 8; e0 < rows; e0 += NW * 8) chunk_rows<D, NW, 8>(a, sm, c, b, g, h0, nh, n, e0, NW * 8, qv, lmv, part, lam);
+    } else if (warp * 4 < rows) {
+        float qv[4][D / 32];
+        fetch_rows<D, NW, 4>(a, sm, b, h0, nh, n, warp * 4, qv);
+        for (int e0 = warp * 4; e0 < rows; e0 += NW * 4) chunk_rows<D, NW, 4>(a, sm, c, b, g, h0, nh, n, e0, NW * 4, qv, lmv, part, lam);
     }
 }
 
@@ -648,21 +700,43 @@ size_t chunk_lam_offset(const Shape& s) {
     return (static_cast<size_t>(s.B) * s.Hq * s.R * chunk_slots(s) * s.d * sizeof(float) + 255) / 256 * 256;
 }
 
-template <int D>
-int launch_chunk_major(const GArgs& a, void* scratch, cudaStream_t stream) {
+// (block, chunk) pairs with blocks of rb tokens, over all KV heads
+long long chunk_ctas(const Shape& s, int rb) {
+    long long n = 0;
+    for (int r = 0; r * rb < s.R; ++r) n += block_chunks(s, rb, r);
+    return n * s.B * s.Hkv;
+}
+
+template <int D, int NW>
+int launch_chunk_kernel(const GArgs& a, int rb, int nh, float* part, float* lam, cudaStream_t stream) {
     const Shape& s = a.s;
     static PerDeviceOnce once;
     if (once.pending()) {
-        if (cudaFuncSetAttribute(generic_chunk_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(ChunkSmem<D>)) != cudaSuccess)
+        if (cudaFuncSetAttribute(generic_chunk_kernel<D, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(ChunkSmem<D, NW>)) != cudaSuccess)
             return HILS_ERR_CUDA;
         once.done();
     }
+    const int nb = (s.R + rb - 1) / rb;
+    int width = 0;
+    for (int y = 0; y < (nb + 1) / 2; ++y) {
+        const int w = block_chunks(s, rb, nb - 1 - y) + (y < nb - 1 - y ? block_chunks(s, rb, y) : 0);
+        width = w > width ? w : width;
+    }
+    return launch_pdl(generic_chunk_kernel<D, NW>, dim3(static_cast<unsigned>(width), static_cast<unsigned>((nb + 1) / 2), static_cast<unsigned>(s.B * s.Hq / nh)), dim3(NW * 32),
+                      sizeof(ChunkSmem<D, NW>), stream, a, rb, nh, part, lam) == cudaSuccess ? 0 : HILS_ERR_CUDA;
+}
+
+template <int D>
+int launch_chunk_major(const GArgs& a, void* scratch, cudaStream_t stream) {
+    const Shape& s = a.s;
     float* part = static_cast<float*>(scratch);
     float* lam = reinterpret_cast<float*>(static_cast<char*>(scratch) + chunk_lam_offset(s));
-    const unsigned chunks = static_cast<unsigned>((s.pos0 + s.R + s.S - 1) / s.S), blocks = static_cast<unsigned>((s.R + kRowBlock - 1) / kRowBlock);
     const long long rows = static_cast<long long>(s.B) * s.Hq * s.R;
-    if (launch_pdl(generic_chunk_kernel<D>, dim3(blocks, chunks, static_cast<unsigned>(s.B * s.Hq)), dim3(kChunkWarps * 32),
-                   sizeof(ChunkSmem<D>), stream, a, part, lam) != cudaSuccess)
+    // Blocks of 128 tokens with all query heads of the KV head and eight warps where there are CTAs enough (3072 tokens, 4 heads, d = 128,
+    // K = 4: 258 -> 151 us for the call; 2635 tokens, 2 heads: 109 -> 89), else blocks of 32 of one head and four warps: more CTAs
+    // with less to do each (600 tokens, 2 heads, d = 128: 25 us, 31 with eight warps; 2048, one head, d = 64: 31, 33).
+    const bool large = chunk_ctas(s, 32) >= 8ll * sm_count();
+    if ((large ? launch_chunk_kernel<D, 8>(a, kRowBlockMax, s.G, part, lam, stream) : launch_chunk_kernel<D, 4>(a, 32, 1, part, lam, stream)) != 0)
         return HILS_ERR_CUDA;
     trace_mark("generic_attend", stream);
     if (launch_pdl(generic_fuse_kernel<D>, dim3(static_cast<unsigned>((rows + kWarpsPerBlock - 1) / kWarpsPerBlock)),
