@@ -18,7 +18,10 @@
 // Bound: HBM (landmarks scanned + selected K / V), and where a call has few units the chain of dependent steps.  One
 // launch per step (decode_fast.cu) drains and ramps between short phases and leaves the memory idle during the
 // selection.  Before / now, B200, us per call through the Python entry points, calls back to back: 1 x 6000 tokens, K = 16:
-// 22.7 / 12.7; 8 x 4K-16K paged, K = 32, W = 512: 49.3 / 28.1; 64 x 64K, K = 32: 142.6 / 118 (5.8 TB/s); 4 x 1M, K = 64: 65.4 / 46.7.
+// 22.7 / 10.7; 8 x 4K-16K paged, K = 32, W = 512: 49.3 / 24.4; 64 x 64K, K = 32: 142.6 / 112.6 (6.1 TB/s); 4 x 1M, K = 64: 65.4 / 43.8;
+// 16 x 8K-32K, four drafts, K = 32: 121 / 56.6.  Before this form of its short steps (landmark tiles asked for ahead of the queries, a
+// tile's biases under its wait, items placed by rank with sel_idx sorted behind the loads, no integer or exactly rounded division on the
+// way) the same calls took 12.7, 28.2, 117.3, 46.8 and 62.2.
 // Draft tokens of one sequence retrieve mostly the same chunks: the union of their selections is loaded once, and all
 // their heads fill the MMA's columns.
 #include "internal.h"
@@ -51,7 +54,7 @@ struct CArgs {
     int* status;
     int cs, lcs;       // CTAs per cluster (a power of two), its logarithm
     int tg;            // tokens of a sequence per unit
-    int gp;            // columns per token: G rounded up to a power of two
+    int lgp;           // logarithm of the columns per token: G rounded up to a power of two
     int list_cap;      // candidates per token a CTA can hold
     // byte offsets behind the buffers
     int off_scores, off_items, off_ids;
@@ -123,27 +126,33 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     uint8_t* bufs = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const Shape& s = a.s;
     const int NW = blockDim.x >> 5, NTH = blockDim.x;
-    const int CS = a.cs, K = s.K, G = s.G, Gp = a.gp;
+    const int CS = a.cs, K = s.K, G = s.G, Gp = 1 << a.lgp;
     uint8_t* tail = bufs + NW * (2 * kHalf) + NW * kLmRow;
     Sm& sm = *reinterpret_cast<Sm*>(tail);
     float* scores = reinterpret_cast<float*>(tail + a.off_scores);           // [TG][list_cap]
     Item* items = reinterpret_cast<Item*>(tail + a.off_items);
-    int* raw_ids = reinterpret_cast<int*>(tail + a.off_ids);                 // [TG][K] the selection, best first
-    int* sel_ids = raw_ids + TG * K;                                         // [TG][K] ascending
+    int* sel_ids = reinterpret_cast<int*>(tail + a.off_ids);                 // [TG][K] the selection, best first
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     uint8_t* kbuf = bufs + warp * (2 * kHalf);                               // this warp's buffers
     uint8_t* vbuf = kbuf + kHalf;
     uint8_t* lmrow = bufs + NW * (2 * kHalf) + warp * kLmRow;
-    const int unit = blockIdx.x / CS, rank = blockIdx.x % CS;
+    const int unit = blockIdx.x >> a.lcs, rank = blockIdx.x & (CS - 1);
+    // quotient by the number of warps (3 or 6) of a number below 98304: the kernel is a chain of short steps, and a division takes as
+    // long as some of them (quotients by CS and by the columns of a token are shifts)
+    auto per_warp = [&](int n) { return static_cast<int>((static_cast<unsigned>(n) * 43691u) >> (NW == 3 ? 17 : 18)); };
     const int kvh = unit % s.Hkv;
     const int ngrp = (s.qps + a.tg - 1) / a.tg;
     const int seq = unit / s.Hkv / ngrp, tok0 = (unit / s.Hkv % ngrp) * a.tg;
     const int ntok = min(a.tg, s.qps - tok0);
     const int query0 = seq * s.qps + tok0;
 
-    if (tid == 0) {
-        for (int i = 0; i < NW; ++i) { mbar_init(&sm.full[i][0], 1); mbar_init(&sm.full[i][1], 1); }
+    if (lane == 0) {                             // (a warp's barriers are its own: it may ask for its first tile before the others are here)
+        mbar_init(&sm.full[warp][0], 1);
+        mbar_init(&sm.full[warp][1], 1);
         mbar_fence_init();
+        fence_proxy_async_smem();
+    }
+    if (tid == 0) {
         tma_prefetch_desc(&map_k);
         tma_prefetch_desc(&map_v);
         tma_prefetch_desc(&map_lm);
@@ -176,6 +185,29 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     const int n_local = ci_max >= 0 ? ci_max - lc_min + 1 : 0;
     const float* bias = a.bias ? a.bias + (static_cast<long long>(seq) * s.Hl + kvh) * s.C : nullptr;
 
+    // tiles of 64 candidates: tile n belongs to CTA n mod CS (its tile n / CS, of warp n / CS mod NW), so that every CTA
+    // sees a sample of the whole sequence
+    const int n_tiles = any_list ? (((nc_max + 63) >> 6) - rank + CS - 1) >> a.lcs : 0;      // this CTA's
+    const int my_tiles = n_tiles > warp ? per_warp(n_tiles - warp + NW - 1) : 0;
+    auto global_id = [&](int i) { return ((((i >> 6) << a.lcs) + rank) << 6) + (i & 63); };   // candidate of list position i
+    const int lm_row0 = (seq * s.Hl + kvh) * s.C;
+
+    // Buffers: the warp's lane 0 refills a buffer once the warp has read it.  Tiles alternate between the two; items put
+    // K (and the landmark row) in the first, V in the second.
+    auto fill_tile = [&](int i) {
+        uint64_t* bar = &sm.full[warp][i & 1];
+        uint8_t* dst = kbuf + (i & 1) * kHalf;
+        const int row = lm_row0 + global_id((warp + i * NW) * 64);
+        mbar_expect_tx(bar, kHalf);
+        tma_load_2d(dst, &map_lm, bar, 0, row);
+        tma_load_2d(dst + 8192, &map_lm, bar, 64, row);
+    };
+    // the first landmark tiles are asked for before everything that the scores need besides
+    if (lane == 0) {
+        if (my_tiles > 0) fill_tile(0);
+        if (my_tiles > 1) fill_tile(1);
+    }
+
     auto item_row = [&](int c) {
         if (c < 0 || c > ci_max) return -1;
         if (!a.block_table) return (seq * s.Hkv + kvh) * s.T + c * kS;
@@ -183,7 +215,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
         return page < 0 || page >= a.num_pages ? -1 : (page * s.Hkv + kvh) * kS;
     };
     // this CTA's share of the local chunks (item q of the unit goes to CTA q mod CS; the local chunks come first)
-    const int my_local = n_local > rank ? (n_local - rank + CS - 1) / CS : 0;
+    const int my_local = n_local > rank ? (n_local - rank + CS - 1) >> a.lcs : 0;
     for (int j = tid; j < my_local; j += NTH) {
         const int c = lc_min + rank + j * CS, row = item_row(c);
         uint32_t f = c < nc_max ? 1u << 16 : 0u;
@@ -196,9 +228,18 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
         items[j] = Item{row < 0 ? -1 : c, row, f};
     }
 
+    // (one token) the rk-th best chunk becomes item n_local + rk of the unit
+    auto place = [&](int rk, int c) {
+        const int at = n_local + rk;
+        if ((at & (CS - 1)) != rank) return;
+        const int row = item_row(c);
+        if (row < 0) set_status(a.status, kDevBadIndex);
+        items[at >> a.lcs] = Item{row < 0 ? -1 : c, row, (1u << 8) | (1u << 16)};
+    };
+
     // column n of the MMAs: token n / Gp, head n % Gp of the group; two words of the column's query per k-step
     auto col_row = [&](const __nv_bfloat16* src, int nt) -> const __nv_bfloat16* {
-        const int col = nt * 8 + g, m = col / Gp, h = col % Gp;
+        const int col = nt * 8 + g, m = col >> a.lgp, h = col & (Gp - 1);
         if (m >= ntok || h >= G) return nullptr;
         return src + (static_cast<long long>(query0 + m) * s.Hq + kvh * G + h) * kD;
     };
@@ -216,23 +257,6 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     uint32_t qf[8][NT][2];
     load_cols(a.q_route, qf);
 
-    // tiles of 64 candidates: tile n belongs to CTA n mod CS (its tile n / CS, of warp n / CS mod NW), so that every CTA
-    // sees a sample of the whole sequence
-    const int n_tiles = any_list ? (((nc_max + 63) >> 6) - rank + CS - 1) >> a.lcs : 0;      // this CTA's
-    const int my_tiles = n_tiles > warp ? (n_tiles - warp + NW - 1) / NW : 0;
-    auto global_id = [&](int i) { return ((((i >> 6) << a.lcs) + rank) << 6) + (i & 63); };   // candidate of list position i
-    const int lm_row0 = (seq * s.Hl + kvh) * s.C;
-
-    // Buffers: the warp's lane 0 refills a buffer once the warp has read it.  Tiles alternate between the two; items put
-    // K (and the landmark row) in the first, V in the second.
-    auto fill_tile = [&](int i) {
-        uint64_t* bar = &sm.full[warp][i & 1];
-        uint8_t* dst = kbuf + (i & 1) * kHalf;
-        const int row = lm_row0 + global_id((warp + i * NW) * 64);
-        mbar_expect_tx(bar, kHalf);
-        tma_load_2d(dst, &map_lm, bar, 0, row);
-        tma_load_2d(dst + 8192, &map_lm, bar, 64, row);
-    };
     auto fill_k = [&](int i) {
         const Item it = items[warp + i * NW];
         uint64_t* bar = &sm.full[warp][0];
@@ -264,8 +288,6 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     const bool early = warp < my_local;           // the warp's first item is a local chunk: requested before the selection
     __syncthreads();
     if (lane == 0) {
-        if (my_tiles > 0) fill_tile(0);
-        if (my_tiles > 1) fill_tile(1);
         if (early && my_tiles == 0) fill_k(0);
         if (early && my_tiles <= 1) fill_v(0);
     }
@@ -274,9 +296,12 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     if (any_list) {
         float umin = INFINITY, umax = -INFINITY;
         for (int i = 0; i < my_tiles; ++i) {
+            const int pos0 = (warp + i * NW) * 64, id0 = global_id(pos0);         // the tile's place in the list, its first candidate
+            float bv[8];                               // (loaded under the wait: behind it, one after the other, they took 5000 cycles)
+#pragma unroll
+            for (int x = 0; x < 8; ++x) bv[x] = bias && id0 + x * 8 + g < nc_max ? bias[id0 + x * 8 + g] : 0.f;
             wait_buf(i & 1);
             const uint32_t tile = smem_u32(kbuf + (i & 1) * kHalf);
-            const int pos0 = (warp + i * NW) * 64, id0 = global_id(pos0);         // the tile's place in the list, its first candidate
             float acc[4][NT][4];
 #pragma unroll
             for (int mt = 0; mt < 4; ++mt)
@@ -303,11 +328,11 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                 for (int hr = 0; hr < 2; ++hr) {
                     const int r = mt * 16 + hr * 8 + g;
                     const bool live = id0 + r < nc_max;
-                    const float bb = (bias && live) ? bias[id0 + r] : 0.f;
+                    const float bb = bv[mt * 2 + hr];
 #pragma unroll
                     for (int nt = 0; nt < NT; ++nt) {
                         // heads of a token: columns m Gp .. m Gp + G - 1
-                        const int h0 = (nt * 8 + 2 * t) % Gp;
+                        const int h0 = (nt * 8 + 2 * t) & (Gp - 1);
                         const float s0 = acc[mt][nt][2 * hr] * s.scale + bb, s1 = acc[mt][nt][2 * hr + 1] * s.scale + bb;
                         auto put = [&](int m, float u, bool writer) {
                             if (m >= ntok || !writer || !live) return;
@@ -322,7 +347,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                             float u = fmaxf(h0 < G ? s0 : -INFINITY, h0 + 1 < G ? s1 : -INFINITY);
                             if (Gp >= 4) u = fmaxf(u, __shfl_xor_sync(kFullMask, u, 1));
                             if (Gp >= 8) u = fmaxf(u, __shfl_xor_sync(kFullMask, u, 2));
-                            put((nt * 8 + 2 * t) / Gp, u, h0 == 0);
+                            put((nt * 8 + 2 * t) >> a.lgp, u, h0 == 0);
                         }
                     }
                 }
@@ -336,8 +361,10 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
         // Each phase below runs once, so its instructions are mostly fetched cold: the loops are rolled and the tokens
         // share the code.  A token's list is walked by NW / ntok warps.
         const int n_list = n_tiles * 64;
-        const int wpt = NW / ntok > 0 ? NW / ntok : 1, li = (warp % wpt) * 32 + lane, ls = wpt * 32;
-        const int m_first = warp / wpt, m_step = NW / wpt;
+        const int wpt = TG == 1 || ntok == 1 ? NW : NW == 3 ? 1 : ntok == 2 ? 3 : ntok == 3 ? 2 : 1;                     // max(1, NW / ntok)
+        const int m_first = wpt == NW ? 0 : wpt == 1 ? warp : wpt == 2 ? warp >> 1 : warp >= 3;                          // warp / wpt
+        const int m_step = wpt == NW ? 1 : wpt == 1 ? NW : wpt == 2 ? 3 : 2;                                             // NW / wpt
+        const int li = (warp - m_first * wpt) * 32 + lane, ls = wpt * 32;
         int n_rank = 0;                            // (rank_all) candidates to rank
         const bool rank_all = nc_max <= Sm::kAll;
         if (rank_all) {
@@ -355,7 +382,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
             __syncthreads();
             // A score that this CTA's share of K of its candidates reach, off a histogram with bins of equal width in the
             // score (the bins of a radix digit are equal in the exponent, and most scores share two or three exponents).
-            const float lo = key_to_float(sm.kmin), inv = static_cast<float>(kBins) / (key_to_float(sm.kmax) - lo);
+            const float lo = key_to_float(sm.kmin), inv = __fdividef(static_cast<float>(kBins), key_to_float(sm.kmax) - lo);
             const bool cut = inv > 0.f && inv < INFINITY;              // (no span: every candidate is collected)
 #pragma unroll 1
             for (int m = m_first; m < ntok; m += m_step) {
@@ -399,7 +426,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                     while (x > 0 && (cum += h[x]) < want) --x;
                     const int b = kBins - kPer * (lane + 1) + x;
                     // (a little below the bin's edge: the bins were found by a rounded product)
-                    if (b > 0) sm.edge[m] = lo + (static_cast<float>(b) - 0.01f) / inv;
+                    if (b > 0) sm.edge[m] = lo + __fdividef(static_cast<float>(b) - 0.01f, inv);
                 }
             }
             cluster_sync(CS);
@@ -515,7 +542,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
             }
         }
         __syncthreads();
-        // the K best by rank, then ascending chunk ids by rank
+        // the K best by rank (their order does not matter to the attention; sel_idx is put in ascending order further down)
 #pragma unroll 1
         for (int m = m_first; m < ntok; m += m_step) {
             if (sm.nc[m] <= K) continue;
@@ -525,19 +552,10 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                 int rk = 0;
 #pragma unroll 4
                 for (int f = 0; f < n; ++f) rk += sm.all[m][f] > mine ? 1 : 0;
-                if (rk < K) raw_ids[m * K + rk] = key_chunk(mine);
-            }
-        }
-        __syncthreads();
-#pragma unroll 1
-        for (int m = m_first; m < ntok; m += m_step) {
-            if (sm.nc[m] <= K) continue;
-            for (int e = li; e < K; e += ls) {
-                const int id = raw_ids[m * K + e];
-                int pos = 0;
-#pragma unroll 4
-                for (int j = 0; j < K; ++j) pos += raw_ids[m * K + j] < id ? 1 : 0;
-                sel_ids[m * K + pos] = id;
+                if (rk < K) {
+                    sel_ids[m * K + rk] = key_chunk(mine);
+                    if (TG == 1) place(rk, key_chunk(mine));
+                }
             }
         }
     }
@@ -545,28 +563,22 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
 #pragma unroll 1
     for (int m = 0; m < ntok; ++m)
         if (sm.nc[m] <= K)
-            for (int e = tid; e < sm.nc[m]; e += NTH) sel_ids[m * K + e] = e;
-    __syncthreads();
+            for (int e = tid; e < sm.nc[m]; e += NTH) {
+                sel_ids[m * K + e] = e;
+                if (TG == 1) place(e, e);
+            }
 
     // ------------------------------------------------------------------------------------------ items
-    int n_items;
-    if (TG == 1) {
-        n_items = n_local + min(K, nc_max);
-        const int my_n = n_items > rank ? (n_items - rank + CS - 1) / CS : 0;
-        for (int j = my_local + tid; j < my_n; j += NTH) {
-            const int c = sel_ids[rank + j * CS - n_local], row = item_row(c);
-            if (row < 0) set_status(a.status, kDevBadIndex);
-            items[j] = Item{row < 0 ? -1 : c, row, (1u << 8) | (1u << 16)};
-        }
-    } else {
-        // union of the tokens' selections in the order (token, id); a chunk belongs to the first token that holds it
-        auto holds = [&](int m, int n, int c) {
-            int l = 0, r = n;
-            while (l < r) {
-                const int mid = (l + r) >> 1;
-                if (sel_ids[m * K + mid] < c) l = mid + 1; else r = mid;
-            }
-            return l < n && sel_ids[m * K + l] == c;
+    int n_items = n_local + min(K, nc_max);
+    if (TG > 1) {
+        __syncthreads();
+        // union of the tokens' selections in the order (token, rank); a chunk belongs to the first token that holds it
+        auto holds = [&](int m, int c) {
+            const int n = c < sm.nc[m] ? min(K, sm.nc[m]) : 0;
+            int hit = 0;
+#pragma unroll 8
+            for (int j = 0; j < n; ++j) hit |= sel_ids[m * K + j] == c ? 1 : 0;
+            return hit != 0;
         };
         int base = n_local;
         for (int x0 = 0; x0 < TG * K; x0 += NTH) {
@@ -579,7 +591,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                 mine = c < lc_min;                                     // chunks of some token's window are local items
 #pragma unroll 1
                 for (int mm = 0; mm < ntok; ++mm)
-                    if (holds(mm, min(K, sm.nc[mm]), c)) {
+                    if (holds(mm, c)) {
                         f |= 1u << (8 + mm);
                         if (mm < m) mine = false;
                     }
@@ -589,12 +601,12 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
             __syncthreads();
             int at = base + __popc(vote & ((1u << lane) - 1u));
             for (int w = 0; w < NW; ++w) { if (w < warp) at += sm.wsum[w]; base += sm.wsum[w]; }
-            if (mine && at % CS == rank) {
+            if (mine && (at & (CS - 1)) == rank) {
                 const int row = item_row(c);
                 if (row < 0) set_status(a.status, kDevBadIndex);
-                items[at / CS] = Item{row < 0 ? -1 : c, row, f};
+                items[at >> a.lcs] = Item{row < 0 ? -1 : c, row, f};
             }
-            __syncthreads();
+            if (x0 + NTH < TG * K) __syncthreads();
         }
         n_items = base;
         for (int j = tid; j < my_local; j += NTH) {
@@ -603,19 +615,28 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
             uint32_t f = items[j].flags;
 #pragma unroll 1
             for (int mm = 0; mm < ntok; ++mm)
-                if (holds(mm, min(K, sm.nc[mm]), c)) f |= 1u << (8 + mm);
+                if (holds(mm, c)) f |= 1u << (8 + mm);
             items[j].flags = f;
         }
     }
     __syncthreads();
-    const int cta_n = n_items > rank ? (n_items - rank + CS - 1) / CS : 0;
-    const int my_n = cta_n > warp ? (cta_n - warp + NW - 1) / NW : 0;           // this warp's items: warp, warp + NW, ...
+    const int cta_n = n_items > rank ? (n_items - rank + CS - 1) >> a.lcs : 0;
+    const int my_n = cta_n > warp ? per_warp(cta_n - warp + NW - 1) : 0;           // this warp's items: warp, warp + NW, ...
     if (lane == 0 && my_n > 0 && !early) { fill_k(0); fill_v(0); }
     if (rank == 0) {
-#pragma unroll 1
-        for (int m = 0; m < ntok; ++m)
-            for (int e = tid; e < K; e += NTH)
-                a.sel[(static_cast<long long>(query0 + m) * s.Hkv + kvh) * K + e] = e < min(K, sm.nc[m]) ? sel_ids[m * K + e] : -1;
+        // ascending chunk ids by rank, then -1
+        for (int x = tid; x < ntok * K; x += NTH) {
+            const int m = TG == 1 ? 0 : x / K, e = x - m * K, nc = sm.nc[m], n = min(K, nc);
+            const int* ids = sel_ids + m * K;
+            const int id = e < n ? ids[e] : -1;
+            int pos = e;
+            if (e < n && nc > K) {
+                pos = 0;
+#pragma unroll 8
+                for (int j = 0; j < n; ++j) pos += ids[j] < id ? 1 : 0;
+            }
+            a.sel[(static_cast<long long>(query0 + m) * s.Hkv + kvh) * K + pos] = id;
+        }
     }
 
     // ------------------------------------------------------------------------------------------ attend
@@ -636,10 +657,11 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
             Mx[nt][x] = kLowestLogit;
             Dn[nt][x] = 0.f;
             const int col = nt * 8 + 2 * t + x;
-            ctok[nt][x] = col % Gp < G ? col / Gp : TG;           // token of the column (TG: none)
+            ctok[nt][x] = (col & (Gp - 1)) < G ? col >> a.lgp : TG;           // token of the column (TG: none)
         }
     for (int i = 0; i < my_n; ++i) {
         const Item it = items[warp + i * NW];
+        const float bb = bias && it.chunk >= 0 && ((it.flags >> 8) & 0xffu) != 0u ? bias[it.chunk] : 0.f;
         wait_buf(0);
         if (it.chunk < 0) {
             wait_buf(1);
@@ -691,7 +713,6 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
         }
         __syncwarp();
         if (lane == 0 && i + 1 < my_n) fill_k(i + 1);
-        const float bb = (bias && any_sel) ? bias[it.chunk] : 0.f;
         float f_[NT][2];
         bool moved = false;
 #pragma unroll
@@ -736,7 +757,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                     const float w = __expf(lam - nm);
                     Dn[nt][x] = fmaf(Dn[nt][x], f_[nt][x], w);
                     Mx[nt][x] = nm;
-                    pw = w / z;
+                    pw = __fdividef(w, z);
                 }
                 moved = moved || f_[nt][x] != 1.f;
 #pragma unroll
@@ -812,16 +833,16 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     }
     __syncthreads();
     auto emit = [&](int cx, int dim, float v, float M, float den) {
-        const int m = cx / G, h = cx % G;
+        const int m = TG == 1 ? 0 : cx / G, h = cx - m * G;
         const bool live = sm.len[m] > 0;
         const long long orow = static_cast<long long>(query0 + m) * s.Hq + kvh * G + h;
-        a.out[orow * kD + dim] = __float2bfloat16_rn(live ? v / den : 0.f);
+        a.out[orow * kD + dim] = __float2bfloat16_rn(live ? __fdividef(v, den) : 0.f);
         if (dim == 0) a.lse[orow] = live ? M + __logf(den) : 0.f;
     };
     // the warps' sums (fixed order: deterministic); a warp takes a column at a time, the result replaces warp 0's
 #pragma unroll 1
     for (int cx = warp; cx < ntok * G; cx += NW) {
-        const int col = (cx / G) * Gp + cx % G;
+        const int m = TG == 1 ? 0 : cx / G, col = m * Gp + cx - m * G;
         const float mw = lane < NW ? sm.col_max[lane][col] : -INFINITY;
         const float M = warp_max(mw), fw = mw == -INFINITY ? 0.f : __expf(mw - M);
         const float den = warp_sum(lane < NW ? sm.col_den[lane][col] * fw : 0.f);
@@ -849,7 +870,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     // a quarter of a column of the unit (32 dimensions) per warp of the cluster
 #pragma unroll 1
     for (int qx = rank * NW + warp; qx < ntok * G * 4; qx += CS * NW) {
-        const int cx = qx >> 2, col = (cx / G) * Gp + cx % G;
+        const int cx = qx >> 2, m = TG == 1 ? 0 : cx / G, col = m * Gp + cx - m * G;
         // lane r: CTA r's maximum and denominator
         const float mr = lane < CS ? ld_peer_f(peer_addr(smem_u32(&sm.col_max[0][col]), lane)) : -INFINITY;
         const float dr = lane < CS ? ld_peer_f(peer_addr(smem_u32(&sm.col_den[0][col]), lane)) : 0.f;
@@ -968,7 +989,7 @@ bool plan_tokens(const Shape& s, int tg, int n_sm, ClusterPlan* p) {
         auto take = [&](size_t bytes) { const size_t at = (off + 15) / 16 * 16; off = at + bytes; return static_cast<int>(at); };
         p->off_scores = take(sizeof(float) * TG * p->list_cap);
         p->off_items = take(sizeof(Item) * ((TG * s.K + local + cs - 1) / cs + 1));
-        p->off_ids = take(sizeof(int) * 2 * TG * s.K);
+        p->off_ids = take(sizeof(int) * TG * s.K);
         p->smem = 1024 + off + static_cast<size_t>(p->warps) * (2 * kHalf + kLmRow);
         if (p->smem <= (per_sm == 2 ? 115712u : 232448u)) return true;
     }
@@ -1018,7 +1039,8 @@ int launch_decode_cluster(const Shape& s, const Tensors& t, cudaStream_t stream)
     a.cs = p.cs;
     a.lcs = p.lcs;
     a.tg = p.tg;
-    a.gp = p.gp;
+    a.lgp = 0;
+    while ((1 << a.lgp) < p.gp) ++a.lgp;
     a.list_cap = p.list_cap;
     a.off_scores = p.off_scores;
     a.off_items = p.off_items;

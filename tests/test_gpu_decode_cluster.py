@@ -107,3 +107,24 @@ def test_lists_that_leave_some_ctas_few_candidates_or_none(n, K, W):
     got = hils.hils_decode(g["q"], g["k"], g["v"], g["landmarks"], g["seq_lens"], 64, K, window=W)
     torch.cuda.synchronize()
     check_decode(cfg, inp, *got, W=W)
+
+
+@pytest.mark.parametrize("B,M,K", [(16, 3, 17), (32, 3, 16), (20, 4, 16), (40, 2, 33)])
+def test_groups_of_draft_tokens_on_six_and_on_three_warps(B, M, K):
+    """A group's tokens share the selection's warps (max(1, warps / tokens) each); the chunks are attended in the order of their
+    scores and reported in ascending order."""
+    cfg = wl.HilsConfig("groups", "decode", B, 32, 8, 64 * 90, 128, 64, K, "bf16", 800 + M * B, n_needles=2, window=1)
+    lens = torch.tensor([64 * 90 - (b * 371) % (64 * 80) for b in range(B)], dtype=torch.int32)
+    t = wl.make_decode_inputs(cfg, DEV, seq_lens=lens.to(DEV))
+    q = torch.randn((B, M, 32, 128), generator=torch.Generator().manual_seed(M)).to(torch.bfloat16).to(DEV)
+    out, lse, sel = hils.hils_decode_multi(q, t["k"], t["v"], t["landmarks"], t["seq_lens"], 64, K)
+    torch.cuda.synchronize()
+    assert hils.last_launch_count() == 1
+    for m in range(M):
+        o, l, s = hils.hils_decode(q[:, m].contiguous(), t["k"], t["v"], t["landmarks"], t["seq_lens"] - (M - 1 - m), 64, K)
+        torch.cuda.synchronize()
+        assert torch.equal(s, sel[:, m])
+        held = torch.where(s < 0, torch.iinfo(torch.int32).max, s)
+        assert (held[..., 1:] >= held[..., :-1]).all()
+        # (two roundings to bf16 of sums in different orders, outputs below 2: twice 2^-8 = 8e-3)
+        assert (o.float() - out[:, m].float()).abs().max() <= 1.6e-2 and (l - lse[:, m]).abs().max() <= 1e-4
