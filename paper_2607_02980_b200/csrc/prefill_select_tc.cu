@@ -103,26 +103,13 @@ __device__ __forceinline__ void bitonic_merge_desc(float (&a)[N]) {
     }
 }
 
-// Entry (score, chunk) to the shared-memory address `at` if the score beats `tau`, and `at` to the next entry.
-__device__ __forceinline__ void append_if(uint32_t& at, float score, float tau, int chunk) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.gt.f32 p, %1, %2;\n\t"
-        "@p st.shared.v2.b32 [%0], {%3, %4};\n\t"
-        "@p add.u32 %0, %0, %5;\n\t}"
-        : "+r"(at) : "f"(score), "f"(tau), "r"(chunk), "r"(__float_as_uint(score)), "n"(8 * kTileTok) : "memory");
+// Entries are compacted by storing each where the kept ones end so far and moving the end only if it is kept.  The addresses are
+// worked out before the stores, each in a register of its own: an address that is advanced behind its store waits until the store
+// has read it (34 cycles per candidate, 2170 of a step's 6230; the stores' predicates and the kept entries' filter the same).
+__device__ __forceinline__ void st_entry(uint32_t at, uint32_t chunk, float score) {
+    asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(at), "r"(chunk), "r"(__float_as_uint(score)) : "memory");
 }
-// The entry to `at` if its score is at least `tau` and `valid`, and `at` to the next entry.
-__device__ __forceinline__ void keep_if(uint32_t& at, unsigned long long raw, float tau, bool valid) {
-    asm volatile(
-        "{\n\t.reg .pred p, v;\n\t"
-        "setp.ne.b32 v, %4, 0;\n\t"
-        "setp.ge.and.f32 p, %2, %3, v;\n\t"
-        "@p st.shared.b64 [%0], %1;\n\t"
-        "@p add.u32 %0, %0, %5;\n\t}"
-        : "+r"(at) : "l"(raw), "f"(__uint_as_float(static_cast<uint32_t>(raw >> 32))), "f"(tau), "r"(static_cast<int>(valid)), "n"(8 * kTileTok)
-        : "memory");
-}
+__device__ __forceinline__ void st_entry(uint32_t at, unsigned long long raw) { asm volatile("st.shared.b64 [%0], %1;" ::"r"(at), "l"(raw) : "memory"); }
 
 // N = length of the per-token sorted score list: 16 for K <= 16, else 32.
 // PERHEAD: one landmark row (and bias) per query head (App. C) instead of one per KV head.  A template parameter, not
@@ -341,7 +328,7 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                         }
                     } else {
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) u16[j] = fmaxf(fmax3(r[0][j], r[1][j], r[2][j]), r[3][j]) * s.scale;
+                        for (int j = 0; j < 16; ++j) u16[j] = fmaf(fmaxf(fmax3(r[0][j], r[1][j], r[2][j]), r[3][j]), s.scale, 0.0f);   // (no -0)
                         if (bias) {
                             const float* bp = bias + cbase;
                             if (cbase + 16 <= s.C) {
@@ -352,8 +339,6 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                                 for (int j = 0; j < 16; ++j) u16[j] += __ldg(bias + min(cbase + j, s.C - 1));
                             }
                         }
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) u16[j] += 0.0f;       // -0 folds into +0: scores compare as numbers
                     }
                     if (tail) {
 #pragma unroll
@@ -375,8 +360,14 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                             acquire();
                         }
                         const float tau = *tau_sm;
+                        uint32_t to[8];
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) append_if(at, u16[8 * h + j], tau, c0 + 8 * h + j);
+                        for (int j = 0; j < 8; ++j) {                    // (there is room for all eight)
+                            to[j] = at;
+                            at += u16[8 * h + j] > tau ? 8 * kTileTok : 0;
+                        }
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) st_entry(to[j], c0 + 8 * h + j, u16[8 * h + j]);
                     }
                 }
             }
@@ -435,10 +426,16 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
 #pragma unroll 1
             for (int e0 = 0; e0 < cnt; e0 += 8) {
                 unsigned long long old[8];
+                uint32_t at[8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) old[j] = pool[(e0 + j) * kTileTok];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) keep_if(to, old[j], tau, e0 + j < cnt);     // to <= the entry: in place, in order
+                for (int j = 0; j < 8; ++j) {                           // (to <= the entry: in place, in order)
+                    at[j] = to;
+                    to += __uint_as_float(static_cast<uint32_t>(old[j] >> 32)) >= tau && e0 + j < cnt ? 8 * kTileTok : 0;
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) st_entry(at[j], old[j]);
             }
             cnt = static_cast<int>(to - pool_at) / (8 * kTileTok);
             uint32_t live = 0;                                  // new entries that stay
@@ -465,8 +462,15 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                     }
             }
             to = pool_at + cnt * (8 * kTileTok);
+            uint32_t at[kRoom];
 #pragma unroll
-            for (int e = 0; e < kRoom; ++e) keep_if(to, raw[e], -INFINITY, ((live >> e) & 1u) != 0);
+            for (int e = 0; e < kRoom; ++e) {
+                at[e] = to;
+                to += ((live >> e) & 1u) * (8 * kTileTok);
+            }
+#pragma unroll
+            for (int e = 0; e < kRoom; ++e)
+                if ((live >> e) & 1u) st_entry(at[e], raw[e]);          // (the pool may be full)
             cnt = static_cast<int>(to - pool_at) / (8 * kTileTok);
         }
         tn += nsteps > 0 ? 1 : 0;
