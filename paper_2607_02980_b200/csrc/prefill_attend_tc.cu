@@ -273,6 +273,10 @@ prefill_attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
                 tc_fence_after_sync();
                 // the tile's P V MMAs are done: after the chunk's last tile its V tile may be overwritten
                 if (ow == 0 && lane == 0 && (flags & 512)) mbar_arrive(&sm.v_empty[run % kVBufs]);
+                if (8 * ow >= (flags & 255)) {           // a ragged tile without entries for this warp: nothing of it is read later
+                    if (lane == 0) mbar_arrive(&sm.o_empty[sl]);
+                    continue;
+                }
                 // The accumulator leaves tensor memory in four quarters of 32 columns; the load of the next quarter runs
                 // under the packing and staging of the current one.
                 uint32_t va[32], vb[32];
@@ -331,7 +335,7 @@ prefill_attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
             const AtcTile& tl = sm.tile[n % kMeta];
             const int pair = tl.pair, i0 = tl.i0;
             // this lane's entry (rows past a ragged tile's last entry repeat that entry)
-            const int e = tl.ent[min(el, (tl.flags & 255) - 1)];
+            const int n_ent = tl.flags & 255, e = tl.ent[min(el, n_ent - 1)];
             tile_done(n);
             const uint32_t qs = n % kQSlots;
             if (n >= kQSlots && !wait(&sm.q_empty[qs], ((n / kQSlots) - 1) & 1)) break;
@@ -340,15 +344,18 @@ prefill_attend_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid
                                        static_cast<long long>(i0) * kD + p16 * 8;
             // the tokens of the warp's entries first (shuffles and copies are both ordered operations: interleaved
             // they would run strictly one after the other)
-            int tokv[kPerWarp / 2];
+            // (a ragged tile without entries for this warp: its rows keep what the slot held, and their results are dropped)
+            if (8 * gw < n_ent) {
+                int tokv[kPerWarp / 2];
 #pragma unroll
-            for (int k = 0; k < kPerWarp / 2; ++k) tokv[k] = __shfl_sync(kFullMask, e, k) >> 8;
+                for (int k = 0; k < kPerWarp / 2; ++k) tokv[k] = __shfl_sync(kFullMask, e, k) >> 8;
 #pragma unroll
-            for (int jj = 0; jj < kPerWarp; ++jj) {
-                const int j = j0 + jj;
-                const int row = 2 * j + hh;
-                const __nv_bfloat16* src = qb0 + (2 * j & 3) * hstride + static_cast<long long>(tokv[jj >> 1]) * kD;
-                cp_async16(qaddr + swz128(row, p16 & 7), src);
+                for (int jj = 0; jj < kPerWarp; ++jj) {
+                    const int j = j0 + jj;
+                    const int row = 2 * j + hh;
+                    const __nv_bfloat16* src = qb0 + (2 * j & 3) * hstride + static_cast<long long>(tokv[jj >> 1]) * kD;
+                    cp_async16(qaddr + swz128(row, p16 & 7), src);
+                }
             }
             // the tile's barrier hears from every gather thread when that thread's copies have landed (no thread waits for them)
             asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&sm.q_full[qs])) : "memory");
