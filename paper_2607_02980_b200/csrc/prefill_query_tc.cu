@@ -24,6 +24,8 @@
 // 750 (two warps per scheduler; special-function unit 37 % busy), weight 200, accumulator's answer 170, probabilities back 190.  The
 // tensor pipe needs 1350 of them.  2 x 6000 tokens, K = 32: 661 -> 587 us with the quotient w / z by the approximate reciprocal (the
 // exactly rounded division took 300 cycles of the chain; its result is rounded to bf16 next) and the next item's barrier asked early.
+// A unit's fixed part: 9300 -> 5000 cycles with the output staged beside the query tile, so that the next unit's queries come with this
+// one's last scores, and the unit's place worked out once, by the list warp (2 x 6000 tokens 587 -> 571 us, 3 x 1000 44.9 -> 41.8).
 // Sixteen softmax warps, half a row's keys or every other item each: 704 and 781 us (more instructions, colder instruction cache).
 #include "internal.h"
 #include "tma.cuh"
@@ -41,8 +43,10 @@ constexpr int kNS = 80;                         // score columns: 64 keys + land
 constexpr int kKBytes = kNS * kD * 2;
 constexpr int kVBytes = kS * kD * 2;
 constexpr int kQBytes = kRows * kD * 2;
-constexpr int kStages = 4;
-constexpr int kMaxC = 160;                      // chunks a unit may see
+constexpr int kStages = 3;
+constexpr int kStgBytes = kTok * 128;           // staging of a softmax warp's output: its 32 rows x 64 dimensions
+constexpr int kMaxK = 64;                       // selected chunks per token
+constexpr int kMaxC = 256;                      // chunks a unit may see
 constexpr int kPCol = 96;                       // columns of a tile: scores 0..79, probabilities 96..127, output 128..255
 constexpr int kOCol = 128;
 constexpr int kMmaWarp = 8, kLoadWarp = 10;           // (and warp 11, the list)
@@ -67,17 +71,27 @@ struct QmSmem {
     uint64_t kv_full[kStages], kv_empty[kStages];
     uint64_t q_full[2], q_empty[2];
     uint64_t s_full[2], s_empty[2], p_full[2], o_done[2];
-    uint64_t list_full[2], list_empty[2];
+    uint64_t list_full[2], list_empty[2], ids_full;
+    alignas(16) int32_t ids[kMaxK * kTok];      // (list builder) selections of 64 tokens (of 32, more than 32 chunks each)
     uint32_t tmem_base;
+    int blk[2], pair[2], seq[2];                // [list] the unit: its block of tokens, (sequence, KV head), sequence
     int n_items[2];                             // items of the unit's list
     int base[2];                                // first chunk of the unit (lists and masks count from it)
-    int parts[2];                               // bit t: tile t has items
     int list[2][kMaxC];                         // chunk | tile 0 needs it << 16 | tile 1 needs it << 17
     uint32_t mask[2][kMaxC];                    // (list builder) [tile][chunk]: tokens that attend it
     int n_tile[2][2];                           // [list][tile]: items of the tile
     int2 titem[2][2][kMaxC];                    // [list][tile][item]: chunk, tokens that attend it
 };
-static_assert(kStages * (kKBytes + kVBytes) + 2 * kQBytes + sizeof(QmSmem) + 1024 <= 232448, "shared memory of the query-major kernel");
+static_assert(kStages * (kKBytes + kVBytes) + 2 * kQBytes + kMmaWarp * kStgBytes + sizeof(QmSmem) + 1024 <= 232448, "shared memory of the query-major kernel");
+
+// bit x of a word (none for x < 0 and x > 31)
+__device__ __forceinline__ uint32_t bit_or_none(int x) {
+    uint32_t r;
+    asm("shl.b32 %0, 1, %1;" : "=r"(r) : "r"(x));                       // (the count is unsigned and saturates at 32)
+    return r;
+}
+// the lowest n bits (n < 0: none, n > 31: all)
+__device__ __forceinline__ uint32_t bits_below(int n) { return bit_or_none(max(n, 0)) - 1u; }
 
 // 2^x of two values on the FMA pipes: x = n + f with f in [-1/2, 1/2] (Cody-Waite), a polynomial of degree 5 in f fitted
 // to the smallest relative error (1e-7), n added to the exponent.  A quarter of a row's exponentials goes this way: the
@@ -104,7 +118,8 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
     uint8_t* kbuf = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* vbuf = kbuf + kStages * kKBytes;
     uint8_t* qbuf = vbuf + kStages * kVBytes;
-    QmSmem& sm = *reinterpret_cast<QmSmem*>(qbuf + 2 * kQBytes);
+    uint8_t* stage = qbuf + 2 * kQBytes;
+    QmSmem& sm = *reinterpret_cast<QmSmem*>(stage + kMmaWarp * kStgBytes);
     const Shape& s = a.s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int pairs = s.B * s.Hkv, blk0 = a.first / kUnitTok, n_blk = (a.n_tok - a.first + kUnitTok - 1) / kUnitTok, n_units = pairs * n_blk;
@@ -112,11 +127,12 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
     if (tid == 0) {
         for (int i = 0; i < kStages; ++i) { mbar_init(&sm.kv_full[i], 1); mbar_init(&sm.kv_empty[i], 2); }
         for (int t = 0; t < 2; ++t) {
-            mbar_init(&sm.q_full[t], 1); mbar_init(&sm.q_empty[t], 4);
+            mbar_init(&sm.q_full[t], 1); mbar_init(&sm.q_empty[t], 1);
             mbar_init(&sm.s_full[t], 1); mbar_init(&sm.s_empty[t], 4);
             mbar_init(&sm.p_full[t], 4); mbar_init(&sm.o_done[t], 1);
             mbar_init(&sm.list_full[t], 1); mbar_init(&sm.list_empty[t], 11);
         }
+        mbar_init(&sm.ids_full, 1);
         mbar_fence_init();
         tma_prefetch_desc(&map_q);
         tma_prefetch_desc(&map_k);
@@ -162,12 +178,10 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
         const float sl2 = s.scale * kLog2e;
         uint32_t n_s = 0, n_u = 0;               // items of this tile / units so far
         for (int idx = blockIdx.x; idx < n_units && ok; idx += gridDim.x, ++n_u) {
-            int blk, pair;
-            unit_of(idx, blk, pair);
             const int ln = n_u & 1;
             if (!wait(&sm.list_full[ln], (n_u >> 1) & 1)) break;
             const int n = sm.n_tile[ln][t];
-            const int b = pair / s.Hkv, gk = pair % s.Hkv;
+            const int blk = sm.blk[ln], pair = sm.pair[ln], b = sm.seq[ln], gk = pair - b * s.Hkv;
             const int tok = blk * kUnitTok + t * kTok + lane;
             const bool live = tok < a.n_tok;
             const int pos = lane_position(s, tok, a.n_tok), lc = local_lo(pos, s.W, kS) / kS;
@@ -277,39 +291,46 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                 // ---- the tile's output rows
                 if (!wait(&sm.o_done[t], (n_s - 1) & 1)) break;
                 tc_fence_after_sync();
-                const float inv = live ? 1.f / den : 0.f;
+                const float inv = live ? __fdividef(1.f, den) : 0.f;
                 const long long orow = (static_cast<long long>(b) * s.Hq + gk * kG + h) * s.R + tok;
                 const bool whole = blk * kUnitTok + t * kTok + kTok <= a.n_tok;
-                uint8_t* stg = qbuf + t * kQBytes + h * 4096;            // this head's rows of the (no longer needed) query tile
+                // 64 dimensions at a time through the warp's own staging rows (not through the query tile: the next unit's queries
+                // are on their way into it)
+                uint8_t* stg = stage + warp * kStgBytes;
 #pragma unroll
-                for (int half = 0; half < 4; ++half) {
-                    uint32_t v[32];
-                    tmem_ld32_issue(t_lane + kOCol + half * 32, v);
-                    tmem_ld_wait32(v);
+                for (int half = 0; half < 2; ++half) {
+                    uint4 w[8];
 #pragma unroll
-                    for (int pc = 0; pc < 4; ++pc) {
-                        uint4 w;
-                        w.x = pack_bf16(__uint_as_float(v[8 * pc]) * inv, __uint_as_float(v[8 * pc + 1]) * inv);
-                        w.y = pack_bf16(__uint_as_float(v[8 * pc + 2]) * inv, __uint_as_float(v[8 * pc + 3]) * inv);
-                        w.z = pack_bf16(__uint_as_float(v[8 * pc + 4]) * inv, __uint_as_float(v[8 * pc + 5]) * inv);
-                        w.w = pack_bf16(__uint_as_float(v[8 * pc + 6]) * inv, __uint_as_float(v[8 * pc + 7]) * inv);
-                        if (whole) *reinterpret_cast<uint4*>(stg + (half >> 1) * 16384 + swz128(lane, (half & 1) * 4 + pc)) = w;
-                        else if (live) *reinterpret_cast<uint4*>(a.out + orow * kD + half * 32 + pc * 8) = w;
+                    for (int q = 0; q < 2; ++q) {
+                        uint32_t v[32];
+                        tmem_ld32_issue(t_lane + kOCol + half * 64 + q * 32, v);
+                        tmem_ld_wait32(v);
+#pragma unroll
+                        for (int pc = 0; pc < 4; ++pc) {
+                            w[4 * q + pc].x = pack_bf16(__uint_as_float(v[8 * pc]) * inv, __uint_as_float(v[8 * pc + 1]) * inv);
+                            w[4 * q + pc].y = pack_bf16(__uint_as_float(v[8 * pc + 2]) * inv, __uint_as_float(v[8 * pc + 3]) * inv);
+                            w[4 * q + pc].z = pack_bf16(__uint_as_float(v[8 * pc + 4]) * inv, __uint_as_float(v[8 * pc + 5]) * inv);
+                            w[4 * q + pc].w = pack_bf16(__uint_as_float(v[8 * pc + 6]) * inv, __uint_as_float(v[8 * pc + 7]) * inv);
+                        }
+                    }
+                    if (whole) {
+                        if (lane == 0) bulk_wait_read<0>();              // (the store before)
+                        __syncwarp();
+#pragma unroll
+                        for (int pc = 0; pc < 8; ++pc) *reinterpret_cast<uint4*>(stg + swz128(lane, pc)) = w[pc];
+                        fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0) {
+                            tma_store_2d(&map_out, stg, half * 64, static_cast<int>(orow), l2_policy_evict_first());
+                            bulk_commit();
+                        }
+                    } else if (live) {
+#pragma unroll
+                        for (int pc = 0; pc < 8; ++pc) *reinterpret_cast<uint4*>(a.out + orow * kD + half * 64 + pc * 8) = w[pc];
                     }
                 }
                 tc_fence_before_sync();
                 if (live) a.lse[orow] = ref + __logf(den);
-                if (whole) {
-                    fence_proxy_async_smem();
-                    __syncwarp();
-                    if (lane < 2) {
-                        tma_store_2d(&map_out, stg + lane * 16384, lane * 64, static_cast<int>(orow) - lane, l2_policy_evict_first());
-                        bulk_commit();
-                        bulk_wait_read<0>();
-                    }
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sm.q_empty[t]);
             }
             if (a.write_sel && h == 0 && live) {
                 int32_t* sel = a.sel + (static_cast<long long>(pair) * s.R + tok) * s.K;
@@ -318,6 +339,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.list_empty[ln]);
         }
+        if (lane == 0) bulk_wait_read<0>();
     } else if (warp < kLoadWarp) {
         // ================================================================ MMA issuer of tile t
         {
@@ -335,6 +357,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                 const int ln = n_u & 1;
                 if (!wait(&sm.list_full[ln], (n_u >> 1) & 1)) break;
                 const int n = sm.n_items[ln];
+                int left = sm.n_tile[ln][t];                             // scores of this tile still to be issued
                 bool have_q = false, first = true;
                 int issued = -1;                                         // last item whose scores were issued
                 auto issue_s = [&](int i) {
@@ -351,8 +374,10 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                             umma_bf16(s_tm, umma_desc_k128(qa + (ks >> 2) * 16384 + (ks & 3) * 32),
                                       umma_desc_k128(ka + (ks >> 2) * (kNS * 128) + (ks & 3) * 32), idesc_s, ks > 0 ? 1u : 0u);
                         umma_commit(&sm.s_full[t]);
+                        if (left == 1) umma_commit(&sm.q_empty[t]);      // the next unit's queries may come
                     }
                     __syncwarp();
+                    --left;
                     ++n_s;
                     issued = i;
                 };
@@ -390,12 +415,26 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
         if (lane == 0) {
             uint32_t g = 0, n_u = 0, n_q[2] = {0, 0};
             for (int idx = blockIdx.x; idx < n_units && ok; idx += gridDim.x, ++n_u) {
+                const int ln = n_u & 1;
                 int blk, pair;
                 unit_of(idx, blk, pair);
-                const int ln = n_u & 1;
-                if (!wait(&sm.list_full[ln], (n_u >> 1) & 1)) break;
-                const int n = sm.n_items[ln], parts = sm.parts[ln], base = sm.base[ln];
-                const int b = pair / s.Hkv, gk = pair % s.Hkv;
+                const int b = pair / s.Hkv, gk = pair - b * s.Hkv;
+                auto load_q = [&] {
+                    for (int t = 0; t < 2 && ok; ++t) {
+                        if (blk * kUnitTok + t * kTok >= a.n_tok) continue;       // (a token attends its own chunk at least)
+                        if (n_q[t] > 0 && !wait(&sm.q_empty[t], (n_q[t] - 1) & 1)) break;
+                        mbar_expect_tx(&sm.q_full[t], kQBytes);
+                        for (int h = 0; h < kG; ++h) {
+                            const int row = (b * s.Hq + gk * kG + h) * s.R + blk * kUnitTok + t * kTok;
+                            tma_load_2d(qbuf + t * kQBytes + h * 4096, &map_q, &sm.q_full[t], 0, row);
+                            tma_load_2d(qbuf + t * kQBytes + 16384 + h * 4096, &map_q, &sm.q_full[t], 64, row);
+                        }
+                        ++n_q[t];
+                    }
+                };
+                if (n_u == 0) load_q();                                  // (under the making of the first list)
+                if (!ok || !wait(&sm.list_full[ln], (n_u >> 1) & 1)) break;
+                const int n = sm.n_items[ln], base = sm.base[ln];
                 auto load_item = [&](int i) {
                     const uint32_t st = g % kStages;
                     const int c = base + (sm.list[ln][i] & 0xffff);
@@ -417,20 +456,10 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                     tma_load_3d(vbuf + st * kVBytes + 8192, &map_v, &sm.kv_full[st], 64, row, pair);
                     ++g;
                 };
-                // the first chunks before the queries: their buffers are free before the last unit's rows have been written
+                // in the order in which the buffers become free: the first chunk's, the queries' with the last unit's last scores
                 int i = 0;
-                for (; i < n && i < kStages && ok; ++i) load_item(i);
-                for (int t = 0; t < 2 && ok; ++t) {
-                    if (!((parts >> t) & 1)) continue;
-                    if (n_q[t] > 0 && !wait(&sm.q_empty[t], (n_q[t] - 1) & 1)) break;
-                    mbar_expect_tx(&sm.q_full[t], kQBytes);
-                    for (int h = 0; h < kG; ++h) {
-                        const int row = (b * s.Hq + gk * kG + h) * s.R + blk * kUnitTok + t * kTok;
-                        tma_load_2d(qbuf + t * kQBytes + h * 4096, &map_q, &sm.q_full[t], 0, row);
-                        tma_load_2d(qbuf + t * kQBytes + 16384 + h * 4096, &map_q, &sm.q_full[t], 64, row);
-                    }
-                    ++n_q[t];
-                }
+                if (n > 0) load_item(i++);
+                if (n_u > 0) load_q();
                 for (; i < n && ok; ++i) load_item(i);
                 mbar_arrive(&sm.list_empty[ln]);
             }
@@ -439,7 +468,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
         }
     } else {
         // ================================================================ the unit's chunk list, one unit ahead
-        uint32_t n_u = 0;
+        uint32_t n_u = 0, n_ids = 0;
         for (int idx = blockIdx.x; idx < n_units && ok; idx += gridDim.x, ++n_u) {
             int blk, pair;
             unit_of(idx, blk, pair);
@@ -448,44 +477,63 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             const int tok0 = blk * kUnitTok;
             const int last = s.pos0 + min(a.n_tok, tok0 + kUnitTok) - 1;
             const int base = a.local ? local_lo(s.pos0 + tok0, s.W, kS) / kS : 0, n_vis = last / kS + 1 - base;
-            for (int c = lane; c < n_vis; c += 32) { sm.mask[0][c] = 0u; sm.mask[1][c] = 0u; }
-            __syncwarp();
-            for (int t = 0; t < 2; ++t) {
-                const int tok = tok0 + t * kTok + lane, pos = s.pos0 + tok;
-                const bool live = tok < a.n_tok;
-                const int lc = live ? local_lo(pos, s.W, kS) / kS : 0;
-                const uint32_t bit = 1u << lane;
-                if (a.local) {
-                    // (nothing to select)
-                } else if (__all_sync(kFullMask, !live || lc <= s.K)) {
-                    // every token takes all its candidates
-                    const int most = __reduce_max_sync(kFullMask, lc);
-                    for (int c = 0; c < most; ++c) {
-                        const unsigned who = __ballot_sync(kFullMask, live && c < lc);
-                        if (lane == 0) sm.mask[t][c] = who;
-                    }
-                } else if (live) {
-                    const int32_t* sel = a.sel + (static_cast<long long>(pair) * s.R + tok) * s.K;
+            // The first list of a CTA is waited for, and its instructions come from memory: short loops.  (2 x 6000 tokens, K = 32, cycles:
+            // an atomic in shared memory per selected chunk 13000 - 26000, bits per token turned by votes, unrolled, 28000.)
+            const bool picks = !a.local && local_lo(last, s.W, kS) / kS > s.K;       // some token has more candidates than places
+            if (picks) {
+                for (int c = lane; c < n_vis; c += 32) { sm.mask[0][c] = 0u; sm.mask[1][c] = 0u; }
+                __syncwarp();
+                // the selections of 64 (32 where they are long) tokens at a time
+                const int step = s.K <= 32 ? kUnitTok : kTok;
+#pragma unroll 1
+                for (int x0 = 0; x0 < kUnitTok; x0 += step) {
+                    const int nx = min(step, a.n_tok - tok0 - x0), words = nx * s.K;
+                    if (nx <= 0) break;
+                    const int32_t* sel = a.sel + (static_cast<long long>(pair) * s.R + tok0 + x0) * s.K;
+                    if (((reinterpret_cast<uintptr_t>(sel) | static_cast<uintptr_t>(4 * words)) & 15) == 0) {
+                        if (lane == 0) {
+                            mbar_expect_tx(&sm.ids_full, 4 * words);
+                            bulk_load(sm.ids, sel, 4 * words, &sm.ids_full);
+                        }
+                        __syncwarp();
+                        if (!wait(&sm.ids_full, n_ids++ & 1)) break;
+                    } else {
 #pragma unroll 8
-                    for (int x = 0; x < s.K; ++x) {
-                        const int c = sel[x];
-                        if (c >= 0 && c < n_vis) atomicOr(&sm.mask[t][c], bit);
+                        for (int y = lane; y < words; y += 32) sm.ids[y] = sel[y];
                     }
+                    __syncwarp();
+                    // lane = token, which starts at its own slot: neighbours' slots lie K words apart
+#pragma unroll 1
+                    for (int y0 = 0; y0 < nx; y0 += kTok) {
+                        const int32_t* id = sm.ids + (y0 + lane) * s.K;
+                        uint32_t* mask = sm.mask[(x0 + y0) / kTok];
+                        if (y0 + lane < nx) {
+                            int e = lane % s.K;
+#pragma unroll 4
+                            for (int i = 0; i < s.K; ++i) {
+                                const int c = id[e];
+                                if (c >= 0 && c < n_vis) atomicOr(mask + c, 1u << lane);
+                                e = e + 1 < s.K ? e + 1 : 0;
+                            }
+                        }
+                        __syncwarp();
+                    }
+                    __syncwarp();
                 }
-                __syncwarp();
-                // chunks of the local windows
-                if (live)
-                    for (int c = lc; c <= pos / kS; ++c) atomicOr(&sm.mask[t][c - base], bit);
-                __syncwarp();
+                if (!ok) break;
             }
             int n = 0, nt[2] = {0, 0};
+#pragma unroll 1
             for (int c0 = 0; c0 < n_vis; c0 += 32) {
                 const int c = c0 + lane;
                 const uint32_t below = (1u << lane) - 1u;
                 uint32_t m[2];
 #pragma unroll
                 for (int t = 0; t < 2; ++t) {
-                    m[t] = c < n_vis ? sm.mask[t][c] : 0u;
+                    // token x of the tile sees chunk c from x = own on, and as a candidate (left of its window) from x = left on
+                    const int first = s.pos0 + tok0 + t * kTok, own = (base + c) * kS - first, left = (base + c + 1) * kS + s.W - 1 - first;
+                    const uint32_t live = bits_below(a.n_tok - tok0 - t * kTok), seen = ~bits_below(own), cand = ~bits_below(left);
+                    m[t] = c < n_vis ? live & ((seen & ~cand) | (a.local ? 0u : picks ? sm.mask[t][c] : cand)) : 0u;
                     const unsigned v = __ballot_sync(kFullMask, m[t] != 0u);
                     if (m[t]) sm.titem[ln][t][nt[t] + __popc(v & below)] = make_int2(base + c, static_cast<int>(m[t]));
                     nt[t] += __popc(v);
@@ -495,11 +543,13 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                 n += __popc(v);
             }
             if (lane == 0) {
+                sm.blk[ln] = blk;
+                sm.pair[ln] = pair;
+                sm.seq[ln] = pair / s.Hkv;
                 sm.n_items[ln] = n;
                 sm.base[ln] = base;
                 sm.n_tile[ln][0] = nt[0];
                 sm.n_tile[ln][1] = nt[1];
-                sm.parts[ln] = (nt[0] > 0 ? 1 : 0) | (nt[1] > 0 ? 2 : 0);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.list_full[ln]);
@@ -517,14 +567,14 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
 
 // Tokens of a call (from its first on) that go this way: a multiple of 128 below the call's length, or all of them.  The
 // split with the largest gain by these costs (SM cycles; fitted to 16K, 2 x 6000 and 3 x 1000 tokens):
-//   here, a unit of 64 tokens: 2200 per chunk it visits (at most every visible one) + 18000, the last unit at least in full;
+//   here, a unit of 64 tokens: 2200 per chunk it visits (at most every visible one) + 12000, the last unit at least in full;
 //   chunk-major (index, attend and fuse kernels): 3830 per 32 tokens and chunk they attend, and 55000 for the launches.
 // With units for every SM the line lies near visible : attended = 5 : 2.  With few (sequence, KV head) pairs the units are a
 // serial chain on some of the SMs, and everything goes chunk-major unless that saves its launches (2 KV heads, a slice of
 // 2190 tokens at 4395, K = 32: 107 us chunk-major, 193 with the first 768 tokens here).  The parts of a call that the library
 // itself cuts into slices keep the whole call's split (Shape::qsplit): the same bits either way.
 int prefill_query_tokens(const Shape& s) {
-    if (s.Hl != s.Hkv || s.K > 64) return 0;
+    if (s.Hl != s.Hkv || s.K > kMaxK) return 0;
     if (s.qsplit >= 0) {
         const int n = s.qsplit - s.pos0;
         return n <= 0 ? 0 : n >= s.R ? s.R : n / 128 * 128;
@@ -535,7 +585,7 @@ int prefill_query_tokens(const Shape& s) {
     int best = 0;
     for (int n = 0; n < s.R;) {
         const int end = n + kUnitTok < s.R ? n + kUnitTok : s.R;
-        const long long vis = (s.pos0 + end - 1) / kS + 1, att = vis < s.K + nl ? vis : s.K + nl, unit = 2200 * vis + 18000;
+        const long long vis = (s.pos0 + end - 1) / kS + 1, att = vis < s.K + nl ? vis : s.K + nl, unit = 2200 * vis + 12000;
         if (vis > kMaxC) break;
         here += pairs * unit;
         there += pairs * (end - n) * att * 3830 / 32;
@@ -550,17 +600,17 @@ int prefill_query_tokens(const Shape& s) {
 }
 
 // Whether the local windows of the chunk-major tokens (from `first` on) go this way too, as one partial output row per token
-// and head (in out and lse, for the fuse kernel) instead of one per window chunk.  A unit visits the nl chunks of a window and
-// one more; costs as above, with a margin that keeps windows of up to five chunks chunk-major, where nothing is gained
-// (W = 256, 8192 tokens, K = 16: 541 us, 544 this way).  W = 512: 60,000 tokens, K = 16: 5.47 -> 4.98 ms; 16K 1.29 -> 1.19 ms; a
-// slice of 2048 tokens at 48K, K = 32: the kernels after the selection 320 -> 297 us.
+// and head (in out and lse, for the fuse kernel) instead of one per window chunk.  SM cycles: a unit visits the nl chunks of a window
+// and one more, 2200 each + 6000, in rounds of a unit per SM, and the launch takes 15000; chunk-major 3400 per 32 tokens and window chunk
+// (their lists are long).  Measured, us chunk-major / here: 16K tokens, K = 16, W = 64 934 / 941, 128 978 / 955, 256 1047 / 978; K = 32,
+// W = 512 1567 / 1403; a slice of 2048 tokens at 48K, K = 32, W = 128 331 / 332, 256 329 / 327, 512 356 / 332; of 300 tokens 71 / 75.
 bool prefill_local_query(const Shape& s, int first) {
     if (s.Hl != s.Hkv) return false;
     if (s.lsplit >= 0) return s.lsplit != 0;
     const int nl = (s.W - 1 + kS - 1) / kS + 1;
-    const long long pairs = static_cast<long long>(s.B) * s.Hkv, sms = sm_count(), toks = s.R - first, unit = 3000 * (nl + 1) + 18000;
-    const long long here = pairs * ((toks + kUnitTok - 1) / kUnitTok) * unit / sms, there = pairs * toks * nl * 3830 / 32 / sms;
-    return (here > unit ? here : unit) * 11 / 10 + 5000 < there;
+    const long long pairs = static_cast<long long>(s.B) * s.Hkv, sms = sm_count(), toks = s.R - first;
+    const long long rounds = (pairs * ((toks + kUnitTok - 1) / kUnitTok) + sms - 1) / sms;
+    return rounds * (2200 * (nl + 1) + 6000) + 15000 < pairs * toks * nl * 3400 / 32 / sms;
 }
 
 int launch_prefill_query_tc(const Shape& s, const Tensors& t, int first, int n_tok, int local, int write_sel, cudaStream_t stream) {
@@ -569,7 +619,7 @@ int launch_prefill_query_tc(const Shape& s, const Tensors& t, int first, int n_t
     if (!make_bf16_2d_map(&map_q, t.q, q_rows, kD, 64, kTok) || !make_kv_map(&map_k, t.k, pairs, s.T, s.pos0 + s.R, kD, 64, kS) ||
         !make_kv_map(&map_v, t.v, pairs, s.T, s.pos0 + s.R, kD, 64, kS) || !make_bf16_2d_map(&map_out, t.out, q_rows, kD, 64, kTok))
         return HILS_ERR_CUDA;
-    const size_t smem = kStages * (kKBytes + kVBytes) + 2 * kQBytes + sizeof(QmSmem) + 1024;
+    const size_t smem = kStages * (kKBytes + kVBytes) + 2 * kQBytes + kMmaWarp * kStgBytes + sizeof(QmSmem) + 1024;
     static PerDeviceOnce once;
     if (once.pending()) {
         if (cudaFuncSetAttribute(prefill_query_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
