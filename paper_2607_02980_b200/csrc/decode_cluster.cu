@@ -77,6 +77,9 @@ __device__ __forceinline__ int4 ld_peer4(uint32_t a) {
     asm volatile("ld.shared::cluster.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
     return v;
 }
+__device__ __forceinline__ void st_peer_f(uint32_t a, float v) { asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync(int cs) {
     if (cs > 1) {
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
@@ -98,7 +101,11 @@ struct CSmem {
     static constexpr int kBins = TG == 1 ? 512 : 256;
     static constexpr int kCand = TG == 1 ? 256 : 128;      // candidates of a token that can be ranked against each other
     static constexpr int kAll = TG == 1 ? 128 : 64;        // up to here all candidates are ranked, without a histogram
-    alignas(16) int hist[TG][kBins];
+    union {
+        alignas(16) int hist[TG][kBins];
+        float recv[TG == 1 ? 32 : 64][32];     // (afterwards) the CTAs' shares of the quarter columns that this CTA writes
+    };
+    float2 recv_md[TG == 1 ? 32 : 64];         // and their maxima and denominators
     unsigned long long own[TG][kCand];         // this CTA's candidates (score key, ~chunk id)
     unsigned long long all[TG][kCand];         // the cluster's
     unsigned kmin, kmax;                       // span of this CTA's scores (ordered keys)
@@ -157,7 +164,8 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
         tma_prefetch_desc(&map_v);
         tma_prefetch_desc(&map_lm);
     }
-    for (int x = tid; x < TG * kBins; x += NTH) (&sm.hist[0][0])[x] = 0;
+    for (int x = tid; x < TG * kBins; x += NTH) sm.hist[x >> (TG == 1 ? 9 : 8)][x & (kBins - 1)] = 0;
+    if (CS > 1) cluster_arrive();                // (waited for below: the others are there, and their histograms clear)
     pdl_wait();
     pdl_launch_dependents();
 
@@ -187,9 +195,12 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
 
     // tiles of 64 candidates: tile n belongs to CTA n mod CS (its tile n / CS, of warp n / CS mod NW), so that every CTA
     // sees a sample of the whole sequence
-    const int n_tiles = any_list ? (((nc_max + 63) >> 6) - rank + CS - 1) >> a.lcs : 0;      // this CTA's
+    // (few candidates: every CTA scores and ranks all of them, and none waits for another)
+    const bool rank_all = any_list && nc_max <= Sm::kAll;
+    const int lcs_t = rank_all ? 0 : a.lcs, rank_t = rank_all ? 0 : rank;
+    const int n_tiles = any_list ? (((nc_max + 63) >> 6) - rank_t + (1 << lcs_t) - 1) >> lcs_t : 0;      // this CTA's
     const int my_tiles = n_tiles > warp ? per_warp(n_tiles - warp + NW - 1) : 0;
-    auto global_id = [&](int i) { return ((((i >> 6) << a.lcs) + rank) << 6) + (i & 63); };   // candidate of list position i
+    auto global_id = [&](int i) { return ((((i >> 6) << lcs_t) + rank_t) << 6) + (i & 63); };   // candidate of list position i
     const int lm_row0 = (seq * s.Hl + kvh) * s.C;
 
     // Buffers: the warp's lane 0 refills a buffer once the warp has read it.  Tiles alternate between the two; items put
@@ -292,6 +303,8 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
         if (early && my_tiles <= 1) fill_v(0);
     }
 
+    if (CS > 1) cluster_wait();
+
     // ------------------------------------------------------------------------------------------ score
     if (any_list) {
         float umin = INFINITY, umax = -INFINITY;
@@ -352,7 +365,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                     }
                 }
         }
-        {
+        if (!rank_all) {
             const unsigned lo = __reduce_min_sync(kFullMask, ordered_key(umin)), hi = __reduce_max_sync(kFullMask, ordered_key(umax));
             if (lane == 0) { atomicMin(&sm.kmin, lo); atomicMax(&sm.kmax, hi); }
         }
@@ -365,19 +378,15 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
         const int m_first = wpt == NW ? 0 : wpt == 1 ? warp : wpt == 2 ? warp >> 1 : warp >= 3;                          // warp / wpt
         const int m_step = wpt == NW ? 1 : wpt == 1 ? NW : wpt == 2 ? 3 : 2;                                             // NW / wpt
         const int li = (warp - m_first * wpt) * 32 + lane, ls = wpt * 32;
-        int n_rank = 0;                            // (rank_all) candidates to rank
-        const bool rank_all = nc_max <= Sm::kAll;
         if (rank_all) {
-            // few candidates: every CTA ranks all of them
-            cluster_sync(CS);
+            __syncthreads();
+            // the scores as ordered keys, padded to a multiple of four by the lowest one
 #pragma unroll 1
-            for (int m = m_first; m < ntok; m += m_step)
-                for (int x = li; x < sm.nc[m]; x += ls) {
-                    const int tile = x >> 6;
-                    const float u = ld_peer_f(peer_addr(smem_u32(&scores[m * a.list_cap + ((tile >> a.lcs) << 6) + (x & 63)]), tile & (CS - 1)));
-                    sm.all[m][x] = select_key(u, x);
-                }
-            n_rank = 1;
+            for (int m = m_first; m < ntok; m += m_step) {
+                unsigned* keys = reinterpret_cast<unsigned*>(sm.all[m]);
+                const int nc = sm.nc[m];
+                for (int x = li; x < nc + 3; x += ls) keys[x] = x < nc ? ordered_key(scores[m * a.list_cap + x]) : 0u;
+            }
         } else {
             __syncthreads();
             // A score that this CTA's share of K of its candidates reach, off a histogram with bins of equal width in the
@@ -546,7 +555,26 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
 #pragma unroll 1
         for (int m = m_first; m < ntok; m += m_step) {
             if (sm.nc[m] <= K) continue;
-            const int n = n_rank ? sm.nc[m] : min(sm.start[m][CS], Sm::kCand);
+            if (rank_all) {
+                const uint4* keys = reinterpret_cast<const uint4*>(sm.all[m]);
+                const int nc = sm.nc[m];
+                for (int e = li; e < nc; e += ls) {
+                    const unsigned mine = reinterpret_cast<const unsigned*>(keys)[e];
+                    int rk = 0;                                      // (equal scores: the lower chunk first)
+#pragma unroll 2
+                    for (int f = 0; f < nc; f += 4) {
+                        const uint4 k = keys[f >> 2];
+                        rk += (k.x > mine || (k.x == mine && f < e)) + (k.y > mine || (k.y == mine && f + 1 < e)) +
+                              (k.z > mine || (k.z == mine && f + 2 < e)) + (k.w > mine || (k.w == mine && f + 3 < e));
+                    }
+                    if (rk < K) {
+                        sel_ids[m * K + rk] = e;
+                        if (TG == 1) place(rk, e);
+                    }
+                }
+                continue;
+            }
+            const int n = min(sm.start[m][CS], Sm::kCand);
             for (int e = li; e < n; e += ls) {
                 const unsigned long long mine = sm.all[m][e];
                 int rk = 0;
@@ -859,35 +887,28 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
 #pragma unroll
             for (int x = 0; x < 4; ++x) emit(cx, lane + 32 * x, v[x], M, den);
         } else {
-            float* dst = reinterpret_cast<float*>(bufs) + col * kRedRow + lane;
+            // a quarter of a column (32 dimensions) goes to the CTA that writes it
 #pragma unroll
-            for (int x = 0; x < 4; ++x) dst[32 * x] = v[x];
-            if (lane == 0) { sm.col_max[0][col] = M; sm.col_den[0][col] = den; }
+            for (int x = 0; x < 4; ++x) {
+                const int qx = cx * 4 + x, at = (qx >> a.lcs << a.lcs) + rank;
+                st_peer_f(peer_addr(smem_u32(&sm.recv[at][lane]), qx & (CS - 1)), v[x]);
+                if (lane < 2) st_peer_f(peer_addr(smem_u32(&sm.recv_md[at]) + 4 * lane, qx & (CS - 1)), lane ? den : M);
+            }
         }
     }
     if (CS == 1) return;
     cluster_sync(CS);
-    // a quarter of a column of the unit (32 dimensions) per warp of the cluster
 #pragma unroll 1
-    for (int qx = rank * NW + warp; qx < ntok * G * 4; qx += CS * NW) {
-        const int cx = qx >> 2, m = TG == 1 ? 0 : cx / G, col = m * Gp + cx - m * G;
+    for (int qx = warp * CS + rank; qx < ntok * G * 4; qx += NW * CS) {
+        const int cx = qx >> 2, at = qx - rank;
         // lane r: CTA r's maximum and denominator
-        const float mr = lane < CS ? ld_peer_f(peer_addr(smem_u32(&sm.col_max[0][col]), lane)) : -INFINITY;
-        const float dr = lane < CS ? ld_peer_f(peer_addr(smem_u32(&sm.col_den[0][col]), lane)) : 0.f;
-        const uint32_t src = smem_u32(reinterpret_cast<float*>(bufs) + col * kRedRow + (qx & 3) * 32 + lane);
-        float v[8];
-#pragma unroll
-        for (int r = 0; r < 8; ++r) v[r] = r < CS ? ld_peer_f(peer_addr(src, r)) : 0.f;
-        const float M = warp_max(mr);
-        const float f = mr == -INFINITY ? 0.f : __expf(mr - M);
-        const float den = warp_sum(dr * f);
+        const float2 md = lane < CS ? sm.recv_md[at + lane] : make_float2(-INFINITY, 0.f);
+        const float M = warp_max(md.x), f = md.x == -INFINITY ? 0.f : __expf(md.x - M), den = warp_sum(md.y * f);
         float n = 0.f;
-#pragma unroll
-        for (int r = 0; r < 8; ++r) n = fmaf(v[r], __shfl_sync(kFullMask, f, r), n);
-        for (int r = 8; r < CS; ++r) n = fmaf(ld_peer_f(peer_addr(src, r)), __shfl_sync(kFullMask, f, r), n);
+#pragma unroll 2
+        for (int r = 0; r < CS; ++r) n = fmaf(sm.recv[at + r][lane], __shfl_sync(kFullMask, f, r), n);
         emit(cx, (qx & 3) * 32 + lane, n, M, den);
     }
-    cluster_sync(CS);                                          // no CTA leaves while another reads its shared memory
 }
 
 template <int NT, int TG>
@@ -985,6 +1006,9 @@ bool plan_tokens(const Shape& s, int tg, int n_sm, ClusterPlan* p) {
         p->cs = cs;
         p->lcs = lcs;
         p->list_cap = ((cand + 63) / 64 + cs - 1) / cs * 64;
+        // (a short list is held whole by every CTA)
+        const int most = multi ? CSmem<4>::kAll : CSmem<1>::kAll, whole = cand < most ? (cand + 63) / 64 * 64 : most;
+        if (p->list_cap < whole) p->list_cap = whole;
         size_t off = multi ? sizeof(CSmem<4>) : sizeof(CSmem<1>);
         auto take = [&](size_t bytes) { const size_t at = (off + 15) / 16 * 16; off = at + bytes; return static_cast<int>(at); };
         p->off_scores = take(sizeof(float) * TG * p->list_cap);
