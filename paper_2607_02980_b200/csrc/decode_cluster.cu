@@ -96,11 +96,15 @@ struct Item {
     uint32_t flags;    // bit m: in token m's local window; bit 8 + m: selected by token m; bit 16: has a landmark row
 };
 
+// Candidates per token up to which every CTA scores and ranks all of them, without a histogram and without waiting for the others:
+// about one per thread.  Us, by histogram / this way: 6K tokens (93 candidates) 11.1 / 8.6, 12K (190) 11.8 / 10.5, 16K (249) 11.7 / 13.8;
+// clusters of one CTA 8K (124) 19.7 / 18.8, 12K 30.8 / 31.1; three warps 6K 49.3 / 47.2, 8K 49.5 / 50.4; four drafts at 8K 34.8 / 37.7.
+__host__ __device__ inline int rank_all_most(bool multi, int warps, int cs) { return multi ? 64 : warps == 3 ? 96 : cs > 1 ? 192 : 128; }
+
 template <int TG>
 struct CSmem {
     static constexpr int kBins = TG == 1 ? 512 : 256;
     static constexpr int kCand = TG == 1 ? 256 : 128;      // candidates of a token that can be ranked against each other
-    static constexpr int kAll = TG == 1 ? 128 : 64;        // up to here all candidates are ranked, without a histogram
     union {
         alignas(16) int hist[TG][kBins];
         float recv[TG == 1 ? 32 : 64][32];     // (afterwards) the CTAs' shares of the quarter columns that this CTA writes
@@ -196,7 +200,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     // tiles of 64 candidates: tile n belongs to CTA n mod CS (its tile n / CS, of warp n / CS mod NW), so that every CTA
     // sees a sample of the whole sequence
     // (few candidates: every CTA scores and ranks all of them, and none waits for another)
-    const bool rank_all = any_list && nc_max <= Sm::kAll;
+    const bool rank_all = any_list && nc_max <= rank_all_most(TG > 1, NW, CS);
     const int lcs_t = rank_all ? 0 : a.lcs, rank_t = rank_all ? 0 : rank;
     const int n_tiles = any_list ? (((nc_max + 63) >> 6) - rank_t + (1 << lcs_t) - 1) >> lcs_t : 0;      // this CTA's
     const int my_tiles = n_tiles > warp ? per_warp(n_tiles - warp + NW - 1) : 0;
@@ -1007,7 +1011,7 @@ bool plan_tokens(const Shape& s, int tg, int n_sm, ClusterPlan* p) {
         p->lcs = lcs;
         p->list_cap = ((cand + 63) / 64 + cs - 1) / cs * 64;
         // (a short list is held whole by every CTA)
-        const int most = multi ? CSmem<4>::kAll : CSmem<1>::kAll, whole = cand < most ? (cand + 63) / 64 * 64 : most;
+        const int most = rank_all_most(multi, p->warps, cs), whole = ((cand < most ? cand : most) + 63) / 64 * 64;
         if (p->list_cap < whole) p->list_cap = whole;
         size_t off = multi ? sizeof(CSmem<4>) : sizeof(CSmem<1>);
         auto take = [&](size_t bytes) { const size_t at = (off + 15) / 16 * 16; off = at + bytes; return static_cast<int>(at); };

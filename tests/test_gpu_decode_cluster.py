@@ -18,6 +18,10 @@ DEV = "cuda"
 @pytest.mark.parametrize("B,T,seq,K,W,G,marks", [
     (3, 64 * 130, [64 * 17 + 1, 64 * 129, 64 * 130], 16, 1, 4, "random"),     # 17, 128 and 129 candidates
     (2, 64 * 70, [64 * 70, 64 * 65 + 1], 64, 65, 8, "random"),                # lists a little longer than K
+    (1, 64 * 194, [64 * 192 + 1], 16, 1, 4, "random"),                        # 192 candidates, every CTA ranks them all
+    (1, 64 * 194, [64 * 193 + 1], 16, 1, 8, "random"),                        # 193
+    (1, 64 * 190, [64 * 190], 32, 1, 3, "equal"),                             # ties among all of them
+    (40, 64 * 100, [64 * 100 - 61 * b for b in range(40)], 16, 1, 4, "three values"),    # three warps: 96 candidates, fewer and more
     (2, 64 * 400, [64 * 400, 64 * 260 + 7], 128, 512, 2, "random"),
     (2, 64 * 300, [64 * 300, 64 * 200], 16, 1, 4, "equal"),                   # every score ties: lowest ids
     (2, 64 * 300, [64 * 300 - 1, 5], 20, 130, 3, "three values"),
