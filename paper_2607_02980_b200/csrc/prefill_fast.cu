@@ -374,7 +374,12 @@ __global__ void __launch_bounds__(kSegLists) invert_scan_kernel(const PArgs a) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // tiles of all earlier segments
     int pre = 0;
-    for (int sg = tid; sg < static_cast<int>(blockIdx.x); sg += kSegLists) pre += a.seg_tiles[sg];
+    if (a.seg_tiles) {
+        for (int sg = tid; sg < static_cast<int>(blockIdx.x); sg += kSegLists) pre += a.seg_tiles[sg];
+    } else {
+#pragma unroll 4
+        for (int l = tid; l < static_cast<int>(blockIdx.x) * kSegLists; l += kSegLists) pre += (a.cnt[l] + a.tile_tok - 1) / a.tile_tok;
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) pre += __shfl_xor_sync(kFullMask, pre, o);
     if (lane == 0) wpre[warp] = pre;
@@ -905,12 +910,19 @@ int launch_prefill_fast(const Shape& s, const Tensors& t, cudaStream_t stream) {
         // From here on every kernel of the call is launched so that its launch and prologue overlap the previous
         // kernel's tail; each of them waits for its predecessors' results before its first dependent access.  None
         // triggers its dependents early: CTAs of the next kernel parked beside a running attend kernel cost 5 %.
-        if (launch_pdl(invert_segsum_kernel, dim3(nseg), dim3(kSegLists), 0, stream, a) != cudaSuccess ||
-            launch_pdl(invert_scan_kernel, dim3(nseg), dim3(kSegLists), 0, stream, a) != cudaSuccess ||
+        // Few lists: the scan's CTAs add up the lists before their own themselves (8192 tokens, K = 16: 430 -> 427 us for the call, a slice of
+        // 2048 tokens at 48K 323 -> 318; in 32 segments a CTA reads 8000 counts)
+        if (nseg <= 32) {
+            a.seg_tiles = nullptr;
+        } else {
+            if (launch_pdl(invert_segsum_kernel, dim3(nseg), dim3(kSegLists), 0, stream, a) != cudaSuccess) return HILS_ERR_CUDA;
+            ++launches;
+        }
+        if (launch_pdl(invert_scan_kernel, dim3(nseg), dim3(kSegLists), 0, stream, a) != cudaSuccess ||
             launch_pdl(invert_fill_kernel, dim3(eb), dim3(kInvThreads), invert_smem(a), stream, a) != cudaSuccess)
             return HILS_ERR_CUDA;
         trace_mark("prefill_invert", stream);
-        launches += 3;
+        launches += 2;
     }
     for (int i0 = t0, blk = 0; i0 < s.R; i0 += a.qb, ++blk) {
         a.i0 = i0;

@@ -165,6 +165,7 @@ prefill_select_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = sm.tmem_base;
+    pdl_wait();
 
     if (warp == kTmaWarp) {
         // ------------------------------------------------------------------ TMA producer
@@ -578,14 +579,15 @@ int launch_prefill_select_tc(const Shape& s, const void* q, const void* landmark
     const unsigned nsm = static_cast<unsigned>(sm_count());
     const unsigned grid = all_tiles < nsm ? all_tiles : nsm;       // one persistent CTA per SM
     const bool perhead = s.Hl != s.Hkv;
+    cudaError_t rc;
     if (s.K <= 16) {
-        if (perhead) prefill_select_tc_kernel<16, true><<<grid, kThreads, smem, stream>>>(map_q, map_lm, a);
-        else prefill_select_tc_kernel<16, false><<<grid, kThreads, smem, stream>>>(map_q, map_lm, a);
+        rc = launch_pdl(perhead ? prefill_select_tc_kernel<16, true> : prefill_select_tc_kernel<16, false>, dim3(grid), dim3(kThreads), smem, stream,
+                        map_q, map_lm, a);
     } else {
-        if (perhead) prefill_select_tc_kernel<32, true><<<grid, kThreads, smem, stream>>>(map_q, map_lm, a);
-        else prefill_select_tc_kernel<32, false><<<grid, kThreads, smem, stream>>>(map_q, map_lm, a);
+        rc = launch_pdl(perhead ? prefill_select_tc_kernel<32, true> : prefill_select_tc_kernel<32, false>, dim3(grid), dim3(kThreads), smem, stream,
+                        map_q, map_lm, a);
     }
-    if (cudaGetLastError() != cudaSuccess) return HILS_ERR_CUDA;
+    if (rc != cudaSuccess) return HILS_ERR_CUDA;
     return a.cnt ? 2 : 1;
 }
 
