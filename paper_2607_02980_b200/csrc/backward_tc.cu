@@ -11,14 +11,18 @@
 // 19 feeds the tile records and entries through a ring.
 // Tensor memory: per tile parity 80 + 64 columns of S and T (at 0 and 240), 2 x 64 of d K^T and d V^T (384 ..), and d Q,
 // which has 96 columns of its own (144 .. 239) and borrows the 32 of its tile's consumed S or T beside them.
-// Bound: the fp32 reductions of d Q in L2 (64 KB per tile; 3100 cycles in requests of whole 128-byte runs, 6200 with a row
-// per lane, which is why the rows are turned in shared memory) and the shared-memory port (about 490 KB per tile).
+// Bound: the read-out warps (93 % of the time busy).  d Q leaves as fp32 reductions, 64 KB per tile, for which L2 takes 2760 cycles
+// whatever carries them (measured alone, 148 SMs: `red` in 128-byte runs, boxes of 512 B to 2 KB, bulk copies of rows).  A row per
+// lane goes to shared memory swizzled and from there by tensor-map reductions, a box of 32 columns of an entry's four heads each: no
+// second pass through registers, and no `red` in the queue of loads and stores that the gather needs.  Per piece of 32 columns a
+// warp spends some 550 cycles until the rows are staged and 570 to issue eight boxes (a box costs its issuer 60 - 80 cycles; one
+// issuing warp for all of them is slower, 3.2 ms for the pass, for half of them 2.10, and one staging buffer per warp 2.54).
+// Backward pass of 16K tokens, K = 16, 32 heads, with its other kernels: 2.02 ms with rows turned through shared memory and added by
+// `red`, 1.83 with the boxes; 1.52 without the reductions.
 // The CTAs walk one (query block, KV head) after the other, so that its rows of q, dO and dq stay in L2.
-// Without the reductions 16K tokens take 1.46 ms instead of 1.65, with half the read-out 1.44: behind the read-out it is the
-// chain gather -> S, T -> statistics -> products.
-// 16K tokens, K = 16, 32 heads: 1.65 ms (3.52 ms with one tile at a time between barriers; 2.56 ms with these roles and d Q
+// History of this kernel alone on that shape: 3.52 ms with one tile at a time between barriers; 2.56 ms with these roles and d Q
 // written over its own S and T, whose slot is then held until the reductions have gone out; 2.38 ms with d Q in columns of
-// its own; 2.00 ms with two thirds of the code).
+// its own; 2.00 ms with two thirds of the code; 1.65 ms before the boxes.
 #include "internal.h"
 #include "tma.cuh"
 
@@ -30,12 +34,16 @@ constexpr int kS = 64;
 constexpr int kG = 4;
 constexpr int kTok = 32;
 constexpr int kRows = kTok * kG;
-constexpr int kNS = 80;                         // score columns: 64 keys + landmark (+ 15 zero rows)
-constexpr int kKBytes = kNS * kD * 2;
+constexpr int kNS = 80;                         // score columns: 64 keys + landmark (+ 15 that nothing reads)
+// Either K block (64 dims) of a chunk: 64 key rows, the landmark row, and 896 bytes that hold other things.  The score product
+// reads them, and what follows the block, as key rows 65 .. 79: what comes out of that stays in columns of its own.
+constexpr int kKBlock = 72 * 128, kKHole = 65 * 128;
+constexpr int kKBytes = 2 * kKBlock;
 constexpr int kVBytes = kS * kD * 2;
 constexpr int kQBytes = kRows * kD * 2;
 constexpr int kDsBytes = kRows * kS * 2;
-constexpr int kMeta = 16;                       // tiles whose records and entries are in shared memory at a time
+constexpr int kStgBytes = 32 * 32 * 4;          // read-out of d Q: 32 rows x 32 columns of a warp, two buffers each
+constexpr int kMeta = 4;                        // tiles whose records and entries are in shared memory at a time
 constexpr int kTCol = 80, kDkCol = 384, kDvCol = 448;
 __device__ __forceinline__ uint32_t slot_col(uint32_t par) { return par * 240u; }          // S of a tile of this parity (T: + kTCol)
 __device__ __forceinline__ uint32_t dq_col(uint32_t par) { return par ? 144u : 112u; }     // its d Q
@@ -64,19 +72,16 @@ struct BArgs {
     int* status;
 };
 
-struct Tile {
+struct alignas(16) Tile {
+    int ent[kTok];                              // (token of the query block) << 8 | slot
     int flags;                                  // entries (0: no more tiles) | first tile of its run << 8 | last << 9 | keys << 16
     int row0;                                   // q, dO, dq row of the query block's first token, head 0 of the KV head
     int kv;                                     // first k, v row of the chunk
     int lm;                                     // landmark row of the chunk (-1: none)
+    int head0, tok0;                            // head 0 of the KV head (of all sequences'), the query block's first token
     int vis;                                    // last visible key of a local row: this + the token
-    int ent[kTok];                              // (token of the query block) << 8 | slot
 };
-struct BSmem {
-    alignas(16) float stg[4][32][36];           // read-out of d Q: a warp's 32 rows x 32 columns (padded rows)
-    alignas(16) float lmf[4][kD];               // the landmark (a copy per read-out warp)
-    alignas(16) Tile tile[kMeta];
-    float dlam[2][kRows];                       // scale * d lambda of a tile's rows
+struct BSmem {                                  // in the first K block's hole, behind d lambda
     uint64_t meta_full[kMeta], meta_empty[kMeta];
     uint64_t q_full[2];
     uint64_t k_ready, k_empty;
@@ -86,26 +91,43 @@ struct BSmem {
     uint64_t acc_empty;
     uint32_t tmem_base;
 };
-constexpr size_t kSmemBytes = 4 * kQBytes + kKBytes + kVBytes + 2 * kDsBytes + sizeof(BSmem) + 1024;
+constexpr int kDlamBytes = kRows * 4;           // scale * d lambda of a tile's rows: in the hole of the K block of its parity
+constexpr int kLmBytes = kD * 2;                // a run's landmark for the read-out: behind d lambda in the second hole, or last
+static_assert(kKHole + kDlamBytes + sizeof(BSmem) <= kKBlock && kKHole + kDlamBytes + kLmBytes <= kKBlock, "what the holes hold");
+constexpr size_t kSmemBytes = 4 * kQBytes + kKBytes + kVBytes + 2 * kDsBytes + 8 * kStgBytes + kMeta * sizeof(Tile) + kLmBytes;
 static_assert(kSmemBytes <= 232448, "shared memory of the backward kernel");
 
 __device__ __forceinline__ void red_add_f32(float* p, float x) {
     asm volatile("red.global.add.f32 [%0], %1;" ::"l"(p), "f"(x) : "memory");
+}
+// Adds one entry's box (32 columns x 1 token x 4 heads, 128B swizzle) to d Q; tracked by the issuing thread's bulk groups.
+__device__ __forceinline__ void tma_red_add_3d(const CUtensorMap* map, const void* src, int x, int y, int z) {
+    asm volatile("cp.reduce.async.bulk.tensor.3d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3, %4}], [%1];"
+                 ::"l"(map), "r"(smem_u32(src)), "r"(x), "r"(y), "r"(z) : "memory");
 }
 __device__ __forceinline__ void red_add_v4(float* p, float x, float y, float z, float w) {
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
-backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const BArgs a) {
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* qbuf = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));   // [2]
+backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
+                   const __grid_constant__ CUtensorMap map_dq, const BArgs a) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t* qbuf = smem_raw;                    // [2]
     uint8_t* obuf = qbuf + 2 * kQBytes;          // dO rows [2]
     uint8_t* kbuf = obuf + 2 * kQBytes;
     uint8_t* vbuf = kbuf + kKBytes;
     uint8_t* dsbuf = vbuf + kVBytes;
     uint8_t* wbuf = dsbuf + kDsBytes;
-    BSmem& sm = *reinterpret_cast<BSmem*>(wbuf + kDsBytes);
+    uint8_t* stgbuf = wbuf + kDsBytes;           // [4][2]
+    Tile* const rec = reinterpret_cast<Tile*>(stgbuf + 8 * kStgBytes);
+    BSmem& sm = *reinterpret_cast<BSmem*>(kbuf + kKHole + kDlamBytes);
+    auto dlam_of = [&](uint32_t par) { return reinterpret_cast<float*>(kbuf + kKHole + par * kKBlock); };
+    // (the swizzled tiles need the 1024-byte alignment that a kernel without static shared memory has; there is no room to round up)
+    if (smem_u32(smem_raw) & 1023u) {
+        if (threadIdx.x == 0) set_status(a.status, kDevTimeout);
+        return;
+    }
     const Shape& s = a.s;
     const int tid = threadIdx.x, warp = __shfl_sync(kFullMask, tid >> 5, 0), lane = tid & 31;
 
@@ -127,10 +149,8 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         mbar_fence_init();
         tma_prefetch_desc(&map_k);
         tma_prefetch_desc(&map_v);
+        tma_prefetch_desc(&map_dq);
     }
-    // rows 64 .. 79 of both K-blocks: the landmark row and zeros (TMA never writes them)
-    for (int x = tid; x < 2 * 16 * 8; x += kThreads)
-        *reinterpret_cast<uint4*>(kbuf + (x >> 7) * (kNS * 128) + swz128(64 + ((x >> 3) & 15), x & 7)) = make_uint4(0u, 0u, 0u, 0u);
     if (warp == kFrontWarp) tmem_alloc(&sm.tmem_base, 512);
     fence_proxy_async_smem();
     tc_fence_before_sync();
@@ -147,7 +167,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     // record of tile n of this CTA (false: there is none)
     auto tile_of = [&](uint32_t n) {
         if (!wait(&sm.meta_full[n % kMeta], (n / kMeta) & 1)) return false;
-        return (sm.tile[n % kMeta].flags & 255) != 0;
+        return (rec[n % kMeta].flags & 255) != 0;
     };
     auto tile_done = [&](uint32_t n) { mbar_arrive(&sm.meta_empty[n % kMeta]); };       // one lane: this warp needs it no more
     const int hs = s.R;                          // rows between two heads of a token
@@ -159,7 +179,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         const uint32_t s_tm = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16) + slot_col(grp);
         const float c2 = s.scale * kLog2e;
         for (uint32_t n = grp; tile_of(n); n += 2) {
-            const Tile& tl = sm.tile[n % kMeta];
+            const Tile& tl = rec[n % kMeta];
             const int n_ent = tl.flags & 255, ent = tl.ent[min(e_row, n_ent - 1)], lmr = tl.lm;
             const bool local = (ent & 255) >= s.K;
             // last visible key of the row; -1 for the rows of a ragged tile's padding
@@ -268,7 +288,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
             };
             // the previous tile's products have read d S and W
             if (n > 0 && !wait(&sm.done[(n - 1) & 1], ((n - 1) >> 1) & 1)) break;
-            sm.dlam[grp][row] = dl;
+            dlam_of(grp)[row] = dl;
 #pragma unroll 1
             for (int q = 0; q < 4; q += 2) {
                 tmem_ld_wait32(va);
@@ -287,71 +307,68 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         // ================================================================ read-out: d Q rows, d K and d V of a run
         const int rw = warp - kReadWarp;
         const uint32_t t_lane = tmem_base + (static_cast<uint32_t>(rw * 32) << 16);
-        float (*stg)[36] = sm.stg[rw];
-        const int row = rw * 32 + lane, e_row = row >> 2;
+        uint8_t* stg0 = stgbuf + 2 * rw * kStgBytes;
+        const int row = rw * 32 + lane;
+        uint32_t run = 0;
+        uint2 lmv = make_uint2(0u, 0u);
         for (uint32_t n = 0; tile_of(n); ++n) {
-            const Tile& tl = sm.tile[n % kMeta];
+            const Tile& tl = rec[n % kMeta];
             const uint32_t sl = n & 1u;
-            const int flags = tl.flags, kv = tl.kv;
+            const int flags = tl.flags, kv = tl.kv, head0 = tl.head0;
             if (flags & 256) {
-                float4 l = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (tl.lm >= 0) {
-                    const uint2 raw = *reinterpret_cast<const uint2*>(a.lm + static_cast<long long>(tl.lm) * kD + 4 * lane);
-                    l = make_float4(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u),
-                                    __uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u));
-                }
-                *reinterpret_cast<float4*>(&sm.lmf[rw][4 * lane]) = l;
+                ++run;
+                lmv = make_uint2(0u, 0u);
+                if (tl.lm >= 0) lmv = __ldg(reinterpret_cast<const uint2*>(a.lm + static_cast<long long>(tl.lm) * kD) + lane);
             }
-            const int orow = e_row < (flags & 255) ? tl.row0 + (row & 3) * hs + (tl.ent[e_row] >> 8) : -1;
+            // lane x < 8 sends the box of the warp's entry x
+            const int e = 8 * rw + (lane & 7), tok = lane < 8 && e < (flags & 255) ? tl.tok0 + (tl.ent[e] >> 8) : -1;
             __syncwarp();
             if (lane == 0) tile_done(n);
             if (!wait(&sm.dq_full, n & 1)) break;
             tc_fence_after_sync();
+            // Two copies by turns, each written by all four warps alike: with this tile's d Q complete every warp is through with
+            // the tile before the last, so nobody reads the run before the last any more.
+            uint8_t* lmt = run & 1u ? reinterpret_cast<uint8_t*>(rec + kMeta) : kbuf + kKBlock + kKHole + kDlamBytes;
+            if (flags & 256) {
+                *reinterpret_cast<uint2*>(lmt + 8 * lane) = lmv;
+                __syncwarp();
+            }
             uint32_t va[32];
             // 32 columns at a time, the borrowed ones first (the first for the even tiles, the last for the odd ones)
             const uint32_t q_tm = t_lane + dq_col(sl);
             const int x0 = sl ? 3 : 0, dx = sl ? -1 : 1;
             tmem_ld32_issue(q_tm + 32 * x0, va);
-            const float dl = sm.dlam[sl][row];
-            float* dst0 = a.dq + (lane & 7) * 4;
-            // through shared memory: a request then adds whole 128-byte runs of four rows
-            int ro[8];
-            float rd[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                ro[i] = __shfl_sync(kFullMask, orow, i * 4 + (lane >> 3));
-                rd[i] = __shfl_sync(kFullMask, dl, i * 4 + (lane >> 3));
-            }
+            const float dl1 = dlam_of(sl)[row];
+            const float2 dl = make_float2(dl1, dl1);
 #pragma unroll 1
             for (int p = 0; p < 4; ++p) {
                 const int x = x0 + dx * p;
+                uint4 lp[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) lp[i] = *reinterpret_cast<const uint4*>(lmt + 64 * x + 16 * i);
                 tmem_ld_wait32(va);
                 if (p == 0 || p == 3) {
                     tc_fence_before_sync();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(p == 0 ? &sm.slot_empty[sl] : &sm.dq_empty);
                 }
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    *reinterpret_cast<uint4*>(&stg[lane][4 * i]) = make_uint4(va[4 * i], va[4 * i + 1], va[4 * i + 2], va[4 * i + 3]);
-                if (p < 3) tmem_ld32_issue(q_tm + 32 * (x + dx), va);
-                const float4 l = *reinterpret_cast<const float4*>(&sm.lmf[rw][32 * x + (lane & 7) * 4]);
+                uint8_t* stg = stg0 + (p & 1) * kStgBytes;
+                if (lane < 8) bulk_wait_read<1>();                     // the last piece but one has left its staging rows
                 __syncwarp();
 #pragma unroll
-                for (int i0 = 0; i0 < 8; i0 += 4) {
-                    float4 g[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) g[i] = *reinterpret_cast<const float4*>(&stg[(i0 + i) * 4 + (lane >> 3)][(lane & 7) * 4]);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int o = ro[i0 + i];
-                        const float d = rd[i0 + i];
-                        if (o >= 0)
-                            red_add_v4(dst0 + static_cast<long long>(o) * kD + 32 * x, fmaf(d, l.x, g[i].x), fmaf(d, l.y, g[i].y),
-                                       fmaf(d, l.z, g[i].z), fmaf(d, l.w, g[i].w));
-                    }
+                for (int i = 0; i < 8; ++i) {
+                    const uint2 l = i & 1 ? make_uint2(lp[i >> 1].z, lp[i >> 1].w) : make_uint2(lp[i >> 1].x, lp[i >> 1].y);
+                    const float2 g0 = __ffma2_rn(dl, make_float2(__uint_as_float(l.x << 16), __uint_as_float(l.x & 0xffff0000u)),
+                                                 make_float2(__uint_as_float(va[4 * i]), __uint_as_float(va[4 * i + 1])));
+                    const float2 g1 = __ffma2_rn(dl, make_float2(__uint_as_float(l.y << 16), __uint_as_float(l.y & 0xffff0000u)),
+                                                 make_float2(__uint_as_float(va[4 * i + 2]), __uint_as_float(va[4 * i + 3])));
+                    *reinterpret_cast<float4*>(stg + swz128(lane, i)) = make_float4(g0.x, g0.y, g1.x, g1.y);
                 }
+                if (p < 3) tmem_ld32_issue(q_tm + 32 * (x + dx), va);
+                fence_proxy_async_smem();
                 __syncwarp();
+                if (tok >= 0) tma_red_add_3d(&map_dq, stg + lane * 512, 32 * x, tok, head0);
+                if (lane < 8) bulk_commit();
             }
             if (flags & 512) {
                 // ---- the run's last tile: d K^T and d V^T leave tensor memory, a lane per dimension
@@ -375,6 +392,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 }
             }
         }
+        if (lane < 8) bulk_wait_all();                                   // own copies in flight
     } else if (warp < kLoadWarp) {
         // ================================================================ gather of the Q and dO rows; d landmark
         // (entry-major, head-minor; an instruction copies two 256-byte rows of one entry, see the forward's gather; a warp
@@ -387,7 +405,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
             const uint32_t sl = n & 1u;
             if (!wait(&sm.ds_full[sl], (n >> 1) & 1)) return;
             // (half a warp sums 16 neighbouring rows)
-            const float4* dl = reinterpret_cast<const float4*>(&sm.dlam[sl][gw * 32 + hh * 16]);
+            const float4* dl = reinterpret_cast<const float4*>(dlam_of(sl) + gw * 32 + hh * 16);
             const uint8_t* qt = qbuf + sl * kQBytes + (p16 >> 3) * 16384;
 #pragma unroll 1
             for (int r = 0; r < 4; ++r) {
@@ -431,7 +449,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
             fl1 = fl0;
             lr1 = lr0;
             if (n >= end) continue;
-            const Tile& tl = sm.tile[n % kMeta];
+            const Tile& tl = rec[n % kMeta];
             const int tok = tl.ent[min(8 * gw + (lane & 7), (tl.flags & 255) - 1)] >> 8, row0 = tl.row0;
             fl0 = tl.flags;
             lr0 = tl.lm;
@@ -465,7 +483,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         // ================================================================ K, V and landmark of the runs
         uint32_t run = 0;
         for (uint32_t n = 0; tile_of(n); ++n) {
-            const Tile& tl = sm.tile[n % kMeta];
+            const Tile& tl = rec[n % kMeta];
             const int flags = tl.flags, pair = tl.kv / s.T, row = tl.kv - pair * s.T, lmr = tl.lm;
             __syncwarp();
             if (lane == 0) tile_done(n);
@@ -483,11 +501,11 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
             if (lane == 0) {
                 mbar_expect_tx(&sm.k_ready, 16384 + kVBytes);
                 tma_load_3d(kbuf, &map_k, &sm.k_ready, 0, row, pair);
-                tma_load_3d(kbuf + kNS * 128, &map_k, &sm.k_ready, 64, row, pair);
+                tma_load_3d(kbuf + kKBlock, &map_k, &sm.k_ready, 64, row, pair);
                 tma_load_3d(vbuf, &map_v, &sm.k_ready, 0, row, pair);
                 tma_load_3d(vbuf + 8192, &map_v, &sm.k_ready, 64, row, pair);
             }
-            if (lane < 16) *reinterpret_cast<uint4*>(kbuf + (lane >> 3) * (kNS * 128) + swz128(64, lane & 7)) = lmp;
+            if (lane < 16) *reinterpret_cast<uint4*>(kbuf + (lane >> 3) * (kKBlock) + swz128(64, lane & 7)) = lmp;
             fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.k_ready);
@@ -501,7 +519,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
             uint32_t run = 0;
             for (uint32_t n = 0; tile_of(n); ++n) {
                 const uint32_t sl = __shfl_sync(kFullMask, n & 1u, 0);
-                const int flags = sm.tile[n % kMeta].flags;
+                const int flags = rec[n % kMeta].flags;
                 __syncwarp();
                 if (lane == 0) tile_done(n);
                 if (flags & 256) { wait(&sm.k_ready, run & 1); ++run; }
@@ -515,7 +533,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 if (elect_one()) {
 #pragma unroll
                     for (int ks = 0; ks < 8; ++ks)
-                        umma_bf16(d, dq0 + (((ks >> 2) * 16384 + (ks & 3) * 32) >> 4), dk0 + (((ks >> 2) * (kNS * 128) + (ks & 3) * 32) >> 4),
+                        umma_bf16(d, dq0 + (((ks >> 2) * 16384 + (ks & 3) * 32) >> 4), dk0 + (((ks >> 2) * (kKBlock) + (ks & 3) * 32) >> 4),
                                   idesc_s, ks > 0 ? 1u : 0u);
 #pragma unroll
                     for (int ks = 0; ks < 8; ++ks)
@@ -531,13 +549,13 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         {
             constexpr uint32_t idesc_q = umma_idesc_bf16(kRows, kD) | kUmmaBMnMajor;
             constexpr uint32_t idesc_kv = umma_idesc_bf16(kD, kS) | kUmmaAMnMajor | kUmmaBMnMajor;
-            const uint64_t kmn = umma_desc_mn128(smem_u32(kbuf), kNS * 128, 1024u);
+            const uint64_t kmn = umma_desc_mn128(smem_u32(kbuf), kKBlock, 1024u);
             const uint64_t dsk = umma_desc_k128(smem_u32(dsbuf));
             const uint64_t dsmn = umma_desc_mn128(smem_u32(dsbuf), 8192u, 1024u), wmn = umma_desc_mn128(smem_u32(wbuf), 8192u, 1024u);
             uint32_t run = 0, n = 0;
             for (; tile_of(n); ++n) {
                 const uint32_t sl = __shfl_sync(kFullMask, n & 1u, 0);
-                const int flags = sm.tile[n % kMeta].flags;
+                const int flags = rec[n % kMeta].flags;
                 const bool first = (flags & 256) != 0;
                 __syncwarp();
                 if (lane == 0) tile_done(n);
@@ -584,11 +602,11 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         int sg = -1;
         long long t = 0, hi = 0;
         int i0 = 0;
-        auto put = [&](int flags, int row0, int kv, int lmr, int vis, int ent) {
-            Tile& tl = sm.tile[n % kMeta];
+        auto put = [&](int flags, int row0, int kv, int lmr, int vis, int head0, int ent) {
+            Tile& tl = rec[n % kMeta];
             if (n >= kMeta && !wait(&sm.meta_empty[n % kMeta], ((n / kMeta) - 1) & 1)) return;
             tl.ent[lane] = ent;
-            if (lane == 0) { tl.flags = flags; tl.row0 = row0; tl.kv = kv; tl.lm = lmr; tl.vis = vis; }
+            if (lane == 0) { tl.flags = flags; tl.row0 = row0; tl.kv = kv; tl.lm = lmr; tl.vis = vis; tl.head0 = head0; tl.tok0 = i0; }
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.meta_full[n % kMeta]);
             ++n;
@@ -612,7 +630,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 if (lane == 0) { px = prev.x; py = prev.y; }
                 if (lane == 31) { nx = after.x; ny = after.y; }
                 const int b = rec.x / s.Hkv, gk = rec.x - b * s.Hkv, c = rec.y;
-                const int row0 = (b * s.Hq + gk * kG) * hs + i0, kv = rec.x * s.T + c * kS;
+                const int head0 = b * s.Hq + gk * kG, row0 = head0 * hs + i0, kv = rec.x * s.T + c * kS;
                 const int lmr = c < s.C ? (b * s.Hl + gk) * s.C + c : -1, vis = s.pos0 + i0 - c * kS;     // (B Hkv C < 2^24)
                 const int flags = min(kS, s.T - c * kS) << 16 | rec.w | (rec.x != px || rec.y != py ? 256 : 0) | (rec.x != nx || rec.y != ny ? 512 : 0);
                 int e0 = a.entries[t * kTok + lane], e1 = nb > 1 ? a.entries[(t + 1) * kTok + lane] : 0;
@@ -620,7 +638,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 for (int x = 0; x < nb && ok; ++x) {
                     const int e2 = x + 2 < nb ? a.entries[(t + x + 2) * kTok + lane] : 0;
                     put(__shfl_sync(kFullMask, flags, x), __shfl_sync(kFullMask, row0, x), __shfl_sync(kFullMask, kv, x),
-                        __shfl_sync(kFullMask, lmr, x), __shfl_sync(kFullMask, vis, x), e0);
+                        __shfl_sync(kFullMask, lmr, x), __shfl_sync(kFullMask, vis, x), __shfl_sync(kFullMask, head0, x), e0);
                     e0 = e1;
                     e1 = e2;
                 }
@@ -631,7 +649,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         }
 #pragma unroll 1
         for (int x = 0; x < 2; ++x)                                     // (one for either statistics group)
-            if (ok) put(0, 0, 0, 0, 0, 0);
+            if (ok) put(0, 0, 0, 0, 0, 0, 0);
     }
     if (!ok && lane == 0) set_status(a.status, kDevTimeout);
     __syncwarp();
@@ -685,9 +703,10 @@ int launch_prefill_backward_fast(const Shape& s, const BackwardTensors& t, cudaS
     InverseIndex ix;
     const int rc = build_inverse_index(s, t.sel_idx, sc + dsum_bytes(s), t.scratch_bytes - dsum_bytes(s), &ix, stream);
     if (rc < 0) return rc;
-    CUtensorMap map_k, map_v;
+    CUtensorMap map_k, map_v, map_dq;
     const uint64_t kv_pairs = static_cast<uint64_t>(s.B) * s.Hkv;
-    if (!make_kv_map(&map_k, t.k, kv_pairs, s.T, s.pos0 + s.R, kD, 64, kS) || !make_kv_map(&map_v, t.v, kv_pairs, s.T, s.pos0 + s.R, kD, 64, kS))
+    if (!make_kv_map(&map_k, t.k, kv_pairs, s.T, s.pos0 + s.R, kD, 64, kS) || !make_kv_map(&map_v, t.v, kv_pairs, s.T, s.pos0 + s.R, kD, 64, kS) ||
+        !make_f32_rows_map(&map_dq, t.dq, static_cast<uint64_t>(s.B) * s.Hq, s.R, kD, 32, kG))
         return HILS_ERR_CUDA;
     static PerDeviceOnce attr_once;
     if (attr_once.pending()) {
@@ -719,7 +738,7 @@ int launch_prefill_backward_fast(const Shape& s, const BackwardTensors& t, cudaS
     a.dlm = t.dlandmarks;
     a.dbias = t.dbias;
     a.status = t.status;
-    if (launch_pdl(backward_tc_kernel, dim3(sm_count()), dim3(kThreads), kSmemBytes, stream, map_k, map_v, a) != cudaSuccess)
+    if (launch_pdl(backward_tc_kernel, dim3(sm_count()), dim3(kThreads), kSmemBytes, stream, map_k, map_v, map_dq, a) != cudaSuccess)
         return HILS_ERR_CUDA;
     trace_mark("backward_attend", stream);
     return rc + 2;

@@ -141,6 +141,8 @@ __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.comm
 template <int N> __device__ __forceinline__ void bulk_wait_read() {
     asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
 }
+// Waits until all of this thread's bulk groups have completed.
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 // 2-D tiled TMA store of one box (shared memory laid out as the map's swizzle prescribes) with an L2 policy,
 // tracked by the issuing thread's bulk groups.  Same fencing rules as bulk_store.
@@ -472,6 +474,19 @@ inline bool make_kv_map(CUtensorMap* map, const void* base, uint64_t pairs, uint
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// fp32 rows of every head, [heads, R, cols] -> boxes of box_cols columns of one row of box_heads heads.
+inline bool make_f32_rows_map(CUtensorMap* map, void* base, uint64_t heads, uint64_t R, uint64_t cols, uint32_t box_cols,
+                              uint32_t box_heads) {
+    EncodeTiledFn fn = get_encode_tiled();
+    if (!fn) return false;
+    cuuint64_t dims[3] = {cols, R, heads};
+    cuuint64_t strides[2] = {cols * 4, R * cols * 4};
+    cuuint32_t box[3] = {box_cols, 1, box_heads};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // packed pairs of fp32 (sm_100): one instruction per two lanes of a row's arithmetic
