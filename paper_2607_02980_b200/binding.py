@@ -125,10 +125,10 @@ def last_launch_count() -> int:
 
 
 def _dtype_code(t: torch.Tensor) -> int:
+    if t.dtype is torch.bfloat16:
+        return HILS_BF16
     if t.dtype == torch.float32:
         return HILS_F32
-    if t.dtype == torch.bfloat16:
-        return HILS_BF16
     raise TypeError("HiLS supports float32 and bfloat16 tensors, got %s" % t.dtype)
 
 
@@ -147,6 +147,36 @@ def _check(t: torch.Tensor, name: str, shape: Tuple[int, ...], dtype, cuda: bool
         raise ValueError("%s must be contiguous" % name)
     if cuda != t.is_cuda:
         raise ValueError("%s must live on %s" % (name, "a CUDA device" if cuda else "the host"))
+
+
+def _check_decode(q, k, v, landmarks, seq_lens, bias, qs, ks, ls, names=("k_cache", "v_cache")):
+    """The checks of a decode call's inputs (k, v of the shape that k must have, ks) in one expression: a short decode step takes
+    about as long on the GPU as the call does on the host.  What fails is named by _check."""
+    dt = q.dtype
+    if (q.is_cuda and k.is_cuda and v.is_cuda and landmarks.is_cuda and seq_lens.is_cuda and k.dtype is dt and v.dtype is dt
+            and landmarks.dtype is dt and seq_lens.dtype is torch.int32 and k.shape == ks and v.shape == ks and landmarks.shape == ls
+            and seq_lens.shape == qs[:1] and q.is_contiguous() and k.is_contiguous() and v.is_contiguous()
+            and landmarks.is_contiguous() and seq_lens.is_contiguous()):
+        if bias is not None:
+            _check(bias, "bias", ls[:3], torch.float32, True)
+        return
+    _check(q, "q", qs, dt, True)
+    _check(k, names[0], ks, dt, True)
+    _check(v, names[1], ks, dt, True)
+    _check(landmarks, "landmarks", ls, dt, True)
+    _check(seq_lens, "seq_lens", qs[:1], torch.int32, True)
+    if bias is not None:
+        _check(bias, "bias", ls[:3], torch.float32, True)
+
+
+def _check_outputs(out, lse, sel_idx, dt, qs, sel_shape):
+    if (out.is_cuda and lse.is_cuda and sel_idx.is_cuda and out.dtype is dt and lse.dtype is torch.float32
+            and sel_idx.dtype is torch.int32 and out.shape == qs and lse.shape == qs[:-1] and sel_idx.shape == sel_shape
+            and out.is_contiguous() and lse.is_contiguous() and sel_idx.is_contiguous()):
+        return
+    _check(out, "out", qs, dt, True)
+    _check(lse, "lse", qs[:-1], torch.float32, True)
+    _check(sel_idx, "sel_idx", sel_shape, torch.int32, True)
 
 
 def make_params(*, B, Hq, Hkv, Hl, L, T_max, C, d, chunk_size, top_k, window=1, scale=0.0, dtype, impl="auto"):
@@ -239,23 +269,16 @@ def hils_decode(q, k_cache, v_cache, landmarks, seq_lens, chunk_size: int, top_k
 
     Returns (out [B,Hq,d], lse [B,Hq], sel_idx [B,Hkv,K])."""
     lib = load_library()
-    B, Hq, d = q.shape
+    qs, ls = tuple(q.shape), landmarks.shape
+    B, Hq, d = qs
     Hkv, T = k_cache.shape[1], k_cache.shape[2]
-    Hl, C = landmarks.shape[1], landmarks.shape[2]
+    Hl, C = ls[1], ls[2]
     dt = q.dtype
-    _check(q, "q", (B, Hq, d), dt, True)
-    _check(k_cache, "k_cache", (B, Hkv, T, d), dt, True)
-    _check(v_cache, "v_cache", (B, Hkv, T, d), dt, True)
-    _check(landmarks, "landmarks", (B, Hl, C, d), dt, True)
-    _check(seq_lens, "seq_lens", (B,), torch.int32, True)
-    if bias is not None:
-        _check(bias, "bias", (B, Hl, C), torch.float32, True)
+    _check_decode(q, k_cache, v_cache, landmarks, seq_lens, bias, qs, (B, Hkv, T, d), (B, Hl, C, d))
     out = torch.empty_like(q) if out is None else out
     lse = torch.empty((B, Hq), dtype=torch.float32, device=q.device) if lse is None else lse
     sel_idx = torch.empty((B, Hkv, top_k), dtype=torch.int32, device=q.device) if sel_idx is None else sel_idx
-    _check(out, "out", (B, Hq, d), dt, True)
-    _check(lse, "lse", (B, Hq), torch.float32, True)
-    _check(sel_idx, "sel_idx", (B, Hkv, top_k), torch.int32, True)
+    _check_outputs(out, lse, sel_idx, dt, qs, (B, Hkv, top_k))
     p = _params_ref(B, Hq, Hkv, Hl, 0, T, C, d, chunk_size, top_k, window, float(scale), _dtype_code(q),
                     _IMPL[impl])
     ws = _scratch(lib.hils_workspace_bytes(p, 1), "hils_workspace_bytes", q.device) if workspace is None else workspace
@@ -265,8 +288,8 @@ def hils_decode(q, k_cache, v_cache, landmarks, seq_lens, chunk_size: int, top_k
                                     _ptr(bias), _ptr(seq_lens), _ptr(out), _ptr(lse), _ptr(sel_idx), _ptr(ws), ws.numel(),
                                     _stream_ptr(stream))
     else:
-        rc = lib.hils_decode(p, _ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(landmarks), _ptr(bias),
-                             _ptr(seq_lens), _ptr(out), _ptr(lse), _ptr(sel_idx), _ptr(ws), ws.numel(),
+        rc = lib.hils_decode(p, q.data_ptr(), k_cache.data_ptr(), v_cache.data_ptr(), landmarks.data_ptr(), _ptr(bias),
+                             seq_lens.data_ptr(), out.data_ptr(), lse.data_ptr(), sel_idx.data_ptr(), ws.data_ptr(), ws.numel(),
                              _stream_ptr(stream))
     if rc != 0:
         raise HilsError(rc, "hils_decode")
@@ -348,27 +371,22 @@ def hils_decode_paged(q, k_pages, v_pages, landmarks, block_table, seq_lens, chu
     """hils_decode over paged caches with page = chunk: k_pages, v_pages [num_pages, Hkv, S, d], block_table [B, C]
     int32 (page of every logical chunk); landmarks / bias stay logical.  Returns (out, lse, sel_idx)."""
     lib = load_library()
-    B, Hq, d = q.shape
+    qs, ls = tuple(q.shape), landmarks.shape
+    B, Hq, d = qs
     P, Hkv, S, _ = k_pages.shape
-    Hl, C = landmarks.shape[1], landmarks.shape[2]
+    Hl, C = ls[1], ls[2]
     dt = q.dtype
-    _check(q, "q", (B, Hq, d), dt, True)
-    _check(k_pages, "k_pages", (P, Hkv, chunk_size, d), dt, True)
-    _check(v_pages, "v_pages", (P, Hkv, chunk_size, d), dt, True)
-    _check(landmarks, "landmarks", (B, Hl, C, d), dt, True)
+    _check_decode(q, k_pages, v_pages, landmarks, seq_lens, bias, qs, (P, Hkv, chunk_size, d), (B, Hl, C, d), ("k_pages", "v_pages"))
     _check(block_table, "block_table", (B, C), torch.int32, True)
-    _check(seq_lens, "seq_lens", (B,), torch.int32, True)
-    if bias is not None:
-        _check(bias, "bias", (B, Hl, C), torch.float32, True)
     p = _params_ref(B, Hq, Hkv, Hl, 0, C * chunk_size, C, d, chunk_size, top_k, window, float(scale),
                     _dtype_code(q), _IMPL["auto"])
     ws = _scratch(lib.hils_workspace_bytes(p, 1), "hils_workspace_bytes", q.device) if workspace is None else workspace
     out = torch.empty((B, Hq, d), dtype=dt, device=q.device) if out is None else out
     lse = torch.empty((B, Hq), dtype=torch.float32, device=q.device) if lse is None else lse
     sel_idx = torch.empty((B, Hkv, top_k), dtype=torch.int32, device=q.device) if sel_idx is None else sel_idx
-    rc = lib.hils_decode_paged(p, _ptr(q), _ptr(k_pages), _ptr(v_pages), _ptr(landmarks), _ptr(bias),
-                               _ptr(block_table), int(P), _ptr(seq_lens), _ptr(out), _ptr(lse), _ptr(sel_idx),
-                               _ptr(ws), ws.numel() * ws.element_size(), _stream_ptr(stream))
+    rc = lib.hils_decode_paged(p, q.data_ptr(), k_pages.data_ptr(), v_pages.data_ptr(), landmarks.data_ptr(), _ptr(bias),
+                               block_table.data_ptr(), int(P), seq_lens.data_ptr(), out.data_ptr(), lse.data_ptr(), sel_idx.data_ptr(),
+                               ws.data_ptr(), ws.numel() * ws.element_size(), _stream_ptr(stream))
     if rc != 0:
         raise HilsError(rc, "hils_decode_paged")
     return out, lse, sel_idx
@@ -507,39 +525,32 @@ def hils_decode_multi(q, k_cache, v_cache, landmarks, seq_lens, chunk_size: int,
     counts them).  Caches [B,Hkv,T,d], or page pools [P,Hkv,S,d] with block_table [B,C].
     Returns (out [B,M,Hq,d], lse [B,M,Hq], sel_idx [B,M,Hkv,K])."""
     lib = load_library()
-    B, M, Hq, d = q.shape
+    qs, ls = tuple(q.shape), landmarks.shape
+    B, M, Hq, d = qs
     Hkv = k_cache.shape[1]
-    Hl, C = landmarks.shape[1], landmarks.shape[2]
+    Hl, C = ls[1], ls[2]
     dt = q.dtype
-    _check(q, "q", (B, M, Hq, d), dt, True)
-    _check(landmarks, "landmarks", (B, Hl, C, d), dt, True)
-    _check(seq_lens, "seq_lens", (B,), torch.int32, True)
     num_pages = 0
     if block_table is None:
         T = k_cache.shape[2]
-        _check(k_cache, "k_cache", (B, Hkv, T, d), dt, True)
-        _check(v_cache, "v_cache", (B, Hkv, T, d), dt, True)
+        _check_decode(q, k_cache, v_cache, landmarks, seq_lens, bias, qs, (B, Hkv, T, d), (B, Hl, C, d))
     else:
         num_pages = k_cache.shape[0]
         T = C * chunk_size
-        _check(k_cache, "k_pages", (num_pages, Hkv, chunk_size, d), dt, True)
-        _check(v_cache, "v_pages", (num_pages, Hkv, chunk_size, d), dt, True)
+        _check_decode(q, k_cache, v_cache, landmarks, seq_lens, bias, qs, (num_pages, Hkv, chunk_size, d), (B, Hl, C, d),
+                      ("k_pages", "v_pages"))
         _check(block_table, "block_table", (B, C), torch.int32, True)
-    if bias is not None:
-        _check(bias, "bias", (B, Hl, C), torch.float32, True)
     out = torch.empty_like(q) if out is None else out
     lse = torch.empty((B, M, Hq), dtype=torch.float32, device=q.device) if lse is None else lse
     sel_idx = torch.empty((B, M, Hkv, top_k), dtype=torch.int32, device=q.device) if sel_idx is None else sel_idx
-    _check(out, "out", (B, M, Hq, d), dt, True)
-    _check(lse, "lse", (B, M, Hq), torch.float32, True)
-    _check(sel_idx, "sel_idx", (B, M, Hkv, top_k), torch.int32, True)
+    _check_outputs(out, lse, sel_idx, dt, qs, (B, M, Hkv, top_k))
     p = _params_ref(B, Hq, Hkv, Hl, 0, T, C, d, chunk_size, top_k, window, float(scale), _dtype_code(q),
                     _IMPL["auto"])
     if workspace is None:
         workspace = _scratch(lib.hils_decode_multi_workspace_bytes(p, int(M)), "hils_decode_multi_workspace_bytes", q.device)
-    rc = lib.hils_decode_multi(p, int(M), _ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(landmarks),
-                               _ptr(bias), _ptr(block_table), int(num_pages), _ptr(seq_lens), _ptr(out), _ptr(lse),
-                               _ptr(sel_idx), _ptr(workspace), workspace.numel(), _stream_ptr(stream))
+    rc = lib.hils_decode_multi(p, int(M), q.data_ptr(), k_cache.data_ptr(), v_cache.data_ptr(), landmarks.data_ptr(),
+                               _ptr(bias), _ptr(block_table), int(num_pages), seq_lens.data_ptr(), out.data_ptr(), lse.data_ptr(),
+                               sel_idx.data_ptr(), workspace.data_ptr(), workspace.numel(), _stream_ptr(stream))
     if rc != 0:
         raise HilsError(rc, "hils_decode_multi")
     return out, lse, sel_idx
