@@ -18,8 +18,8 @@
 // Bound: HBM (landmarks scanned + selected K / V), and where a call has few units the chain of dependent steps.  One
 // launch per step (decode_fast.cu) drains and ramps between short phases and leaves the memory idle during the
 // selection.  Before / now, B200, us per call through the Python entry points, calls back to back: 1 x 6000 tokens, K = 16:
-// 22.7 / 10.7; 8 x 4K-16K paged, K = 32, W = 512: 49.3 / 24.4; 64 x 64K, K = 32: 142.6 / 112.6 (6.1 TB/s); 4 x 1M, K = 64: 65.4 / 43.8;
-// 16 x 8K-32K, four drafts, K = 32: 121 / 56.6.  Before this form of its short steps (landmark tiles asked for ahead of the queries, a
+// 22.7 / 9.3; 8 x 4K-16K paged, K = 32, W = 512: 49.3 / 22.7; 64 x 64K, K = 32: 142.6 / 113.8 (6.1 TB/s); 4 x 1M, K = 64: 65.4 / 43.5;
+// 16 x 8K-32K, four drafts, K = 32: 121 / 56.7.  Before this form of its short steps (landmark tiles asked for ahead of the queries, a
 // tile's biases under its wait, items placed by rank with sel_idx sorted behind the loads, no integer or exactly rounded division on the
 // way) the same calls took 12.7, 28.2, 117.3, 46.8 and 62.2.
 // Draft tokens of one sequence retrieve mostly the same chunks: the union of their selections is loaded once, and all
