@@ -747,12 +747,19 @@ int launch_chunk_major(const GArgs& a, void* scratch, cudaStream_t stream) {
     float* part = static_cast<float*>(scratch);
     float* lam = reinterpret_cast<float*>(static_cast<char*>(scratch) + chunk_lam_offset(s));
     const long long rows = static_cast<long long>(s.B) * s.Hq * s.R;
-    // Blocks of 128 tokens with all query heads of the KV head and eight warps where there are CTAs enough (3072 tokens, 4 heads, d = 128,
-    // K = 4: 258 -> 151 us for the call; 2635 tokens, 2 heads: 109 -> 89), else blocks of 32 of one head and four warps: more CTAs
-    // with less to do each (600 tokens, 2 heads, d = 128: 25 us, 31 with eight warps; 2048, one head, d = 64: 31, 33).
-    const bool large = chunk_ctas(s, 32) >= 8ll * sm_count();
-    if ((large ? launch_chunk_kernel<D, 8>(a, kRowBlockMax, s.G, part, lam, stream) : launch_chunk_kernel<D, 4>(a, 32, 1, part, lam, stream)) != 0)
-        return HILS_ERR_CUDA;
+    // Three block sizes: 32 tokens of one query head (most CTAs, least work each), 64 tokens of one head, 128 tokens with all query heads
+    // of the KV head (a K or V value is fetched for the most rows); four warps at d = 64, eight at d = 128.  The lines lie where the
+    // counts of 32-token CTAs below cross, K = 8, us for the call (32 / 64 / 128 tokens):
+    //   d = 128: 841 tokens, 4 heads (2 KV heads) 48 / 54 / 67; 2048, one head 51 / 47 / 54; 2048, 4 heads (2) 149 / 128 / 142;
+    //            3000, 2 heads (1) 141 / 112 / 110; 4096, 4 heads (2) 448 / 316 / 259
+    //   d = 64:  8 x 841, one head 55 / 62 / 65; 2048, 2 heads (1) 51 / 52 / 60; 2048, 4 heads (2) 87 / 82 / 90; 3 x 2048, 4 heads (2)
+    //            227 / 203 / 221; 3 x 3300, 4 heads (2) 459 / 371 / 346
+    // (with four warps for 32 tokens everywhere and eight for 128, one line between them: 56, 55, 142, 110, 260; 66, 51, 101, 227, 380)
+    constexpr int kNW = D == 64 ? 4 : 8;
+    const long long ctas = chunk_ctas(s, 32), heads = ctas * s.G, sms = sm_count();
+    const bool all_heads = ctas >= (D == 64 ? 60 : 15) * sms;
+    const int rb = all_heads ? kRowBlockMax : heads >= (D == 64 ? 24 : 7) * sms ? 64 : 32;
+    if (launch_chunk_kernel<D, kNW>(a, rb, all_heads ? s.G : 1, part, lam, stream) != 0) return HILS_ERR_CUDA;
     trace_mark("generic_attend", stream);
     if (launch_pdl(generic_fuse_kernel<D>, dim3(static_cast<unsigned>((rows + kWarpsPerBlock - 1) / kWarpsPerBlock)),
                    dim3(kWarpsPerBlock * 32), 0, stream, a, static_cast<const float*>(part), static_cast<const float*>(lam)) != cudaSuccess)

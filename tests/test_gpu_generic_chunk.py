@@ -1,5 +1,5 @@
-"""The fp32 chunk-major kernel in both of its forms (blocks of 128 tokens with all heads of a KV head, eight rows per warp; blocks
-of 32 tokens of one head) against the CPU oracle: head counts that do not divide a warp's rows, blocks and chunks that end in the
+"""The fp32 chunk-major kernel in its forms (blocks of 128 tokens with all heads of a KV head; blocks of 64 or 32 tokens of one
+head) against the CPU oracle: head counts that do not divide a warp's rows, blocks and chunks that end in the
 middle of one another, an odd and an even number of blocks, slices, landmarks per query head, a routing query."""
 import numpy as np
 import pytest
@@ -15,10 +15,12 @@ DEV = "cuda"
 
 
 @pytest.mark.parametrize("B,Hq,Hkv,L,d,S,K,W,bias,per_head", [
-    (2, 4, 2, 1300, 128, 64, 4, 1, False, False),      # large: 8 rows per warp, 11 blocks
-    (2, 6, 2, 1217, 64, 48, 3, 100, True, True),       # large: three heads, chunks of 48, per-head landmarks
-    (4, 2, 2, 1281, 64, 64, 8, 65, True, False),       # large: one head per KV head
-    (1, 3, 1, 230, 128, 64, 4, 70, True, True),        # small: one head per CTA, 8 blocks of 32
+    (2, 4, 2, 1300, 128, 64, 4, 1, False, False),      # 64 tokens, 21 blocks, eight warps
+    (2, 6, 2, 1217, 64, 48, 3, 100, True, True),       # 64 tokens, three heads, chunks of 48, per-head landmarks
+    (4, 2, 2, 1281, 64, 64, 8, 65, True, False),       # 32 tokens, one head per KV head, 41 blocks
+    (1, 3, 1, 230, 128, 64, 4, 70, True, True),        # 32 tokens, 8 blocks, eight warps
+    (3, 4, 2, 1300, 128, 64, 4, 1, True, False),       # 128 tokens, all heads, 11 blocks, eight warps
+    (3, 6, 2, 1217, 64, 16, 5, 1, True, True),         # 128 tokens, three heads, chunks of 16, four warps
     (1, 2, 1, 31, 64, 16, 2, 1, False, False),
 ])
 def test_against_the_oracle(B, Hq, Hkv, L, d, S, K, W, bias, per_head):
