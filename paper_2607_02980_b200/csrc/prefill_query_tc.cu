@@ -518,6 +518,9 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                         }
                         __syncwarp();
                     }
+                    // The next rows may come the other way: ordinary accesses to sm.ids are ordered before a bulk copy into it by a proxy
+                    // fence of the lane that made them alone.  (One CTA meets both ways where top_k is no multiple of 4.)
+                    fence_proxy_async_smem();
                     __syncwarp();
                 }
                 if (!ok) break;
