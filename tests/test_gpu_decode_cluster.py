@@ -132,3 +132,23 @@ def test_groups_of_draft_tokens_on_six_and_on_three_warps(B, M, K):
         assert (held[..., 1:] >= held[..., :-1]).all()
         # (two roundings to bf16 of sums in different orders, outputs below 2: twice 2^-8 = 8e-3)
         assert (o.float() - out[:, m].float()).abs().max() <= 1.6e-2 and (l - lse[:, m]).abs().max() <= 1e-4
+
+
+@pytest.mark.parametrize("T,W", [(64 * 150, 512), (64 * 12, 512)])
+def test_pages_of_local_chunks_out_of_range(T, W):
+    """A warp's first item is asked for by one lane ahead of the cluster's first barrier, and given up there where it has no page:
+    with a list of candidates to score and without one, the other sequence's results stay the same."""
+    from test_gpu_paged import paginate
+    cfg = wl.HilsConfig("gone", "decode", 2, 8, 2, T, 128, 64, 16, "bf16", 971, window=W)
+    inp = wl.make_decode_inputs(cfg, "cpu", seq_lens=torch.tensor([T, T - 9], dtype=torch.int32))
+    kp, vp, table = paginate(inp, cfg, 2)
+    p = hils.make_params(B=2, Hq=8, Hkv=2, Hl=2, L=0, T_max=T, C=cfg.C, d=128, chunk_size=64, top_k=16, window=W, dtype=1)
+    ws = hils.alloc_workspace(p, True, DEV)
+    run = lambda: hils.hils_decode_paged(inp["q"].to(DEV), kp.to(DEV), vp.to(DEV), inp["landmarks"].to(DEV), table.to(DEV),
+                                         inp["seq_lens"].to(DEV), 64, 16, window=W, workspace=ws)
+    good = run()
+    assert hils.poll_status(ws) == 0 and hils.last_launch_count() == 1
+    table[0, T // 64 - 8:] = -1                                # (every chunk of the window but its oldest)
+    out, lse, sel = run()
+    assert hils.poll_status(ws) == -7
+    assert torch.equal(sel, good[2]) and torch.equal(out[1], good[0][1]) and torch.equal(lse[1], good[1][1])
