@@ -197,6 +197,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                 const bool local = c >= lc;
                 const bool act = ((who >> lane) & 1u) != 0u;
                 if (!s_ready && !wait(&sm.s_full[t], n_s & 1)) break;
+                __syncwarp();                        // (s_ready is a lane's own answer, and the loads take the whole warp)
                 tc_fence_after_sync();
                 float v[64], lm4[4];
                 tmem_ld64_4(t_lane, t_lane + 64, v, lm4);
@@ -255,6 +256,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                 // the previous chunk's value product has read its probabilities and left the accumulator
                 if (i > 0) {
                     if (!o_ready && !wait(&sm.o_done[t], (n_s - 1) & 1)) break;
+                    __syncwarp();
                     if (__any_sync(kFullMask, grow != 1.f)) {
                         tc_fence_after_sync();
 #pragma unroll 1
