@@ -329,10 +329,8 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
             // Two copies by turns, each written by all four warps alike: with this tile's d Q complete every warp is through with
             // the tile before the last, so nobody reads the run before the last any more.
             uint8_t* lmt = run & 1u ? reinterpret_cast<uint8_t*>(rec + kMeta) : kbuf + kKBlock + kKHole + kDlamBytes;
-            if (flags & 256) {
-                *reinterpret_cast<uint2*>(lmt + 8 * lane) = lmv;
-                __syncwarp();
-            }
+            if (flags & 256) *reinterpret_cast<uint2*>(lmt + 8 * lane) = lmv;
+            __syncwarp();                            // (also ahead of the loads below, which take the whole warp)
             uint32_t va[32];
             // 32 columns at a time, the borrowed ones first (the first for the even tiles, the last for the odd ones)
             const uint32_t q_tm = t_lane + dq_col(sl);
@@ -369,6 +367,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                 __syncwarp();
                 if (tok >= 0) tma_red_add_3d(&map_dq, stg + lane * 512, 32 * x, tok, head0);
                 if (lane < 8) bulk_commit();
+                __syncwarp();                                            // (the wait for the next piece takes the whole warp)
             }
             if (flags & 512) {
                 // ---- the run's last tile: d K^T and d V^T leave tensor memory, a lane per dimension
