@@ -292,6 +292,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             if (n > 0) {
                 // ---- the tile's output rows
                 if (!wait(&sm.o_done[t], (n_s - 1) & 1)) break;
+                __syncwarp();
                 tc_fence_after_sync();
                 const float inv = live ? __fdividef(1.f, den) : 0.f;
                 const long long orow = (static_cast<long long>(b) * s.Hq + gk * kG + h) * s.R + tok;
@@ -330,6 +331,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
 #pragma unroll
                         for (int pc = 0; pc < 8; ++pc) *reinterpret_cast<uint4*>(a.out + orow * kD + half * 64 + pc * 8) = w[pc];
                     }
+                    __syncwarp();                    // (the next half's loads take the whole warp)
                 }
                 tc_fence_before_sync();
                 if (live) a.lse[orow] = ref + __logf(den);
