@@ -321,6 +321,13 @@ int hils_poll_status(const void* workspace, void* stream);
 /* Number of kernels the last hils_prefill / hils_decode call of this thread enqueued. */
 int hils_last_launch_count(void);
 
+/* Form that a call of these sizes takes on the current device, for tests and tuning: four numbers to form, all 0 where
+ * neither of these kernels runs.
+ *   Decode in one launch (is_decode = 1, tokens_per_seq newest tokens per sequence): tokens that share a unit, warps per CTA,
+ *     CTAs per cluster, candidates per token up to which every CTA ranks all of them.
+ *   fp32 prefill, chunk-major: tokens per CTA, query heads per CTA, warps per CTA, 0. */
+int hils_call_form(const hils_params* params, int is_decode, int32_t tokens_per_seq, int32_t* form);
+
 /* Per-kernel timing for profiling (no counterpart in the paper; Sec. 7.1 reports end-to-end latency
  * only).  hils_trace_enable(1) creates CUDA events once for the calling thread; while on, each
  * hils_prefill / hils_decode records an event after every kernel it enqueues.  hils_trace_read

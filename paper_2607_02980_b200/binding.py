@@ -28,6 +28,7 @@ EXPORTS = [
     "hils_landmark_summary", "hils_decode_paged", "hils_prefill_at", "hils_prefill_at_workspace_bytes",
     "hils_prefill_routed", "hils_decode_routed", "hils_chunk_overlap", "hils_prefill_backward",
     "hils_prefill_backward_workspace_bytes", "hils_decode_multi", "hils_decode_multi_workspace_bytes",
+    "hils_call_form",
 ]
 
 
@@ -101,6 +102,8 @@ def load_library() -> ctypes.CDLL:
     lib.hils_poll_status.restype = ctypes.c_int
     lib.hils_poll_status.argtypes = [vp, vp]
     lib.hils_last_launch_count.restype = ctypes.c_int
+    lib.hils_call_form.restype = ctypes.c_int
+    lib.hils_call_form.argtypes = [pp, ctypes.c_int, ctypes.c_int32, ctypes.POINTER(ctypes.c_int32)]
     lib.hils_status_string.restype = ctypes.c_char_p
     lib.hils_status_string.argtypes = [ctypes.c_int]
     lib.hils_version.restype = ctypes.c_char_p
@@ -122,6 +125,15 @@ def version() -> str:
 
 def last_launch_count() -> int:
     return int(load_library().hils_last_launch_count())
+
+
+def call_form(params: HilsParams, is_decode: bool, tokens_per_seq: int = 1) -> Tuple[int, ...]:
+    """The form that a call of these sizes takes on the current device (see include/hils.h), for tests and tuning."""
+    form = (ctypes.c_int32 * 4)()
+    rc = load_library().hils_call_form(ctypes.byref(params), 1 if is_decode else 0, tokens_per_seq, form)
+    if rc != 0:
+        raise HilsError(rc, "hils_call_form")
+    return tuple(form)
 
 
 def _dtype_code(t: torch.Tensor) -> int:

@@ -667,6 +667,25 @@ int hils_poll_status(const void* workspace, void* stream) {
 
 int hils_last_launch_count(void) { return g_last_launches; }
 
+int hils_call_form(const hils_params* params, int is_decode, int32_t tokens_per_seq, int32_t* form) {
+    Shape s;
+    if (!form || tokens_per_seq < 1) return HILS_ERR_INVALID_ARG;
+    int rc = make_shape(params, is_decode, &s);
+    if (rc != HILS_OK) return rc;
+    if (is_decode) {
+        if (static_cast<long long>(s.B) * tokens_per_seq > (1 << 24)) return HILS_ERR_INVALID_ARG;
+        s.B *= tokens_per_seq;
+        s.qps = tokens_per_seq;
+    }
+    Path path;
+    rc = pick_path(s, params, &path);
+    if (rc != HILS_OK) return rc;
+    for (int i = 0; i < 4; ++i) form[i] = 0;
+    if (path == Path::DecodeFast) decode_cluster_form(s, form);
+    if (path == Path::Generic) generic_chunk_form(s, params->dtype, form);
+    return HILS_OK;
+}
+
 int hils_trace_enable(int on) {
     Trace& t = g_trace;
     if (on && !t.have_events) {

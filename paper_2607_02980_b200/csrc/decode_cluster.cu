@@ -1055,6 +1055,15 @@ bool decode_cluster_supports(const Shape& s) {
     return s.Hl == s.Hkv && (s.K >= 16 || s.T > 4096) && s.K <= kMaxK && plan_cluster(s, sm_count(), &p);
 }
 
+void decode_cluster_form(const Shape& s, int32_t* form) {
+    ClusterPlan p;
+    if (!decode_cluster_supports(s) || !plan_cluster(s, sm_count(), &p)) return;
+    form[0] = p.tg;
+    form[1] = p.warps;
+    form[2] = p.cs;
+    form[3] = rank_all_most(p.tg > 1, p.warps, p.cs);
+}
+
 int launch_decode_cluster(const Shape& s, const Tensors& t, cudaStream_t stream) {
     ClusterPlan p;
     if (!plan_cluster(s, sm_count(), &p)) return HILS_ERR_UNSUPPORTED;

@@ -722,6 +722,22 @@ long long chunk_ctas(const Shape& s, int rb) {
     return n * s.B * s.Hkv;
 }
 
+// Three block sizes: 32 tokens of one query head (most CTAs, least work each), 64 tokens of one head, 128 tokens with all query heads
+// of the KV head (a K or V value is fetched for the most rows); four warps at d = 64, eight at d = 128.  The lines lie where the
+// counts of 32-token CTAs below cross, K = 8, us for the call (32 / 64 / 128 tokens):
+//   d = 128: 841 tokens, 4 heads (2 KV heads) 48 / 54 / 67; 2048, one head 51 / 47 / 54; 2048, 4 heads (2) 149 / 128 / 142;
+//            3000, 2 heads (1) 141 / 112 / 110; 4096, 4 heads (2) 448 / 316 / 259
+//   d = 64:  8 x 841, one head 55 / 62 / 65; 2048, 2 heads (1) 51 / 52 / 60; 2048, 4 heads (2) 87 / 82 / 90; 3 x 2048, 4 heads (2)
+//            227 / 203 / 221; 3 x 3300, 4 heads (2) 459 / 371 / 346
+// (with four warps for 32 tokens everywhere and eight for 128, one line between them: 56, 55, 142, 110, 260; 66, 51, 101, 227, 380)
+struct ChunkForm { int tokens, heads, warps; };        // per CTA: tokens, query heads of a KV head, warps
+ChunkForm chunk_form(const Shape& s) {
+    const long long ctas = chunk_ctas(s, 32), heads = ctas * s.G, sms = sm_count();
+    const int warps = s.d == 64 ? 4 : 8;
+    if (ctas >= (s.d == 64 ? 60 : 15) * sms) return {kRowBlockMax, s.G, warps};
+    return {heads >= (s.d == 64 ? 24 : 7) * sms ? 64 : 32, 1, warps};
+}
+
 template <int D, int NW>
 int launch_chunk_kernel(const GArgs& a, int rb, int nh, float* part, float* lam, cudaStream_t stream) {
     const Shape& s = a.s;
@@ -747,19 +763,8 @@ int launch_chunk_major(const GArgs& a, void* scratch, cudaStream_t stream) {
     float* part = static_cast<float*>(scratch);
     float* lam = reinterpret_cast<float*>(static_cast<char*>(scratch) + chunk_lam_offset(s));
     const long long rows = static_cast<long long>(s.B) * s.Hq * s.R;
-    // Three block sizes: 32 tokens of one query head (most CTAs, least work each), 64 tokens of one head, 128 tokens with all query heads
-    // of the KV head (a K or V value is fetched for the most rows); four warps at d = 64, eight at d = 128.  The lines lie where the
-    // counts of 32-token CTAs below cross, K = 8, us for the call (32 / 64 / 128 tokens):
-    //   d = 128: 841 tokens, 4 heads (2 KV heads) 48 / 54 / 67; 2048, one head 51 / 47 / 54; 2048, 4 heads (2) 149 / 128 / 142;
-    //            3000, 2 heads (1) 141 / 112 / 110; 4096, 4 heads (2) 448 / 316 / 259
-    //   d = 64:  8 x 841, one head 55 / 62 / 65; 2048, 2 heads (1) 51 / 52 / 60; 2048, 4 heads (2) 87 / 82 / 90; 3 x 2048, 4 heads (2)
-    //            227 / 203 / 221; 3 x 3300, 4 heads (2) 459 / 371 / 346
-    // (with four warps for 32 tokens everywhere and eight for 128, one line between them: 56, 55, 142, 110, 260; 66, 51, 101, 227, 380)
-    constexpr int kNW = D == 64 ? 4 : 8;
-    const long long ctas = chunk_ctas(s, 32), heads = ctas * s.G, sms = sm_count();
-    const bool all_heads = ctas >= (D == 64 ? 60 : 15) * sms;
-    const int rb = all_heads ? kRowBlockMax : heads >= (D == 64 ? 24 : 7) * sms ? 64 : 32;
-    if (launch_chunk_kernel<D, kNW>(a, rb, all_heads ? s.G : 1, part, lam, stream) != 0) return HILS_ERR_CUDA;
+    const ChunkForm f = chunk_form(s);
+    if (launch_chunk_kernel<D, D == 64 ? 4 : 8>(a, f.tokens, f.heads, part, lam, stream) != 0) return HILS_ERR_CUDA;
     trace_mark("generic_attend", stream);
     if (launch_pdl(generic_fuse_kernel<D>, dim3(static_cast<unsigned>((rows + kWarpsPerBlock - 1) / kWarpsPerBlock)),
                    dim3(kWarpsPerBlock * 32), 0, stream, a, static_cast<const float*>(part), static_cast<const float*>(lam)) != cudaSuccess)
@@ -810,6 +815,14 @@ bool generic_supports(const Shape& s) {
 size_t generic_scratch_bytes(const Shape& s, int dtype) {
     if (!chunk_major(s, dtype)) return 0;
     return chunk_lam_offset(s) + sizeof(float) * static_cast<size_t>(s.B) * s.Hq * s.R * chunk_slots(s);
+}
+
+void generic_chunk_form(const Shape& s, int dtype, int32_t* form) {
+    if (!chunk_major(s, dtype)) return;
+    const ChunkForm f = chunk_form(s);
+    form[0] = f.tokens;
+    form[1] = f.heads;
+    form[2] = f.warps;
 }
 
 int launch_generic(const Shape& s, int dtype, const Tensors& t, cudaStream_t stream) {

@@ -64,6 +64,9 @@ size_t decode_fast_scratch_bytes(const Shape& s);
 // Decode in one launch of thread-block clusters (one landmark row per KV head).
 bool decode_cluster_supports(const Shape& s);
 int launch_decode_cluster(const Shape& s, const Tensors& t, cudaStream_t stream);
+// What hils_call_form reports (form is left alone where the kernels do not apply).
+void decode_cluster_form(const Shape& s, int32_t* form);
+void generic_chunk_form(const Shape& s, int dtype, int32_t* form);
 
 // Decode fast path run on the library's own static device scratch (see hils_decode_noalloc).
 int launch_decode_noalloc(const Shape& s, const Tensors& t, int32_t* device_status, cudaStream_t stream);
