@@ -24,6 +24,8 @@
 // way) the same calls took 12.7, 28.2, 117.3, 46.8 and 62.2.
 // Draft tokens of one sequence retrieve mostly the same chunks: the union of their selections is loaded once, and all
 // their heads fill the MMA's columns.
+#include <stddef.h>
+
 #include "internal.h"
 #include "tma.cuh"
 
@@ -57,7 +59,7 @@ struct CArgs {
     int lgp;           // logarithm of the columns per token: G rounded up to a power of two
     int list_cap;      // candidates per token a CTA can hold
     // byte offsets behind the buffers
-    int off_scores, off_items, off_ids;
+    int off_items, off_ids;
 };
 
 // Distributed shared memory
@@ -112,13 +114,6 @@ template <int TG>
 struct CSmem {
     static constexpr int kBins = TG == 1 ? 512 : 256;
     static constexpr int kCand = TG == 1 ? 256 : 128;      // candidates of a token that can be ranked against each other
-    union {
-        alignas(16) int hist[TG][kBins];
-        float recv[TG == 1 ? 32 : 64][32];     // (afterwards) the CTAs' shares of the quarter columns that this CTA writes
-    };
-    float2 recv_md[TG == 1 ? 32 : 64];         // and their maxima and denominators
-    unsigned long long own[TG][kCand];         // this CTA's candidates (score key, ~chunk id)
-    unsigned long long all[TG][kCand];         // the cluster's
     unsigned kmin, kmax;                       // span of this CTA's scores (ordered keys)
     float edge[TG];                            // published: score that this CTA's share of K of its candidates reach
     unsigned long long thr[TG];                // candidates from this key on are collected
@@ -128,9 +123,27 @@ struct CSmem {
     int bad;                                   // tokens whose candidates do not fit (bit m)
     unsigned long long prefix;
     int remaining;
-    float col_max[kMaxWarps][16], col_den[kMaxWarps][16];   // the warps' running maximum and denominator per column; row 0: the CTA's
+    float col_max[kMaxWarps][16], col_den[kMaxWarps][16];   // the warps' running maximum and denominator per column
     int wsum[kMaxWarps];
     uint64_t full[kMaxWarps][2];
+    alignas(16) unsigned long long all[TG][kCand];         // the cluster's candidates (score key, ~chunk id)
+    unsigned long long own[TG][kCand];         // this CTA's
+    int hist[TG][kBins];                       // (last, with the scores behind it: see Shares)
+};
+
+// Where the CTAs of a cluster leave their shares of the quarter columns (32 dimensions) that this CTA writes, kRows of them, with
+// their maxima and denominators.  They arrive while this CTA may still be at work, so they lie in what nobody has used since the
+// last cluster barrier, the histogram and the scores behind it, and take no room from the lists (a group of four tokens with lists of
+// 1000 candidates, or 5900 candidates of one, fill a CTA): the scores have been read by the barrier that published the counts.  Where every CTA
+// ranks all candidates the last barrier is the first one, and their scores, which are few, lie behind the shares.
+template <int TG>
+struct Shares {
+    static constexpr int kRows = TG == 1 ? 32 : 64;
+    static constexpr int kBehind = kRows * (32 * 4 + 8) - static_cast<int>(sizeof(CSmem<TG>::hist));       // bytes of them behind the histogram
+    static_assert(offsetof(CSmem<TG>, hist) + sizeof(CSmem<TG>::hist) == sizeof(CSmem<TG>) && sizeof(CSmem<TG>) % 16 == 0 && kBehind % 16 == 0,
+                  "the scores follow the histogram");
+    float row[kRows][32];
+    float2 md[kRows];
 };
 
 // NT: MMA column tiles of 8 (token x head columns), TG: tokens per unit at most.
@@ -147,7 +160,6 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     const int CS = a.cs, K = s.K, G = s.G, Gp = 1 << a.lgp;
     uint8_t* tail = bufs + NW * (2 * kHalf) + NW * kLmRow;
     Sm& sm = *reinterpret_cast<Sm*>(tail);
-    float* scores = reinterpret_cast<float*>(tail + a.off_scores);           // [TG][list_cap]
     Item* items = reinterpret_cast<Item*>(tail + a.off_items);
     int* sel_ids = reinterpret_cast<int*>(tail + a.off_ids);                 // [TG][K] the selection, best first
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
@@ -211,6 +223,8 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     const int lcs_t = rank_all ? 0 : a.lcs, rank_t = rank_all ? 0 : rank;
     const int n_tiles = any_list ? (((nc_max + 63) >> 6) - rank_t + (1 << lcs_t) - 1) >> lcs_t : 0;      // this CTA's
     const int my_tiles = n_tiles > warp ? per_warp(n_tiles - warp + NW - 1) : 0;
+    const int cap = TG == 1 ? 0 : rank_all ? (nc_max + 63) & ~63 : a.list_cap;
+    float* scores = reinterpret_cast<float*>(tail + sizeof(Sm) + (rank_all && CS > 1 ? Shares<TG>::kBehind : 0));      // [TG][cap]
     auto global_id = [&](int i) { return ((((i >> 6) << lcs_t) + rank_t) << 6) + (i & 63); };   // candidate of list position i
     const int lm_row0 = (seq * s.Hl + kvh) * s.C;
 
@@ -360,7 +374,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                         const float s0 = acc[mt][nt][2 * hr] * s.scale + bb, s1 = acc[mt][nt][2 * hr + 1] * s.scale + bb;
                         auto put = [&](int m, float u, bool writer) {
                             if (m >= ntok || !writer || !live) return;
-                            scores[m * a.list_cap + pos0 + r] = u;
+                            scores[m * cap + pos0 + r] = u;
                             umin = fminf(umin, u);
                             umax = fmaxf(umax, u);
                         };
@@ -396,7 +410,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
             for (int m = m_first; m < ntok; m += m_step) {
                 unsigned* keys = reinterpret_cast<unsigned*>(sm.all[m]);
                 const int nc = sm.nc[m];
-                for (int x = li; x < nc + 3; x += ls) keys[x] = x < nc ? ordered_key(scores[m * a.list_cap + x]) : 0u;
+                for (int x = li; x < nc + 3; x += ls) keys[x] = x < nc ? ordered_key(scores[m * cap + x]) : 0u;
             }
         } else {
             __syncthreads();
@@ -411,7 +425,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
 #pragma unroll 4
                 for (int i = li; i < n_list; i += ls)
                     if (global_id(i) < nc)
-                        atomicAdd(&sm.hist[m][min(kBins - 1, max(0, static_cast<int>((scores[m * a.list_cap + i] - lo) * inv)))], 1);
+                        atomicAdd(&sm.hist[m][min(kBins - 1, max(0, static_cast<int>((scores[m * cap + i] - lo) * inv)))], 1);
             }
             __syncthreads();
 #pragma unroll 1
@@ -467,7 +481,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
 #pragma unroll 4
                     for (int i = li; i < n_list; i += ls) {
                         const int id = global_id(i);
-                        const unsigned long long key = select_key(scores[m * a.list_cap + i], id);
+                        const unsigned long long key = select_key(scores[m * cap + i], id);
                         if (id < nc && key >= thr) {
                             const int p = atomicAdd(&sm.cnt[m], 1);
                             if (p < Sm::kCand) sm.own[m][p] = key;
@@ -503,7 +517,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                         __syncthreads();
                         for (int i = tid; i < n_list; i += NTH) {
                             const int id = global_id(i);
-                            const unsigned long long key = select_key(scores[m * a.list_cap + i], id);
+                            const unsigned long long key = select_key(scores[m * cap + i], id);
                             if (id < sm.nc[m] && (key & mask) == prefix) atomicAdd(&sm.hist[m][(key >> shift) & 255u], 1);
                         }
                         cluster_sync(CS);
@@ -878,7 +892,8 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
         a.out[orow * kD + dim] = __float2bfloat16_rn(live ? __fdividef(v, den) : 0.f);
         if (dim == 0) a.lse[orow] = live ? M + __logf(den) : 0.f;
     };
-    // the warps' sums (fixed order: deterministic); a warp takes a column at a time, the result replaces warp 0's
+    // the warps' sums (fixed order: deterministic); a warp takes a column at a time
+    Shares<TG>& shares = reinterpret_cast<Shares<TG>&>(sm.hist);
 #pragma unroll 1
     for (int cx = warp; cx < ntok * G; cx += NW) {
         const int m = TG == 1 ? 0 : cx / G, col = m * Gp + cx - m * G;
@@ -902,8 +917,8 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
 #pragma unroll
             for (int x = 0; x < 4; ++x) {
                 const int qx = cx * 4 + x, at = (qx >> a.lcs << a.lcs) + rank;
-                st_peer_f(peer_addr(smem_u32(&sm.recv[at][lane]), qx & (CS - 1)), v[x]);
-                if (lane < 2) st_peer_f(peer_addr(smem_u32(&sm.recv_md[at]) + 4 * lane, qx & (CS - 1)), lane ? den : M);
+                st_peer_f(peer_addr(smem_u32(&shares.row[at][lane]), qx & (CS - 1)), v[x]);
+                if (lane < 2) st_peer_f(peer_addr(smem_u32(&shares.md[at]) + 4 * lane, qx & (CS - 1)), lane ? den : M);
             }
         }
     }
@@ -913,11 +928,11 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
     for (int qx = warp * CS + rank; qx < ntok * G * 4; qx += NW * CS) {
         const int cx = qx >> 2, at = qx - rank;
         // lane r: CTA r's maximum and denominator
-        const float2 md = lane < CS ? sm.recv_md[at + lane] : make_float2(-INFINITY, 0.f);
+        const float2 md = lane < CS ? shares.md[at + lane] : make_float2(-INFINITY, 0.f);
         const float M = warp_max(md.x), f = md.x == -INFINITY ? 0.f : __expf(md.x - M), den = warp_sum(md.y * f);
         float n = 0.f;
 #pragma unroll 2
-        for (int r = 0; r < CS; ++r) n = fmaf(sm.recv[at + r][lane], __shfl_sync(kFullMask, f, r), n);
+        for (int r = 0; r < CS; ++r) n = fmaf(shares.row[at + r][lane], __shfl_sync(kFullMask, f, r), n);
         emit(cx, (qx & 3) * 32 + lane, n, M, den);
     }
 }
@@ -958,7 +973,7 @@ int launch(const CArgs& a, const CUtensorMap& mk, const CUtensorMap& mv, const C
 }
 
 struct ClusterPlan {
-    int cs, lcs, warps, tg, gp, nt, list_cap, off_scores, off_items, off_ids, units;
+    int cs, lcs, warps, tg, gp, nt, list_cap, off_items, off_ids, units;
     size_t smem;
 };
 
@@ -1017,12 +1032,19 @@ bool plan_tokens(const Shape& s, int tg, int n_sm, ClusterPlan* p) {
         p->cs = cs;
         p->lcs = lcs;
         p->list_cap = ((cand + 63) / 64 + cs - 1) / cs * 64;
-        // (a short list is held whole by every CTA)
-        const int most = rank_all_most(multi, p->warps, cs), whole = ((cand < most ? cand : most) + 63) / 64 * 64;
-        if (p->list_cap < whole) p->list_cap = whole;
+        // Long lists of units that take turns on the SMs.  Groups: apart, on three warps, is as fast or faster (20 x 51,200 tokens, four
+        // drafts, us grouped / apart: 8 query heads per KV head 131 / 117, 4 heads 114 / 113; while all units are resident, 16 x 64K, 67 / 79).
+        // Two CTAs per SM only where they do not add a turn (K = 16 - 32, us two / one: 32 x 108K tokens, 256 units, 48 / 52; 40 x 90K, 320
+        // units, 88 / 85).
+        const auto turns = [&](long long at_once) { return (units + at_once - 1) / at_once; };
+        if (multi ? units > n_sm && p->list_cap > 768 : per_sm == 2 && p->list_cap > 1344 && 2 * turns(2 * n_sm) > turns(n_sm)) continue;
         size_t off = multi ? sizeof(CSmem<4>) : sizeof(CSmem<1>);
         auto take = [&](size_t bytes) { const size_t at = (off + 15) / 16 * 16; off = at + bytes; return static_cast<int>(at); };
-        p->off_scores = take(sizeof(float) * TG * p->list_cap);
+        // the scores, or those of a short list that every CTA holds whole, behind the shares of the output
+        const int most = rank_all_most(multi, p->warps, cs), whole = ((cand < most ? cand : most) + 63) / 64 * 64;
+        const size_t list = sizeof(float) * TG * p->list_cap, shares = cs == 1 ? 0 : multi ? Shares<4>::kBehind : Shares<1>::kBehind;
+        const size_t ranked = shares + sizeof(float) * TG * whole;
+        take(list > ranked ? list : ranked);
         p->off_items = take(sizeof(Item) * ((TG * s.K + local + cs - 1) / cs + 1));
         p->off_ids = take(sizeof(int) * TG * s.K);
         p->smem = 1024 + off + static_cast<size_t>(p->warps) * (2 * kHalf + kLmRow);
@@ -1086,7 +1108,6 @@ int launch_decode_cluster(const Shape& s, const Tensors& t, cudaStream_t stream)
     a.lgp = 0;
     while ((1 << a.lgp) < p.gp) ++a.lgp;
     a.list_cap = p.list_cap;
-    a.off_scores = p.off_scores;
     a.off_items = p.off_items;
     a.off_ids = p.off_ids;
     const int seqs = s.B / s.qps;

@@ -113,12 +113,22 @@ def test_lists_that_leave_some_ctas_few_candidates_or_none(n, K, W):
     check_decode(cfg, inp, *got, W=W)
 
 
-@pytest.mark.parametrize("B,M,K", [(16, 3, 17), (32, 3, 16), (20, 4, 16), (40, 2, 33)])
-def test_groups_of_draft_tokens_on_six_and_on_three_warps(B, M, K):
+def form(cfg, M=1):
+    p = hils.make_params(B=cfg.B, Hq=cfg.Hq, Hkv=cfg.Hkv, Hl=cfg.Hkv, L=0, T_max=cfg.L, C=cfg.C, d=128, chunk_size=64, top_k=cfg.K,
+                         window=cfg.window, dtype=1)
+    return hils.call_form(p, True, M)[:3]
+
+
+# want: tokens per unit, warps per CTA (no room for clusters of more than one)
+@pytest.mark.parametrize("B,M,K,T,want", [(16, 3, 17, 64 * 90, (3, 6)), (32, 3, 16, 64 * 90, (3, 6)), (20, 4, 16, 64 * 90, (4, 6)),
+                                          (40, 2, 33, 64 * 90, (2, 6)), (32, 4, 12, 64 * 65, (4, 3)), (40, 3, 8, 64 * 65, (3, 3)),
+                                          (64, 2, 14, 64 * 65, (2, 3))])
+def test_groups_of_draft_tokens_on_six_and_on_three_warps(B, M, K, T, want):
     """A group's tokens share the selection's warps (max(1, warps / tokens) each); the chunks are attended in the order of their
     scores and reported in ascending order."""
-    cfg = wl.HilsConfig("groups", "decode", B, 32, 8, 64 * 90, 128, 64, K, "bf16", 800 + M * B, n_needles=2, window=1)
-    lens = torch.tensor([64 * 90 - (b * 371) % (64 * 80) for b in range(B)], dtype=torch.int32)
+    cfg = wl.HilsConfig("groups", "decode", B, 32, 8, T, 128, 64, K, "bf16", 800 + M * B, n_needles=2, window=1)
+    assert form(cfg, M) == want + (1,)
+    lens = torch.tensor([T - (b * 371) % (T - 640) for b in range(B)], dtype=torch.int32)
     t = wl.make_decode_inputs(cfg, DEV, seq_lens=lens.to(DEV))
     q = torch.randn((B, M, 32, 128), generator=torch.Generator().manual_seed(M)).to(torch.bfloat16).to(DEV)
     out, lse, sel = hils.hils_decode_multi(q, t["k"], t["v"], t["landmarks"], t["seq_lens"], 64, K)
@@ -152,3 +162,48 @@ def test_pages_of_local_chunks_out_of_range(T, W):
     out, lse, sel = run()
     assert hils.poll_status(ws) == -7
     assert torch.equal(sel, good[2]) and torch.equal(out[1], good[0][1]) and torch.equal(lse[1], good[1][1])
+
+
+@pytest.mark.parametrize("T,marks", [(64 * 70, "random"), (64 * 300 + 5, "random"), (64 * 300, "equal"), (64 * 12, "random")])
+def test_groups_in_clusters(T, marks):
+    """Groups of four drafts on two CTAs, whose shares of the output meet in what ranking, listing (and, with ties, the radix
+    selection) leave: every candidate ranked, a list, a list of equal scores, nothing to select."""
+    B, M, K, W = 8, 4, 16, 512
+    cfg = wl.HilsConfig("pairs", "decode", B, 32, 8, T, 128, 64, K, "bf16", 960, n_needles=2, window=W)
+    assert form(cfg, M) == (4, 6, 2)
+    lens = torch.tensor([T - 17 * b for b in range(B)], dtype=torch.int32)
+    t = wl.make_decode_inputs(cfg, DEV, seq_lens=lens.to(DEV))
+    if marks == "equal":
+        t["landmarks"][:] = t["landmarks"][:1, :1, :1].clone()
+    bias = None if marks == "equal" else wl.make_bias(cfg, DEV)
+    q = torch.randn((B, M, 32, 128), generator=torch.Generator().manual_seed(T)).to(torch.bfloat16).to(DEV)
+    out, lse, sel = hils.hils_decode_multi(q, t["k"], t["v"], t["landmarks"], t["seq_lens"], 64, K, window=W, bias=bias)
+    torch.cuda.synchronize()
+    assert hils.last_launch_count() == 1
+    for m in range(M):
+        o, l, s = hils.hils_decode(q[:, m].contiguous(), t["k"], t["v"], t["landmarks"], t["seq_lens"] - (M - 1 - m), 64, K, window=W, bias=bias)
+        torch.cuda.synchronize()
+        assert torch.equal(s, sel[:, m])
+        # (two roundings to bf16 of sums in different orders, outputs below 2: twice 2^-8 = 8e-3)
+        assert (o.float() - out[:, m].float()).abs().max() <= 1.6e-2 and (l - lse[:, m]).abs().max() <= 1e-4
+
+
+@pytest.mark.parametrize("B,M,chunks,K,want", [(10, 1, 6200, 32, (1, 6, 1)), (16, 4, 1000, 32, (4, 6, 1)), (32, 1, 1700, 16, (1, 3, 1))])
+def test_lists_that_fill_a_cta(B, M, chunks, K, want):
+    """Against the same sequences one by one (other splits of the lists); the caches are pages that the sequences share."""
+    cfg = wl.HilsConfig("long", "decode", B, 32, 8, 64 * chunks, 128, 64, K, "bf16", 961)
+    assert form(cfg, M) == want
+    g = torch.Generator(device=DEV).manual_seed(chunks)
+    rnd = lambda *shape: torch.randn(shape, device=DEV, generator=g).to(torch.bfloat16)
+    q, kp, vp, lm = rnd(B, M, 32, 128), rnd(97, 8, 64, 128), rnd(97, 8, 64, 128), rnd(B, 8, chunks, 128)
+    table = torch.randint(0, 97, (B, chunks), device=DEV, generator=g).to(torch.int32)
+    lens = torch.tensor([64 * chunks - 131 * b for b in range(B)], dtype=torch.int32, device=DEV)
+    out, lse, sel = hils.hils_decode_multi(q, kp, vp, lm, lens, 64, K, block_table=table)
+    torch.cuda.synchronize()
+    assert hils.last_launch_count() == 1
+    for b in range(B):
+        for m in range(M):
+            o, l, s = hils.hils_decode_paged(q[b:b + 1, m].contiguous(), kp, vp, lm[b:b + 1], table[b:b + 1], lens[b:b + 1] - (M - 1 - m), 64, K)
+            torch.cuda.synchronize()
+            assert torch.equal(s[0], sel[b, m])
+            assert (o[0].float() - out[b, m].float()).abs().max() <= 1.6e-2 and (l[0] - lse[b, m]).abs().max() <= 1e-4
