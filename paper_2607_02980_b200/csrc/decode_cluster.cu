@@ -416,7 +416,10 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
             __syncthreads();
             // A score that this CTA's share of K of its candidates reach, off a histogram with bins of equal width in the
             // score (the bins of a radix digit are equal in the exponent, and most scores share two or three exponents).
-            const float lo = key_to_float(sm.kmin), inv = __fdividef(static_cast<float>(kBins), key_to_float(sm.kmax) - lo);
+            // (both scaled by 2^-8: a mask of the lowest finite number spans more than 2^126, beyond which this division returns 0, and without
+            // bins every candidate is collected and goes through the radix selection: 8 x 25,600 tokens, K = 16, 70 % masked 25.0 us, 20.4
+            // with the bins)
+            const float lo = key_to_float(sm.kmin), inv = __fdividef(kBins * 0x1p-8f, (key_to_float(sm.kmax) - lo) * 0x1p-8f);
             const bool cut = inv > 0.f && inv < INFINITY;              // (no span: every candidate is collected)
 #pragma unroll 1
             for (int m = m_first; m < ntok; m += m_step) {

@@ -141,3 +141,26 @@ def test_a_query_that_is_not_a_number_spoils_its_own_row_only(L, K):
 def test_masks_of_the_lowest_finite_number(mode, L, K, impl, share):
     cfg = wl.HilsConfig("lowest", mode, 1, 8, 2, L, 128, 64, K, "bf16", 1400 + K)
     (decode if mode == "decode" else prefill)(cfg, share, impl=impl, mask=torch.finfo(torch.float32).min)
+
+
+def test_masks_of_the_lowest_finite_number_take_the_short_path():
+    """A list with such masks has a histogram like any other (up to 256 of its chunks are ranked), where its span of 3.4e38 must not
+    turn the bins' width into nothing: the kernel takes as long as with masks of -1e30.  (Without a histogram the radix selection
+    over the cluster takes a quarter more.)"""
+    B, T, K = 8, 64 * 400, 16
+    cfg = wl.HilsConfig("path", "decode", B, 32, 8, T, 128, 64, K, "bf16", 1450)
+    t = wl.make_decode_inputs(cfg, DEV)
+    masked = torch.rand((B, 8, cfg.C), generator=torch.Generator().manual_seed(7)) < 0.7
+    lowest = [torch.where(masked, m, torch.zeros(())).contiguous().to(DEV) for m in (-1e30, torch.finfo(torch.float32).min)]
+    times, sels = ([], []), []
+    hils.trace_enable(True)
+    try:
+        for i in range(60):
+            got = hils.hils_decode(t["q"], t["k"], t["v"], t["landmarks"], t["seq_lens"], 64, K, bias=lowest[i & 1])
+            (name, ms), = hils.trace_read()
+            times[i & 1].append(ms)
+            sels.append(got[2])
+    finally:
+        hils.trace_enable(False)
+    assert name == "decode_cluster" and torch.equal(sels[0], sels[1])
+    assert min(times[1]) <= 1.1 * min(times[0]), (min(times[0]), min(times[1]))
