@@ -22,10 +22,10 @@
 //   warp 11          builds the unit's list of chunks (and which tile needs them, with a bit per token), one unit ahead
 // Bound: the softmax warps' serial chain per chunk, 2000 cycles: answer of the barrier 290, tensor-memory load 100, maximum 200, exponentials
 // 750 (two warps per scheduler; special-function unit 37 % busy), weight 200, accumulator's answer 170, probabilities back 190.  The
-// tensor pipe needs 1350 of them.  2 x 6000 tokens, K = 32: 661 -> 587 us with the quotient w / z by the approximate reciprocal (the
-// exactly rounded division took 300 cycles of the chain; its result is rounded to bf16 next) and the next item's barrier asked early.
+// tensor pipe needs 1350 of them.  The rounded division of w by z took 300 cycles of the chain: 2 x 6000 tokens, K = 32, us for the call with
+// it 739, with quotient() 694 (with the approximate quotient, which loses two bits, 686); the next item's barrier is asked early.
 // A unit's fixed part: 9300 -> 5000 cycles with the output staged beside the query tile, so that the next unit's queries come with this
-// one's last scores, and the unit's place worked out once, by the list warp (2 x 6000 tokens 587 -> 571 us, 3 x 1000 44.9 -> 41.8).
+// one's last scores, and the unit's place worked out once, by the list warp (this kernel on 2 x 6000 tokens 587 -> 571 us, the call on 3 x 1000 44.9 -> 42.0).
 // Sixteen softmax warps, half a row's keys or every other item each: 704 and 781 us (more instructions, colder instruction cache).
 #include "internal.h"
 #include "tma.cuh"
@@ -251,7 +251,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                 }
                 const float w = act ? __expf(lam - ref) : 0.f;
                 den += w;
-                const float pw = act ? __fdividef(w, z) : 0.f;
+                const float qz = quotient(w, z), pw = act ? qz : 0.f;
                 const float2 pw2 = make_float2(pw, pw);
                 // the previous chunk's value product has read its probabilities and left the accumulator
                 if (i > 0) {
@@ -294,7 +294,7 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                 if (!wait(&sm.o_done[t], (n_s - 1) & 1)) break;
                 __syncwarp();
                 tc_fence_after_sync();
-                const float inv = live ? __fdividef(1.f, den) : 0.f;
+                const float inv = live ? 1.f / den : 0.f;
                 const long long orow = (static_cast<long long>(b) * s.Hq + gk * kG + h) * s.R + tok;
                 const bool whole = blk * kUnitTok + t * kTok + kTok <= a.n_tok;
                 // 64 dimensions at a time through the warp's own staging rows (not through the query tile: the next unit's queries
