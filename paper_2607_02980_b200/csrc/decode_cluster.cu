@@ -18,10 +18,11 @@
 // Bound: HBM (landmarks scanned + selected K / V), and where a call has few units the chain of dependent steps.  One
 // launch per step (decode_fast.cu) drains and ramps between short phases and leaves the memory idle during the
 // selection.  Before / now, B200, us per call through the Python entry points, calls back to back: 1 x 6000 tokens, K = 16:
-// 22.7 / 9.3; 8 x 4K-16K paged, K = 32, W = 512: 49.3 / 22.7; 64 x 64K, K = 32: 142.6 / 113.8 (6.1 TB/s); 4 x 1M, K = 64: 65.4 / 43.5;
+// 22.7 / 9.2; 8 x 4K-16K paged, K = 32, W = 512: 49.3 / 22.7; 64 x 64K, K = 32: 142.6 / 111 (6.2 TB/s); 4 x 1M, K = 64: 65.4 / 43.5;
 // 16 x 8K-32K, four drafts, K = 32: 121 / 56.7.  Before this form of its short steps (landmark tiles asked for ahead of the queries, a
-// tile's biases under its wait, items placed by rank with sel_idx sorted behind the loads, no integer or exactly rounded division on the
-// way) the same calls took 12.7, 28.2, 117.3, 46.8 and 62.2.
+// tile's biases under its wait, items placed by rank with sel_idx sorted behind the loads, no integer division on the way) the same calls
+// took 12.7, 28.2, 117.3, 46.8 and 62.2.  (The output's rounded division is 0.1 us of the first: without it means that lie half way between
+// two bf16 numbers came out on the wrong side.)
 // Draft tokens of one sequence retrieve mostly the same chunks: the union of their selections is loaded once, and all
 // their heads fill the MMA's columns.
 #include <stddef.h>
@@ -813,7 +814,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
                     const float w = __expf(lam - nm);
                     Dn[nt][x] = fmaf(Dn[nt][x], f_[nt][x], w);
                     Mx[nt][x] = nm;
-                    pw = __fdividef(w, z);
+                    pw = quotient(w, z);
                 }
                 moved = moved || f_[nt][x] != 1.f;
 #pragma unroll
@@ -892,7 +893,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_co
         const int m = TG == 1 ? 0 : cx / G, h = cx - m * G;
         const bool live = sm.len[m] > 0;
         const long long orow = static_cast<long long>(query0 + m) * s.Hq + kvh * G + h;
-        a.out[orow * kD + dim] = __float2bfloat16_rn(live ? __fdividef(v, den) : 0.f);
+        a.out[orow * kD + dim] = __float2bfloat16_rn(live ? v / den : 0.f);
         if (dim == 0) a.lse[orow] = live ? M + __logf(den) : 0.f;
     };
     // the warps' sums (fixed order: deterministic); a warp takes a column at a time

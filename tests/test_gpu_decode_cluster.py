@@ -207,3 +207,40 @@ def test_lists_that_fill_a_cta(B, M, chunks, K, want):
             torch.cuda.synchronize()
             assert torch.equal(s[0], sel[b, m])
             assert (o[0].float() - out[b, m].float()).abs().max() <= 1.6e-2 and (l[0] - lse[b, m]).abs().max() <= 1e-4
+
+
+def test_a_mean_of_chunks_is_rounded_once():
+    """Keys and landmarks of zeros: the n chunks of a sequence and the one token behind them weigh 1 each, and the output is the sum
+    of their values, exact in fp32, over n + 1.  The values make it lie half way between two bf16 numbers, where a quotient that is off
+    in its last place rounds to the wrong one."""
+    B, T, K = 32, 64 * 33, 32
+    cfg = wl.HilsConfig("mean", "decode", B, 8, 2, T, 128, 64, K, "bf16", 972)
+    zeros = lambda *shape: torch.zeros(shape, dtype=torch.bfloat16)
+    v = torch.ones((B, 2, T, 128))
+    tie = 2 * (torch.arange(128) % 80) + 1                    # the means: 1 + tie / 256, tie odd
+    for b in range(B):
+        n = b + 2                                             # chunks, the last one's single token among them
+        # n tie / 256 in numbers of eight bits: even steps of 1 / 256 above one, any below
+        left = n * tie
+        if n % 2 == 1:
+            v[b, :, 64 * (n - 1):] -= 1 / 256
+            left = left + 1
+        for c in range(n - n % 2):
+            step = torch.round(left / (2 * (n - n % 2 - c))) * 2
+            v[b, :, 64 * c:64 * (c + 1) if c < n - 1 else T] += step / 256
+            left = left - step
+        assert (left == 0).all()
+    want = (1 + torch.where(tie % 4 == 1, tie - 1, tie + 1) / 256).expand(B, 8, 128)      # (ties to even)
+    assert torch.equal(v, v.to(torch.bfloat16).float())
+    lens = torch.tensor([64 * (b + 1) + 1 for b in range(B)], dtype=torch.int32, device=DEV)
+    q = torch.randn((B, 8, 128), generator=torch.Generator().manual_seed(1)).to(torch.bfloat16)
+    args = [x.to(DEV) for x in (zeros(B, 2, T, 128), v.to(torch.bfloat16), zeros(B, 2, T // 64, 128))]
+    out, lse, sel = hils.hils_decode(q.to(DEV), *args, lens, 64, K)
+    torch.cuda.synchronize()
+    assert hils.last_launch_count() == 1
+    assert torch.equal(out.float().cpu(), want)
+    qm = torch.stack([q, q], 1).to(DEV)
+    many = [x.repeat(3, 1, 1, 1) for x in args]
+    out = hils.hils_decode_multi(qm.repeat(3, 1, 1, 1), *many, lens.repeat(3) , 64, K)[0]
+    torch.cuda.synchronize()
+    assert torch.equal(out[:, 1].float().cpu(), want.repeat(3, 1, 1))
