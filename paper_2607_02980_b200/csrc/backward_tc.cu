@@ -112,7 +112,7 @@ __device__ __forceinline__ void red_add_v4(float* p, float x, float y, float z, 
 __global__ void __launch_bounds__(kThreads, 1)
 backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                    const __grid_constant__ CUtensorMap map_dq, const BArgs a) {
-    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    extern __shared__ __align__(1024) uint8_t smem_raw[];     // (no room to round up: see tiles_aligned)
     uint8_t* qbuf = smem_raw;                    // [2]
     uint8_t* obuf = qbuf + 2 * kQBytes;          // dO rows [2]
     uint8_t* kbuf = obuf + 2 * kQBytes;
@@ -123,11 +123,6 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     Tile* const rec = reinterpret_cast<Tile*>(stgbuf + 8 * kStgBytes);
     BSmem& sm = *reinterpret_cast<BSmem*>(kbuf + kKHole + kDlamBytes);
     auto dlam_of = [&](uint32_t par) { return reinterpret_cast<float*>(kbuf + kKHole + par * kKBlock); };
-    // (the swizzled tiles need the 1024-byte alignment that a kernel without static shared memory has; there is no room to round up)
-    if (smem_u32(smem_raw) & 1023u) {
-        if (threadIdx.x == 0) set_status(a.status, kDevTimeout);
-        return;
-    }
     const Shape& s = a.s;
     const int tid = threadIdx.x, warp = __shfl_sync(kFullMask, tid >> 5, 0), lane = tid & 31;
 
@@ -682,8 +677,26 @@ size_t dsum_bytes(const Shape& s) { return (static_cast<size_t>(s.B) * s.Hq * s.
 
 }  // namespace
 
+// The swizzled tiles start on multiples of 1024 bytes if the kernel's dynamic shared memory does, which lies behind what the system
+// reserves (1024 bytes) and the kernel's static part (none).  Where a toolchain lays this out in another way the generic kernel
+// takes the calls.  (Asked once per device; true where no device answers, e.g. a workspace-size query on a host without a GPU.)
+static bool tiles_aligned() {
+    static int known[64] = {};                   // 1: aligned, 2: not
+    const int dev = PerDeviceOnce::device();
+    if (dev < 0) return true;
+    if (known[dev] == 0) {
+        int reserved = 0;
+        cudaFuncAttributes attr;
+        if (cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess ||
+            cudaFuncGetAttributes(&attr, backward_tc_kernel) != cudaSuccess)
+            return true;
+        known[dev] = (static_cast<size_t>(reserved) + attr.sharedSizeBytes) % 1024 == 0 ? 1 : 2;
+    }
+    return known[dev] == 1;
+}
+
 bool prefill_backward_fast_supports(const Shape& s, int dtype) {
-    return prefill_fast_supports(s, dtype) && s.Hl == s.Hkv && s.K + 17 <= 255 &&
+    return prefill_fast_supports(s, dtype) && tiles_aligned() && s.Hl == s.Hkv && s.K + 17 <= 255 &&
            static_cast<long long>(s.B) * s.Hq * s.R < (1ll << 31);
 }
 
