@@ -325,7 +325,7 @@ int hils_last_launch_count(void);
  * neither of these kernels runs.
  *   Decode in one launch (is_decode = 1, tokens_per_seq newest tokens per sequence): tokens that share a unit, warps per CTA,
  *     CTAs per cluster, candidates per token up to which every CTA ranks all of them.
- *   fp32 prefill, chunk-major: tokens per CTA, query heads per CTA, warps per CTA, 0. */
+ *   fp32 prefill, chunk-major: tokens per CTA, query heads per CTA, warps per CTA, 1 where the tokens are walked from the middle on. */
 int hils_call_form(const hils_params* params, int is_decode, int32_t tokens_per_seq, int32_t* form);
 
 /* Per-kernel timing for profiling (no counterpart in the paper; Sec. 7.1 reports end-to-end latency

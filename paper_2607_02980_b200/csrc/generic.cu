@@ -593,19 +593,21 @@ __device__ __forceinline__ void chunk_rows(const GArgs& a, ChunkSmem<D, NW>& sm,
     __syncwarp();
 }
 
-// NW: warps per CTA and most rows of a warp at a time, row_block: tokens (nb blocks), nh: query heads (of one KV head)
+// NW: warps per CTA and most rows of a warp at a time, row_block: tokens (nb blocks), nh: query heads (of one KV head), mid_first: whether
+// the blocks are walked from the middle ones on (see chunk_form)
 template <int D, int NW>
 __global__ void __launch_bounds__(NW * 32, 16 / NW)
-generic_chunk_kernel(const GArgs a, int row_block, int nb, int nh, float* part, float* lam) {
+generic_chunk_kernel(const GArgs a, int row_block, int nb, int nh, int mid_first, float* part, float* lam) {
     extern __shared__ uint8_t chunk_raw[];
     ChunkSmem<D, NW>& sm = *reinterpret_cast<ChunkSmem<D, NW>*>(chunk_raw);
     const Shape& s = a.s;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // blocks of tokens y (from the last one on) and y (from the first one on) share a row of CTAs, one per chunk up to their last tokens
-    const int hi = nb - 1 - blockIdx.y, n_hi = block_chunks(s, row_block, hi);
-    const bool low = static_cast<int>(blockIdx.x) >= n_hi;
-    const int blk = low ? blockIdx.y : hi, c = low ? blockIdx.x - n_hi : blockIdx.x;
-    if (low && (blk == hi || c >= block_chunks(s, row_block, blk))) return;
+    // two blocks of tokens, as far from the first one as from the last, share a row of CTAs, one per chunk up to their last tokens: from the
+    // ends on with the late one first, or from the middle on with the early one, whose tokens attend most of their chunks, first
+    const int y = mid_first ? gridDim.y - 1 - blockIdx.y : nb - 1 - blockIdx.y, n_y = block_chunks(s, row_block, y);
+    const bool other = static_cast<int>(blockIdx.x) >= n_y;
+    const int blk = other ? nb - 1 - y : y, c = other ? blockIdx.x - n_y : blockIdx.x;
+    if (other && (blk == y || c >= block_chunks(s, row_block, blk))) return;
     int b = 0, g = blockIdx.z, h0 = 0;                                      // z: (sequence, KV head, nh of its query heads)
     if (nh < s.G) {
         const int per = s.G / nh;
@@ -730,16 +732,21 @@ long long chunk_ctas(const Shape& s, int rb) {
 //   d = 64:  8 x 841, one head 55 / 62 / 65; 2048, 2 heads (1) 51 / 52 / 60; 2048, 4 heads (2) 87 / 82 / 90; 3 x 2048, 4 heads (2)
 //            227 / 203 / 221; 3 x 3300, 4 heads (2) 459 / 371 / 346
 // (with four warps for 32 tokens everywhere and eight for 128, one line between them: 56, 55, 142, 110, 260; 66, 51, 101, 227, 380)
-struct ChunkForm { int tokens, heads, warps; };        // per CTA: tokens, query heads of a KV head, warps
+// Where a few of the 32-token CTAs are left over from the first that are resident (four per SM at d = 64, two at 128), the blocks are walked
+// from the middle on, which leaves the last blocks' chunks, with the fewest rows, for the end; elsewhere from the ends on (us, one head,
+// d = 64, from the middle / from the ends: 1612 tokens, K = 8, 1.14 times the resident CTAs, 29.2 / 31.4; 1800, 1.42 times, 31.0 / 32.6; 2048
+// tokens, K = 4, 1.78 times, 29.5 / 28.1).
+struct ChunkForm { int tokens, heads, warps, mid_first; };        // per CTA: tokens, query heads of a KV head, warps
 ChunkForm chunk_form(const Shape& s) {
     const long long ctas = chunk_ctas(s, 32), heads = ctas * s.G, sms = sm_count();
     const int warps = s.d == 64 ? 4 : 8;
-    if (ctas >= (s.d == 64 ? 60 : 15) * sms) return {kRowBlockMax, s.G, warps};
-    return {heads >= (s.d == 64 ? 24 : 7) * sms ? 64 : 32, 1, warps};
+    if (ctas >= (s.d == 64 ? 60 : 15) * sms) return {kRowBlockMax, s.G, warps, 0};
+    if (heads >= (s.d == 64 ? 24 : 7) * sms) return {64, 1, warps, 0};
+    return {32, 1, warps, 10 * heads <= 16 * (16 / warps) * sms ? 1 : 0};
 }
 
 template <int D, int NW>
-int launch_chunk_kernel(const GArgs& a, int rb, int nh, float* part, float* lam, cudaStream_t stream) {
+int launch_chunk_kernel(const GArgs& a, int rb, int nh, int mid_first, float* part, float* lam, cudaStream_t stream) {
     const Shape& s = a.s;
     static PerDeviceOnce once;
     if (once.pending()) {
@@ -754,7 +761,7 @@ int launch_chunk_kernel(const GArgs& a, int rb, int nh, float* part, float* lam,
         width = w > width ? w : width;
     }
     return launch_pdl(generic_chunk_kernel<D, NW>, dim3(static_cast<unsigned>(width), static_cast<unsigned>((nb + 1) / 2), static_cast<unsigned>(s.B * s.Hq / nh)), dim3(NW * 32),
-                      sizeof(ChunkSmem<D, NW>), stream, a, rb, nb, nh, part, lam) == cudaSuccess ? 0 : HILS_ERR_CUDA;
+                      sizeof(ChunkSmem<D, NW>), stream, a, rb, nb, nh, mid_first, part, lam) == cudaSuccess ? 0 : HILS_ERR_CUDA;
 }
 
 template <int D>
@@ -764,7 +771,7 @@ int launch_chunk_major(const GArgs& a, void* scratch, cudaStream_t stream) {
     float* lam = reinterpret_cast<float*>(static_cast<char*>(scratch) + chunk_lam_offset(s));
     const long long rows = static_cast<long long>(s.B) * s.Hq * s.R;
     const ChunkForm f = chunk_form(s);
-    if (launch_chunk_kernel<D, D == 64 ? 4 : 8>(a, f.tokens, f.heads, part, lam, stream) != 0) return HILS_ERR_CUDA;
+    if (launch_chunk_kernel<D, D == 64 ? 4 : 8>(a, f.tokens, f.heads, f.mid_first, part, lam, stream) != 0) return HILS_ERR_CUDA;
     trace_mark("generic_attend", stream);
     if (launch_pdl(generic_fuse_kernel<D>, dim3(static_cast<unsigned>((rows + kWarpsPerBlock - 1) / kWarpsPerBlock)),
                    dim3(kWarpsPerBlock * 32), 0, stream, a, static_cast<const float*>(part), static_cast<const float*>(lam)) != cudaSuccess)
@@ -823,6 +830,7 @@ void generic_chunk_form(const Shape& s, int dtype, int32_t* form) {
     form[0] = f.tokens;
     form[1] = f.heads;
     form[2] = f.warps;
+    form[3] = f.mid_first;
 }
 
 int launch_generic(const Shape& s, int dtype, const Tensors& t, cudaStream_t stream) {

@@ -26,16 +26,19 @@ def test_errors_and_other_kernels():
 
 
 @pytest.mark.parametrize("B,Hq,Hkv,L,d,S,K,W,want", [
-    (2, 4, 2, 1300, 128, 64, 4, 1, (64, 1, 8)),
-    (2, 6, 2, 1217, 64, 48, 3, 100, (64, 1, 4)),
-    (4, 2, 2, 1281, 64, 64, 8, 65, (32, 1, 4)),
-    (1, 3, 1, 230, 128, 64, 4, 70, (32, 1, 8)),
-    (3, 4, 2, 1300, 128, 64, 4, 1, (128, 2, 8)),
-    (3, 6, 2, 1217, 64, 16, 5, 1, (128, 3, 4)),
-    (1, 2, 1, 31, 64, 16, 2, 1, (32, 1, 4)),
+    (2, 4, 2, 1300, 128, 64, 4, 1, (64, 1, 8, 0)),
+    (2, 6, 2, 1217, 64, 48, 3, 100, (64, 1, 4, 0)),
+    (4, 2, 2, 1281, 64, 64, 8, 65, (32, 1, 4, 0)),
+    (1, 3, 1, 230, 128, 64, 4, 70, (32, 1, 8, 1)),
+    (3, 4, 2, 1300, 128, 64, 4, 1, (128, 2, 8, 0)),
+    (3, 6, 2, 1217, 64, 16, 5, 1, (128, 3, 4, 0)),
+    (1, 2, 1, 31, 64, 16, 2, 1, (32, 1, 4, 1)),
+    (1, 1, 1, 1612, 64, 64, 8, 1, (32, 1, 4, 1)),
+    (1, 1, 1, 1730, 64, 48, 8, 40, (32, 1, 4, 0)),
+    (1, 2, 1, 1000, 64, 64, 8, 130, (32, 1, 4, 1)),
 ])
 def test_fp32_prefill(B, Hq, Hkv, L, d, S, K, W, want):
-    assert hils.call_form(params(B, Hq, Hkv, L, d, S, K, 0, W=W), False) == want + (0,)
+    assert hils.call_form(params(B, Hq, Hkv, L, d, S, K, 0, W=W), False) == want
 
 
 @pytest.mark.parametrize("B,Hkv,T,K,W,G,want", [

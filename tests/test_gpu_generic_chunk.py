@@ -22,6 +22,9 @@ DEV = "cuda"
     (3, 4, 2, 1300, 128, 64, 4, 1, True, False),       # 128 tokens, all heads, 11 blocks, eight warps
     (3, 6, 2, 1217, 64, 16, 5, 1, True, True),         # 128 tokens, three heads, chunks of 16, four warps
     (1, 2, 1, 31, 64, 16, 2, 1, False, False),
+    (1, 1, 1, 1612, 64, 64, 8, 1, False, False),       # 32 tokens, 51 blocks from the middle on
+    (1, 1, 1, 1730, 64, 48, 8, 40, True, False),       # 55 from the ends on
+    (1, 2, 1, 1000, 64, 64, 8, 130, True, False),      # 32 from the middle on
 ])
 def test_against_the_oracle(B, Hq, Hkv, L, d, S, K, W, bias, per_head):
     cfg = wl.HilsConfig("fp32", "prefill", B, Hq, Hkv, L, d, S, K, "f32", 900 + L, window=W)
