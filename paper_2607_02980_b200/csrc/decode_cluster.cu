@@ -107,8 +107,9 @@ struct Item {
 };
 
 // Candidates per token up to which every CTA scores and ranks all of them, without a histogram and without waiting for the others:
-// about one per thread.  Us, by histogram / this way: 6K tokens (93 candidates) 11.1 / 8.6, 12K (190) 11.8 / 10.5, 16K (249) 11.7 / 13.8;
-// clusters of one CTA 8K (124) 19.7 / 18.8, 12K 30.8 / 31.1; three warps 6K 49.3 / 47.2, 8K 49.5 / 50.4; four drafts at 8K 34.8 / 37.7.
+// about one per thread.  Us per call, by histogram / this way: 6K tokens (93 candidates) 11.8 / 9.3, 12K (190) 11.9 / 11.0, 16K (249) 11.9 /
+// 14.1; clusters of one CTA 8K (124) 20.0 / 19.0, 12K 20.2 / 20.5; three warps 6K 50.6 / 48.5, 8K 50.8 / 51.4; four drafts 4K (63) 32.9 / 31.9,
+// 8K 35.2 / 38.0.
 __host__ __device__ inline int rank_all_most(bool multi, int warps, int cs) { return multi ? 64 : warps == 3 ? 96 : cs > 1 ? 192 : 128; }
 
 template <int TG>

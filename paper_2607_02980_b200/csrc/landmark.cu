@@ -379,7 +379,8 @@ int launch_landmark_summary(int dtype, int B, int Hkv, int Hl, int C, int d, int
             attr_once.done();
         }
         const unsigned blocks = static_cast<unsigned>(total < sm_count() ? total : sm_count());
-        // (launched so that a call's start overlaps the end of the kernel before it: 8 x 64K ragged tokens 125.2 -> 124.4 us)
+        // (launched so that a call's start overlaps the end of the kernel before it: calls of 4 x 1.7K tokens back to back 7.8 -> 7.2 us; 8 x 64K
+        // tokens take 125 either way, to 0.6 %)
         return launch_pdl(landmark_summary_tc_kernel, dim3(blocks), dim3(kTcWarps * 32), smem, stream, map_k, a) == cudaSuccess ? 1 : HILS_ERR_CUDA;
     }
     return dtype == HILS_F32 ? launch_typed<float>(a, d, stream) : launch_typed<__nv_bfloat16>(a, d, stream);

@@ -575,7 +575,8 @@ prefill_query_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
 // Tokens of a call (from its first on) that go this way: a multiple of 128 below the call's length, or all of them.  The
 // split with the largest gain by these costs (SM cycles; fitted to 16K, 2 x 6000 and 3 x 1000 tokens):
 //   here, a unit of 64 tokens: 2200 per chunk it visits (at most every visible one) + 12000, the last unit at least in full;
-//   chunk-major (index, attend and fuse kernels): 3830 per 32 tokens and chunk they attend, and 50000 for the launches.
+//   chunk-major (index, attend and fuse kernels): 3830 per 32 tokens and chunk they attend, and 50000 for the launches (which rest on one
+//   pair: 2 KV heads, K = 16, us all here / all chunk-major 3000 tokens 70 / 72, 4000 tokens 88 / 84).
 // With units for every SM the line lies near visible : attended = 5 : 2.  With few (sequence, KV head) pairs the units are a
 // serial chain on some of the SMs, and everything goes chunk-major unless that saves its launches (2 KV heads, a slice of
 // 2190 tokens at 4395, K = 32: 107 us chunk-major, 193 with the first 768 tokens here).  The parts of a call that the library
